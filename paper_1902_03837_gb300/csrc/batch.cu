@@ -10,9 +10,10 @@
 //   1. every problem's host set-up runs once (chi0_batch_create).  The
 //      problems of one system (one context at several q indices) share its
 //      coefficients and its mixed grids, computed once per system;
-//   2. the oscillator strengths of all problems run in ONE persistent launch
-//      over a device task table: blocks take the next (problem, k-pair, n,
-//      m-chunk) work item from a counter, so uneven problems balance;
+//   2. the oscillator strengths of all problems run in one persistent launch
+//      per grid size (the column transforms are compiled per size) over a
+//      device task table: blocks take the next (problem, k-pair, n, m-chunk)
+//      work item from a counter, so uneven problems balance;
 //   3. the remaining kernels of every problem (weights, operand split,
 //      contraction, reduction, Dyson) go on a few helper streams.  Problems
 //      are assigned to the streams longest first, each to the stream with the
@@ -56,11 +57,16 @@ struct chi0_batch {
   cudaGraphExec_t exec = nullptr;
   cudaStream_t capture_stream = nullptr;
   bool fp64 = false;
+  // the rho tasks in groups of one grid size (RhoGeom::nfft), each group one
+  // persistent launch with its own block counter
+  struct RhoGroup {
+    int nfft, first, count;
+    int64_t total;
+    size_t smem;
+  };
+  std::vector<RhoGroup> groups;
   DevBuf tasks, counter;
-  int ntasks = 0;
-  int64_t total_blocks = 0;
   int jm = 4;
-  size_t smem = 0;
   int nsm = 148;
   cudaStream_t last_stream = nullptr;  // stream of the last replay
   bool replayed = false;
@@ -74,12 +80,15 @@ std::map<std::string, int> g_tune;  // geometry key -> chosen m bands per block
 
 template <typename T, typename TOUT>
 chi0_status build_tasks(chi0_batch* b, int jm_max, std::vector<chi0::RhoTask<T, TOUT>>& tasks,
-                        size_t* smem, int64_t* total) {
+                        std::vector<chi0_batch::RhoGroup>& groups) {
   tasks.clear();
-  *smem = 0;
-  *total = 0;
-  for (chi0_ctx* c : b->items) {
-    if (c->nt == 0) continue;
+  groups.clear();
+  std::vector<chi0_ctx*> items;
+  for (chi0_ctx* c : b->items)
+    if (c->nt > 0) items.push_back(c);
+  std::stable_sort(items.begin(), items.end(),
+                   [](const chi0_ctx* x, const chi0_ctx* y) { return x->geom.nfft < y->geom.nfft; });
+  for (chi0_ctx* c : items) {
     chi0::RhoTask<T, TOUT> tk;
     size_t sm = 0;
     int64_t nb = 0;
@@ -89,42 +98,48 @@ chi0_status build_tasks(chi0_batch* b, int jm_max, std::vector<chi0::RhoTask<T, 
         (const typename chi0::C2<T>::t*)c->d_tw1.p, (const typename chi0::C2<T>::t*)c->d_tw2.p,
         (TOUT*)c->d_R.p, jm_max, &tk, &sm, &nb);
     if (e != cudaSuccess) return CHI0_EUNSUPPORTED;
-    tk.block0 = *total;
-    *total += nb;
-    *smem = std::max(*smem, sm);
+    if (groups.empty() || groups.back().nfft != c->geom.nfft)
+      groups.push_back({c->geom.nfft, (int)tasks.size(), 0, 0, 0});
+    chi0_batch::RhoGroup& g = groups.back();
+    tk.block0 = g.total;
+    g.total += nb;
+    g.smem = std::max(g.smem, sm);
+    ++g.count;
+    if (g.smem > 227 * 1024) return CHI0_EUNSUPPORTED;
     tasks.push_back(tk);
   }
-  if (*smem > 227 * 1024) return CHI0_EUNSUPPORTED;
   return CHI0_OK;
 }
 
 template <typename T, typename TOUT>
 chi0_status upload_tasks(chi0_batch* b, int jm) {
   std::vector<chi0::RhoTask<T, TOUT>> tasks;
-  size_t smem = 0;
-  int64_t total = 0;
-  chi0_status s = build_tasks<T, TOUT>(b, jm, tasks, &smem, &total);
+  std::vector<chi0_batch::RhoGroup> groups;
+  chi0_status s = build_tasks<T, TOUT>(b, jm, tasks, groups);
   if (s != CHI0_OK) return s;
   chi0_ctx* c0 = b->items[0];
   if ((s = chi0::ctx_ensure(c0, b->tasks, tasks.size() * sizeof(tasks[0]) + 16, "batch tasks")) != CHI0_OK) return s;
-  if ((s = chi0::ctx_ensure(c0, b->counter, 16, "batch counter")) != CHI0_OK) return s;
+  if ((s = chi0::ctx_ensure(c0, b->counter, groups.size() * 8, "batch counters")) != CHI0_OK) return s;
   if (!tasks.empty() &&
       cudaMemcpy(b->tasks.p, tasks.data(), tasks.size() * sizeof(tasks[0]), cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaGetLastError();
     return CHI0_ECUDA;
   }
-  b->ntasks = (int)tasks.size();
-  b->total_blocks = total;
+  b->groups = groups;
   b->jm = jm;
-  b->smem = smem;
   return CHI0_OK;
 }
 
 template <typename T, typename TOUT>
 cudaError_t launch_tasks(chi0_batch* b, cudaStream_t st) {
-  return chi0::launch_rho_batch<T, TOUT>((const chi0::RhoTask<T, TOUT>*)b->tasks.p, b->ntasks,
-                                         b->total_blocks, b->jm, b->smem,
-                                         (unsigned long long*)b->counter.p, b->nsm, st);
+  if (b->groups.empty()) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(b->counter.p, 0, b->groups.size() * 8, st);
+  for (size_t i = 0; i < b->groups.size() && e == cudaSuccess; ++i) {
+    const chi0_batch::RhoGroup& g = b->groups[i];
+    e = chi0::launch_rho_batch<T, TOUT>((const chi0::RhoTask<T, TOUT>*)b->tasks.p + g.first, g.count, g.total, g.nfft,
+                                        b->jm, g.smem, (unsigned long long*)b->counter.p + i, b->nsm, st);
+  }
+  return e;
 }
 
 cudaError_t launch_batched_rho(chi0_batch* b, cudaStream_t st) {
@@ -139,8 +154,8 @@ std::string tune_key(const chi0_batch* b) {
   std::string k = b->fp64 ? "f64" : "f32";
   for (const chi0_ctx* c : b->items) {
     const RhoGeom& g = c->geom;
-    char buf[160];
-    snprintf(buf, sizeof(buf), "|%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d", g.N1, g.N2, g.NZ, g.HX, g.HY, g.HZ,
+    char buf[176];
+    snprintf(buf, sizeof(buf), "|%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d", g.nfft, g.N1, g.N2, g.NZ, g.HX, g.HY, g.HZ,
              g.ng, g.nk, g.Nn, g.Nm, g.nb);
     k += buf;
   }
@@ -274,6 +289,18 @@ chi0_status chi0_batch_create(chi0_ctx* const* ctxs, const int* iqs, void* const
       b->items.push_back(c);
     }
   }
+  // the q points of one system share its grids: one size for all of them
+  for (int i = 0; i < n && s == CHI0_OK; ++i) s = chi0::plan_geometry(b->items[i], b->iqs[i]);
+  for (int pass = 0; pass < 2 && s == CHI0_OK; ++pass)
+    for (int i = 0; i < n && s == CHI0_OK; ++i) {
+      chi0_ctx* c = b->items[i];
+      for (int j = 0; j < n; ++j)
+        if (ctxs[j] == ctxs[i]) {
+          c->rho_need_floor = std::max(c->rho_need_floor, b->items[j]->rho_need);
+          c->rho_generic |= pass == 1 && b->items[j]->geom.nfft == 0;
+        }
+      if (pass == 0) s = chi0::plan_geometry(c, b->iqs[i]);
+    }
   // plan rho; the first problem of a system with transitions owns the mixed
   // grids, the system's other problems borrow them
   std::vector<chi0_ctx*> owner(n, nullptr);
@@ -438,7 +465,7 @@ chi0_status chi0_batch_run(chi0_batch* b, void* stream) {
     }
     join(0);
     if (s == CHI0_OK && launch_batched_rho(b, st) != cudaSuccess) s = CHI0_ECUDA;
-    if (!b->items.empty()) b->items[0]->launches += 1;
+    if (!b->items.empty()) b->items[0]->launches += (int64_t)b->groups.size();
     // the rest of every problem on its stream, in the planned order
     fork(b->evs[2 * ns + 1]);
     for (int i : b->order) {

@@ -199,17 +199,12 @@ chi0_status check_device_error(chi0_ctx* c) {
 
 namespace chi0 {
 
-chi0_status plan_rho(chi0_ctx* c, int iq) {
-  if (!c) return CHI0_EINVAL;
-  if (iq < 0 || iq >= c->cfg.nq) return fail(c, CHI0_EINVAL, "iq %d out of range", iq);
-  for (int ik = 0; ik < c->nk; ++ik)
-    if (!c->wf_set[ik]) return fail(c, CHI0_ESTATE, "wavefunctions of k %d not set", ik);
-  if (!c->energies_set) return fail(c, CHI0_ESTATE, "energies not set");
-  if (c->rho_planned_epoch == c->plan_epoch && c->plan_rho_iq == iq) {
-    c->rho_iq = c->chi_iq = c->eps_iq = -1;   // the plan holds; the results are stale
-    return CHI0_OK;
-  }
-  chi0_status s;
+constexpr int kBgChunk = 4096;   // difference vectors per launch of the extrapolar densities
+
+// Host set-up of a q point: response set, k-pairs, transition block, extents
+// and the smallest alias-free grid (rho_need), which is what batch.cu needs of
+// every q point before it shares one system's grids between them.
+chi0_status plan_geometry(chi0_ctx* c, int iq) {
   // ---- q-point setup on the host
   response_set(c, iq, c->h_gresp);
   kpairs(c, iq, c->h_kq, c->h_g0);
@@ -281,7 +276,10 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
     if (A[2] != B[2]) return A[2] < B[2];
     return A[0] < B[0];
   });
-  // the real-space product must not alias onto the response set
+  // the real-space product must not alias onto the response set,
+  // and a column transform holds frequencies of [-n/2, n/2) only; the
+  // extrapolar correction's densities reach the differences of the set
+  int need = 0;
   for (int d = 0; d < 3; ++d) {
     const int n = c->cfg.fft[d];
     const int hmax = std::max(std::abs(lo[d]), std::abs(hi[d])) + g0max;
@@ -289,7 +287,45 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
       return fail(c, CHI0_EINVAL,
                   "fft[%d] = %d aliases: need > 2*%d + %d for these spheres and response set", d,
                   n, L[d], hmax);
+    const int reach = c->bg_on ? std::max(hmax, hi[d] - lo[d]) : hmax;
+    need = std::max({need, 2 * L[d] + reach + 1, 2 * reach + 1});
   }
+  c->rho_need = std::max(need, c->rho_need_floor);
+  // rho does not depend on the grid as long as it is alias free: take the
+  // smallest cubic one the column transforms know (rho_fft.cuh), and the
+  // caller's grid where that does not reach
+  chi0::rho_fft_tables(c->h_gresp.data(), g, c->h_rows, c->h_lut);
+  if (!c->rho_generic)
+    g.nfft = c->fp64 ? chi0::rho_fft_size<double>(g, c->rho_need) : chi0::rho_fft_size<float>(g, c->rho_need);
+  if (g.nfft && c->bg_on) {   // the difference set's chunks go through the same kernel
+    RhoGeom gd = g;
+    gd.HX = 2 * (hi[0] - lo[0]) + 1;
+    gd.HY = 2 * (hi[1] - lo[1]) + 1;
+    gd.HZ = 2 * (hi[2] - lo[2]) + 1;
+    gd.npair = gd.HY * gd.HZ;
+    gd.ng = kBgChunk;
+    const int n = c->fp64 ? chi0::rho_fft_size<double>(gd, c->rho_need) : chi0::rho_fft_size<float>(gd, c->rho_need);
+    if (n == 0) g.nfft = 0;
+  }
+  if (g.nfft) g.N1 = g.N2 = g.N3 = g.nfft;
+  return CHI0_OK;
+}
+
+chi0_status plan_rho(chi0_ctx* c, int iq) {
+  if (!c) return CHI0_EINVAL;
+  if (iq < 0 || iq >= c->cfg.nq) return fail(c, CHI0_EINVAL, "iq %d out of range", iq);
+  for (int ik = 0; ik < c->nk; ++ik)
+    if (!c->wf_set[ik]) return fail(c, CHI0_ESTATE, "wavefunctions of k %d not set", ik);
+  if (!c->energies_set) return fail(c, CHI0_ESTATE, "energies not set");
+  if (c->rho_planned_epoch == c->plan_epoch && c->plan_rho_iq == iq) {
+    c->rho_iq = c->chi_iq = c->eps_iq = -1;   // the plan holds; the results are stale
+    return CHI0_OK;
+  }
+  chi0_status s;
+  if ((s = plan_geometry(c, iq)) != CHI0_OK) return s;
+  RhoGeom& g = c->geom;
+  const std::vector<int32_t>& rows = c->h_rows;
+  const std::vector<int16_t>& lut = c->h_lut;
   const bool streamed = c->stream_nb > 0;
   if (streamed) {
     if (c->bg_on || c->term_params || c->grp_thresh > 0.0)
@@ -308,7 +344,7 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
   }
   // ---- device buffers
   const size_t cb = cplx_bytes(c);
-  const size_t plane_bytes = (size_t)g.N1 * g.NZ * g.N2 * cb;
+  const size_t plane_bytes = chi0::rho_volume(g) * cb;
   // streamed: the m-band grids of every k (resident) and one block's n grids
   const size_t ubytes = streamed ? (size_t)c->nk * c->Nm * plane_bytes : (size_t)c->nk * c->nb * plane_bytes;
   if ((s = ensure(c, c->d_U, ubytes, "mixed-grid wavefunctions")) != CHI0_OK) return s;
@@ -318,11 +354,17 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
   if ((s = ensure(c, c->d_R, (size_t)(streamed ? c->nt_blk : c->nt) * g.ng * cb, "rho")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_gresp, (size_t)g.ng * 12, "G set")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_gperm, (size_t)g.ng * 4, "G order")) != CHI0_OK) return s;
+  const size_t rows_bytes = (rows.size() * 4 + 15) / 16 * 16;
+  if ((s = ensure(c, c->d_rtab, rows_bytes + lut.size() * 2, "response tables")) != CHI0_OK) return s;
+  g.rows = (const int32_t*)c->d_rtab.p;
+  g.lut = (const int16_t*)((const char*)c->d_rtab.p + rows_bytes);
   if ((s = ensure(c, c->d_kq, (size_t)c->nk * 4, "k pairs")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_g0, (size_t)c->nk * 12, "umklapp")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_tw1, (size_t)g.N1 * cb, "twiddles")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_tw2, (size_t)g.N2 * cb, "twiddles")) != CHI0_OK) return s;
   CK(cudaMemcpyAsync(c->d_gresp.p, c->h_gresp.data(), (size_t)g.ng * 12, cudaMemcpyHostToDevice, c->st), "G set H2D");
+  CK(cudaMemcpyAsync((void*)g.rows, rows.data(), rows.size() * 4, cudaMemcpyHostToDevice, c->st), "rows H2D");
+  CK(cudaMemcpyAsync((void*)g.lut, lut.data(), lut.size() * 2, cudaMemcpyHostToDevice, c->st), "lut H2D");
   CK(cudaMemcpyAsync(c->d_kq.p, c->h_kq.data(), (size_t)c->nk * 4, cudaMemcpyHostToDevice, c->st), "kq H2D");
   CK(cudaMemcpyAsync(c->d_gperm.p, c->h_gperm.data(), (size_t)g.ng * 4, cudaMemcpyHostToDevice, c->st), "G order H2D");
   CK(cudaMemcpyAsync(c->d_g0.p, c->h_g0.data(), (size_t)c->nk * 12, cudaMemcpyHostToDevice, c->st), "g0 H2D");
@@ -351,17 +393,24 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
     a1.bytes = (double)c->nk * c->nb * ((double)c->npw_max * (cb + 12) + ubytes / ((double)c->nk * c->nb));
     a1.flops = 8.0 * (double)c->nk * c->nb * g.NZ *
                ((double)g.NX * g.N2 * g.NY + (double)g.N1 * g.N2 * g.NX);
-    // rho: every transition reads two N1 x NZ x N2 mixed grids and writes ng values;
-    // executed work per transition and x plane: the z correlation (N2 HZ NZ
-    // complex multiply-adds), the pruned y transform (HY HZ N2 / 4 multiply-adds
-    // plus 6 HZ N2 flops of radix-4 butterflies when N2 % 4 == 0, else HY HZ N2
-    // multiply-adds), the x accumulation (ng multiply-adds)
+    // rho: the grids read once and ng values written per transition; executed
+    // work of the mixed-grid kernel per transition and x plane: the z
+    // correlation (N2 HZ NZ complex multiply-adds), the pruned y transform
+    // (HY HZ N2 / 4 multiply-adds plus 6 HZ N2 flops of radix-4 butterflies
+    // when N2 % 4 == 0, else HY HZ N2 multiply-adds), the x accumulation (ng
+    // multiply-adds)
     auto& a2 = c->stage[CHI0_STAGE_RHO];
     a2.bytes = (double)c->nt * g.ng * cb + (double)ubytes;
     const double ywork = (g.N2 % 4 == 0) ? 8.0 * g.HY * g.HZ * (g.N2 / 4) + 6.0 * g.HZ * g.N2
                                          : 8.0 * g.HY * g.HZ * g.N2;
     a2.flops = (double)c->nt * g.N1 *
                (8.0 * g.N2 * g.HZ * g.NZ + ywork + 8.0 * g.ng);
+    if (g.nfft) {
+      // column transforms at 5 N log2 N flops, and the products
+      const double n = g.nfft, col = 5.0 * n * std::log2(n);
+      a1.flops = (double)c->nk * c->nb * col * ((double)g.NY * g.NZ + n * g.NZ + n * n);
+      a2.flops = (double)c->nt * (6.0 * n * n * n + col * (n * n + n * g.HZ + g.npair));
+    }
   }
   c->rho_planned_epoch = c->plan_epoch;
   ++c->rho_plan_serial;
@@ -412,7 +461,7 @@ chi0_status launch_rho_pipelined(chi0_ctx* c) {
     need[ch] = std::max(need[ch], std::max(ch, chunk_of(c->h_kq[k])));
   }
   const RhoGeom& g0 = c->geom;
-  const size_t band = (size_t)g0.N1 * g0.NZ * g0.N2;   // complex entries of one band's mixed grid
+  const size_t band = chi0::rho_volume(g0);   // complex entries of one state on the grid
   const size_t cbytes = cplx_bytes(c);
   for (int w = 0; w < nch; ++w) {
     const int k0 = w * per, k1 = std::min(nk, k0 + per);
@@ -457,7 +506,12 @@ chi0_status launch_rho_pipelined(chi0_ctx* c) {
 chi0_status launch_rho(chi0_ctx* c, bool with_pairs) {
   const int iq = c->plan_rho_iq;
   if (iq < 0) return fail(c, CHI0_ESTATE, "rho not planned");
-  if (with_pairs && c->nt > 0 && !c->grid_shared && c->stream_nb == 0 && c->nk >= 2 * kWfChunks) {
+  // in chunks only while coefficient copies that no earlier call waited for
+  // are in flight: eight partial launches of each kernel leave the GPU partly
+  // idle eight times
+  const bool uploading = c->up_count != c->up_taken;
+  c->up_taken = c->up_count;
+  if (uploading && with_pairs && c->nt > 0 && !c->grid_shared && c->stream_nb == 0 && c->nk >= 2 * kWfChunks) {
     chi0_status s = launch_rho_pipelined(c);
     if (s != CHI0_OK) return s;
     c->rho_iq = iq;
@@ -582,7 +636,7 @@ chi0_status plan_bg(chi0_ctx* c) {
                   "fft[%d] = %d aliases for the extrapolar densities: need > 2*%d + %d", a,
                   c->cfg.fft[a], L, dmax);
   }
-  constexpr int kChunk = 4096;
+  constexpr int kChunk = kBgChunk;
   const int nch = (nd + kChunk - 1) / kChunk;
   if (nch > chi0::kBgMaxChunks)
     return fail(c, CHI0_EUNSUPPORTED, "%d difference vectors: more than %d chunks", nd, chi0::kBgMaxChunks);
@@ -590,6 +644,9 @@ chi0_status plan_bg(chi0_ctx* c) {
   chi0::BgChunks ch{};
   ch.n = nch;
   c->bg_geom.assign(nch, g);
+  std::vector<std::vector<int32_t>> rows(nch);
+  std::vector<std::vector<int16_t>> luts(nch);
+  std::vector<size_t> taboff(nch + 1, 0);
   for (int k = 0; k < nch; ++k) {
     const int a0 = k * kChunk, a1 = std::min(nd, a0 + kChunk);
     ch.start[k] = a0;
@@ -615,6 +672,8 @@ chi0_status plan_bg(chi0_ctx* c) {
     gc.g0max = 0;
     gc.g0z_min = 0;
     gc.g0z_max = 0;
+    chi0::rho_fft_tables(D[a0].data(), gc, rows[k], luts[k]);
+    taboff[k + 1] = taboff[k] + (rows[k].size() * 4 + luts[k].size() * 2 + 15) / 16 * 16;
   }
   ch.start[nch] = nd;
   // extrapolar weights wbar[iw][k * Nm + m] (same pole form as the weights kernel)
@@ -639,6 +698,15 @@ chi0_status plan_bg(chi0_ctx* c) {
   const size_t cb = cplx_bytes(c);
   if ((s = ensure(c, c->d_bgd, dflat.size() * 4, "difference vectors")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_bgperm, ident.size() * 4, "difference order")) != CHI0_OK) return s;
+  if ((s = ensure(c, c->d_bgtab, taboff[nch], "difference tables")) != CHI0_OK) return s;
+  for (int k = 0; k < nch; ++k) {
+    char* tab = (char*)c->d_bgtab.p + taboff[k];
+    c->bg_geom[k].rows = (const int32_t*)tab;
+    c->bg_geom[k].lut = (const int16_t*)(tab + rows[k].size() * 4);
+    CK(cudaMemcpyAsync(tab, rows[k].data(), rows[k].size() * 4, cudaMemcpyHostToDevice, c->st), "rows H2D");
+    CK(cudaMemcpyAsync(tab + rows[k].size() * 4, luts[k].data(), luts[k].size() * 2, cudaMemcpyHostToDevice, c->st),
+       "lut H2D");
+  }
   if ((s = ensure(c, c->d_bgkq, kid.size() * 4, "k map")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_bgg0, zero.size() * 4, "zero umklapp")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_bgrd, (size_t)ntd * nd * cb, "diagonal densities")) != CHI0_OK) return s;
@@ -1860,7 +1928,7 @@ void chi0_destroy(chi0_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->st);
   DevBuf* bufs[] = {&c->d_gvec, &c->d_npw, &c->d_coef, &c->d_eps, &c->d_occ, &c->d_stage,
-                    &c->d_gresp, &c->d_gperm, &c->d_kq, &c->d_g0, &c->d_tw1, &c->d_tw2, &c->d_U, &c->d_R,
+                    &c->d_gresp, &c->d_gperm, &c->d_rtab, &c->d_bgtab, &c->d_kq, &c->d_g0, &c->d_tw1, &c->d_tw2, &c->d_U, &c->d_R,
                     &c->d_w, &c->d_part, &c->d_chi, &c->d_A, &c->d_colp, &c->d_rowp, &c->d_pinv,
                     &c->d_err, &c->d_vsqrt, &c->d_omim, &c->d_tc, &c->d_termx, &c->d_termy,
                     &c->d_termq, &c->d_termw, &c->d_termc, &c->d_bgd, &c->d_bgperm, &c->d_bgkq,

@@ -70,7 +70,14 @@ struct chi0_ctx {
   int n_lo = 0, Nn = 0, Nm = 0;
   int64_t nt = 0;
   RhoGeom geom{};
-  DevBuf d_gresp, d_gperm, d_kq, d_g0, d_tw1, d_tw2, d_U, d_R, d_w, d_part, d_chi, d_A, d_colp, d_rowp,
+  // grid of the states (RhoGeom::nfft): points per axis that the q point
+  // needs; a batch sets the floor to what every q point of a system needs, so
+  // that they share one grid, and rho_generic where one of them has none
+  int rho_need = 0, rho_need_floor = 0;
+  bool rho_generic = false;
+  std::vector<int32_t> h_rows;
+  std::vector<int16_t> h_lut;
+  DevBuf d_gresp, d_gperm, d_rtab, d_kq, d_g0, d_tw1, d_tw2, d_U, d_R, d_w, d_part, d_chi, d_A, d_colp, d_rowp,
       d_pinv, d_err, d_vsqrt, d_omim, d_tc;
   int nchunks = 1, kchunk = 0;
   void* tc = nullptr;  // tensor-core path state (tc.cu)
@@ -95,7 +102,7 @@ struct chi0_ctx {
   int64_t bg_ntd = 0;                  // states (k, m < Nm) with diagonal densities
   std::vector<RhoGeom> bg_geom;        // rho geometry of each chunk of the difference set
   chi0::BgChunks bg_ch{};
-  DevBuf d_bgd, d_bgperm, d_bgkq, d_bgg0, d_bgrd, d_bgw, d_bgP, d_bgidx;
+  DevBuf d_bgd, d_bgperm, d_bgtab, d_bgkq, d_bgg0, d_bgrd, d_bgw, d_bgP, d_bgidx;
   // degenerate-pole grouping (Appendix B) and the double-grid frequency factor
   double grp_thresh = 0.0;             // Ha; 0: every pole its own factor
   DevBuf d_dpole;                      // [nt] pole energy of each transition's group representative
@@ -150,7 +157,7 @@ struct chi0_ctx {
   cudaStream_t s_up = nullptr;
   std::vector<cudaEvent_t> ev_up;
   std::vector<int64_t> up_seq;
-  int64_t up_count = 0;
+  int64_t up_count = 0, up_taken = 0;   // copies queued; those that a compute_rho has waited for
   cudaEvent_t ev_wf_done = nullptr;
   cudaEvent_t ev_join_dy2 = nullptr;
   std::vector<cudaEvent_t> ev_freq;  // [nw] contraction (and reduction) of frequency w done
@@ -219,6 +226,7 @@ std::vector<DevBuf*> tc_scratch_slots(chi0_ctx* c);
 chi0_status tc_tune_split(chi0_ctx* c, float* best_ms);
 // plan (host set-up, allocation, uploads; may synchronise) and launch
 // (kernels only, capturable) halves of compute_rho / build_chi0 / invert_eps
+chi0_status plan_geometry(chi0_ctx* c, int iq);
 chi0_status plan_rho(chi0_ctx* c, int iq);
 chi0_status launch_rho(chi0_ctx* c, bool with_pairs);
 chi0_status plan_chi0(chi0_ctx* c, int iq);

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace chi0 {
 
 template <typename T> struct C2;
@@ -37,7 +39,20 @@ struct RhoGeom {
   // local k whose first band is bu0; the m grids in an array of nbm bands per
   // (global) k, separate from the n grids when the task's Um is set.
   int k0, nbu, bu0, nbm;
+  // > 0: the states are in real space on the nfft^3 grid, U[x][z][y], and rho
+  // goes through the column transforms of rho_fft.cuh (N1 = N2 = N3 = nfft);
+  // 0: mixed grids and the kernels of rho.cu.  rows / lut (device): the
+  // (y, z) pairs that hold response vectors and the vectors of each pair
+  // (rho_fft_tables).
+  int nfft, npair;
+  const int32_t* rows;
+  const int16_t* lut;
 };
+
+// Complex entries of one state on the grid.
+inline size_t rho_volume(const RhoGeom& g) {
+  return g.nfft ? (size_t)g.nfft * g.nfft * g.nfft : (size_t)g.N1 * g.NZ * g.N2;
+}
 
 // Zero padding of the n plane in the rho kernel's shared memory.
 struct RhoSmem {
@@ -60,10 +75,21 @@ struct RhoTask {
   const typename C2<T>::t* tw2;
   TOUT* R;
   int jm;          // m bands per block (<= the kernel's JM)
+  int xc;          // x planes per pass (column transforms only)
   int64_t block0;  // first global block of this task in a batched launch
 };
 
 // ---- launchers (stream-ordered; return cudaGetLastError()) ----
+
+// Smallest grid the column transforms take that has at least `need` points
+// per axis and whose work fits a block's shared memory; 0: none.  g: the
+// extents (L, H), ng and npair of the problem.
+template <typename T>
+int rho_fft_size(const RhoGeom& g, int need);
+// Tables of a response set (gset[ng][3], host) with the extents in g: sets
+// g.npair; rows[HZ] = first pair << 16 | first hy << 8 | number of hy;
+// lut[hx][pair] = response index or -1.
+void rho_fft_tables(const int32_t* gset, RhoGeom& g, std::vector<int32_t>& rows, std::vector<int16_t>& lut);
 
 // a1: sphere -> mixed grid U[k][band][x][gz][y] for every k and band, or
 // (nkr > 0) for the k points k0 .. k0 + nkr - 1 and bands b0 .. b0 + nbo - 1
@@ -92,11 +118,25 @@ cudaError_t rho_task_make(const RhoGeom& g, const typename C2<T>::t* U, const in
                           const typename C2<T>::t* tw1, const typename C2<T>::t* tw2, TOUT* R,
                           int jm_max, RhoTask<T, TOUT>* tk, size_t* smem, int64_t* nblocks);
 
-// Persistent rho over many tasks in one launch (tasks_dev: device array with
-// block0 prefix offsets; total: all blocks; counter: device scratch).
+// Persistent rho over many tasks of one nfft in one launch (tasks_dev: device
+// array with block0 prefix offsets; total: all blocks; counter: device
+// scratch, zero when the launch starts).
 template <typename T, typename TOUT>
-cudaError_t launch_rho_batch(const RhoTask<T, TOUT>* tasks_dev, int ntasks, int64_t total, int jm,
+cudaError_t launch_rho_batch(const RhoTask<T, TOUT>* tasks_dev, int ntasks, int64_t total, int nfft, int jm,
                              size_t smem, unsigned long long* counter, int nsm, cudaStream_t s);
+
+// Kernels of rho_fft.cuh by grid size (rho_fft32.cu, rho_fft64.cu).
+namespace rfft {
+template <typename T>
+cudaError_t wf_dispatch(const RhoGeom& g, const int32_t* gvec, const int32_t* npw, const typename C2<T>::t* coef,
+                        typename C2<T>::t* U, cudaStream_t s, int k0, int nkr, int b0, int nbo);
+template <typename T>
+cudaError_t rho_dispatch(const RhoTask<T, typename C2<T>::t>& tk, size_t smem, int threads, int64_t nblocks,
+                         cudaStream_t s);
+template <typename T>
+cudaError_t batch_dispatch(int nfft, const RhoTask<T, typename C2<T>::t>* tasks, int ntasks, int64_t total,
+                           size_t smem, unsigned long long* counter, int nsm, cudaStream_t s);
+}  // namespace rfft
 
 // a3: real transition weights w[iw][t] (FP64).
 // With bg != 0 each weight is reduced by the extrapolar weight of its m

@@ -21,6 +21,12 @@
 // and JM m bands, streams the x planes of the two mixed grids through shared
 // memory and accumulates rho for all its transitions in registers, so the
 // large intermediate of a staged FFT never reaches HBM.
+//
+// These kernels serve the grids that the column transforms of rho_fft.cuh do
+// not reach (more than 36 points per axis needed, or a sphere whose box does
+// not fit a block's shared memory); every other problem goes there.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace chi0 {
@@ -685,8 +691,6 @@ cudaError_t launch_wf_to_mixed(const RhoGeom& g, const int32_t* gvec, const int3
                                const typename C2<T>::t* tw2, typename C2<T>::t* U,
                                cudaStream_t s, int k0, int nkr, int b0, int nbo) {
   using T2 = typename C2<T>::t;
-  const size_t smem = ((size_t)g.NZ * g.NX * g.NY + (size_t)g.NX * g.N2) * sizeof(T2);
-  if (smem > 227 * 1024) return cudaErrorInvalidValue;
   if (nkr <= 0) {  // every k and band
     k0 = 0;
     nkr = g.nk;
@@ -694,6 +698,9 @@ cudaError_t launch_wf_to_mixed(const RhoGeom& g, const int32_t* gvec, const int3
     nbo = g.nb;
   }
   if (k0 < 0 || b0 < 0 || nbo <= 0 || k0 + nkr > g.nk || b0 + nbo > g.nb) return cudaErrorInvalidValue;
+  if (g.nfft) return rfft::wf_dispatch<T>(g, gvec, npw, coef, U, s, k0, nkr, b0, nbo);
+  const size_t smem = ((size_t)g.NZ * g.NX * g.NY + (size_t)g.NX * g.N2) * sizeof(T2);
+  if (smem > 227 * 1024) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(k_wf_to_mixed<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
@@ -711,13 +718,98 @@ static cudaError_t launch_rho_jm(const RhoTask<T, TOUT>& tk, size_t smem, int64_
   return cudaGetLastError();
 }
 
+// ---- column transforms (rho_fft.cuh): sizes and shared memory
+
+static constexpr int kRhoFftSizes[] = {8, 10, 12, 15, 16, 18, 20, 24, 30, 32, 36};
+static constexpr size_t kRhoFftTwo = 104 << 10;   // two blocks on an SM, and some L1 for the states
+static constexpr size_t kRhoFftOne = 227 << 10;
+
+// Planes per pass and shared memory of a block of jm transitions; false: does
+// not fit.  A pass holds jm HZ (N | 1) values per plane; as many planes as two
+// blocks on an SM allow, in passes of equal size.
+static bool rho_fft_fit(const RhoGeom& g, int n, int jm, size_t cb, int* xc, size_t* smem) {
+  const size_t xb = (size_t)jm * n * g.npair * cb, row = (size_t)jm * g.ng * cb;
+  const size_t per = (size_t)jm * g.HZ * (n | 1) * cb;
+  const size_t lim = xb + std::max(row, 2 * per) <= kRhoFftTwo ? kRhoFftTwo : kRhoFftOne;
+  if (xb + std::max(row, per) > lim) return false;
+  const int fit = (int)std::min<size_t>(n, (lim - xb) / per);
+  const int passes = (n + fit - 1) / fit;
+  *xc = (n + passes - 1) / passes;
+  *smem = xb + std::max(row, *xc * per);
+  return true;
+}
+
+template <typename T>
+int rho_fft_size(const RhoGeom& g, int need) {
+  for (int n : kRhoFftSizes) {
+    if (n < need) continue;
+    int xc;
+    size_t smem;
+    const size_t cb = sizeof(typename C2<T>::t);
+    const bool wf = ((size_t)n * g.NY * g.NZ + (size_t)n * g.NZ) * cb <= kRhoFftOne;
+    return wf && g.npair <= 32767 && g.HX < 256 && g.HY < 256 && rho_fft_fit(g, n, 1, cb, &xc, &smem) ? n : 0;
+  }
+  return 0;
+}
+
+void rho_fft_tables(const int32_t* gset, RhoGeom& g, std::vector<int32_t>& rows, std::vector<int16_t>& lut) {
+  std::vector<int> lo(g.HZ, g.HY), hi(g.HZ, -1);
+  for (int i = 0; i < g.ng; ++i) {
+    const int y = gset[3 * i + 1] - g.My_lo, z = gset[3 * i + 2] - g.Mz_lo;
+    lo[z] = std::min(lo[z], y);
+    hi[z] = std::max(hi[z], y);
+  }
+  std::vector<int> first(g.HZ);
+  rows.assign(g.HZ, 0);
+  g.npair = 0;
+  for (int z = 0; z < g.HZ; ++z) {
+    const int cnt = std::max(0, hi[z] - lo[z] + 1);
+    first[z] = g.npair;
+    if (cnt > 0) rows[z] = g.npair << 16 | (lo[z] & 0xff) << 8 | (cnt & 0xff);
+    g.npair += cnt;
+  }
+  lut.assign((size_t)g.HX * g.npair, -1);
+  for (int i = 0; i < g.ng; ++i) {
+    const int x = gset[3 * i] - g.Mx_lo, y = gset[3 * i + 1] - g.My_lo, z = gset[3 * i + 2] - g.Mz_lo;
+    lut[(size_t)x * g.npair + first[z] + y - lo[z]] = (int16_t)i;
+  }
+}
+
+// Threads of a block: the count that leaves the fewest idle lanes over the
+// z, y and x columns of a block (the z columns carry the loads and products).
+static int rho_fft_threads(const RhoGeom& g, int jm, int xc) {
+  int best = 256;
+  double best_cost = 1e30;
+  for (int t : {256, 224, 192, 160, 128}) {
+    double c = 0.0;
+    for (int x0 = 0; x0 < g.nfft; x0 += xc) {
+      const int nx = std::min(xc, g.nfft - x0);
+      c += 1.4 * jm * ((nx * g.nfft + t - 1) / t) + (jm * nx * g.HZ + t - 1) / t;
+    }
+    c = (c + (jm * g.npair + t - 1) / t) * t;
+    if (c < best_cost) {
+      best_cost = c;
+      best = t;
+    }
+  }
+  return best;
+}
+
 template <typename T, typename TOUT>
 cudaError_t rho_task_make(const RhoGeom& g, const typename C2<T>::t* U, const int32_t* kq,
                           const int32_t* g0, const int32_t* gresp, const int32_t* gperm,
                           const typename C2<T>::t* tw1, const typename C2<T>::t* tw2, TOUT* R,
                           int jm_max, RhoTask<T, TOUT>* tk, size_t* smem, int64_t* nblocks) {
   if (g.Nn > 65535 || g.HX >= 32768 || g.HY * g.HZ >= 65536) return cudaErrorInvalidValue;
-  RhoSmem sm;
+  RhoSmem sm{};
+  if (g.nfft) {
+    int jm = jm_max, xc = 1;
+    while (jm > 1 && (jm > g.Nm || !rho_fft_fit(g, g.nfft, jm, sizeof(TOUT), &xc, smem))) jm /= 2;
+    if (!rho_fft_fit(g, g.nfft, jm, sizeof(TOUT), &xc, smem)) return cudaErrorInvalidValue;
+    *tk = RhoTask<T, TOUT>{g, sm, U, nullptr, kq, g0, gresp, gperm, tw1, tw2, R, jm, xc, 0};
+    *nblocks = (int64_t)g.nk * g.Nn * ((g.Nm + jm - 1) / jm);
+    return cudaSuccess;
+  }
   // rows of the zero-padded n plane: row = padz + hz + b, b in [0, NZ), hz over
   // every tile of every k-pair: [Mz_lo - G0z_max, Mz_lo + nhb * kHZT - 1 - G0z_min]
   const int nhb = (g.HZ + kHZT - 1) / kHZT;
@@ -754,6 +846,21 @@ cudaError_t launch_rho_pairs(const RhoGeom& g, const typename C2<T>::t* U, const
                              const typename C2<T>::t* tw1, const typename C2<T>::t* tw2, TOUT* R,
                              cudaStream_t s, const typename C2<T>::t* Um) {
   if (g.Nn <= 0 || g.Nm <= 0 || g.nk <= 0) return cudaSuccess;
+  if (g.nfft) {
+    // the most m bands per block (they share the n columns) that still leave
+    // room for two blocks on an SM and four blocks for every SM
+    RhoTask<T, TOUT> tk;
+    size_t smem = 0;
+    int64_t nb = 0;
+    for (int jm : {4, 2, 1}) {
+      const cudaError_t e = rho_task_make<T, TOUT>(g, U, kq, g0, gresp, gperm, tw1, tw2, R, jm, &tk, &smem, &nb);
+      if (e != cudaSuccess) return e;
+      if (tk.jm == jm && smem <= kRhoFftTwo && nb >= 4 * 152) break;
+    }
+    tk.Um = Um;
+    if (nb > 0x7fffffff) return cudaErrorInvalidValue;
+    return rfft::rho_dispatch<T>(tk, smem, rho_fft_threads(g, tk.jm, tk.xc), nb, s);
+  }
   for (int jm : {4, 2, 1}) {
     RhoTask<T, TOUT> tk;
     size_t smem = 0;
@@ -772,14 +879,12 @@ cudaError_t launch_rho_pairs(const RhoGeom& g, const typename C2<T>::t* U, const
 }
 
 template <typename T, typename TOUT>
-cudaError_t launch_rho_batch(const RhoTask<T, TOUT>* tasks_dev, int ntasks, int64_t total, int jm,
+cudaError_t launch_rho_batch(const RhoTask<T, TOUT>* tasks_dev, int ntasks, int64_t total, int nfft, int jm,
                              size_t smem, unsigned long long* counter, int nsm, cudaStream_t s) {
   if (ntasks == 0 || total == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
-  int per_sm = 1;
+  if (nfft) return rfft::batch_dispatch<T>(nfft, tasks_dev, ntasks, total, smem, counter, nsm, s);
+  cudaError_t e = cudaSuccess;
   const int grid = nsm * 2;
-  (void)per_sm;
   switch (jm) {
     case 4:
       e = cudaFuncSetAttribute(k_rho_batch<T, 4, TOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -799,6 +904,8 @@ cudaError_t launch_rho_batch(const RhoTask<T, TOUT>* tasks_dev, int ntasks, int6
   return cudaGetLastError();
 }
 
+template int rho_fft_size<double>(const RhoGeom&, int);
+template int rho_fft_size<float>(const RhoGeom&, int);
 template cudaError_t launch_wf_to_mixed<double>(const RhoGeom&, const int32_t*, const int32_t*,
                                                 const double2*, const double2*, const double2*,
                                                 double2*, cudaStream_t, int, int, int, int);
@@ -813,9 +920,9 @@ template cudaError_t rho_task_make<float, float2>(const RhoGeom&, const float2*,
                                                   const int32_t*, const int32_t*, const int32_t*,
                                                   const float2*, const float2*, float2*, int,
                                                   RhoTask<float, float2>*, size_t*, int64_t*);
-template cudaError_t launch_rho_batch<double, double2>(const RhoTask<double, double2>*, int, int64_t, int,
+template cudaError_t launch_rho_batch<double, double2>(const RhoTask<double, double2>*, int, int64_t, int, int,
                                                        size_t, unsigned long long*, int, cudaStream_t);
-template cudaError_t launch_rho_batch<float, float2>(const RhoTask<float, float2>*, int, int64_t, int,
+template cudaError_t launch_rho_batch<float, float2>(const RhoTask<float, float2>*, int, int64_t, int, int,
                                                      size_t, unsigned long long*, int, cudaStream_t);
 template cudaError_t launch_rho_pairs<double, double2>(const RhoGeom&, const double2*,
                                                        const int32_t*, const int32_t*,
