@@ -1122,9 +1122,9 @@ chi0_status plan_eps(chi0_ctx* c, int iq, double2* A) {
   const int nw = c->cfg.nw, ng = c->cfg.ng;
   chi0_status s;
   if ((s = ensure(c, c->d_vsqrt, (size_t)ng * 8, "coulomb")) != CHI0_OK) return s;
-  if ((s = ensure(c, c->d_colp, (size_t)nw * ng * 32 * 16, "panels")) != CHI0_OK) return s;
-  if ((s = ensure(c, c->d_rowp, (size_t)nw * ng * 32 * 16, "panels")) != CHI0_OK) return s;
-  if ((s = ensure(c, c->d_pinv, (size_t)nw * 32 * 32 * 16, "pivot blocks")) != CHI0_OK) return s;
+  if ((s = ensure(c, c->d_colp, (size_t)nw * ng * 16 * 16, "panels")) != CHI0_OK) return s;
+  if ((s = ensure(c, c->d_rowp, (size_t)nw * ng * 16 * 16, "panels")) != CHI0_OK) return s;
+  if ((s = ensure(c, c->d_pinv, (size_t)nw * 512 * 16, "pivot blocks")) != CHI0_OK) return s;
   std::vector<double> v(ng);
   int64_t qi[3];
   q_integers(c, iq, qi);
@@ -1191,7 +1191,7 @@ chi0_status launch_eps(chi0_ctx* c) {
         : chi0::launch_dyson(chi, (const double*)c->d_vsqrt.p, ng, i1 - i0, out, (double2*)c->d_colp.p,
                              (double2*)c->d_rowp.p, (double2*)c->d_pinv.p, (int*)c->d_err.p, c->st);
     if (e != cudaSuccess) return cuda_fail(c, e, "dyson launch");
-    nlaunch += (general ? 1 : 2) + 3 * ((ng + 31) / 32);
+    nlaunch += chi0::dyson_launches(ng);
     i0 = i1;
   }
   chi0::stage_end(c, CHI0_STAGE_DYSON, nlaunch);
@@ -1234,7 +1234,6 @@ chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
   // own panel scratch (the group's slice of the per-frequency buffers), so
   // that the pivot-block inverses of one group (one SM per matrix) overlap
   // the rank-32 updates of the other.
-  const int nT = (ng + 31) / 32;
   int grp = 0;
   auto general = [&](int iw) { return c->has_real && c->h_vi[iw] >= 0; };
   auto first_v = [&](int iw) { return c->has_real ? c->h_vr[iw] : iw; };   // list entries of frequency iw
@@ -1265,15 +1264,15 @@ chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
     chi0::stage_begin(c, CHI0_STAGE_DYSON);
     const double2* chi = (const double2*)c->d_chi.p + w0 * n2;
     double2* out = c->plan_eps_out + w0 * n2;
-    double2* colp = (double2*)c->d_colp.p + (size_t)w0 * ng * 32;
-    double2* rowp = (double2*)c->d_rowp.p + (size_t)w0 * ng * 32;
-    double2* pinv = (double2*)c->d_pinv.p + (size_t)w0 * 32 * 32;
+    double2* colp = (double2*)c->d_colp.p + (size_t)w0 * ng * 16;
+    double2* rowp = (double2*)c->d_rowp.p + (size_t)w0 * ng * 16;
+    double2* pinv = (double2*)c->d_pinv.p + (size_t)w0 * 512;
     e = general(w0) ? chi0::launch_dyson_general(chi, (const double*)c->d_vsqrt.p, ng, gw, out, colp, rowp, pinv,
                                                  (int*)c->d_err.p, c->st)
                     : chi0::launch_dyson(chi, (const double*)c->d_vsqrt.p, ng, gw, out, colp, rowp, pinv,
                                          (int*)c->d_err.p, c->st);
     if (e != cudaSuccess) s = cuda_fail(c, e, "dyson launch");
-    chi0::stage_end(c, CHI0_STAGE_DYSON, (general(w0) ? 1 : 2) + 3 * nT);
+    chi0::stage_end(c, CHI0_STAGE_DYSON, chi0::dyson_launches(ng));
     // a host output receives each group as soon as it is inverted, so that
     // only the last group's copy follows the last contraction
     if (s == CHI0_OK && host_out) {

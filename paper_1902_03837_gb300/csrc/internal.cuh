@@ -194,7 +194,8 @@ cudaError_t launch_chi0_fp64_partials(const double2* R, const double* w, int64_t
 cudaError_t launch_chi0_reduce(const double2* part, int nchunks, int ng, int nw, double2* chi,
                                cudaStream_t s, int accumulate = 0);
 
-// a5: eps~ = 1 - V chi V, then in-place blocked Gauss-Jordan inverse.
+// a5: eps~ = 1 - V chi V, then blocked Gauss-Jordan inverse in A (which may be
+// chi).  Scratch per matrix: ng * 16 entries in each panel, 512 in pinv.
 cudaError_t launch_dyson(const double2* chi, const double* vsqrt, int ng, int nw, double2* A,
                          double2* colpanel, double2* rowpanel, double2* pinv, int* err_flag,
                          cudaStream_t s);
@@ -202,6 +203,8 @@ cudaError_t launch_dyson(const double2* chi, const double* vsqrt, int ng, int nw
 cudaError_t launch_dyson_general(const double2* chi, const double* vsqrt, int ng, int nw, double2* A,
                                  double2* colpanel, double2* rowpanel, double2* pinv, int* err_flag,
                                  cudaStream_t s);
+// Kernel launches of either.
+int dyson_launches(int ng);
 // The Dyson kernels prefer the whole shared-memory carveout, the setting of
 // the tensor-core contraction, so that both can share an SM.
 cudaError_t dyson_prepare();

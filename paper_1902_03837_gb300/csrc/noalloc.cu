@@ -5,11 +5,11 @@
 // every byte it hands out), or a service that must keep a fixed device-memory
 // footprint once it has started, so that a later allocation can neither fail
 // nor push another tenant of the GPU out of memory.  This entry point runs the
-// same blocked Gauss-Jordan kernels as chi0_invert_eps, one frequency after
-// another, with all of their scratch (the row/column panels, the pivot-block
-// inverse, the Coulomb factors and the error flag) in one file-scope device
-// array whose size is fixed at build time.  Every GPU that loads the library
-// holds that array until the process exits.  The first call on a device
+// same blocked Gauss-Jordan kernels as chi0_invert_eps, as many frequencies at
+// a time as its panels hold, with all of their scratch (the row/column panels,
+// the pivot-block inverses, the Coulomb factors and the error flag) in one
+// file-scope device array whose size is fixed at build time.  Every GPU that
+// loads the library holds that array until the process exits.  The first call on a device
 // looks up the array's device address (cudaGetSymbolAddress, once per
 // device, with that device current); make that first call before any stream
 // capture begins.
@@ -25,12 +25,14 @@
 namespace {
 
 constexpr int kNoallocMaxNg = 2048;  // largest N_G this entry point accepts
-constexpr int kPanelW = 32;          // pivot-block width of the Gauss-Jordan kernels
+constexpr int kPanelW = 16;          // pivot-block width of the Gauss-Jordan kernels
+constexpr int kPanelEntries = 29 * kNoallocMaxNg;  // entries of each panel
+constexpr int kMaxGroup = 24;        // frequencies at a time (pivot blocks: two of 16 x 16 each)
 
 // layout of the scratch array (bytes)
-constexpr size_t kColBytes = (size_t)kNoallocMaxNg * kPanelW * sizeof(double2);
-constexpr size_t kRowBytes = (size_t)kPanelW * kNoallocMaxNg * sizeof(double2);
-constexpr size_t kPivBytes = (size_t)kPanelW * kPanelW * sizeof(double2);
+constexpr size_t kColBytes = (size_t)kPanelEntries * sizeof(double2);
+constexpr size_t kRowBytes = (size_t)kPanelEntries * sizeof(double2);
+constexpr size_t kPivBytes = (size_t)kMaxGroup * 2 * kPanelW * kPanelW * sizeof(double2);
 constexpr size_t kVBytes = (size_t)kNoallocMaxNg * sizeof(double);
 constexpr size_t kErrBytes = 256;
 constexpr size_t kOffCol = 0;
@@ -92,11 +94,16 @@ extern "C" chi0_status chi0_invert_eps_noalloc(const void* chi0, const double* v
     cudaGetLastError();
     return CHI0_ECUDA;
   }
+  // as many frequencies at a time as the panels hold: with one after the other
+  // the chain of pivots leaves most of the GPU idle (12 matrices of N_G =
+  // 300 fit)
   const size_t n2 = (size_t)ng * ng;
-  for (int iw = 0; iw < nw; ++iw) {
+  const int group = kPanelEntries / (ng * kPanelW) < kMaxGroup ? kPanelEntries / (ng * kPanelW) : kMaxGroup;
+  for (int iw = 0; iw < nw; iw += group) {
     const double2* c = static_cast<const double2*>(chi0) + iw * n2;
     double2* o = static_cast<double2*>(out) + iw * n2;
-    if (chi0::launch_dyson(c, vs, ng, 1, o, colp, rowp, pinv, err, st) != cudaSuccess) {
+    const int n = nw - iw < group ? nw - iw : group;
+    if (chi0::launch_dyson(c, vs, ng, n, o, colp, rowp, pinv, err, st) != cudaSuccess) {
       cudaGetLastError();
       return CHI0_ECUDA;
     }
