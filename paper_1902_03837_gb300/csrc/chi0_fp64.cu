@@ -39,10 +39,10 @@ __global__ void k_weights(int nk, int n_lo, int Nn, int Nm, int nb, const int32_
                           const double* __restrict__ omega_im, const int* __restrict__ vkind, int nw,
                           double eta, double pref, double occ_tol, int bg, double eps_bar,
                           const double* __restrict__ dpole, const double* __restrict__ epsd, int nd,
-                          double* __restrict__ w, int k0) {
-  const int64_t nt = (int64_t)nk * Nn * Nm;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nt) return;
+                          double* __restrict__ w, int k0, const int64_t* __restrict__ perm, int64_t nrow) {
+  const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (row >= nrow) return;
+  const int64_t t = perm ? perm[row] : row;
   const int m = (int)(t % Nm);
   const int64_t r = t / Nm;
   const int n = n_lo + (int)(r % Nn);
@@ -74,7 +74,7 @@ __global__ void k_weights(int nk, int n_lo, int Nn, int Nm, int nb, const int32_
       v = pref * df * f;
     }
     if (bg && fm > occ_tol) v -= pref * fm * pole_weight(kind, omega_im[iw], eta, dbar);
-    w[(size_t)iw * nt + t] = v;
+    w[(size_t)iw * nrow + row] = v;
   }
 }
 
@@ -92,7 +92,7 @@ __device__ __forceinline__ void tri_decode(int tile, int& I, int& J) {
 // part[kc][iw][i][j] = sum_{t in chunk kc} w_t R_ti conj(R_tj) on lower tiles I >= J.
 __global__ void __launch_bounds__(256)
 k_chi0_fp64(const double2* __restrict__ R, const double* __restrict__ w, int64_t nt, int ng,
-            int nw, int kchunk, double2* __restrict__ part) {
+            int nw, int kchunk, double2* __restrict__ part, const int64_t* __restrict__ perm) {
   __shared__ double2 As[kKB][kT];
   __shared__ double2 Bs[kKB][kT];
   __shared__ double ws[kKB];
@@ -112,10 +112,10 @@ k_chi0_fp64(const double2* __restrict__ R, const double* __restrict__ w, int64_t
   for (int64_t tt = t0; tt < t1; tt += kKB) {
     for (int e = tid; e < kKB * kT; e += 256) {
       const int r = e / kT, c = e % kT;
-      const int64_t t = tt + r;
+      const int64_t t = tt + r < t1 ? (perm ? perm[tt + r] : tt + r) : -1;
       const int ia = I * kT + c, ib = J * kT + c;
-      As[r][c] = (t < t1 && ia < ng) ? R[t * ng + ia] : make_double2(0.0, 0.0);
-      Bs[r][c] = (t < t1 && ib < ng) ? R[t * ng + ib] : make_double2(0.0, 0.0);
+      As[r][c] = (t >= 0 && ia < ng) ? R[t * ng + ia] : make_double2(0.0, 0.0);
+      Bs[r][c] = (t >= 0 && ib < ng) ? R[t * ng + ib] : make_double2(0.0, 0.0);
     }
     if (tid < kKB) ws[tid] = (tt + tid < t1) ? wv[tt + tid] : 0.0;
     __syncthreads();
@@ -184,21 +184,21 @@ cudaError_t launch_weights(int nk, int n_lo, int Nn, int Nm, int nb, const int32
                            const double* eps, const double* occ, const double* omega_im,
                            const int* vkind, int nw, double eta, double pref,
                            double occ_tol, int bg, double eps_bar, const double* dpole, const double* epsd,
-                           int nd, double* w, cudaStream_t s, int k0) {
-  const int64_t nt = (int64_t)nk * Nn * Nm;
-  if (nt == 0) return cudaSuccess;
-  const int64_t blocks = (nt + 255) / 256;
+                           int nd, double* w, cudaStream_t s, int k0, const int64_t* perm, int64_t nrow) {
+  if (!perm) nrow = (int64_t)nk * Nn * Nm;
+  if (nrow == 0) return cudaSuccess;
+  const int64_t blocks = (nrow + 255) / 256;
   k_weights<<<(unsigned)blocks, 256, 0, s>>>(nk, n_lo, Nn, Nm, nb, kq, eps, occ, omega_im, vkind, nw, eta,
-                                            pref, occ_tol, bg, eps_bar, dpole, epsd, nd, w, k0);
+                                            pref, occ_tol, bg, eps_bar, dpole, epsd, nd, w, k0, perm, nrow);
   return cudaGetLastError();
 }
 
 cudaError_t launch_chi0_fp64_partials(const double2* R, const double* w, int64_t nt, int ng,
                                       int nw, int kchunk, int nchunks, double2* part,
-                                      cudaStream_t s) {
+                                      cudaStream_t s, const int64_t* perm) {
   const int nT = (ng + kT - 1) / kT;
   dim3 grid(nT * (nT + 1) / 2, nchunks, nw);
-  k_chi0_fp64<<<grid, 256, 0, s>>>(R, w, nt, ng, nw, kchunk, part);
+  k_chi0_fp64<<<grid, 256, 0, s>>>(R, w, nt, ng, nw, kchunk, part, perm);
   return cudaGetLastError();
 }
 

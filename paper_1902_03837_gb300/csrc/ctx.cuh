@@ -115,8 +115,14 @@ struct chi0_ctx {
   int64_t kgrp = 0;                    // transitions in group order, each group padded to 64
   DevBuf d_tperm;                      // [kgrp] int64 transition of each row (-1: padding)
   DevBuf d_grange;                     // [ngroups] int2 (first k-block, k-blocks) of each group
-  DevBuf d_ga;                         // [nt] double pref (f_m - f_n)
+  DevBuf d_ga;                         // [kgrp] double pref (f_m - f_n) of each row
   DevBuf d_gfac;                       // [nwv][ngroups] float F_g(w) of the representatives
+  // transitions with weight (f_m - f_n > tol, or f_m > tol with the extrapolar
+  // correction): rho covers the dense (k, n, m) block, of which a metal's
+  // weights leave half; the weights and the contraction run over the nwt rows
+  // d_wperm[row].  nwt = 0: over the whole block.
+  int64_t nwt = 0;
+  DevBuf d_wperm;
   // sign shared by every transition weight of the imaginary-axis frequencies
   // (-1: all <= 0, +1: all >= 0, 0: mixed or not known); nonzero lets the
   // Hermitian contraction take the one-operand form chi0 = sign S S^H with
@@ -167,6 +173,11 @@ struct chi0_ctx {
 
 
 namespace chi0 {
+// rows of the weights and of the contraction, and the transition of each (NULL: itself)
+inline int64_t weighted_rows(const chi0_ctx* c) { return c->nwt > 0 ? c->nwt : c->nt; }
+inline const int64_t* weighted_perm(const chi0_ctx* c) {
+  return c->nwt > 0 ? (const int64_t*)c->d_wperm.p : nullptr;
+}
 // record msg on c and return s
 chi0_status ctx_fail(chi0_ctx* c, chi0_status s, const char* msg);
 // grow b to at least bytes (device memory; contents not preserved)
@@ -188,10 +199,11 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw);
 chi0_status tc_plan_grouped(chi0_ctx* c, int ng, int nw);
 chi0_status tc_launch_grouped(chi0_ctx* c, double2* chi, const cudaEvent_t* ev_freq);
 // accumulate: chi += this contraction (the transitions come in blocks)
+// perm: row t of the sum is transition perm[t] of R
 chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, int ng, int nw,
                       double2* chi, const cudaEvent_t* ev_freq = nullptr,
                       const cudaEvent_t* ev_prep = nullptr, const chi0::BgApply* bg = nullptr,
-                      const int* vkind = nullptr, int accumulate = 0);
+                      const int* vkind = nullptr, int accumulate = 0, const int64_t* perm = nullptr);
 void tc_release(chi0_ctx* c);
 // one bounded mbarrier wait that can never be satisfied (failure detection)
 cudaError_t launch_wait_probe(int* err, cudaStream_t s);

@@ -138,7 +138,8 @@ cudaError_t batch_dispatch(int nfft, const RhoTask<T, typename C2<T>::t>* tasks,
                            size_t smem, unsigned long long* counter, int nsm, cudaStream_t s);
 }  // namespace rfft
 
-// a3: real transition weights w[iw][t] (FP64).
+// a3: real transition weights w[iw][t] (FP64), or w[iw][row] of the nrow
+// transitions perm[row] (perm != NULL).
 // With bg != 0 each weight is reduced by the extrapolar weight of its m
 // (a transition from m into an empty state at eps_bar): the closure form of
 // the Bruneval-Gonze correction.
@@ -155,7 +156,8 @@ cudaError_t launch_weights(int nk, int n_lo, int Nn, int Nm, int nb, const int32
                            const double* eps, const double* occ, const double* omega_im,
                            const int* vkind, int nw, double eta, double pref,
                            double occ_tol, int bg, double eps_bar, const double* dpole, const double* epsd,
-                           int nd, double* w, cudaStream_t s, int k0 = 0);
+                           int nd, double* w, cudaStream_t s, int k0 = 0, const int64_t* perm = nullptr,
+                           int64_t nrow = 0);
 // chi[iw] = H[vr[iw]] + i H[vi[iw]] (vi[iw] < 0: chi[iw] = H[vr[iw]])
 cudaError_t launch_combine_freq(const double2* H, const int* vr, const int* vi, int ng, int nw, double2* chi,
                                 cudaStream_t s);
@@ -185,10 +187,11 @@ struct BgApply {
 };
 
 // a4 (FP64 form): split-K partials of chi0 = sum_t w_t R_t R_t^H, lower
-// triangle tiles; part[kc][iw][i][j] (complex128).
+// triangle tiles; part[kc][iw][i][j] (complex128).  perm: row t of the sum is
+// transition perm[t].
 cudaError_t launch_chi0_fp64_partials(const double2* R, const double* w, int64_t nt, int ng,
                                       int nw, int kchunk, int nchunks, double2* part,
-                                      cudaStream_t s);
+                                      cudaStream_t s, const int64_t* perm = nullptr);
 // Sum of the partials, Hermitian completion: chi[iw][i][j] (accumulate: added
 // to what chi holds, the sum over earlier transition blocks).
 cudaError_t launch_chi0_reduce(const double2* part, int nchunks, int ng, int nw, double2* chi,

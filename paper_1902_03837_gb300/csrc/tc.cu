@@ -746,7 +746,8 @@ struct PrepOut {
 };
 
 // perm (optional): row t of the operand is transition perm[t] of R (-1: a
-// zero row), for nt rows; without it row t is transition t.
+// zero row), for nt rows; without it row t is transition t.  Weights are
+// indexed by row.
 __global__ void __launch_bounds__(256)
 k_prep(const float2* __restrict__ R, int ngrp, int64_t nt, int ng, int mpad, const __grid_constant__ PrepOut out,
        const int64_t* __restrict__ perm) {
@@ -765,7 +766,7 @@ k_prep(const float2* __restrict__ R, int ngrp, int64_t nt, int ng, int mpad, con
   __syncthreads();
   for (int e = threadIdx.x; e < ngrp * kPT; e += 256) {
     const int g = e / kPT, tl = e % kPT;
-    const int64_t t = src[tl];
+    const int64_t t = src[tl] >= 0 ? t0 + tl : -1;   // the weights are in row order
     if (out.wr[g] && t >= 0) {
       const double wv = out.wr[g][t];
       // sqrt|w| in FP32 (2^-24 relative, far below the split's 2^-17; the
@@ -1222,7 +1223,7 @@ chi0_status tc_launch_grouped(chi0_ctx* c, double2* chi, const cudaEvent_t* ev_f
 
 chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, int ng, int nw,
                       double2* chi, const cudaEvent_t* ev_freq, const cudaEvent_t* ev_prep,
-                      const BgApply* bg, const int* vkind, int accumulate) {
+                      const BgApply* bg, const int* vkind, int accumulate, const int64_t* perm) {
   if (!c->tc) return ctx_fail(c, CHI0_ESTATE, "tensor-core contraction not planned");
   TcState& t = *static_cast<TcState*>(c->tc);
   const dim3 pgrid((unsigned)(t.kpad / kPT), (unsigned)(t.mpad / 2 / kPI));
@@ -1255,7 +1256,7 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
     ob.hi[0] = (__nv_bfloat16*)t.bh.p;
     ob.lo[0] = (__nv_bfloat16*)t.bl.p;
     stage_begin(c, CHI0_STAGE_WEIGHTS);
-    k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)R, 1, nt, ng, t.mpad, ob, nullptr);
+    k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)R, 1, nt, ng, t.mpad, ob, perm);
     stage_end(c, CHI0_STAGE_WEIGHTS, 1);
   }
   const int nunits = t.ntiles * t.nchunks, nunits_f = t.ntiles_f * t.nchunks_f;
@@ -1274,7 +1275,7 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
       oa.sq[g] = one_op && !jb.cplx;
     }
     stage_begin(c, CHI0_STAGE_WEIGHTS);
-    k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)R, gw, nt, ng, t.mpad, oa, nullptr);
+    k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)R, gw, nt, ng, t.mpad, oa, perm);
     stage_end(c, CHI0_STAGE_WEIGHTS, 1);
     if (ev_prep)
       for (int g = 0; g < gw; ++g) {
@@ -1386,14 +1387,14 @@ chi0_status tc_tune_split(chi0_ctx* c, float* best_ms) {
     PrepOut ob{};
     ob.hi[0] = (__nv_bfloat16*)t.bh.p;
     ob.lo[0] = (__nv_bfloat16*)t.bl.p;
-    k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)c->d_R.p, 1, c->nt, ng, t.mpad, ob, nullptr);
+    k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)c->d_R.p, 1, weighted_rows(c), ng, t.mpad, ob, weighted_perm(c));
   }
   PrepOut oa{};
   oa.hi[0] = (__nv_bfloat16*)t.ah[0].p;
   oa.lo[0] = (__nv_bfloat16*)t.al[0].p;
   oa.wr[0] = (const double*)c->d_w.p;
   oa.sq[0] = one_op;
-  k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)c->d_R.p, 1, c->nt, ng, t.mpad, oa, nullptr);
+  k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)c->d_R.p, 1, weighted_rows(c), ng, t.mpad, oa, weighted_perm(c));
   const size_t cap = t.part.bytes / ((size_t)t.tile_elems * 16);
   const int base_split = (t.total_kb + t.kbpc - 1) / t.kbpc;
   int best_kbpc = t.kbpc, best_n = t.nchunks;
