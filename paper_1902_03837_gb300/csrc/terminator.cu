@@ -27,153 +27,342 @@ constexpr int kI = 5, kH = 128, kO = 2;
 constexpr int kP = kH * kI + kH + kH * kH + kH + kO * kH + kO;  // 17538
 constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kH * kI, kOffW2 = kOffB1 + kH, kOffB2 = kOffW2 + kH * kH,
               kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kO * kH;
-constexpr int kS = 32;         // samples per block
+constexpr int kS = 32;         // samples per block of the training kernel
+constexpr int kSP = 64;        // samples per pass of the prediction kernel
 constexpr int kThreads = 256;
+constexpr int kLd = kH + 4;    // padded row: eight rows' 16-byte pieces fall into distinct banks
 
 __device__ __forceinline__ float rb(float v, int bf16) {
   return bf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v;
 }
 
-// Forward (and optionally backward) for kS samples per block.  Gradients of
-// the block go to part[block][kP] (summed later in a fixed order).
-template <bool kBackward>
-__global__ void __launch_bounds__(kThreads)
-k_mlp(const float* __restrict__ prm, const float* __restrict__ x, const float* __restrict__ t,
-      int64_t batch, int bf16, float* __restrict__ part, float* __restrict__ y_out,
-      float* __restrict__ loss_part) {
-  extern __shared__ float sm[];
-  float* W2 = sm;                       // [H][H+1] (rounded)
-  float* h1 = W2 + kH * (kH + 1);       // [S][H]
-  float* h2 = h1 + kS * kH;             // [S][H]
-  float* xs = h2 + kS * kH;             // [S][I]
-  float* ys = xs + kS * kI;             // [S][O] -> dy
-  float* dz2 = ys + kS * kO;            // [S][H]
-  float* dz1 = dz2 + kS * kH;           // [S][H]
-  float* red = dz1 + kS * kH;           // [kThreads]
+// acc[i][j] += sum_k A[s_i][k] B[h_j][k], k ascending (rows of kLd floats in
+// shared memory; s_i = 8 i + lane / 4, h_j = 32 j + 4 warp + lane % 4).  Both
+// layers of the network are bound by the FP32 pipe once the operands come as
+// 16-byte pieces for NS x 4 outputs per thread (one load per 2 NS x 8 / (NS + 4)
+// multiply-adds; a scalar pair of loads per multiply-add was bound by shared
+// memory).  Every output keeps its own chain of fused multiply-adds in the
+// order of k, so the results do not depend on the tiling.
+template <int NS>
+__device__ __forceinline__ void rows_dot(const float* __restrict__ A, const float* __restrict__ B, float (&acc)[NS][4]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float* a = A + (lane >> 2) * kLd;
+  const float* b = B + (warp * 4 + (lane & 3)) * kLd;
+#pragma unroll 2
+  for (int k = 0; k < kH; k += 4) {
+    float4 av[NS], bv[4];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) av[i] = *reinterpret_cast<const float4*>(a + i * 8 * kLd + k);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(b + j * 32 * kLd + k);
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        acc[i][j] = fmaf(bv[j].x, av[i].x, acc[i][j]);
+        acc[i][j] = fmaf(bv[j].y, av[i].y, acc[i][j]);
+        acc[i][j] = fmaf(bv[j].z, av[i].z, acc[i][j]);
+        acc[i][j] = fmaf(bv[j].w, av[i].w, acc[i][j]);
+      }
+  }
+}
+
+// The parameters as every pass of a block uses them: products' operands rounded.
+struct alignas(16) MlpWeights {
+  alignas(16) float W2[kH * kLd];
+  alignas(16) float w3[kO * kH];
+  float w1[kH * kI], b1[kH], b2[kH], b3[kO];
+};
+__device__ __forceinline__ void load_weights(MlpWeights& w, const float* __restrict__ prm, int bf16) {
   const int tid = threadIdx.x;
-  const int64_t s0 = (int64_t)blockIdx.x * kS;
-  const int ns = (batch - s0 < kS) ? (int)(batch - s0) : kS;
-  for (int e = tid; e < kH * kH; e += kThreads) {
-    const int r = e / kH, c = e % kH;
-    W2[r * (kH + 1) + c] = rb(prm[kOffW2 + e], bf16);
+#pragma unroll 8
+  for (int e = tid; e < kH * kH; e += kThreads)   // (the caller's vector is only 4-byte aligned)
+    w.W2[(e / kH) * kLd + e % kH] = rb(prm[kOffW2 + e], bf16);
+  for (int e = tid; e < kH * kI; e += kThreads) w.w1[e] = rb(prm[kOffW1 + e], bf16);
+  for (int e = tid; e < kO * kH; e += kThreads) w.w3[e] = rb(prm[kOffW3 + e], bf16);
+  if (tid < kH) {
+    w.b1[tid] = prm[kOffB1 + tid];
+    w.b2[tid] = prm[kOffB2 + tid];
   }
-  for (int e = tid; e < kS * kI; e += kThreads) {
-    const int s = e / kI;
-    xs[e] = (s < ns) ? rb(x[(s0 + s) * kI + e % kI], bf16) : 0.f;
+  if (tid < kO) w.b3[tid] = prm[kOffB3 + tid];
+}
+
+__device__ __forceinline__ float layer1(const MlpWeights& w, const float* __restrict__ xs, int s, int h) {
+  float z = w.b1[h];
+#pragma unroll
+  for (int i = 0; i < kI; ++i) z = fmaf(w.w1[h * kI + i], xs[s * kI + i], z);
+  return tanhf(z);
+}
+
+// y[s][o] of rows h2[s] (rounded)
+__device__ __forceinline__ float layer3(const MlpWeights& w, const float* __restrict__ h2, int s, int o) {
+  float z = w.b3[o];
+#pragma unroll 4
+  for (int k = 0; k < kH; k += 4) {
+    const float4 a = *reinterpret_cast<const float4*>(h2 + s * kLd + k);
+    const float4 b = *reinterpret_cast<const float4*>(w.w3 + o * kH + k);
+    z = fmaf(b.x, a.x, z);
+    z = fmaf(b.y, a.y, z);
+    z = fmaf(b.z, a.z, z);
+    z = fmaf(b.w, a.w, z);
   }
-  __syncthreads();
-  // layer 1
-  for (int e = tid; e < kS * kH; e += kThreads) {
-    const int s = e / kH, h = e % kH;
-    float z = prm[kOffB1 + h];
-    for (int i = 0; i < kI; ++i) z = fmaf(rb(prm[kOffW1 + h * kI + i], bf16), xs[s * kI + i], z);
-    h1[e] = tanhf(z);
-  }
-  __syncthreads();
-  // layer 2
-  for (int e = tid; e < kS * kH; e += kThreads) {
-    const int s = e / kH, h = e % kH;
-    float z = prm[kOffB2 + h];
-    const float* w = W2 + h * (kH + 1);
-    const float* a = h1 + s * kH;
-    for (int k = 0; k < kH; ++k) z = fmaf(w[k], rb(a[k], bf16), z);
-    h2[e] = tanhf(z);
-  }
-  __syncthreads();
-  // layer 3
-  for (int e = tid; e < kS * kO; e += kThreads) {
-    const int s = e / kO, o = e % kO;
-    float z = prm[kOffB3 + o];
-    for (int k = 0; k < kH; ++k) z = fmaf(rb(prm[kOffW3 + o * kH + k], bf16), rb(h2[s * kH + k], bf16), z);
-    ys[e] = z;
-    if (!kBackward && s < ns) y_out[(s0 + s) * kO + o] = z;
-  }
-  if (!kBackward) return;
-  __syncthreads();
-  // loss and dy = (y - t) / B
-  float lsum = 0.f;
-  for (int e = tid; e < kS * kO; e += kThreads) {
-    const int s = e / kO;
-    float r = 0.f;
-    if (s < ns) r = ys[e] - t[(s0 + s) * kO + e % kO];
-    lsum += r * r;
-    ys[e] = r / (float)batch;
-  }
-  red[tid] = lsum;
-  __syncthreads();
-  for (int w = kThreads / 2; w > 0; w >>= 1) {
-    if (tid < w) red[tid] += red[tid + w];
+  return z;
+}
+
+// Prediction: two blocks per SM stay for the whole launch and take kSP samples
+// at a time, so that the parameters are staged once per block.  Bound by the
+// FP32 pipe (17.3 k multiply-adds and 256 tanh per sample): 10^6 samples 5180 ->
+// 929 us (0.67 ms of issue slots).
+struct PredictSmem {
+  MlpWeights w;
+  alignas(16) float h[kSP * kLd];
+  float xs[kSP * kI];
+};
+__global__ void __launch_bounds__(kThreads, 2)
+k_mlp_predict(const float* __restrict__ prm, const float* __restrict__ x, int64_t batch, int bf16,
+              float* __restrict__ y) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  PredictSmem& sm = *reinterpret_cast<PredictSmem*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  load_weights(sm.w, prm, bf16);
+  for (int64_t s0 = (int64_t)blockIdx.x * kSP; s0 < batch; s0 += (int64_t)gridDim.x * kSP) {
+    const int ns = (int)min((int64_t)kSP, batch - s0);
+    for (int e = tid; e < kSP * kI; e += kThreads) sm.xs[e] = e < ns * kI ? rb(x[s0 * kI + e], bf16) : 0.f;
     __syncthreads();
+    for (int s = tid / kH; s < kSP; s += kThreads / kH)
+      sm.h[s * kLd + tid % kH] = rb(layer1(sm.w, sm.xs, s, tid % kH), bf16);
+    __syncthreads();
+    float acc[kSP / 8][4];
+#pragma unroll
+    for (int i = 0; i < kSP / 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = sm.w.b2[j * 32 + warp * 4 + (lane & 3)];
+    rows_dot(sm.h, sm.w.W2, acc);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSP / 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        sm.h[(i * 8 + (lane >> 2)) * kLd + j * 32 + warp * 4 + (lane & 3)] = rb(tanhf(acc[i][j]), bf16);
+    __syncthreads();
+    if (tid < kSP * kO) {
+      const int s = tid % kSP, o = tid / kSP;
+      const float z = layer3(sm.w, sm.h, s, o);
+      if (s < ns) y[(s0 + s) * kO + o] = z;
+    }
+    // the next pass writes xs (read before the last barrier but one) and h
+    // (behind its own first barrier)
   }
-  if (tid == 0) loss_part[blockIdx.x] = 0.5f * red[0] / (float)batch;
-  // dz2 = (dy W3) * (1 - h2^2)
-  for (int e = tid; e < kS * kH; e += kThreads) {
-    const int s = e / kH, h = e % kH;
-    float g = 0.f;
-    for (int o = 0; o < kO; ++o) g = fmaf(rb(ys[s * kO + o], bf16), rb(prm[kOffW3 + o * kH + h], bf16), g);
-    const float hv = h2[e];
-    dz2[e] = (s < ns) ? g * (1.f - hv * hv) : 0.f;
+}
+
+// Forward and backward for kS samples per block.  Gradients of the block go to
+// part[block][kP] (summed later in a fixed order).  Per-sample values are the
+// same chains as in the prediction; the three products of 32 x 128 x 128 (h2,
+// dz1, dW2) take 4 x 4, 4 x 4 and 8 x 8 outputs per thread.  A block holds an SM
+// (one per SM at the minibatch of 4096): a training step there, with the
+// reduction and Adam, 91.7 -> 36.3 us.
+struct TrainSmem {
+  MlpWeights w;
+  alignas(16) float h1[kS * kLd], h2[kS * kLd], d2[kS * kLd], d1[kS * kLd];   // rounded operands
+  alignas(16) float r2[kS * kLd], r1[kS * kLd];                               // dz2, dz1 as computed
+  float xs[kS * kI], ys[kS * kO], red[kThreads / 32];
+};
+__global__ void __launch_bounds__(kThreads, 1)
+k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const float* __restrict__ t, int64_t batch,
+            int bf16, float* __restrict__ part, float* __restrict__ loss_part) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TrainSmem& sm = *reinterpret_cast<TrainSmem*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t s0 = (int64_t)blockIdx.x * kS;
+  const int ns = (int)min((int64_t)kS, batch - s0);
+  load_weights(sm.w, prm, bf16);
+  for (int e = tid; e < kS * kI; e += kThreads) sm.xs[e] = e < ns * kI ? rb(x[s0 * kI + e], bf16) : 0.f;
+  __syncthreads();
+  const int sr = lane >> 2;                        // rows sr + 8 i
+  const int hc = warp * 4 + (lane & 3);            // layer 2: columns hc + 32 j
+  const int kc = hc * 4;                           // layer 1: columns kc + j
+  float h1v[4][4], h2v[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float4 r;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h1v[i][j] = layer1(sm.w, sm.xs, sr + 8 * i, kc + j);
+    r = make_float4(rb(h1v[i][0], bf16), rb(h1v[i][1], bf16), rb(h1v[i][2], bf16), rb(h1v[i][3], bf16));
+    *reinterpret_cast<float4*>(sm.h1 + (sr + 8 * i) * kLd + kc) = r;
   }
   __syncthreads();
-  // dz1 = (dz2 W2) * (1 - h1^2)
-  for (int e = tid; e < kS * kH; e += kThreads) {
-    const int s = e / kH, k = e % kH;
-    float g = 0.f;
-    for (int h = 0; h < kH; ++h) g = fmaf(rb(dz2[s * kH + h], bf16), W2[h * (kH + 1) + k], g);
-    const float hv = h1[e];
-    dz1[e] = (s < ns) ? g * (1.f - hv * hv) : 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h2v[i][j] = sm.w.b2[hc + 32 * j];
+  rows_dot(sm.h1, sm.w.W2, h2v);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      h2v[i][j] = tanhf(h2v[i][j]);
+      sm.h2[(sr + 8 * i) * kLd + hc + 32 * j] = rb(h2v[i][j], bf16);
+    }
+  __syncthreads();
+  // layer 3, loss and dy = (y - t) / B
+  float lsum = 0.f;
+  if (tid < kS * kO) {
+    const int s = tid / kO, o = tid % kO;
+    float r = 0.f;
+    if (s < ns) r = layer3(sm.w, sm.h2, s, o) - t[(s0 + s) * kO + o];
+    lsum = r * r;
+    sm.ys[tid] = r / (float)batch;
+  }
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, w);
+  if (lane == 0) sm.red[warp] = lsum;
+  __syncthreads();
+  if (tid == 0) loss_part[blockIdx.x] = 0.5f * (sm.red[0] + sm.red[1]) / (float)batch;   // kS kO = 64 values
+  // dz2 = (dy W3) * (1 - h2^2)
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int s = sr + 8 * i, h = hc + 32 * j;
+      float g = 0.f;
+#pragma unroll
+      for (int o = 0; o < kO; ++o) g = fmaf(rb(sm.ys[s * kO + o], bf16), sm.w.w3[o * kH + h], g);
+      const float hv = h2v[i][j];
+      const float d = s < ns ? g * (1.f - hv * hv) : 0.f;
+      sm.r2[s * kLd + h] = d;
+      sm.d2[s * kLd + h] = rb(d, bf16);
+    }
+  __syncthreads();
+  // dz1 = (dz2 W2) * (1 - h1^2), h ascending
+  {
+    float g[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) g[i][j] = 0.f;
+#pragma unroll 2
+    for (int h = 0; h < kH; h += 4) {
+      float4 dv[4], wv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) dv[i] = *reinterpret_cast<const float4*>(sm.d2 + (sr + 8 * i) * kLd + h);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) wv[q] = *reinterpret_cast<const float4*>(sm.w.W2 + (h + q) * kLd + kc);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float dq[4] = {dv[i].x, dv[i].y, dv[i].z, dv[i].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          g[i][0] = fmaf(dq[q], wv[q].x, g[i][0]);
+          g[i][1] = fmaf(dq[q], wv[q].y, g[i][1]);
+          g[i][2] = fmaf(dq[q], wv[q].z, g[i][2]);
+          g[i][3] = fmaf(dq[q], wv[q].w, g[i][3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int s = sr + 8 * i;
+      float d[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float hv = h1v[i][j];
+        d[j] = s < ns ? g[i][j] * (1.f - hv * hv) : 0.f;
+      }
+      *reinterpret_cast<float4*>(sm.r1 + s * kLd + kc) = make_float4(d[0], d[1], d[2], d[3]);
+      *reinterpret_cast<float4*>(sm.d1 + s * kLd + kc) =
+          make_float4(rb(d[0], bf16), rb(d[1], bf16), rb(d[2], bf16), rb(d[3], bf16));
+    }
   }
   __syncthreads();
   float* gp = part + (size_t)blockIdx.x * kP;
+  // dW2[h][k] = sum_s dz2[s][h] h1[s][k]
+  {
+    const int h0 = (tid >> 4) * 8, k0 = (tid & 15) * 8;
+    float g[8][8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int b = 0; b < 8; ++b) g[a][b] = 0.f;
+    for (int s = 0; s < kS; ++s) {
+      const float4 d0 = *reinterpret_cast<const float4*>(sm.d2 + s * kLd + h0);
+      const float4 d1 = *reinterpret_cast<const float4*>(sm.d2 + s * kLd + h0 + 4);
+      const float4 a0 = *reinterpret_cast<const float4*>(sm.h1 + s * kLd + k0);
+      const float4 a1 = *reinterpret_cast<const float4*>(sm.h1 + s * kLd + k0 + 4);
+      const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+      const float h[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) g[a][b] = fmaf(d[a], h[b], g[a][b]);
+    }
+    if (((uintptr_t)gp & 7) == 0) {   // kP and kOffW2 are even: 8-byte pieces where the caller's buffer allows
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; b += 2)
+          *reinterpret_cast<float2*>(gp + kOffW2 + (h0 + a) * kH + k0 + b) = make_float2(g[a][b], g[a][b + 1]);
+    } else {
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) gp[kOffW2 + (h0 + a) * kH + k0 + b] = g[a][b];
+    }
+  }
   // dW3[o][h] = sum_s dy[s][o] h2[s][h];  db3
-  for (int e = tid; e < kO * kH; e += kThreads) {
-    const int o = e / kH, h = e % kH;
+  {
+    const int o = tid / kH, h = tid % kH;
     float g = 0.f;
-    for (int s = 0; s < kS; ++s) g = fmaf(rb(ys[s * kO + o], bf16), rb(h2[s * kH + h], bf16), g);
-    gp[kOffW3 + e] = g;
+    for (int s = 0; s < kS; ++s) g = fmaf(rb(sm.ys[s * kO + o], bf16), sm.h2[s * kLd + h], g);
+    gp[kOffW3 + tid] = g;
   }
   if (tid < kO) {
     float g = 0.f;
-    for (int s = 0; s < kS; ++s) g += ys[s * kO + tid];
+    for (int s = 0; s < kS; ++s) g += sm.ys[s * kO + tid];
     gp[kOffB3 + tid] = g;
   }
-  // dW2[h][k] = sum_s dz2[s][h] h1[s][k];  db2
-  for (int e = tid; e < kH * kH; e += kThreads) {
-    const int h = e / kH, k = e % kH;
+  {  // db2, db1
+    const int h = tid % kH;
+    const float* r = tid < kH ? sm.r2 : sm.r1;
     float g = 0.f;
-    for (int s = 0; s < kS; ++s) g = fmaf(rb(dz2[s * kH + h], bf16), rb(h1[s * kH + k], bf16), g);
-    gp[kOffW2 + e] = g;
-  }
-  for (int h = tid; h < kH; h += kThreads) {
-    float g2 = 0.f, g1 = 0.f;
-    for (int s = 0; s < kS; ++s) {
-      g2 += dz2[s * kH + h];
-      g1 += dz1[s * kH + h];
-    }
-    gp[kOffB2 + h] = g2;
-    gp[kOffB1 + h] = g1;
+    for (int s = 0; s < kS; ++s) g += r[s * kLd + h];
+    gp[(tid < kH ? kOffB2 : kOffB1) + h] = g;
   }
   // dW1[h][i] = sum_s dz1[s][h] x[s][i]
   for (int e = tid; e < kH * kI; e += kThreads) {
     const int h = e / kI, i = e % kI;
     float g = 0.f;
-    for (int s = 0; s < kS; ++s) g = fmaf(rb(dz1[s * kH + h], bf16), xs[s * kI + i], g);
+    for (int s = 0; s < kS; ++s) g = fmaf(sm.d1[s * kLd + h], sm.xs[s * kI + i], g);
     gp[kOffW1 + e] = g;
   }
 }
+static_assert(sizeof(MlpWeights) % 16 == 0 && kLd % 4 == 0, "16-byte pieces");
+static_assert(kS * kO == 64 && kThreads == 2 * kH && kO * kH == kThreads, "thread maps of k_mlp_train");
 
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nblk, const float* __restrict__ lpart,
-                             float* __restrict__ grad, float* __restrict__ loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+// Sum of the block partials in a fixed order: four interleaved sums per
+// parameter (their loads are independent), then the four.
+constexpr int kRedP = 64, kRedW = 4;
+__global__ void __launch_bounds__(kRedP * kRedW)
+k_mlp_reduce(const float* __restrict__ part, int nblk, const float* __restrict__ lpart, float* __restrict__ grad,
+             float* __restrict__ loss) {
+  __shared__ float sums[kRedW][kRedP];
+  const int p = blockIdx.x * kRedP + threadIdx.x % kRedP, w = threadIdx.x / kRedP;
+  float g = 0.f;
   if (p < kP) {
-    float g = 0.f;
-    for (int b = 0; b < nblk; ++b) g += part[(size_t)b * kP + p];
+#pragma unroll 8
+    for (int b = w; b < nblk; b += kRedW) g += part[(size_t)b * kP + p];
+  }
+  sums[w][threadIdx.x % kRedP] = g;
+  __syncthreads();
+  if (w == 0 && p < kP) {
+    for (int q = 1; q < kRedW; ++q) g += sums[q][threadIdx.x];
     grad[p] = g;
   }
-  if (p == 0 && loss) {
+  if (blockIdx.x == 0 && loss && threadIdx.x < 32) {
     float l = 0.f;
-    for (int b = 0; b < nblk; ++b) l += lpart[b];
-    *loss = l;
+    for (int b = threadIdx.x; b < nblk; b += 32) l += lpart[b];
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) l += __shfl_xor_sync(0xffffffffu, l, q);
+    if (threadIdx.x == 0) *loss = l;
   }
 }
 
@@ -190,10 +379,6 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
   p[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
 }
 
-size_t mlp_smem() {
-  return sizeof(float) * ((size_t)kH * (kH + 1) + 4 * (size_t)kS * kH + kS * kI + kS * kO + kThreads);
-}
-
 }  // namespace
 
 int mlp_nparams() { return kP; }
@@ -201,21 +386,21 @@ int mlp_nparams() { return kP; }
 cudaError_t mlp_loss_grad(const float* prm, const float* x, const float* t, int64_t batch, int bf16,
                           float* grad, float* loss, float* part, float* lpart, cudaStream_t st) {
   const int nblk = (int)((batch + kS - 1) / kS);
-  const size_t smem = mlp_smem();
-  cudaError_t e = cudaFuncSetAttribute(k_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(TrainSmem));
   if (e != cudaSuccess) return e;
-  k_mlp<true><<<nblk, kThreads, smem, st>>>(prm, x, t, batch, bf16, part, nullptr, lpart);
-  k_mlp_reduce<<<(kP + 255) / 256, 256, 0, st>>>(part, nblk, lpart, grad, loss);
+  k_mlp_train<<<nblk, kThreads, sizeof(TrainSmem), st>>>(prm, x, t, batch, bf16, part, lpart);
+  k_mlp_reduce<<<(kP + kRedP - 1) / kRedP, kRedP * kRedW, 0, st>>>(part, nblk, lpart, grad, loss);
   return cudaGetLastError();
 }
 
 cudaError_t mlp_predict(const float* prm, const float* x, int64_t batch, int bf16, float* y,
                         cudaStream_t st) {
-  const int64_t nblk = (batch + kS - 1) / kS;
-  const size_t smem = mlp_smem();
-  cudaError_t e = cudaFuncSetAttribute(k_mlp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int64_t passes = (batch + kSP - 1) / kSP;
+  cudaError_t e =
+      cudaFuncSetAttribute(k_mlp_predict, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(PredictSmem));
   if (e != cudaSuccess) return e;
-  k_mlp<false><<<(unsigned)nblk, kThreads, smem, st>>>(prm, x, nullptr, batch, bf16, nullptr, y, nullptr);
+  k_mlp_predict<<<(unsigned)(passes < 2 * 152 ? passes : 2 * 152), kThreads, sizeof(PredictSmem), st>>>(prm, x, batch,
+                                                                                                       bf16, y);
   return cudaGetLastError();
 }
 
