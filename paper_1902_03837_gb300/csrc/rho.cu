@@ -777,14 +777,15 @@ void rho_fft_tables(const int32_t* gset, RhoGeom& g, std::vector<int32_t>& rows,
 
 // Threads of a block: the count that leaves the fewest idle lanes over the
 // z, y and x columns of a block (the z columns carry the loads and products).
-static int rho_fft_threads(const RhoGeom& g, int jm, int xc) {
+static int rho_fft_threads(const RhoGeom& g, int jm, int xc, bool resident) {
   int best = 256;
   double best_cost = 1e30;
   for (int t : {256, 224, 192, 160, 128}) {
     double c = 0.0;
     for (int x0 = 0; x0 < g.nfft; x0 += xc) {
       const int nx = std::min(xc, g.nfft - x0);
-      c += 1.4 * jm * ((nx * g.nfft + t - 1) / t) + (jm * nx * g.HZ + t - 1) / t;
+      c += 1.4 * (resident ? jm * ((nx * g.nfft + t - 1) / t) : (jm * nx * g.nfft + t - 1) / t) +
+           (jm * nx * g.HZ + t - 1) / t;
     }
     c = (c + (jm * g.npair + t - 1) / t) * t;
     if (c < best_cost) {
@@ -859,7 +860,7 @@ cudaError_t launch_rho_pairs(const RhoGeom& g, const typename C2<T>::t* U, const
     }
     tk.Um = Um;
     if (nb > 0x7fffffff) return cudaErrorInvalidValue;
-    return rfft::rho_dispatch<T>(tk, smem, rho_fft_threads(g, tk.jm, tk.xc), nb, s);
+    return rfft::rho_dispatch<T>(tk, smem, rho_fft_threads(g, tk.jm, tk.xc, sizeof(T) == 4 && g.nfft <= 24), nb, s);
   }
   for (int jm : {4, 2, 1}) {
     RhoTask<T, TOUT> tk;

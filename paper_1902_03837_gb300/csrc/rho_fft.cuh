@@ -13,7 +13,7 @@
 // (states and rho together, one GB300): 6x6x6 k, 16 + 184 bands, N_G = 1000,
 // 48^3 -> 24^3, FP32: 181 -> 20.2 ms; 4x4x4 k, 64 bands, N_G = 431, 30^3 ->
 // 20^3, FP32: 13.7 -> 1.5 ms; 4x4x4 k, 8 + 24 bands, N_G = 59, 24^3 -> 12^3,
-// FP64: 12.3 -> 1.06 ms.
+// FP64: 12.3 -> 0.85 ms.
 //
 // Per transition the three axes are transformed one after the other and cut
 // to the response set after each: z columns straight from the two states'
@@ -32,6 +32,9 @@ namespace chi0 {
 namespace rfft {
 
 constexpr int kMaxThreads = 256;
+// Blocks that the registers of rho's kernel leave room for on an SM.
+template <typename T, int N>
+constexpr int kRhoBlocks = sizeof(T) == 4 || N <= 16 ? 2 : 1;
 
 // frequency of output (and input) i of an N-point column, in [-N/2, N/2)
 template <int N, int I>
@@ -124,9 +127,12 @@ __device__ __forceinline__ T2 cjmul(const T2 a, const T2 b) {
 // rho of one n at k and up to jm consecutive m at k - q (the same block order
 // and output as the generic kernel of rho.cu).
 //
-// Bound by the FP32 (FP64) pipes.  The n column stays in registers over the
-// block's m bands while both fit (kResident); the states are read from L2 once
-// per block (1 + 1/jm volumes per transition).  zs is padded to an odd row so
+// Bound by the FP32 (FP64) pipes.  In FP32 the n column stays in registers over
+// the block's m bands while both fit (kResident); the states are read from L2
+// once per block (1 + 1/jm volumes per transition).  In FP64 the registers are
+// worth more as resident warps, and the columns of all m bands are dealt out
+// one by one, so that fewer lanes idle in the last warp (12^3, 12288
+// transitions: 900 -> 695 us, of which the FP64 operations take 600).  zs is padded to an odd row so
 // that the y columns of a warp (stride N | 1) fall into distinct banks.
 // ---------------------------------------------------------------------------
 template <typename T, int N>
@@ -134,7 +140,7 @@ __device__ __forceinline__ void rho_fft_block(const RhoTask<T, typename C2<T>::t
                                               unsigned char* smem_raw) {
   using T2 = typename C2<T>::t;
   constexpr int NP = N | 1;
-  constexpr bool kResident = sizeof(T) == 4 ? N <= 24 : N <= 20;
+  constexpr bool kResident = sizeof(T) == 4 && N <= 24;
   const RhoGeom& g = tk.g;
   const int tid = threadIdx.x, nth = blockDim.x;
   const int jm = tk.jm, xc = tk.xc, P = g.npair, HZ = g.HZ, HX = g.HX;
@@ -161,26 +167,40 @@ __device__ __forceinline__ void rho_fft_block(const RhoTask<T, typename C2<T>::t
   for (int x0 = 0; x0 < N; x0 += xc) {
     const int nx = min(xc, N - x0);
     // z columns of the products: zs[j][xl][hz][y]
-    for (int u = tid; u < nx * N; u += nth) {
-      const int xl = u / N, y = u - xl * N;
-      const size_t off = (size_t)(x0 + xl) * (N * N) + y;
-      T2 un[N];
-      if constexpr (kResident)
+    auto store = [&](const T2 (&a)[N], T2* o) {
+      fft::static_for<0, N>([&](auto ic) {
+        constexpr int i = decltype(ic)::value, h = kFreq<N, i>;
+        if ((unsigned)(h - hz_base) < (unsigned)HZ) o[h * NP] = a[i];
+      });
+    };
+    if constexpr (kResident) {
+      for (int u = tid; u < nx * N; u += nth) {
+        const int xl = u / N, y = u - xl * N;
+        const size_t off = (size_t)(x0 + xl) * (N * N) + y;
+        T2 un[N];
         fft::static_for<0, N>([&](auto ic) { un[ic.value] = __ldg(Un + off + ic.value * N); });
-      T2* o = zs + ((size_t)xl * HZ - hz_base) * NP + y;
-      for (int j = 0; j < cm; ++j) {
+        T2* o = zs + ((size_t)xl * HZ - hz_base) * NP + y;
+        for (int j = 0; j < cm; ++j) {
+          const T2* __restrict__ um = Um + (size_t)j * vol + off;
+          T2 a[N];
+          fft::static_for<0, N>([&](auto ic) { a[ic.value] = __ldg(um + ic.value * N); });
+          fft::static_for<0, N>([&](auto ic) { a[ic.value] = cjmul(un[ic.value], a[ic.value]); });
+          fft::column<N>(a);
+          store(a, o);
+          o += (size_t)nx * HZ * NP;
+        }
+      }
+    } else {
+      for (int u = tid; u < cm * nx * N; u += nth) {
+        const int r = u / N, y = u - r * N;   // r = j nx + xl
+        const int j = r / nx;
+        const size_t off = (size_t)(x0 + r - j * nx) * (N * N) + y;
         const T2* __restrict__ um = Um + (size_t)j * vol + off;
         T2 a[N];
         fft::static_for<0, N>([&](auto ic) { a[ic.value] = __ldg(um + ic.value * N); });
-        if constexpr (!kResident)
-          fft::static_for<0, N>([&](auto ic) { un[ic.value] = __ldg(Un + off + ic.value * N); });
-        fft::static_for<0, N>([&](auto ic) { a[ic.value] = cjmul(un[ic.value], a[ic.value]); });
+        fft::static_for<0, N>([&](auto ic) { a[ic.value] = cjmul(__ldg(Un + off + ic.value * N), a[ic.value]); });
         fft::column<N>(a);
-        fft::static_for<0, N>([&](auto ic) {
-          constexpr int i = decltype(ic)::value, h = kFreq<N, i>;
-          if ((unsigned)(h - hz_base) < (unsigned)HZ) o[h * NP] = a[i];
-        });
-        o += (size_t)nx * HZ * NP;
+        store(a, zs + ((size_t)r * HZ - hz_base) * NP + y);
       }
     }
     __syncthreads();
@@ -230,7 +250,7 @@ __device__ __forceinline__ void rho_fft_block(const RhoTask<T, typename C2<T>::t
 }
 
 template <typename T, int N>
-__global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(kMaxThreads, kRhoBlocks<T, N>)
 k_rho_fft(const RhoTask<T, typename C2<T>::t> tk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   rho_fft_block<T, N>(tk, blockIdx.x, smem_raw);
@@ -238,7 +258,7 @@ k_rho_fft(const RhoTask<T, typename C2<T>::t> tk) {
 
 // Persistent form over the tasks of one grid size (as k_rho_batch of rho.cu).
 template <typename T, int N>
-__global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(kMaxThreads, kRhoBlocks<T, N>)
 k_rho_fft_batch(const RhoTask<T, typename C2<T>::t>* __restrict__ tasks, int ntasks, int64_t total,
                 unsigned long long* __restrict__ counter) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
