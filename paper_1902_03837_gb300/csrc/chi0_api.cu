@@ -948,13 +948,7 @@ chi0_status plan_chi0(chi0_ctx* c, int iq) {
     CK(cudaMemcpyAsync(c->d_vkind.p, c->h_vkind.data(), nw * 4, cudaMemcpyHostToDevice, c->st), "kinds H2D");
     CK(cudaStreamSynchronize(c->st), "synchronize");
     if (c->fp64) {
-      // split the transitions into chunks so that the grid fills the GPU
-      const int nT = (ng + 31) / 32;
-      const int64_t tiles = (int64_t)nT * (nT + 1) / 2 * nw;
-      int64_t want = std::max<int64_t>(1, (4 * 152 + tiles - 1) / tiles);
-      const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(8ull << 30) / (int64_t)(n2 * nw * 16));
-      want = std::min<int64_t>({want, mem_cap, (ntc + 63) / 64});
-      c->nchunks = (int)std::max<int64_t>(1, want);
+      c->nchunks = chi0::chi0_fp64_chunks(ntc, ng, nw);
       c->kchunk = (int)((ntc + c->nchunks - 1) / c->nchunks);
       if ((s = ensure(c, c->d_part, n2 * nw * c->nchunks * 16, "chi0 partials")) != CHI0_OK) return s;
     } else if (c->grouped) {

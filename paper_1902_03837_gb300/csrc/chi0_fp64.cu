@@ -10,6 +10,8 @@
 //
 // is accumulated over bounded transition chunks (the paper's reduction over
 // the k/c/v distribution becomes an on-device sum of chunk partials).
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace chi0 {
@@ -78,11 +80,13 @@ __global__ void k_weights(int nk, int n_lo, int Nn, int Nm, int nb, const int32_
   }
 }
 
-constexpr int kT = 32;   // output tile (complex entries per side)
-constexpr int kKB = 16;  // transitions per shared-memory stage
+constexpr int kT = 16;     // output tile (complex entries per side)
+constexpr int kKB = 32;    // transitions per shared-memory stage
+constexpr int kFThreads = 128;
+constexpr int kFUnits = 152 * 18;   // blocks: three rounds of six on every SM
 
 __device__ __forceinline__ void tri_decode(int tile, int& I, int& J) {
-  int i = (int)((sqrt(8.0 * (double)tile + 1.0) - 1.0) * 0.5);
+  int i = (int)((sqrtf(8.0f * (float)tile + 1.0f) - 1.0f) * 0.5f);
   while ((i + 1) * (i + 2) / 2 <= tile) ++i;
   while (i * (i + 1) / 2 > tile) --i;
   I = i;
@@ -90,92 +94,119 @@ __device__ __forceinline__ void tri_decode(int tile, int& I, int& J) {
 }
 
 // part[kc][iw][i][j] = sum_{t in chunk kc} w_t R_ti conj(R_tj) on lower tiles I >= J.
-__global__ void __launch_bounds__(256)
+//
+// Bound by the FP64 units (2 multiply-adds per clock and SM, 4 per entry and
+// transition), so what counts is how few of them are spent beside the lower
+// triangle and how evenly the SMs share them: 16 x 16 tiles (N_G = 137: 82% of
+// the entries computed are kept, 62% with 32 x 32), the weight multiplied in
+// when a row is staged (a thirty-second of the multiply-adds; per use it was a
+// fifth), a quadrant of the tile per warp and two entries per lane.  Two stages:
+// the rows of one are fetched while the other is summed.  Measured against 32 x
+// 32 tiles with four entries per thread: N_G = 137, 5164 rows, 3 frequencies
+// 2496 -> 1212 us (1000 us of multiply-adds in the triangle); N_G = 59, 12288 rows
+// 338 -> 216 us; N_G = 9, 120 rows 88 -> 6 us (two blocks did all of it).
+__global__ void __launch_bounds__(kFThreads, 6)
 k_chi0_fp64(const double2* __restrict__ R, const double* __restrict__ w, int64_t nt, int ng,
             int nw, int kchunk, double2* __restrict__ part, const int64_t* __restrict__ perm) {
-  __shared__ double2 As[kKB][kT];
-  __shared__ double2 Bs[kKB][kT];
-  __shared__ double ws[kKB];
+  __shared__ double2 As[kKB][kT];   // w_t R_ti
+  __shared__ double2 Bs[kKB][kT];   // R_tj
   int I, J;
   tri_decode(blockIdx.x, I, J);
   const int kc = blockIdx.y, iw = blockIdx.z;
   const int64_t t0 = (int64_t)kc * kchunk;
   const int64_t t1 = min(nt, t0 + kchunk);
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  double2 acc[2][2];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 2; ++b) acc[a][b] = make_double2(0.0, 0.0);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lr = (warp >> 1) * 8 + (lane >> 2), lc = (warp & 1) * 8 + (lane & 3) * 2;
+  const int sc = tid % kT, sr = tid / kT;   // staging: column sc, rows sr, sr + 8, ...
+  constexpr int kRows = kKB * kT / kFThreads;
+  const int ia = I * kT + sc, ib = J * kT + sc;
   const double* wv = w + (size_t)iw * nt;
-  for (int64_t tt = t0; tt < t1; tt += kKB) {
-    for (int e = tid; e < kKB * kT; e += 256) {
-      const int r = e / kT, c = e % kT;
-      const int64_t t = tt + r < t1 ? (perm ? perm[tt + r] : tt + r) : -1;
-      const int ia = I * kT + c, ib = J * kT + c;
-      As[r][c] = (t >= 0 && ia < ng) ? R[t * ng + ia] : make_double2(0.0, 0.0);
-      Bs[r][c] = (t >= 0 && ib < ng) ? R[t * ng + ib] : make_double2(0.0, 0.0);
-    }
-    if (tid < kKB) ws[tid] = (tt + tid < t1) ? wv[tt + tid] : 0.0;
-    __syncthreads();
-#pragma unroll 4
-    for (int r = 0; r < kKB; ++r) {
-      const double wt = ws[r];
-      double2 a[2], b[2];
+  double2 fa[kRows], fb[kRows];
+  double fw[kRows];
+  auto fetch = [&](int64_t tt) {
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const double2 av = As[r][ty * 2 + u];
-        a[u] = make_double2(wt * av.x, wt * av.y);
-        b[u] = Bs[r][tx * 2 + u];
+    for (int q = 0; q < kRows; ++q) {
+      const int64_t row = tt + sr + q * (kFThreads / kT);
+      fa[q] = fb[q] = make_double2(0.0, 0.0);
+      fw[q] = 0.0;
+      if (row < t1) {
+        const double2* r = R + (perm ? perm[row] : row) * ng;
+        if (ia < ng) fa[q] = r[ia];
+        if (ib < ng) fb[q] = r[ib];
+        fw[q] = wv[row];
       }
+    }
+  };
+  double2 x0 = make_double2(0.0, 0.0), x1 = x0;
+  fetch(t0);
+  for (int64_t tt = t0; tt < t1; tt += kKB) {
+    __syncthreads();
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {  // acc += a conj(b)
-          acc[u][v].x = fma(a[u].x, b[v].x, acc[u][v].x);
-          acc[u][v].x = fma(a[u].y, b[v].y, acc[u][v].x);
-          acc[u][v].y = fma(a[u].y, b[v].x, acc[u][v].y);
-          acc[u][v].y = fma(-a[u].x, b[v].y, acc[u][v].y);
-        }
+    for (int q = 0; q < kRows; ++q) {
+      const int r = sr + q * (kFThreads / kT);
+      As[r][sc] = make_double2(fw[q] * fa[q].x, fw[q] * fa[q].y);
+      Bs[r][sc] = fb[q];
     }
     __syncthreads();
+    if (tt + kKB < t1) fetch(tt + kKB);
+    const int n = (int)min((int64_t)kKB, t1 - tt);
+#pragma unroll 4
+    for (int r = 0; r < n; ++r) {
+      const double2 a = As[r][lr], b0 = Bs[r][lc], b1 = Bs[r][lc + 1];
+      x0.x = fma(a.x, b0.x, x0.x);   // a conj(b)
+      x0.y = fma(a.y, b0.x, x0.y);
+      x1.x = fma(a.x, b1.x, x1.x);
+      x1.y = fma(a.y, b1.x, x1.y);
+      x0.x = fma(a.y, b0.y, x0.x);
+      x0.y = fma(-a.x, b0.y, x0.y);
+      x1.x = fma(a.y, b1.y, x1.x);
+      x1.y = fma(-a.x, b1.y, x1.y);
+    }
   }
   double2* out = part + ((size_t)kc * nw + iw) * (size_t)ng * ng;
-#pragma unroll
-  for (int u = 0; u < 2; ++u)
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      const int i = I * kT + ty * 2 + u, j = J * kT + tx * 2 + v;
-      if (i < ng && j < ng) out[(size_t)i * ng + j] = acc[u][v];
-    }
+  const int i = I * kT + lr, j = J * kT + lc;
+  if (i < ng && j < ng) out[(size_t)i * ng + j] = x0;
+  if (i < ng && j + 1 < ng) out[(size_t)i * ng + j + 1] = x1;
 }
 
 // chi[iw][i][j] (i >= j) = sum_kc part, then chi[iw][j][i] = conj(chi[iw][i][j]).
-__global__ void k_chi0_reduce(const double2* __restrict__ part, int nchunks, int ng, int nw,
-                              double2* __restrict__ chi, int accumulate) {
+// 32 entries of a row per block, their chunks summed by eight warps (a
+// thread per entry walked up to hundreds of chunks one load after the other).
+constexpr int kRedW = 8;
+__global__ void __launch_bounds__(32 * kRedW)
+k_chi0_reduce(const double2* __restrict__ part, int nchunks, int ng, int nw, double2* __restrict__ chi,
+              int accumulate) {
+  __shared__ double2 sums[kRedW][32];
   const int64_t n2 = (int64_t)ng * ng;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n2 * nw) return;
-  const int iw = (int)(e / n2);
-  const int64_t ij = e - (int64_t)iw * n2;
+  const int iw = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t ij = (int64_t)blockIdx.x * 32 + lane;
   const int i = (int)(ij / ng), j = (int)(ij - (int64_t)i * ng);
-  if (i < j) return;
-  double sx = 0.0, sy = 0.0;
-  for (int c = 0; c < nchunks; ++c) {
-    const double2 v = part[((size_t)c * nw + iw) * n2 + ij];
-    sx += v.x;
-    sy += v.y;
+  const bool live = ij < n2 && i >= j;
+  double2 s = make_double2(0.0, 0.0);
+  if (live) {
+#pragma unroll 4
+    for (int c = warp; c < nchunks; c += kRedW) {
+      const double2 v = part[((size_t)c * nw + iw) * n2 + ij];
+      s.x += v.x;
+      s.y += v.y;
+    }
+  }
+  sums[warp][lane] = s;
+  __syncthreads();
+  if (warp != 0 || !live) return;
+  for (int q = 1; q < kRedW; ++q) {
+    s.x += sums[q][lane].x;
+    s.y += sums[q][lane].y;
   }
   double2* o = chi + (size_t)iw * n2;
-  if (i == j) sy = 0.0;  // Hermitian: real diagonal
-  if (accumulate) {      // add to the sum of the earlier transition blocks
-    const double2 a = o[(size_t)i * ng + j];
-    sx += a.x;
-    sy += a.y;
+  if (i == j) s.y = 0.0;  // Hermitian: real diagonal
+  if (accumulate) {       // add to the sum of the earlier transition blocks
+    const double2 a = o[ij];
+    s.x += a.x;
+    s.y += a.y;
   }
-  o[(size_t)i * ng + j] = make_double2(sx, sy);
-  if (i != j) o[(size_t)j * ng + i] = make_double2(sx, -sy);
+  o[ij] = s;
+  if (i != j) o[(size_t)j * ng + i] = make_double2(s.x, -s.y);
 }
 
 }  // namespace
@@ -193,12 +224,19 @@ cudaError_t launch_weights(int nk, int n_lo, int Nn, int Nm, int nb, const int32
   return cudaGetLastError();
 }
 
+int chi0_fp64_chunks(int64_t nt, int ng, int nw) {
+  const int64_t nT = (ng + kT - 1) / kT, tiles = nT * (nT + 1) / 2 * nw;
+  const int64_t want = (kFUnits + tiles - 1) / tiles;
+  const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(8ull << 30) / ((int64_t)ng * ng * nw * 16));
+  return (int)std::max<int64_t>(1, std::min({want, mem_cap, (nt + kKB / 2 - 1) / (kKB / 2), (int64_t)65535}));
+}
+
 cudaError_t launch_chi0_fp64_partials(const double2* R, const double* w, int64_t nt, int ng,
                                       int nw, int kchunk, int nchunks, double2* part,
                                       cudaStream_t s, const int64_t* perm) {
   const int nT = (ng + kT - 1) / kT;
-  dim3 grid(nT * (nT + 1) / 2, nchunks, nw);
-  k_chi0_fp64<<<grid, 256, 0, s>>>(R, w, nt, ng, nw, kchunk, part, perm);
+  dim3 grid((unsigned)(nT * (nT + 1) / 2), (unsigned)nchunks, (unsigned)nw);
+  k_chi0_fp64<<<grid, kFThreads, 0, s>>>(R, w, nt, ng, nw, kchunk, part, perm);
   return cudaGetLastError();
 }
 
@@ -226,8 +264,8 @@ cudaError_t launch_combine_freq(const double2* H, const int* vr, const int* vi, 
 
 cudaError_t launch_chi0_reduce(const double2* part, int nchunks, int ng, int nw, double2* chi,
                                cudaStream_t s, int accumulate) {
-  const int64_t n = (int64_t)ng * ng * nw;
-  k_chi0_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, nchunks, ng, nw, chi, accumulate);
+  const dim3 grid((unsigned)(((int64_t)ng * ng + 31) / 32), (unsigned)nw);
+  k_chi0_reduce<<<grid, 32 * kRedW, 0, s>>>(part, nchunks, ng, nw, chi, accumulate);
   return cudaGetLastError();
 }
 

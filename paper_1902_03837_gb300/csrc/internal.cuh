@@ -186,6 +186,9 @@ struct BgApply {
   int nd;
 };
 
+// Chunks that the FP64 contraction splits nt transitions into: enough blocks
+// for every SM, of 16 transitions at least, partials within 8 GB.
+int chi0_fp64_chunks(int64_t nt, int ng, int nw);
 // a4 (FP64 form): split-K partials of chi0 = sum_t w_t R_t R_t^H, lower
 // triangle tiles; part[kc][iw][i][j] (complex128).  perm: row t of the sum is
 // transition perm[t].
