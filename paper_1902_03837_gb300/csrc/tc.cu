@@ -25,27 +25,15 @@
 // accumulated transitions, ~2e-6 relative per 512), so each TMEM accumulation
 // is limited to 128 transitions; the epilogue warps fold those sub-sums into
 // compensated FP32 sums, and the per-CTA partials are added in FP64.  Only the
-// lower-triangle 128 x 128 tiles of D are computed (chi0 is Hermitian).
+// tiles on and below the diagonal of D are computed (chi0 is Hermitian).
 //
-// Kernel structure (one CTA = one tile x one range of transitions, 6 warps):
-//   warp 0      TMA producer: Ah, Al, Bh, Bl tiles (128 x 64 BF16, 128-byte
-//               swizzle) into a 3-stage shared-memory ring (mbarrier tx counts)
-//   warp 1      TMEM allocation (2 x 128 columns); one elected thread issues
-//               tcgen05.mma (M = N = 128, K = 16, BF16 -> FP32) into the two
-//               accumulators in turn and tcgen05.commit
-//   warps 2-5   epilogue: tcgen05.ld of a finished 128 x 128 accumulator,
-//               combination of 2 x 2 real blocks into complex entries,
-//               compensated accumulation in registers, final FP64 partial
+// The kernel, k_herk_wide, works in tiles of 128 x 256 with N = 256 products
+// (its comment has the structure): over the lower-triangle tiles (real
+// weights), over every tile (the complex weights of a real frequency), or over
+// every tile with FP32 tiles out (the self-energy product).
 // Every mbarrier wait is bounded: on timeout the kernel raises the device
 // error flag (reported as CHI0_ETIMEOUT), skips the remaining work, frees its
 // TMEM and returns.
-// Every contraction now runs the wide variant of this kernel, k_herk_wide:
-// 128 x 256 tiles, N = 256 products, twelve warps (see its comment), over the
-// lower-triangle tiles (real weights), over every tile (the complex weights
-// of a real frequency), or over every tile with FP32 tiles out (the
-// self-energy product).  k_herk_bf16x3 below, the 128 x 128 form, is no longer
-// launched; its comment describes the work units and the pipeline that
-// k_herk_wide widens.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -62,14 +50,9 @@ namespace chi0 {
 namespace {
 
 constexpr int kBM = 128;             // tile rows (real), = 64 complex G
-constexpr int kBN = 128;             // tile cols (real)
+constexpr int kBN = 128;             // columns of an epilogue warp (half a tile)
 constexpr int kBK = 64;              // transitions per pipeline stage (128 bytes of BF16)
-constexpr int kStages = 3;
 constexpr int kSubKB = 2;           // k-blocks per TMEM accumulation (128 transitions)
-constexpr int kTileBytes = kBM * kBK * 2;         // 16 KB per operand tile
-constexpr int kStageBytes = 4 * kTileBytes;       // Ah, Al, Bh, Bl
-constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*align*/ + 256 /*barriers*/;
-constexpr int kThreads = 192;
 constexpr long long kSpinCycles = 4000000000LL;   // ~2 s at 2 GHz
 constexpr int kErrTimeout = 2;
 
@@ -192,14 +175,6 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
          ((uint32_t)(m >> 4) << 24);
 }
 
-__device__ __forceinline__ void tri_decode(int tile, int& I, int& J) {
-  int i = (int)((sqrt(8.0 * (double)tile + 1.0) - 1.0) * 0.5);
-  while ((i + 1) * (i + 2) / 2 <= tile) ++i;
-  while (i * (i + 1) / 2 > tile) --i;
-  I = i;
-  J = tile - i * (i + 1) / 2;
-}
-
 // Compensated accumulation (Neumaier): s + c carries the running sum.
 __device__ __forceinline__ void nsum(float& s, float& c, float x) {
   const float t = s + x;
@@ -207,255 +182,24 @@ __device__ __forceinline__ void nsum(float& s, float& c, float x) {
   s = t;
 }
 
-// Work unit = one lower-triangle tile (I, J) x one range of k-blocks (a
-// split) -- or, with nI > 0, one tile of the full grid of nI row tiles of A
-// by ntiles / nI row tiles of B (I = tile % nI, J = tile / nI; A and B then
-// have their own row paddings mpad and mpad_b); unit u is tile u % ntiles of
-// split u / ntiles, so the CTAs resident
-// at one time read the same k-blocks (shared in L2).  The kernel is
-// persistent: CTA c takes units c, c + gridDim.x, ...; the stage ring and the
-// accumulator ping-pong run on across units, so the next unit's operands
-// stream in while the epilogue finishes the last one, and the CTA holds its SM
-// for the whole launch (blocks of a concurrent kernel fill what it leaves).
-// The MMA thread alternates between two TMEM accumulators, one per sub-chunk
-// of kSubKB k-blocks; the epilogue warps drain a finished sub-chunk (complex
-// combination, compensated FP32 sums held in registers) while the other one
-// fills, so the tensor core's FP32 accumulation never runs longer than
-// kSubKB * 64 transitions.
-// At most 224 registers: two warps of this CTA share a sub-partition, and
-// 2 x 224 x 32 leaves 2048 of its 16384 registers for a 64-register warp of
-// a concurrent Dyson block.
-__global__ void __maxnreg__(224)
-k_herk_bf16x3(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ CUtensorMap tm_al,
-              const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CUtensorMap tm_bl,
-              int total_kb, int kb_per_split, int mpad, double2* __restrict__ part, int ntiles,
-              int nunits, int* __restrict__ err, int nI, int mpad_b, int f32out,
-              const int2* __restrict__ ranges) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  unsigned char* gbase = smem_raw + (base - raw);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + kStages * kStageBytes);
-  const uint32_t bar_full = smem_u32(bars);                   // [kStages]
-  const uint32_t bar_empty = smem_u32(bars + kStages);        // [kStages]
-  const uint32_t bar_accf = smem_u32(bars + 2 * kStages);     // [2] accumulator full
-  const uint32_t bar_acce = smem_u32(bars + 2 * kStages + 2); // [2] accumulator drained
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 4);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  {  // an earlier CTA timed out: skip the work (one read, so the whole CTA agrees)
-    volatile int* skip = reinterpret_cast<volatile int*>(tmem_slot + 2);
-    if (threadIdx.x == 0) *skip = *(volatile int*)(err + 1);
-    __syncthreads();
-    if (*skip) return;
-  }
-  // k-block range of a unit
-  auto unit_range = [&](int u, int& kb0, int& nkb) {
-    if (ranges) {  // k-block range of split u / ntiles from the table (a pole group)
-      const int2 r = ranges[u / ntiles];
-      kb0 = r.x;
-      nkb = r.y;
-      return;
-    }
-    kb0 = (u / ntiles) * kb_per_split;
-    nkb = max(0, min(total_kb, kb0 + kb_per_split) - kb0);
-  };
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(bar_full + 8 * s, 1);
-      mbar_init(bar_empty + 8 * s, 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(bar_accf + 8 * b, 1);
-      mbar_init(bar_acce + 8 * b, 4);  // one arrival per epilogue warp
-    }
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0 && lane == 0) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tm_ah) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tm_al) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tm_bh) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tm_bl) : "memory");
-  }
-  if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 2 * kBN);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-
-  if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer
-      int gk = 0;  // k-blocks loaded by this CTA so far (stage ring position)
-      bool ok = true;
-      for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
-        int I, J, kb0, nkb;
-        const int tile = u % ntiles;
-        if (nI > 0) {
-          I = tile % nI;
-          J = tile / nI;
-        } else {
-          tri_decode(tile, I, J);
-        }
-        unit_range(u, kb0, nkb);
-        for (int k = 0; k < nkb; ++k, ++gk) {
-          const int s = gk % kStages;
-          const uint32_t ph = (uint32_t)((gk / kStages) & 1);
-          if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort_flag, err)) {
-            ok = false;
-            break;
-          }
-          const uint32_t st = base + s * kStageBytes;
-          mbar_expect_tx(bar_full + 8 * s, kStageBytes);
-          // k-blocked layout: block kb starts at row kb * mpad (A) and kb * mpad_b (B)
-          const int row = (kb0 + k) * mpad, row_b = (kb0 + k) * mpad_b;
-          tma_load_2d(st, &tm_ah, 0, row + I * kBM, bar_full + 8 * s);
-          tma_load_2d(st + kTileBytes, &tm_al, 0, row + I * kBM, bar_full + 8 * s);
-          tma_load_2d(st + 2 * kTileBytes, &tm_bh, 0, row_b + J * kBN, bar_full + 8 * s);
-          tma_load_2d(st + 3 * kTileBytes, &tm_bl, 0, row_b + J * kBN, bar_full + 8 * s);
-        }
-      }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
-      constexpr uint32_t idesc = idesc_bf16(kBM, kBN);
-      int gk = 0, gsc = 0;  // stage ring position, sub-chunks issued by this CTA
-      bool ok = true;
-      for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
-        int kb0, nkb;
-        unit_range(u, kb0, nkb);
-        const int nsub = (nkb + kSubKB - 1) / kSubKB;
-        int k = 0;
-        for (int sc = 0; sc < nsub; ++sc, ++gsc) {
-          const int b = gsc & 1;
-          if (!mbar_wait(bar_acce + 8 * b, (uint32_t)(((gsc >> 1) & 1) ^ 1), abort_flag, err)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t acc = tmem + (uint32_t)(b * kBN);
-          const int kend = min(nkb, (sc + 1) * kSubKB);
-          for (int kk0 = 0; k < kend; ++k, ++kk0, ++gk) {
-            const int s = gk % kStages;
-            const uint32_t ph = (uint32_t)((gk / kStages) & 1);
-            if (!mbar_wait(bar_full + 8 * s, ph, abort_flag, err)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t st = base + s * kStageBytes;
-            const uint64_t dah = desc_sw128(st);
-            const uint64_t dal = desc_sw128(st + kTileBytes);
-            const uint64_t dbh = desc_sw128(st + 2 * kTileBytes);
-            const uint64_t dbl = desc_sw128(st + 3 * kTileBytes);
-#pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-              const uint64_t off = (uint64_t)((kk * 32) >> 4);  // 16 BF16 = 32 bytes along K
-              umma_bf16(acc, dah + off, dbh + off, idesc, (kk0 > 0 || kk > 0) ? 1u : 0u);
-              umma_bf16(acc, dah + off, dbl + off, idesc, 1u);
-              umma_bf16(acc, dal + off, dbh + off, idesc, 1u);
-            }
-            umma_commit(bar_empty + 8 * s);  // stage free once these MMAs have read it
-          }
-          if (!ok) break;
-          umma_commit(bar_accf + 8 * b);     // sub-chunk sum ready in accumulator b
-        }
-      }
-    }
-  } else {
-    // ---------------- epilogue (warps 2..5 -> TMEM lane quadrants 2, 3, 0, 1)
-    const int q = warp & 3;
-    const bool odd = (lane & 1) != 0;
-    int gsc = 0;  // sub-chunks drained by this CTA
-    bool ok = true;
-    for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
-      int kb0, nkb;
-      unit_range(u, kb0, nkb);
-      const int nsub = (nkb + kSubKB - 1) / kSubKB;
-      float accs[32][2], accc[32][2];  // compensated sums: [complex entry][re, im]
-#pragma unroll
-      for (int e = 0; e < 32; ++e) accs[e][0] = accs[e][1] = accc[e][0] = accc[e][1] = 0.f;
-      for (int sc = 0; sc < nsub; ++sc, ++gsc) {
-        const int b = gsc & 1;
-        ok = __all_sync(0xffffffffu,
-                        mbar_wait(bar_accf + 8 * b, (uint32_t)((gsc >> 1) & 1), abort_flag, err) ? 1 : 0) != 0;
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * kBN);
-#pragma unroll
-        for (int cb = 0; cb < kBN / 16; ++cb) {
-          uint32_t v[16];
-          tmem_ld16(acc + (uint32_t)(cb * 16), v);
-          // rows 2i (even lane) and 2i+1 (odd lane); each lane combines 4 of the 8 complex columns
-          float recv[8];
-#pragma unroll
-          for (int k2 = 0; k2 < 8; ++k2) {
-            const float send = __uint_as_float(odd ? v[k2] : v[8 + k2]);
-            recv[k2] = __shfl_xor_sync(0xffffffffu, send, 1);
-          }
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            const float r0c0 = odd ? recv[2 * jj] : __uint_as_float(v[2 * jj]);           // D[2i][2j]
-            const float r0c1 = odd ? recv[2 * jj + 1] : __uint_as_float(v[2 * jj + 1]);   // D[2i][2j+1]
-            const float r1c0 = odd ? __uint_as_float(v[8 + 2 * jj]) : recv[2 * jj];       // D[2i+1][2j]
-            const float r1c1 = odd ? __uint_as_float(v[9 + 2 * jj]) : recv[2 * jj + 1];   // D[2i+1][2j+1]
-            const int e = cb * 4 + jj;
-            nsum(accs[e][0], accc[e][0], r0c0 + r1c1);
-            nsum(accs[e][1], accc[e][1], r1c0 - r0c1);
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_acce + 8 * b) : "memory");
-      }
-      if (!ok) break;
-      const int il = (q * 32 + lane) >> 1;  // complex row of the tile
-      const size_t obase = ((size_t)(u / ntiles) * ntiles + (u % ntiles)) * (size_t)(kBM / 2) * (kBN / 2) +
-                           (size_t)il * (kBN / 2) + (odd ? 4 : 0);
-      if (f32out) {  // the compensated sums rounded to FP32 (the tile layout of part, 8-byte entries)
-        float2* out = reinterpret_cast<float2*>(part) + obase;
-#pragma unroll
-        for (int cb = 0; cb < kBN / 16; ++cb)
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            const int e = cb * 4 + jj;
-            out[cb * 8 + jj] = make_float2(accs[e][0] + accc[e][0], accs[e][1] + accc[e][1]);
-          }
-      } else {
-        double2* out = part + obase;
-#pragma unroll
-        for (int cb = 0; cb < kBN / 16; ++cb)
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            const int e = cb * 4 + jj;
-            out[cb * 8 + jj] = make_double2((double)accs[e][0] + (double)accc[e][0],
-                                            (double)accs[e][1] + (double)accc[e][1]);
-          }
-      }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tmem, 2 * kBN);
-  }
-}
-
-// ---- wide tiles: 128 rows of A x 256 rows of B per unit ---------------------
-// The Hermitian contraction with N = 256 per MMA: each k-block stages Ah, Al
-// (128 rows) and Bh, Bl (256 rows, two TMA boxes each) and issues 12
-// tcgen05.mma of 128 x 256 x 16, so one operand byte feeds twice the products
-// of a 128 x 128 tile (half the shared-memory and L2 traffic per product of
-// A, and twice the work per stage in flight).  Two stages of 96 KB.  The
+// ---- the contraction kernel: 128 rows of A x 256 rows of B per unit ----------
+// Work unit = one tile (I, J) x one range of k-blocks (a split): unit u is tile
+// u % ntiles of split u / ntiles, so the CTAs resident at one time read the same
+// k-blocks (shared in L2).  The kernel is persistent: CTA c takes units c, c +
+// gridDim.x, ...; the stage ring and the accumulator ping-pong run on across
+// units, so the next unit's operands stream in while the epilogue finishes the
+// last one.  The MMA thread alternates between two TMEM accumulators, one per
+// sub-chunk of kSubKB k-blocks; the epilogue warps drain a finished sub-chunk
+// (complex combination, compensated FP32 sums held in registers) while the
+// other one fills, so the tensor core's FP32 accumulation never runs longer
+// than kSubKB * 64 transitions.
+// Each k-block stages Ah, Al (128 rows) and Bh, Bl (256 rows, two TMA boxes
+// each) and issues 12 tcgen05.mma of 128 x 256 x 16, so one operand byte feeds
+// twice the products of a 128 x 128 tile (half the shared-memory and L2 traffic
+// per product of A, and twice the work per stage in flight).  Two stages of 96 KB.  The
 // accumulators take all 512 TMEM columns (two of 256, ping-pong); eight
 // epilogue warps drain them, two per TMEM lane quadrant, each holding the
-// compensated sums of 128 of the 256 columns (as many as the narrow kernel's
-// four).  Warps 0..3 (producer, MMA issuer, two idle) give registers to the
+// compensated sums of 128 of the 256 columns.  Warps 0..3 (producer, MMA issuer, two idle) give registers to the
 // epilogue warpgroups: 384 threads launched at 144 registers (55,296), then
 // 4 x 32 x 40 + 8 x 32 x 192 = 54,272 after the hand-over, which leaves a
 // 128-thread, 64-register Dyson block room beside it (10,240 registers,
@@ -836,33 +580,26 @@ k_prep(const float2* __restrict__ R, int ngrp, int64_t nt, int ng, int mpad, con
 
 // chi[i][j] (i >= j) = sum over chunks of the partials (FP64), mirrored.
 // Position of the complex entry (i, j), i >= j, among the Hermitian
-// contraction's partial tiles: narrow 64 x 64 tiles in lower-triangle order,
-// or wide 64 x 128 tiles (I = i / 64, J = j / 128, I >= 2J) column by column.
-__device__ __forceinline__ void herm_pos(int i, int j, int wide, int nI, int& tile, size_t& off) {
-  if (wide) {
-    const int I = i / (kBM / 2), J = j / (kWN / 2);
-    tile = J * nI - J * (J - 1) + (I - 2 * J);
-    off = (size_t)(i % (kBM / 2)) * (kWN / 2) + (j % (kWN / 2));
-  } else {
-    const int I = i / (kBM / 2), J = j / (kBN / 2);
-    tile = I * (I + 1) / 2 + J;
-    off = (size_t)(i % (kBM / 2)) * (kBN / 2) + (j % (kBN / 2));
-  }
+// contraction's partial tiles: 64 x 128 complex tiles (I = i / 64, J = j / 128,
+// I >= 2J) column by column.
+__device__ __forceinline__ void herm_pos(int i, int j, int nI, int& tile, size_t& off) {
+  const int I = i / (kBM / 2), J = j / (kWN / 2);
+  tile = J * nI - J * (J - 1) + (I - 2 * J);
+  off = (size_t)(i % (kBM / 2)) * (kWN / 2) + (j % (kWN / 2));
 }
 
 __global__ void k_tc_reduce(const double2* __restrict__ part, int nchunks, int ntiles, int ng,
-                            double2* __restrict__ chi, int accumulate, int wide, int nI, int tile_elems,
-                            double sign) {
+                            double2* __restrict__ chi, int accumulate, int nI, double sign) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ng * ng) return;
   const int i = (int)(e / ng), j = (int)(e % ng);
   if (i < j) return;
   int tile;
   size_t off;
-  herm_pos(i, j, wide, nI, tile, off);
+  herm_pos(i, j, nI, tile, off);
   double sx = 0.0, sy = 0.0;
   for (int c = 0; c < nchunks; ++c) {
-    const double2 v = part[((size_t)c * ntiles + tile) * tile_elems + off];
+    const double2 v = part[((size_t)c * ntiles + tile) * kWPart + off];
     sx += v.x;
     sy += v.y;
   }
@@ -879,19 +616,17 @@ __global__ void k_tc_reduce(const double2* __restrict__ part, int nchunks, int n
 }
 
 // chi[i][j] = sum over chunks of the partials of the full tile grid (A rows i,
-// B rows j: tile (i / 64) + (j / cols) nT with cols = 64 complex columns per
-// 128 x 128 tile or 128 per 128 x 256 tile), every entry (no Hermitian
-// symmetry).
+// B rows j: tile (i / 64) + (j / 128) nT), every entry (no Hermitian symmetry).
 __global__ void k_tc_reduce_full(const double2* __restrict__ part, int nchunks, int ntiles, int nT, int ng,
-                                 double2* __restrict__ chi, int accumulate, int cols) {
+                                 double2* __restrict__ chi, int accumulate) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ng * ng) return;
   const int i = (int)(e / ng), j = (int)(e % ng);
-  const int tile = i / (kBM / 2) + (j / cols) * nT;
-  const size_t off = (size_t)(i % (kBM / 2)) * cols + (j % cols);
+  const int tile = i / (kBM / 2) + (j / (kWN / 2)) * nT;
+  const size_t off = (size_t)(i % (kBM / 2)) * (kWN / 2) + (j % (kWN / 2));
   double sx = 0.0, sy = 0.0;
   for (int c = 0; c < nchunks; ++c) {
-    const double2 v = part[((size_t)c * ntiles + tile) * (kBM / 2) * cols + off];
+    const double2 v = part[((size_t)c * ntiles + tile) * kWPart + off];
     sx += v.x;
     sy += v.y;
   }
@@ -910,24 +645,14 @@ struct TcState {
   int ntiles_f = 0, kbpc_f = 0, nchunks_f = 0;   // full tile grid (complex weights)
   int group = 1;  // frequencies per operand-split pass (A buffers in use)
   int nsm = 1;    // persistent contraction grid
-  // Hermitian contraction: wide tiles (128 x 256, k_herk_wide) or narrow ones
-  // (128 x 128, k_herk_bf16x3); nI row tiles of 128 (and nJ column tiles of
-  // 256 when wide); tile_elems complex entries per partial tile
-  int wide = 1, nI = 0, nJ = 0, tile_elems = (kBM / 2) * (kBN / 2);
+  int nI = 0, nJ = 0;   // row tiles of 128 and column tiles of 256 of the Hermitian contraction
 };
 
 // Tile layout of the Hermitian contraction for an operand of mpad rows.
 void herm_tiles(TcState& t) {
   t.nI = t.mpad / kBM;
-  if (t.wide) {
-    t.nJ = t.mpad / kWN;
-    t.ntiles = t.nI * t.nJ - t.nJ * (t.nJ - 1);
-    t.tile_elems = kWPart;
-  } else {
-    t.nJ = t.nI;
-    t.ntiles = t.nI * (t.nI + 1) / 2;
-    t.tile_elems = (kBM / 2) * (kBN / 2);
-  }
+  t.nJ = t.mpad / kWN;
+  t.ntiles = t.nI * t.nJ - t.nJ * (t.nJ - 1);
 }
 
 // One Hermitian contraction launch (lower-triangle tiles x transition splits).
@@ -937,14 +662,9 @@ cudaError_t launch_herm(chi0_ctx* c, TcState& t, int g, int kbpc, int nunits, co
   const unsigned grid = (unsigned)std::min(nunits, std::max(1, t.nsm));
   const CUtensorMap& mbh = one_op ? t.m_ah[g] : t.m_bh;
   const CUtensorMap& mbl = one_op ? t.m_al[g] : t.m_bl;
-  if (t.wide)
-    k_herk_wide<<<grid, kWThreads, kWSmemBytes, c->st>>>(t.m_ah[g], t.m_al[g], mbh, mbl, t.total_kb, kbpc, t.mpad,
-                                                          (double2*)t.part.p, t.ntiles, nunits, (int*)c->d_err.p,
-                                                          t.nI, ranges, 0, t.mpad, 0);
-  else
-    k_herk_bf16x3<<<grid, kThreads, kSmemBytes, c->st>>>(t.m_ah[g], t.m_al[g], mbh, mbl, t.total_kb, kbpc, t.mpad,
-                                                          (double2*)t.part.p, t.ntiles, nunits, (int*)c->d_err.p, 0,
-                                                          t.mpad, 0, ranges);
+  k_herk_wide<<<grid, kWThreads, kWSmemBytes, c->st>>>(t.m_ah[g], t.m_al[g], mbh, mbl, t.total_kb, kbpc, t.mpad,
+                                                        (double2*)t.part.p, t.ntiles, nunits, (int*)c->d_err.p,
+                                                        t.nI, ranges, 0, t.mpad, 0);
   return cudaGetLastError();
 }
 
@@ -979,7 +699,6 @@ bool make_map(CUtensorMap* m, void* ptr, int64_t kpad, int mpad) {
 chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   if (!c->tc) c->tc = new TcState();
   TcState& t = *static_cast<TcState*>(c->tc);
-  t.wide = 1;
   t.mpad = (2 * ng + kWN - 1) / kWN * kWN;   // a multiple of the wide tile's 256 columns
   t.kpad = (nt + kBK - 1) / kBK * kBK;
   const int nT = t.mpad / kBM;
@@ -1014,8 +733,7 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   };
   choose_split(t.ntiles, t.kbpc, t.nchunks);
   // the full tile grid of the complex contraction of a real-axis frequency
-  // (128 x 256 tiles with the wide kernel)
-  t.ntiles_f = t.wide ? nT * (t.mpad / kWN) : nT * nT;
+  t.ntiles_f = nT * (t.mpad / kWN);
   choose_split(t.ntiles_f, t.kbpc_f, t.nchunks_f);
   if (t.kpad / kPT > 0x7fffffff / t.mpad)
     return ctx_fail(c, CHI0_EUNSUPPORTED, "too many transitions for one contraction");
@@ -1031,9 +749,8 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   // a batch problem (group_cap > 0) keeps room for twice the planned
   // partials, for the split candidates of tc_tune_split
   const size_t room = c->group_cap > 0 ? 2 : 1;
-  const size_t nbytes = std::max((size_t)t.nchunks * t.ntiles * room * t.tile_elems,
-                                  c->has_real ? (size_t)t.nchunks_f * t.ntiles_f * (kBM / 2) * (t.wide ? kWN : kBN) / 2
-                                              : (size_t)0);
+  const size_t nbytes = std::max((size_t)t.nchunks * t.ntiles * room * kWPart,
+                                  c->has_real ? (size_t)t.nchunks_f * t.ntiles_f * kWPart : (size_t)0);
   if ((s = ctx_ensure(c, t.part, nbytes * 16, "chunk partials")) != CHI0_OK)
     return s;
   // A buffers for up to kPrepGroup frequencies, as far as half of the free
@@ -1059,10 +776,7 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   }
   if (need_b && (!make_map(&t.m_bh, t.bh.p, t.kpad, t.mpad) || !make_map(&t.m_bl, t.bl.p, t.kpad, t.mpad)))
     return ctx_fail(c, CHI0_ECUDA, "cuTensorMapEncodeTiled failed");
-  cudaError_t e = cudaFuncSetAttribute(k_herk_bf16x3, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_herk_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(k_herk_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmemBytes);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_herk_wide, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
@@ -1070,9 +784,6 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   // an SM running a contraction CTA (193 KB) keeps room for the small blocks
   // of the Dyson step of the previous frequency (a carveout sized to the CTA
   // alone would leave none).
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_herk_bf16x3, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_prep, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
@@ -1096,19 +807,19 @@ namespace {
 constexpr int kCombW = 8;
 __global__ void __launch_bounds__(256)
 k_grp_combine(const double2* __restrict__ part, const float* __restrict__ F, int ngroups, int ntiles, int ng,
-              int w0, int nwc, double2* __restrict__ chi, int wide, int nI, int tile_elems) {
+              int w0, int nwc, double2* __restrict__ chi, int nI) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ng * ng) return;
   const int i = (int)(e / ng), j = (int)(e % ng);
   if (i < j) return;
   int tile;
   size_t off;
-  herm_pos(i, j, wide, nI, tile, off);
+  herm_pos(i, j, nI, tile, off);
   float sx[kCombW], sy[kCombW], cx[kCombW], cy[kCombW];
 #pragma unroll
   for (int w = 0; w < kCombW; ++w) sx[w] = sy[w] = cx[w] = cy[w] = 0.f;
   for (int g = 0; g < ngroups; ++g) {
-    const double2 p = part[((size_t)g * ntiles + tile) * tile_elems + off];
+    const double2 p = part[((size_t)g * ntiles + tile) * kWPart + off];
     const float px = (float)p.x, py = (float)p.y;
 #pragma unroll
     for (int w = 0; w < kCombW; ++w) {
@@ -1137,7 +848,6 @@ k_grp_combine(const double2* __restrict__ part, const float* __restrict__ F, int
 chi0_status tc_plan_grouped(chi0_ctx* c, int ng, int nw) {
   if (!c->tc) c->tc = new TcState();
   TcState& t = *static_cast<TcState*>(c->tc);
-  t.wide = 1;
   t.mpad = (2 * ng + kWN - 1) / kWN * kWN;
   t.kpad = c->kgrp;
   herm_tiles(t);
@@ -1154,16 +864,11 @@ chi0_status tc_plan_grouped(chi0_ctx* c, int ng, int nw) {
   DevBuf* ops[] = {&t.ah[0], &t.al[0]};   // one operand (S S^H form)
   for (DevBuf* b : ops)
     if ((s = ctx_ensure(c, *b, opb, "grouped operands")) != CHI0_OK) return s;
-  if ((s = ctx_ensure(c, t.part, (size_t)c->ngroups * t.ntiles * t.tile_elems * 16, "group sums")) != CHI0_OK)
+  if ((s = ctx_ensure(c, t.part, (size_t)c->ngroups * t.ntiles * kWPart * 16, "group sums")) != CHI0_OK)
     return s;
   if (!make_map(&t.m_ah[0], t.ah[0].p, t.kpad, t.mpad) || !make_map(&t.m_al[0], t.al[0].p, t.kpad, t.mpad))
     return ctx_fail(c, CHI0_ECUDA, "cuTensorMapEncodeTiled failed");
-  cudaError_t e = cudaFuncSetAttribute(k_herk_bf16x3, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_herk_bf16x3, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_herk_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(k_herk_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmemBytes);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_herk_wide, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
@@ -1202,12 +907,12 @@ chi0_status tc_launch_grouped(chi0_ctx* c, double2* chi, const cudaEvent_t* ev_f
   for (int w0 = 0; w0 < nw; w0 += kCombW, ++nlaunch) {
     const int nwc = std::min(kCombW, nw - w0);
     k_grp_combine<<<cgrid, 256, 0, c->st>>>((const double2*)t.part.p, (const float*)c->d_gfac.p, c->ngroups,
-                                            t.ntiles, ng, w0, nwc, chi, t.wide, t.nI, t.tile_elems);
+                                            t.ntiles, ng, w0, nwc, chi, t.nI);
     if (ev_freq)
       for (int w = w0; w < w0 + nwc; ++w) cudaEventRecord(ev_freq[w], c->st);
   }
   stage_end(c, CHI0_STAGE_REDUCE, nlaunch);
-  const double tile_bytes = (double)t.tile_elems * 16;
+  const double tile_bytes = (double)kWPart * 16;
   c->stage[CHI0_STAGE_WEIGHTS].bytes = (double)c->nt * ng * 8 + 4.0 * t.mpad * t.kpad;
   c->stage[CHI0_STAGE_CONTRACT].bytes = 4.0 * t.mpad * t.kpad + (double)nunits * tile_bytes;
   // the work done: one Hermitian contraction over the transitions in group
@@ -1215,7 +920,7 @@ chi0_status tc_launch_grouped(chi0_ctx* c, double2* chi, const cudaEvent_t* ev_f
   c->stage[CHI0_STAGE_CONTRACT].flops = 4.0 * (double)ng * (ng + 1) * (double)t.kpad;
   c->stage[CHI0_STAGE_REDUCE].flops = 2.0 * (double)ng * (ng + 1) * (double)c->ngroups * nw;
   c->stage[CHI0_STAGE_REDUCE].bytes = (double)nlaunch * nunits * tile_bytes + (double)n2 * nw * 16;
-  c->tc_issued_flops = 3.0 * 2.0 * kBM * (t.wide ? kWN : kBN) * (double)t.kpad * t.ntiles;
+  c->tc_issued_flops = 3.0 * 2.0 * kBM * kWN * (double)t.kpad * t.ntiles;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return ctx_fail(c, CHI0_ECUDA, cudaGetErrorString(e));
   return CHI0_OK;
@@ -1287,14 +992,9 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
       double2* out = chi + (size_t)jb.v * n2;
       stage_begin(c, CHI0_STAGE_CONTRACT);
       if (jb.cplx) {
-        if (t.wide)
-          k_herk_wide<<<hgrid_f, kWThreads, kWSmemBytes, c->st>>>(
-              t.m_ah[g], t.m_al[g], t.m_bh, t.m_bl, t.total_kb, t.kbpc_f, t.mpad, (double2*)t.part.p, t.ntiles_f,
-              nunits_f, (int*)c->d_err.p, nT, nullptr, 1, t.mpad, 0);
-        else
-          k_herk_bf16x3<<<hgrid_f, kThreads, kSmemBytes, c->st>>>(
-              t.m_ah[g], t.m_al[g], t.m_bh, t.m_bl, t.total_kb, t.kbpc_f, t.mpad, (double2*)t.part.p, t.ntiles_f,
-              nunits_f, (int*)c->d_err.p, nT, t.mpad, 0, nullptr);
+        k_herk_wide<<<hgrid_f, kWThreads, kWSmemBytes, c->st>>>(
+            t.m_ah[g], t.m_al[g], t.m_bh, t.m_bl, t.total_kb, t.kbpc_f, t.mpad, (double2*)t.part.p, t.ntiles_f,
+            nunits_f, (int*)c->d_err.p, nT, nullptr, 1, t.mpad, 0);
         ++nfull;
       } else {
         launch_herm(c, t, g, t.kbpc, nunits, nullptr, one_op);
@@ -1304,11 +1004,11 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
       stage_begin(c, CHI0_STAGE_REDUCE);
       if (jb.cplx)
         k_tc_reduce_full<<<(unsigned)((n2 + 255) / 256), 256, 0, c->st>>>(
-            (const double2*)t.part.p, t.nchunks_f, t.ntiles_f, nT, ng, out, accumulate, (t.wide ? kWN : kBN) / 2);
+            (const double2*)t.part.p, t.nchunks_f, t.ntiles_f, nT, ng, out, accumulate);
       else
         k_tc_reduce<<<(unsigned)((n2 + 255) / 256), 256, 0, c->st>>>((const double2*)t.part.p, t.nchunks, t.ntiles,
-                                                                      ng, out, accumulate, t.wide, t.nI,
-                                                                      t.tile_elems, one_op ? (double)c->herk_sign : 1.0);
+                                                                      ng, out, accumulate, t.nI,
+                                                                      one_op ? (double)c->herk_sign : 1.0);
       int nk = 1;
       if (bg) {
         launch_bg_apply(bg->P + (size_t)jb.v * bg->nd, bg->didx, ng, bg->nd, 1, out, c->st, 0);
@@ -1325,8 +1025,7 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
       }
     }
   }
-  const double tile_bytes = (double)t.tile_elems * 16;
-  const double tile_bytes_f = (double)(kBM / 2) * ((t.wide ? kWN : kBN) / 2) * 16;
+  const double tile_bytes = (double)kWPart * 16;
   // operand split: R read once per pass, hi/lo written (B once if needed, A per job)
   c->stage[CHI0_STAGE_WEIGHTS].bytes += (double)(passes + (need_b ? 1 : 0)) * nt * ng * 8 +
                                         (double)(jobs.size() + (need_b ? 1 : 0)) * 4.0 * t.mpad * t.kpad;
@@ -1334,13 +1033,13 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
   // in the one-operand form and two otherwise, and writes its chunk partials
   c->stage[CHI0_STAGE_CONTRACT].bytes =
       (double)nherm * (one_op ? 4.0 : 8.0) * t.mpad * t.kpad + (double)nfull * 8.0 * t.mpad * t.kpad +
-      (double)nherm * t.nchunks * t.ntiles * tile_bytes + (double)nfull * t.nchunks_f * t.ntiles_f * tile_bytes_f;
+      (double)nherm * t.nchunks * t.ntiles * tile_bytes + (double)nfull * t.nchunks_f * t.ntiles_f * tile_bytes;
   c->stage[CHI0_STAGE_REDUCE].bytes =
-      (double)nherm * t.nchunks * t.ntiles * tile_bytes + (double)nfull * t.nchunks_f * t.ntiles_f * tile_bytes_f +
+      (double)nherm * t.nchunks * t.ntiles * tile_bytes + (double)nfull * t.nchunks_f * t.ntiles_f * tile_bytes +
       (double)(nherm + nfull) * n2 * 16;
   // tensor-core work actually issued: 3 BF16 products over the tiles of each launch
   c->tc_issued_flops = 3.0 * 2.0 * kBM * (double)t.kpad *
-                      ((double)(t.wide ? kWN : kBN) * (t.ntiles * nherm + t.ntiles_f * nfull));
+                      ((double)kWN * (t.ntiles * nherm + t.ntiles_f * nfull));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return ctx_fail(c, CHI0_ECUDA, cudaGetErrorString(e));
   return CHI0_OK;
@@ -1395,7 +1094,7 @@ chi0_status tc_tune_split(chi0_ctx* c, float* best_ms) {
   oa.wr[0] = (const double*)c->d_w.p;
   oa.sq[0] = one_op;
   k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)c->d_R.p, 1, weighted_rows(c), ng, t.mpad, oa, weighted_perm(c));
-  const size_t cap = t.part.bytes / ((size_t)t.tile_elems * 16);
+  const size_t cap = t.part.bytes / ((size_t)kWPart * 16);
   const int base_split = (t.total_kb + t.kbpc - 1) / t.kbpc;
   int best_kbpc = t.kbpc, best_n = t.nchunks;
   float best = 1e30f;
@@ -1467,7 +1166,7 @@ cudaError_t launch_wait_probe(int* err, cudaStream_t s) {
 // chi0 contraction, C_ij = sum_K A_K(i) conj(B_K(j)), with K = G' (ng values)
 // instead of the transitions: A = W^d (rows 2 i + c), B = rho of the
 // transitions t of the quasiparticle window (rows 2 t + c), the full grid of
-// 128 x 128 tiles, one k range per tile (no chunk partials: each tile's sum
+// 128 x 256 tiles, one k range per tile (no chunk partials: each tile's sum
 // is Y itself, rounded to FP32).  Transitions are ordered t = ((k nb) + m) nqp + a,
 // so that the partners a of one (k, m) are adjacent columns of Y.
 
