@@ -205,8 +205,10 @@ __device__ __forceinline__ void nsum(float& s, float& c, float x) {
 // 128-thread, 64-register Dyson block room beside it (10,240 registers,
 // 2,816 per sub-partition).
 // Tiles: (I, J) with I in [2J, nI), nI = mpad / 128 row tiles of A and nJ =
-// mpad / 256 column tiles of B (mpad a multiple of 256): every real entry
-// (r, c) with r >= c lies in one of them.  Tile index = sum_{J' < J} (nI - 2J')
+// ceil(mpad / 256) column tiles of B: every real entry (r, c) with r >= c lies
+// in one of them.  Where mpad is an odd multiple of 128, the second box of the
+// last column tile reads the first rows of the next k-block (zeros after the
+// last one): its columns lie beyond the matrix and nothing reads their sums.  Tile index = sum_{J' < J} (nI - 2J')
 // + (I - 2J).  Partial output: 64 complex rows x 128 complex columns per
 // unit.
 constexpr int kWN = 256;                          // tile cols (real)
@@ -235,12 +237,25 @@ __device__ __forceinline__ void setmaxnreg_inc192() {
   asm volatile("setmaxnreg.inc.sync.aligned.u32 192;" ::: "memory");
 }
 
+// Operands of one launch: A (hi, lo) of up to kPrepGroup frequencies, and B (hi,
+// lo) common to them, or A's own where both tiles come from one operand.
+constexpr int kPrepGroup = 8;
+struct HerkMaps {
+  CUtensorMap ah[kPrepGroup], al[kPrepGroup], bh, bl;
+  int own;   // 1: B is A's operand
+};
+
+// Units of several frequencies (upf each, frequency by frequency) in one launch:
+// with few tiles and transitions a launch per frequency leaves SMs idle or
+// splits the transitions so finely that the chunk partials and the ramp of
+// each unit cost more than its products.  N_G = 431 with 58 k rows: 200 -> 142 us
+// per frequency (four per launch, and 16 tiles in place of 20: rows padded to
+// 128), N_G = 220 with 61 k rows: 105 -> 51 us (eight), 24 real frequencies of N_G =
+// 400: 498 -> 394 us each (four).
 __global__ void __maxnreg__(144)
-k_herk_wide(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ CUtensorMap tm_al,
-            const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CUtensorMap tm_bl, int total_kb,
-            int kb_per_split, int mpad, double2* __restrict__ part, int ntiles, int nunits,
-            int* __restrict__ err, int nI, const int2* __restrict__ ranges, int full, int mpad_b,
-            int f32out) {
+k_herk_wide(const __grid_constant__ HerkMaps maps, int total_kb, int kb_per_split, int mpad,
+            double2* __restrict__ part, int ntiles, int upf, int nunits, int* __restrict__ err, int nI,
+            const int2* __restrict__ ranges, int full, int mpad_b, int f32out, size_t f32stride) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -260,7 +275,7 @@ k_herk_wide(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ C
     __syncthreads();
     if (*skip) return;
   }
-  auto unit_range = [&](int u, int& kb0, int& nkb) {
+  auto unit_range = [&](int u, int& kb0, int& nkb) {   // u within its frequency
     if (ranges) {
       const int2 r = ranges[u / ntiles];
       kb0 = r.x;
@@ -283,11 +298,9 @@ k_herk_wide(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ C
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0 && lane == 0) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tm_ah) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tm_al) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tm_bh) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tm_bl) : "memory");
+  if (warp == 0 && lane < (nunits + upf - 1) / upf) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&maps.ah[lane]) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&maps.al[lane]) : "memory");
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 2 * kWN);
   tc_fence_before();
@@ -301,8 +314,11 @@ k_herk_wide(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ C
       // ---------------- TMA producer
       int gk = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+      for (int uu = blockIdx.x; uu < nunits && ok; uu += gridDim.x) {
         int I, J, kb0, nkb;
+        const int g = uu / upf, u = uu - g * upf;
+        const CUtensorMap *tm_ah = &maps.ah[g], *tm_al = &maps.al[g];
+        const CUtensorMap *tm_bh = maps.own ? tm_ah : &maps.bh, *tm_bl = maps.own ? tm_al : &maps.bl;
         if (full) {   // every tile: I fastest
           I = (u % ntiles) % nI;
           J = (u % ntiles) / nI;
@@ -320,12 +336,12 @@ k_herk_wide(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ C
           const uint32_t sb = base + st * kWStageBytes;
           mbar_expect_tx(bar_full + 8 * st, kWStageBytes);
           const int row = (kb0 + k) * mpad, rowb = (kb0 + k) * mpad_b;
-          tma_load_2d(sb, &tm_ah, 0, row + I * kBM, bar_full + 8 * st);
-          tma_load_2d(sb + kWTileA, &tm_al, 0, row + I * kBM, bar_full + 8 * st);
-          tma_load_2d(sb + 2 * kWTileA, &tm_bh, 0, rowb + J * kWN, bar_full + 8 * st);
-          tma_load_2d(sb + 2 * kWTileA + kWTileA, &tm_bh, 0, rowb + J * kWN + kBM, bar_full + 8 * st);
-          tma_load_2d(sb + 2 * kWTileA + kWTileB, &tm_bl, 0, rowb + J * kWN, bar_full + 8 * st);
-          tma_load_2d(sb + 2 * kWTileA + kWTileB + kWTileA, &tm_bl, 0, rowb + J * kWN + kBM, bar_full + 8 * st);
+          tma_load_2d(sb, tm_ah, 0, row + I * kBM, bar_full + 8 * st);
+          tma_load_2d(sb + kWTileA, tm_al, 0, row + I * kBM, bar_full + 8 * st);
+          tma_load_2d(sb + 2 * kWTileA, tm_bh, 0, rowb + J * kWN, bar_full + 8 * st);
+          tma_load_2d(sb + 2 * kWTileA + kWTileA, tm_bh, 0, rowb + J * kWN + kBM, bar_full + 8 * st);
+          tma_load_2d(sb + 2 * kWTileA + kWTileB, tm_bl, 0, rowb + J * kWN, bar_full + 8 * st);
+          tma_load_2d(sb + 2 * kWTileA + kWTileB + kWTileA, tm_bl, 0, rowb + J * kWN + kBM, bar_full + 8 * st);
         }
       }
     } else if (warp == 1 && lane == 0) {
@@ -335,7 +351,7 @@ k_herk_wide(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ C
       bool ok = true;
       for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
         int kb0, nkb;
-        unit_range(u, kb0, nkb);
+        unit_range(u % upf, kb0, nkb);
         const int nsub = (nkb + kSubKB - 1) / kSubKB;
         int k = 0;
         for (int sc = 0; sc < nsub; ++sc, ++gsc) {
@@ -385,7 +401,7 @@ k_herk_wide(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ C
     bool ok = true;
     for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
       int kb0, nkb;
-      unit_range(u, kb0, nkb);
+      unit_range(u % upf, kb0, nkb);
       const int nsub = (nkb + kSubKB - 1) / kSubKB;
       float accs[32][2], accc[32][2];
 #pragma unroll
@@ -429,9 +445,9 @@ k_herk_wide(const __grid_constant__ CUtensorMap tm_ah, const __grid_constant__ C
         // complex tiles of the full grid of 128-row B tiles: this warp's 64
         // columns are tile I + (2 J + hcol) nI (one k range per tile), which
         // exists while its B rows lie within mpad_b
-        const int tile = u % ntiles, I = tile % nI, Jn = 2 * (tile / nI) + hcol;
+        const int tile = u % upf % ntiles, I = tile % nI, Jn = 2 * (tile / nI) + hcol;
         if (Jn * kBN < mpad_b) {
-          float2* out = reinterpret_cast<float2*>(part) + ((size_t)Jn * nI + I) * (size_t)(kBM / 2) * (kBN / 2) +
+          float2* out = reinterpret_cast<float2*>(part) + (u / upf) * f32stride + ((size_t)Jn * nI + I) * (size_t)(kBM / 2) * (kBN / 2) +
                         (size_t)il * (kBN / 2) + (odd ? 4 : 0);
 #pragma unroll
           for (int cb = 0; cb < kBN / 16; ++cb)
@@ -480,7 +496,6 @@ constexpr int kPI = 32;  // complex G per tile
 // -2.8e-6 relative on every chi0_ii, where the two-operand form's dropped
 // terms have no sign); the split then stores lo' = lo + lo^2 / (2 hi) in
 // place of lo, which makes the diagonal's products hi^2 + 2 hi lo' = x^2.
-constexpr int kPrepGroup = 8;
 struct PrepOut {
   __nv_bfloat16* hi[kPrepGroup];
   __nv_bfloat16* lo[kPrepGroup];
@@ -592,6 +607,8 @@ __global__ void k_tc_reduce(const double2* __restrict__ part, int nchunks, int n
                             double2* __restrict__ chi, int accumulate, int nI, double sign) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ng * ng) return;
+  part += (size_t)blockIdx.y * nchunks * ntiles * kWPart;   // frequency of the launch
+  chi += (size_t)blockIdx.y * ng * ng;
   const int i = (int)(e / ng), j = (int)(e % ng);
   if (i < j) return;
   int tile;
@@ -621,6 +638,8 @@ __global__ void k_tc_reduce_full(const double2* __restrict__ part, int nchunks, 
                                  double2* __restrict__ chi, int accumulate) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ng * ng) return;
+  part += (size_t)blockIdx.y * nchunks * ntiles * kWPart;
+  chi += (size_t)blockIdx.y * 2 * ng * ng;   // (each real frequency is two entries of the list)
   const int i = (int)(e / ng), j = (int)(e % ng);
   const int tile = i / (kBM / 2) + (j / (kWN / 2)) * nT;
   const size_t off = (size_t)(i % (kBM / 2)) * (kWN / 2) + (j % (kWN / 2));
@@ -639,10 +658,13 @@ __global__ void k_tc_reduce_full(const double2* __restrict__ part, int nchunks, 
 
 struct TcState {
   DevBuf ah[kPrepGroup], al[kPrepGroup], bh, bl, part;
-  CUtensorMap m_ah[kPrepGroup], m_al[kPrepGroup], m_bh, m_bl;
+  HerkMaps maps{};
   int64_t kpad = 0;
-  int mpad = 0, ntiles = 0, total_kb = 0, kbpc = 0, nchunks = 0;
-  int ntiles_f = 0, kbpc_f = 0, nchunks_f = 0;   // full tile grid (complex weights)
+  // tiles, k-blocks per split, splits, and frequencies per launch of the
+  // contraction over the lower triangle and over the full tile grid (complex
+  // weights)
+  int mpad = 0, ntiles = 0, total_kb = 0, kbpc = 0, nchunks = 0, per = 1;
+  int ntiles_f = 0, kbpc_f = 0, nchunks_f = 0, per_f = 1;
   int group = 1;  // frequencies per operand-split pass (A buffers in use)
   int nsm = 1;    // persistent contraction grid
   int nI = 0, nJ = 0;   // row tiles of 128 and column tiles of 256 of the Hermitian contraction
@@ -651,20 +673,27 @@ struct TcState {
 // Tile layout of the Hermitian contraction for an operand of mpad rows.
 void herm_tiles(TcState& t) {
   t.nI = t.mpad / kBM;
-  t.nJ = t.mpad / kWN;
+  t.nJ = (t.mpad + kWN - 1) / kWN;
   t.ntiles = t.nI * t.nJ - t.nJ * (t.nJ - 1);
 }
 
-// One Hermitian contraction launch (lower-triangle tiles x transition splits).
-// one_op: the one-operand form D = S S^T, both tiles read from operand g;
-// otherwise A is operand g and B the unit-weight operand.
-cudaError_t launch_herm(chi0_ctx* c, TcState& t, int g, int kbpc, int nunits, const int2* ranges, bool one_op) {
+// Contraction of the nf operands from A buffer g0 on: over the lower-triangle
+// tiles (one_op: the one-operand form D = S S^T, both tiles read from an
+// operand; otherwise B is the unit-weight operand), or over the full grid.
+cudaError_t launch_herm(chi0_ctx* c, TcState& t, int g0, int nf, int kbpc, int nchunks, const int2* ranges,
+                        bool one_op, bool full) {
+  HerkMaps m;
+  for (int g = 0; g < nf; ++g) {
+    m.ah[g] = t.maps.ah[g0 + g];
+    m.al[g] = t.maps.al[g0 + g];
+  }
+  m.bh = t.maps.bh;
+  m.bl = t.maps.bl;
+  m.own = one_op;
+  const int ntiles = full ? t.ntiles_f : t.ntiles, upf = ntiles * nchunks, nunits = upf * nf;
   const unsigned grid = (unsigned)std::min(nunits, std::max(1, t.nsm));
-  const CUtensorMap& mbh = one_op ? t.m_ah[g] : t.m_bh;
-  const CUtensorMap& mbl = one_op ? t.m_al[g] : t.m_bl;
-  k_herk_wide<<<grid, kWThreads, kWSmemBytes, c->st>>>(t.m_ah[g], t.m_al[g], mbh, mbl, t.total_kb, kbpc, t.mpad,
-                                                        (double2*)t.part.p, t.ntiles, nunits, (int*)c->d_err.p,
-                                                        t.nI, ranges, 0, t.mpad, 0);
+  k_herk_wide<<<grid, kWThreads, kWSmemBytes, c->st>>>(m, t.total_kb, kbpc, t.mpad, (double2*)t.part.p, ntiles, upf,
+                                                        nunits, (int*)c->d_err.p, t.nI, ranges, full, t.mpad, 0, 0);
   return cudaGetLastError();
 }
 
@@ -699,7 +728,7 @@ bool make_map(CUtensorMap* m, void* ptr, int64_t kpad, int mpad) {
 chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   if (!c->tc) c->tc = new TcState();
   TcState& t = *static_cast<TcState*>(c->tc);
-  t.mpad = (2 * ng + kWN - 1) / kWN * kWN;   // a multiple of the wide tile's 256 columns
+  t.mpad = (2 * ng + kBM - 1) / kBM * kBM;
   t.kpad = (nt + kBK - 1) / kBK * kBK;
   const int nT = t.mpad / kBM;
   herm_tiles(t);
@@ -713,46 +742,7 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
     cudaGetLastError();
   }
   t.nsm = nsm;
-  auto choose_split = [&](int ntiles, int& kbpc, int& nchunks) {
-    int nsplit = 1;
-    double best = 1e30;
-    for (int sp = 1; sp <= 64; ++sp) {
-      const int kbps = (t.total_kb + sp - 1) / sp;
-      if (sp > 1 && kbps < 8 * kSubKB) break;  // keep every CTA busy for a while
-      const int ctas = ntiles * sp;
-      const int waves = (ctas + nsm - 1) / nsm;
-      // time ~ waves * work per CTA; prefer fewer partials on ties
-      const double cost = (double)waves * kbps + 4.0 * sp;
-      if (cost < best) {
-        best = cost;
-        nsplit = sp;
-      }
-    }
-    kbpc = (t.total_kb + nsplit - 1) / nsplit;
-    nchunks = (t.total_kb + kbpc - 1) / kbpc;
-  };
-  choose_split(t.ntiles, t.kbpc, t.nchunks);
-  // the full tile grid of the complex contraction of a real-axis frequency
-  t.ntiles_f = nT * (t.mpad / kWN);
-  choose_split(t.ntiles_f, t.kbpc_f, t.nchunks_f);
-  if (t.kpad / kPT > 0x7fffffff / t.mpad)
-    return ctx_fail(c, CHI0_EUNSUPPORTED, "too many transitions for one contraction");
   const size_t opb = (size_t)t.mpad * t.kpad * 2;
-  chi0_status s;
-  // the unit-weight operand B is read only by the two-operand form (weights
-  // of mixed signs) and by the complex contractions of real frequencies
-  const bool need_b = c->herk_sign == 0 || c->has_real;
-  if (need_b) {
-    if ((s = ctx_ensure(c, t.bh, opb, "B hi")) != CHI0_OK) return s;
-    if ((s = ctx_ensure(c, t.bl, opb, "B lo")) != CHI0_OK) return s;
-  }
-  // a batch problem (group_cap > 0) keeps room for twice the planned
-  // partials, for the split candidates of tc_tune_split
-  const size_t room = c->group_cap > 0 ? 2 : 1;
-  const size_t nbytes = std::max((size_t)t.nchunks * t.ntiles * room * kWPart,
-                                  c->has_real ? (size_t)t.nchunks_f * t.ntiles_f * kWPart : (size_t)0);
-  if ((s = ctx_ensure(c, t.part, nbytes * 16, "chunk partials")) != CHI0_OK)
-    return s;
   // A buffers for up to kPrepGroup frequencies, as far as half of the free
   // device memory allows (one pair is always needed)
   {
@@ -768,13 +758,56 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
     while (g > std::max(1, have) && (double)(g - have) * 2.0 * (double)opb > 0.5 * (double)free_b) --g;
     t.group = g;
   }
+  // Splits of the transitions and frequencies per launch, in units of one
+  // k-block's products (0.8 us): whole waves of one CTA per SM, each unit 3
+  // for its ramp and the write of its partial, each launch 8, and each split of
+  // a tile 0.06 for the partial that the reduction reads.  More frequencies
+  // per launch only where that gains over a per cent each: their results come
+  // together, and the Dyson step of the first waits for the last.
+  auto choose_split = [&](int ntiles, int& kbpc, int& nchunks, int& per) {
+    double best = 1e30;
+    for (int nf = 1; nf <= t.group; nf *= 2)
+      for (int sp = 1; sp <= 64; ++sp) {
+        const int kbps = (t.total_kb + sp - 1) / sp;
+        if (sp > 1 && kbps < 8 * kSubKB) break;  // keep every CTA busy for a while
+        const int64_t waves = ((int64_t)ntiles * sp * nf + nsm - 1) / nsm;
+        const double cost = ((double)(waves * (kbps + 3) + 8) / nf + 0.06 * ntiles * sp) * (1.0 + 0.01 * nf);
+        if (cost < best) {
+          best = cost;
+          kbpc = kbps;
+          per = nf;
+        }
+      }
+    nchunks = (t.total_kb + kbpc - 1) / kbpc;
+  };
+  choose_split(t.ntiles, t.kbpc, t.nchunks, t.per);
+  // the full tile grid of the complex contraction of a real-axis frequency
+  t.ntiles_f = nT * t.nJ;
+  choose_split(t.ntiles_f, t.kbpc_f, t.nchunks_f, t.per_f);
+  if (t.kpad / kPT > 0x7fffffff / t.mpad)
+    return ctx_fail(c, CHI0_EUNSUPPORTED, "too many transitions for one contraction");
+  chi0_status s;
+  // the unit-weight operand B is read only by the two-operand form (weights
+  // of mixed signs) and by the complex contractions of real frequencies
+  const bool need_b = c->herk_sign == 0 || c->has_real;
+  if (need_b) {
+    if ((s = ctx_ensure(c, t.bh, opb, "B hi")) != CHI0_OK) return s;
+    if ((s = ctx_ensure(c, t.bl, opb, "B lo")) != CHI0_OK) return s;
+  }
+  // a batch problem (group_cap > 0) keeps room for twice the planned
+  // partials, for the split candidates of tc_tune_split
+  const size_t room = c->group_cap > 0 ? 2 : 1;
+  const size_t nbytes = std::max((size_t)t.per * t.nchunks * t.ntiles * room * kWPart,
+                                  c->has_real ? (size_t)t.per_f * t.nchunks_f * t.ntiles_f * kWPart : (size_t)0);
+  if ((s = ctx_ensure(c, t.part, nbytes * 16, "chunk partials")) != CHI0_OK)
+    return s;
   for (int g = 0; g < t.group; ++g) {
     if ((s = ctx_ensure(c, t.ah[g], opb, "A hi")) != CHI0_OK) return s;
     if ((s = ctx_ensure(c, t.al[g], opb, "A lo")) != CHI0_OK) return s;
-    if (!make_map(&t.m_ah[g], t.ah[g].p, t.kpad, t.mpad) || !make_map(&t.m_al[g], t.al[g].p, t.kpad, t.mpad))
+    if (!make_map(&t.maps.ah[g], t.ah[g].p, t.kpad, t.mpad) || !make_map(&t.maps.al[g], t.al[g].p, t.kpad, t.mpad))
       return ctx_fail(c, CHI0_ECUDA, "cuTensorMapEncodeTiled failed");
   }
-  if (need_b && (!make_map(&t.m_bh, t.bh.p, t.kpad, t.mpad) || !make_map(&t.m_bl, t.bl.p, t.kpad, t.mpad)))
+  if (need_b && (!make_map(&t.maps.bh, t.bh.p, t.kpad, t.mpad) || !make_map(&t.maps.bl, t.bl.p, t.kpad, t.mpad)))
     return ctx_fail(c, CHI0_ECUDA, "cuTensorMapEncodeTiled failed");
   cudaError_t e = cudaFuncSetAttribute(k_herk_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmemBytes);
   if (e == cudaSuccess)
@@ -848,7 +881,7 @@ k_grp_combine(const double2* __restrict__ part, const float* __restrict__ F, int
 chi0_status tc_plan_grouped(chi0_ctx* c, int ng, int nw) {
   if (!c->tc) c->tc = new TcState();
   TcState& t = *static_cast<TcState*>(c->tc);
-  t.mpad = (2 * ng + kWN - 1) / kWN * kWN;
+  t.mpad = (2 * ng + kBM - 1) / kBM * kBM;
   t.kpad = c->kgrp;
   herm_tiles(t);
   t.total_kb = (int)(t.kpad / kBK);
@@ -866,7 +899,7 @@ chi0_status tc_plan_grouped(chi0_ctx* c, int ng, int nw) {
     if ((s = ctx_ensure(c, *b, opb, "grouped operands")) != CHI0_OK) return s;
   if ((s = ctx_ensure(c, t.part, (size_t)c->ngroups * t.ntiles * kWPart * 16, "group sums")) != CHI0_OK)
     return s;
-  if (!make_map(&t.m_ah[0], t.ah[0].p, t.kpad, t.mpad) || !make_map(&t.m_al[0], t.al[0].p, t.kpad, t.mpad))
+  if (!make_map(&t.maps.ah[0], t.ah[0].p, t.kpad, t.mpad) || !make_map(&t.maps.al[0], t.al[0].p, t.kpad, t.mpad))
     return ctx_fail(c, CHI0_ECUDA, "cuTensorMapEncodeTiled failed");
   cudaError_t e = cudaFuncSetAttribute(k_herk_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmemBytes);
   if (e == cudaSuccess)
@@ -898,7 +931,7 @@ chi0_status tc_launch_grouped(chi0_ctx* c, double2* chi, const cudaEvent_t* ev_f
   // one unit per (tile, group): the group sums M_g, tile by tile
   const int nunits = t.ntiles * c->ngroups;
   stage_begin(c, CHI0_STAGE_CONTRACT);
-  launch_herm(c, t, 0, t.total_kb, nunits, (const int2*)c->d_grange.p, true);
+  launch_herm(c, t, 0, 1, t.total_kb, c->ngroups, (const int2*)c->d_grange.p, true, false);
   stage_end(c, CHI0_STAGE_CONTRACT, 1);
   // chi0 at every frequency from the group sums and the groups' factors
   const unsigned cgrid = (unsigned)((n2 + 255) / 256);
@@ -964,9 +997,6 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
     k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)R, 1, nt, ng, t.mpad, ob, perm);
     stage_end(c, CHI0_STAGE_WEIGHTS, 1);
   }
-  const int nunits = t.ntiles * t.nchunks, nunits_f = t.ntiles_f * t.nchunks_f;
-  const unsigned hgrid = (unsigned)std::min(nunits, std::max(1, t.nsm));
-  const unsigned hgrid_f = (unsigned)std::min(nunits_f, std::max(1, t.nsm));
   int passes = 0, nherm = 0, nfull = 0;
   for (size_t j0 = 0; j0 < jobs.size(); j0 += t.group, ++passes) {
     const int gw = (int)std::min<size_t>(t.group, jobs.size() - j0);
@@ -987,52 +1017,50 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
         cudaEventRecord(ev_prep[jobs[j0 + g].v], c->st);
         if (jobs[j0 + g].cplx) cudaEventRecord(ev_prep[jobs[j0 + g].v + 1], c->st);
       }
-    for (int g = 0; g < gw; ++g) {
-      const Job& jb = jobs[j0 + g];
-      double2* out = chi + (size_t)jb.v * n2;
+    // launches of up to per (per_f) jobs of one kind
+    for (int g = 0, nf; g < gw; g += nf) {
+      const bool cplx = jobs[j0 + g].cplx;
+      const int most = cplx ? t.per_f : t.per;
+      for (nf = 1; nf < most && g + nf < gw && jobs[j0 + g + nf].cplx == cplx;) ++nf;
+      const int v0 = jobs[j0 + g].v, step = cplx ? 2 : 1;   // entries v0, v0 + step, ...
+      double2* out = chi + (size_t)v0 * n2;
       stage_begin(c, CHI0_STAGE_CONTRACT);
-      if (jb.cplx) {
-        k_herk_wide<<<hgrid_f, kWThreads, kWSmemBytes, c->st>>>(
-            t.m_ah[g], t.m_al[g], t.m_bh, t.m_bl, t.total_kb, t.kbpc_f, t.mpad, (double2*)t.part.p, t.ntiles_f,
-            nunits_f, (int*)c->d_err.p, nT, nullptr, 1, t.mpad, 0);
-        ++nfull;
-      } else {
-        launch_herm(c, t, g, t.kbpc, nunits, nullptr, one_op);
-        ++nherm;
-      }
+      launch_herm(c, t, g, nf, cplx ? t.kbpc_f : t.kbpc, cplx ? t.nchunks_f : t.nchunks, nullptr, one_op && !cplx, cplx);
+      (cplx ? nfull : nherm) += nf;
       stage_end(c, CHI0_STAGE_CONTRACT, 1);
       stage_begin(c, CHI0_STAGE_REDUCE);
-      if (jb.cplx)
-        k_tc_reduce_full<<<(unsigned)((n2 + 255) / 256), 256, 0, c->st>>>(
-            (const double2*)t.part.p, t.nchunks_f, t.ntiles_f, nT, ng, out, accumulate);
+      const dim3 rgrid((unsigned)((n2 + 255) / 256), (unsigned)nf);
+      if (cplx)
+        k_tc_reduce_full<<<rgrid, 256, 0, c->st>>>((const double2*)t.part.p, t.nchunks_f, t.ntiles_f, nT, ng, out,
+                                                   accumulate);
       else
-        k_tc_reduce<<<(unsigned)((n2 + 255) / 256), 256, 0, c->st>>>((const double2*)t.part.p, t.nchunks, t.ntiles,
-                                                                      ng, out, accumulate, t.nI,
-                                                                      one_op ? (double)c->herk_sign : 1.0);
+        k_tc_reduce<<<rgrid, 256, 0, c->st>>>((const double2*)t.part.p, t.nchunks, t.ntiles, ng, out, accumulate, t.nI,
+                                              one_op ? (double)c->herk_sign : 1.0);
       int nk = 1;
-      if (bg) {
-        launch_bg_apply(bg->P + (size_t)jb.v * bg->nd, bg->didx, ng, bg->nd, 1, out, c->st, 0);
+      if (bg && !cplx) {
+        launch_bg_apply(bg->P + (size_t)v0 * bg->nd, bg->didx, ng, bg->nd, nf, out, c->st, 0);
         ++nk;
-        if (jb.cplx) {   // + i (Hermitised P of the imaginary parts)
-          launch_bg_apply(bg->P + (size_t)(jb.v + 1) * bg->nd, bg->didx, ng, bg->nd, 1, out, c->st, 1);
-          ++nk;
-        }
+      }
+      for (int q = 0; bg && cplx && q < nf; ++q, nk += 2) {   // + P_r + i P_i (Hermitised parts of the complex weights)
+        const double2* P = bg->P + (size_t)(v0 + 2 * q) * bg->nd;
+        launch_bg_apply(P, bg->didx, ng, bg->nd, 1, out + 2 * q * n2, c->st, 0);
+        launch_bg_apply(P + bg->nd, bg->didx, ng, bg->nd, 1, out + 2 * q * n2, c->st, 1);
       }
       stage_end(c, CHI0_STAGE_REDUCE, nk);
-      if (ev_freq) {
-        cudaEventRecord(ev_freq[jb.v], c->st);
-        if (jb.cplx) cudaEventRecord(ev_freq[jb.v + 1], c->st);
-      }
+      if (ev_freq)
+        for (int v = v0; v < v0 + step * nf; ++v) cudaEventRecord(ev_freq[v], c->st);
     }
   }
   const double tile_bytes = (double)kWPart * 16;
   // operand split: R read once per pass, hi/lo written (B once if needed, A per job)
   c->stage[CHI0_STAGE_WEIGHTS].bytes += (double)(passes + (need_b ? 1 : 0)) * nt * ng * 8 +
                                         (double)(jobs.size() + (need_b ? 1 : 0)) * 4.0 * t.mpad * t.kpad;
-  // contraction: each launch streams its operands (hi and lo) once, one set
-  // in the one-operand form and two otherwise, and writes its chunk partials
+  // contraction: each frequency streams its operands (hi and lo; the rows of
+  // whole column tiles) once, one set in the one-operand form and two
+  // otherwise, and writes its chunk partials
+  const double rows = (double)t.nJ * kWN;
   c->stage[CHI0_STAGE_CONTRACT].bytes =
-      (double)nherm * (one_op ? 4.0 : 8.0) * t.mpad * t.kpad + (double)nfull * 8.0 * t.mpad * t.kpad +
+      (double)nherm * (one_op ? 4.0 : 8.0) * rows * t.kpad + (double)nfull * 8.0 * rows * t.kpad +
       (double)nherm * t.nchunks * t.ntiles * tile_bytes + (double)nfull * t.nchunks_f * t.ntiles_f * tile_bytes;
   c->stage[CHI0_STAGE_REDUCE].bytes =
       (double)nherm * t.nchunks * t.ntiles * tile_bytes + (double)nfull * t.nchunks_f * t.ntiles_f * tile_bytes +
@@ -1073,8 +1101,8 @@ std::vector<DevBuf*> tc_scratch_slots(chi0_ctx* c) {
   return v;
 }
 
-// The contraction of the first entry of the frequency list (its operands
-// split as tc_launch does) timed for the planned transition split and for
+// The contraction of the first entries of the frequency list (those of one
+// launch, their operands split as tc_launch does) timed for the planned transition split and for
 // half and twice as many splits; the fastest is kept for the later launches.
 chi0_status tc_tune_split(chi0_ctx* c, float* best_ms) {
   if (!c->tc || c->nt == 0) return CHI0_OK;
@@ -1088,12 +1116,17 @@ chi0_status tc_tune_split(chi0_ctx* c, float* best_ms) {
     ob.lo[0] = (__nv_bfloat16*)t.bl.p;
     k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)c->d_R.p, 1, weighted_rows(c), ng, t.mpad, ob, weighted_perm(c));
   }
+  // the first t.per entries of the frequency list (real parts of the weights
+  // where an entry is one of a real frequency: the time does not depend on it)
+  const int nf = std::min(t.per, c->nwv);
   PrepOut oa{};
-  oa.hi[0] = (__nv_bfloat16*)t.ah[0].p;
-  oa.lo[0] = (__nv_bfloat16*)t.al[0].p;
-  oa.wr[0] = (const double*)c->d_w.p;
-  oa.sq[0] = one_op;
-  k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)c->d_R.p, 1, weighted_rows(c), ng, t.mpad, oa, weighted_perm(c));
+  for (int g = 0; g < nf; ++g) {
+    oa.hi[g] = (__nv_bfloat16*)t.ah[g].p;
+    oa.lo[g] = (__nv_bfloat16*)t.al[g].p;
+    oa.wr[g] = (const double*)c->d_w.p + (size_t)g * weighted_rows(c);
+    oa.sq[g] = one_op;
+  }
+  k_prep<<<pgrid, 256, 0, c->st>>>((const float2*)c->d_R.p, nf, weighted_rows(c), ng, t.mpad, oa, weighted_perm(c));
   const size_t cap = t.part.bytes / ((size_t)kWPart * 16);
   const int base_split = (t.total_kb + t.kbpc - 1) / t.kbpc;
   int best_kbpc = t.kbpc, best_n = t.nchunks;
@@ -1106,14 +1139,11 @@ chi0_status tc_tune_split(chi0_ctx* c, float* best_ms) {
   for (int sp : {base_split, std::max(1, base_split / 2), 2 * base_split}) {
     const int kbpc = (t.total_kb + sp - 1) / sp;
     const int nchunks = (t.total_kb + kbpc - 1) / kbpc;
-    if ((size_t)nchunks * t.ntiles > cap) continue;
-    const int nunits = t.ntiles * nchunks;
-    const unsigned grid = (unsigned)std::min(nunits, std::max(1, t.nsm));
+    if ((size_t)nf * nchunks * t.ntiles > cap) continue;
     float ms = 0.f;
     for (int rep = 0; rep < 2; ++rep) {   // the first run warms the caches
       cudaEventRecord(e0, c->st);
-      launch_herm(c, t, 0, kbpc, nunits, nullptr, one_op);
-      (void)grid;
+      launch_herm(c, t, 0, nf, kbpc, nchunks, nullptr, one_op, false);
       cudaEventRecord(e1, c->st);
       if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
         cudaGetLastError();
@@ -1130,7 +1160,7 @@ chi0_status tc_tune_split(chi0_ctx* c, float* best_ms) {
   cudaEventDestroy(e1);
   t.kbpc = best_kbpc;
   t.nchunks = best_n;
-  if (best_ms) *best_ms = best;
+  if (best_ms) *best_ms = best / nf;   // per frequency
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CHI0_OK : ctx_fail(c, CHI0_ECUDA, cudaGetErrorString(e));
 }
@@ -1174,7 +1204,7 @@ namespace {
 
 struct SigTc {
   DevBuf ah, al, bh, bl;
-  CUtensorMap m_ah, m_al, m_bh, m_bl;
+  HerkMaps maps{};
   int64_t kpad = 0, T = 0, mpad_b = 0;
   int ng = 0, mpad_a = 0, nI = 0, nJ = 0, nsm = 1;
 };
@@ -1256,8 +1286,8 @@ chi0_status sig_tc_plan(chi0_ctx* c, int64_t T, int ng) {
   if ((s = ctx_ensure(c, t.al, opa, "W^delta lo")) != CHI0_OK) return s;
   if ((s = ctx_ensure(c, t.bh, opb, "rho hi")) != CHI0_OK) return s;
   if ((s = ctx_ensure(c, t.bl, opb, "rho lo")) != CHI0_OK) return s;
-  if (!make_map(&t.m_ah, t.ah.p, t.kpad, t.mpad_a) || !make_map(&t.m_al, t.al.p, t.kpad, t.mpad_a) ||
-      !make_map(&t.m_bh, t.bh.p, t.kpad, (int)t.mpad_b) || !make_map(&t.m_bl, t.bl.p, t.kpad, (int)t.mpad_b))
+  if (!make_map(&t.maps.ah[0], t.ah.p, t.kpad, t.mpad_a) || !make_map(&t.maps.al[0], t.al.p, t.kpad, t.mpad_a) ||
+      !make_map(&t.maps.bh, t.bh.p, t.kpad, (int)t.mpad_b) || !make_map(&t.maps.bl, t.bl.p, t.kpad, (int)t.mpad_b))
     return ctx_fail(c, CHI0_ECUDA, "cuTensorMapEncodeTiled failed");
   int dev = 0, nsm = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1293,9 +1323,9 @@ cudaError_t sig_tc_contract(chi0_ctx* c, float2* Y) {
   const int ntiles = t.nI * ((t.nJ + 1) / 2);
   const int total_kb = (int)(t.kpad / kBK);
   const unsigned grid = (unsigned)std::min(ntiles, t.nsm);
-  k_herk_wide<<<grid, kWThreads, kWSmemBytes, c->st>>>(t.m_ah, t.m_al, t.m_bh, t.m_bl, total_kb, total_kb, t.mpad_a,
-                                                        reinterpret_cast<double2*>(Y), ntiles, ntiles,
-                                                        (int*)c->d_err.p, t.nI, nullptr, 1, (int)t.mpad_b, 1);
+  k_herk_wide<<<grid, kWThreads, kWSmemBytes, c->st>>>(t.maps, total_kb, total_kb, t.mpad_a,
+                                                        reinterpret_cast<double2*>(Y), ntiles, ntiles, ntiles,
+                                                        (int*)c->d_err.p, t.nI, nullptr, 1, (int)t.mpad_b, 1, 0);
   return cudaGetLastError();
 }
 
