@@ -1247,11 +1247,14 @@ chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
   cudaStreamWaitEvent(c->s_dy2, c->ev_fork, 0);
   c->st = c->s_ct;
   s = launch_chi0(c, c->ev_freq.data(), c->ev_prep.data(), /*defer_combine=*/true);
-  // Dyson steps in groups of 4 frequencies: the pivot-block inverses of a
-  // group run side by side (one SM each), which a single frequency's chain
-  // of 32 dependent pivot steps cannot hide.  The last four frequencies go
-  // as 2, 1, 1, so that after the last contraction only one frequency's
-  // Dyson step is left.  A group holds frequencies of one kind (imaginary
+  // Dyson steps in groups of frequencies.  A group's chain of pivot blocks takes
+  // about 30 us a step whatever its size, and a matrix's update 54 clocks per 16
+  // x 16 tile of the whole GPU's FP64 units, so a group holds at least 4 and at
+  // least the q matrices whose updates fit into the chain.  Where the
+  // contraction takes longer than the Dyson steps, the last groups halve down to
+  // q, so that little is left after the last contraction (N_G = 1000: 2, 1, 1);
+  // where the Dyson steps take longer, small last groups would only add
+  // chains.  A group holds frequencies of one kind (imaginary
   // axis: Hermitian eps~; real axis: general eps~, whose chi0 is first
   // combined from its two contractions H_r + i H_i).
   // Consecutive groups alternate between two Dyson streams, each with its
@@ -1259,12 +1262,19 @@ chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
   // that the pivot-block inverses of one group (one SM per matrix) overlap
   // the rank-32 updates of the other.
   int grp = 0;
+  const double nt16 = (ng + 15) / 16;
+  const double step_s = 54.0 * (c->has_real ? nt16 * nt16 : 0.5 * nt16 * (nt16 + 1.0)) / 1.93e9;   // of one matrix
+  const int q = std::max(1, (int)std::min(30e-6 / step_s, 1e6)), size = std::max(4, q);
+  const bool dyson_bound = nt16 * step_s / 0.85 > c->tc_issued_flops / nw / 1.2e15;
   auto general = [&](int iw) { return c->has_real && c->h_vi[iw] >= 0; };
   auto first_v = [&](int iw) { return c->has_real ? c->h_vr[iw] : iw; };   // list entries of frequency iw
   auto last_v = [&](int iw) { return general(iw) ? c->h_vi[iw] : first_v(iw); };
   for (int w0 = 0; w0 < nw && s == CHI0_OK;) {
     const int r = nw - w0;
-    int gw = r > 4 ? std::min(4, r - 4) : (r == 4 ? 2 : 1);
+    int gw;
+    if (dyson_bound) gw = r <= size + size / 2 ? r : size;
+    else if (r > size) gw = std::min(size, r - size);
+    else gw = r <= q ? r : std::max(q, r / 2);
     for (int g = 1; g < gw; ++g)
       if (general(w0 + g) != general(w0)) {
         gw = g;
