@@ -1684,15 +1684,20 @@ chi0_status chi0_build_sigma_i(chi0_ctx* c, int iq, int qp_lo, int qp_hi, const 
   const int64_t nI = (ng + 63) / 64, nJ = (T + 63) / 64;
   const size_t osz = (size_t)c->nk * nb * nqp * nqp * 16;   // I of one frequency
   if ((s = ensure(c, c->d_sigR, (size_t)T * ng * cb, "quasiparticle rho")) != CHI0_OK) return s;
-  if ((s = ensure(c, c->d_sigY, (size_t)nI * nJ * 4096 * cb * 2, "W^delta rho* tiles")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_sigRT, (size_t)nI * nJ * 4096 * cb, "rho tiles")) != CHI0_OK) return s;
   if (!out_on_device && (s = ensure(c, c->d_sigI, osz, "I staging")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_vsqrt, (size_t)ng * 8, "coulomb")) != CHI0_OK) return s;
   if (c->fp64) {
     if ((s = ensure(c, c->d_sigWd, (size_t)ng * ng * 16, "W^delta")) != CHI0_OK) return s;
-  } else if ((s = chi0::sig_tc_plan(c, T, ng)) != CHI0_OK) {
+  } else if ((s = chi0::sig_tc_plan(c, T, ng, nw)) != CHI0_OK) {
     return s;
   }
+  // frequencies per launch of the contraction and the dot products (with a
+  // device output), and per split of W^delta
+  const int nper = c->fp64 || !out_on_device ? 1 : chi0::sig_tc_freqs(c);
+  const int nsplit = c->fp64 ? 1 : chi0::sig_tc_split_freqs(c);
+  const size_t ytile = (size_t)nI * nJ * 4096;   // entries of Y of one frequency
+  if ((s = ensure(c, c->d_sigY, ytile * cb * (c->fp64 ? 1 : nper), "W^delta rho* tiles")) != CHI0_OK) return s;
   if (!c->d_err.p) {
     if ((s = ensure(c, c->d_err, 16, "error flag")) != CHI0_OK) return s;
     CK(cudaMemsetAsync(c->d_err.p, 0, 16, c->st), "clear error flag");
@@ -1744,24 +1749,29 @@ chi0_status chi0_build_sigma_i(chi0_ctx* c, int iq, int qp_lo, int qp_hi, const 
   const size_t n2 = (size_t)ng * ng;
   const double* v = (const double*)c->d_vsqrt.p;
   void* Y = c->d_sigY.p;   // FP64 (FP64 form) or FP32 (mixed form) tiles
-  for (int iw = 0; iw < nw; ++iw) {
+  for (int iw = 0, nf; iw < nw; iw += nf) {
+    const int s0 = iw % nsplit;   // place of the frequency in its split
+    nf = std::min({nper, nw - iw, nsplit - s0});
     const double2* E = (const double2*)eps_inv + iw * n2;
     double2* I = out_on_device ? (double2*)((char*)out + iw * osz) : (double2*)c->d_sigI.p;
-    chi0::stage_begin(c, CHI0_STAGE_WEIGHTS);
-    e = c->fp64 ? chi0::launch_sig_wd64(E, v, ng, (double2*)c->d_sigWd.p, c->st) : chi0::sig_tc_split_a(c, E, v);
-    if (e != cudaSuccess) return cuda_fail(c, e, "W^delta launch");
-    chi0::stage_end(c, CHI0_STAGE_WEIGHTS, 1);
+    if (s0 == 0) {
+      chi0::stage_begin(c, CHI0_STAGE_WEIGHTS);
+      e = c->fp64 ? chi0::launch_sig_wd64(E, v, ng, (double2*)c->d_sigWd.p, c->st)
+                  : chi0::sig_tc_split_a(c, E, v, std::min(nsplit, nw - iw));
+      if (e != cudaSuccess) return cuda_fail(c, e, "W^delta launch");
+      chi0::stage_end(c, CHI0_STAGE_WEIGHTS, 1);
+    }
     chi0::stage_begin(c, CHI0_STAGE_CONTRACT);
     e = c->fp64 ? chi0::launch_sig_gemm64((const double2*)c->d_sigWd.p, (const double2*)c->d_sigR.p, ng, T, nqp, nb,
                                           (double2*)Y, c->st)
-                : chi0::sig_tc_contract(c, (float2*)Y);
+                : chi0::sig_tc_contract(c, (float2*)Y, s0, nf);
     if (e != cudaSuccess) return cuda_fail(c, e, "W^delta rho* contraction launch");
     chi0::stage_end(c, CHI0_STAGE_CONTRACT, 1);
     chi0::stage_begin(c, CHI0_STAGE_REDUCE);
     e = c->fp64 ? chi0::launch_sig_dot<double2, double2>((const double2*)c->d_sigRT.p, (const double2*)Y, ng, T, nqp,
                                                          pref, I, c->st)
                 : chi0::launch_sig_dot<float2, float2>((const float2*)c->d_sigRT.p, (const float2*)Y, ng, T, nqp, pref,
-                                                       I, c->st);
+                                                       I, c->st, nf, ytile, osz / 16);
     if (e != cudaSuccess) return cuda_fail(c, e, "I launch");
     chi0::stage_end(c, CHI0_STAGE_REDUCE, 1);
     if (!out_on_device)

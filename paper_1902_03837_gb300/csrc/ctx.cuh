@@ -210,12 +210,17 @@ cudaError_t launch_wait_probe(int* err, cudaStream_t s);
 // self-energy kernel I (Eq. I_c) on the tensor cores: Y(i, t) = sum_j
 // W^d_ij conj(rho_t(j)) for T transitions of the quasiparticle window, written
 // in FP32 as 64 x 64 complex tiles, tile (i / 64) + (t / 64) * ceil(ng / 64)
-chi0_status sig_tc_plan(chi0_ctx* c, int64_t T, int ng);
+chi0_status sig_tc_plan(chi0_ctx* c, int64_t T, int ng, int nw);
+// frequencies that sig_tc_split_a takes at a time and that sig_tc_contract
+// takes per launch
+int sig_tc_split_freqs(const chi0_ctx* c);
+int sig_tc_freqs(const chi0_ctx* c);
 // rho of the window (the rho kernel's order ((k nqp) + a) nb + m) into the B operand
 cudaError_t sig_tc_split_b(chi0_ctx* c, const float2* R, int nqp, int nb);
-// W^d of one frequency from eps~^-1 (E) and V into the A operand
-cudaError_t sig_tc_split_a(chi0_ctx* c, const double2* E, const double* vsqrt);
-cudaError_t sig_tc_contract(chi0_ctx* c, float2* Y);
+// W^d of nf frequencies from eps~^-1 (E) and V into the A operands 0 .. nf - 1
+cudaError_t sig_tc_split_a(chi0_ctx* c, const double2* E, const double* vsqrt, int nf);
+// Y of the A operands a0 .. a0 + nf - 1, one behind the other
+cudaError_t sig_tc_contract(chi0_ctx* c, float2* Y, int a0, int nf);
 void sig_tc_release(chi0_ctx* c);
 // learned terminator: network kernels and the correction of a built chi0
 int mlp_nparams();

@@ -218,7 +218,8 @@ cudaError_t dyson_prepare();
 // Self-energy kernel I (Eq. I_c; sigma.cu).  W^d of one frequency in FP64
 // from eps~^-1 (E) and V; Y(i, t) = sum_j W^d_ij conj(rho_t(j)) in plain
 // FP64 (rho in the rho kernel's order of the quasiparticle window, Y in
-// 64 x 64 tiles); I[g][a][b] = pref sum_i rho_(g,a)(i) Y(i, (g,b)).
+// 64 x 64 tiles); I[g][a][b] = pref sum_i rho_(g,a)(i) Y(i, (g,b)) (nf
+// frequencies, ystride and ostride entries apart).
 cudaError_t launch_sig_wd64(const double2* E, const double* vsqrt, int ng, double2* Wd, cudaStream_t s);
 cudaError_t launch_sig_gemm64(const double2* Wd, const double2* R, int ng, int64_t T, int nqp, int nb,
                               double2* Y, cudaStream_t s);
@@ -227,6 +228,6 @@ template <typename TR>
 cudaError_t launch_sig_rhot(const TR* R, int64_t T, int nqp, int nb, int ng, TR* RT, cudaStream_t s);
 template <typename TR, typename TY>
 cudaError_t launch_sig_dot(const TR* RT, const TY* Y, int ng, int64_t T, int nqp, double pref, double2* out,
-                           cudaStream_t s);
+                           cudaStream_t s, int nf = 1, size_t ystride = 0, size_t ostride = 0);
 
 }  // namespace chi0

@@ -1203,10 +1203,11 @@ cudaError_t launch_wait_probe(int* err, cudaStream_t s) {
 namespace {
 
 struct SigTc {
-  DevBuf ah, al, bh, bl;
+  DevBuf ah, al, bh, bl;   // A: nsplit operands one behind the other
   HerkMaps maps{};
   int64_t kpad = 0, T = 0, mpad_b = 0;
   int ng = 0, mpad_a = 0, nI = 0, nJ = 0, nsm = 1;
+  int nsplit = 1, per = 1;   // frequencies per split of W^d, and per contraction launch
 };
 
 __device__ __forceinline__ void split_store(float x0, float x1, __nv_bfloat16* hi, __nv_bfloat16* lo, size_t off) {
@@ -1241,8 +1242,11 @@ k_sig_bsplit(const float2* __restrict__ R, int64_t T, int nqp, int nb, int ng, i
 // A: row 2 i + c, column j holds W^d_ij.c, Eq. (W_delta) with W = V E V:
 // W^d_ij = V_i V_j [ (Im E_ij + Im E_ji) / 2 - i (Re E_ij - Re E_ji) / 2 ].
 __global__ void __launch_bounds__(256)
-k_sig_asplit(const double2* __restrict__ E, const double* __restrict__ v, int ng, int mpad_a,
+k_sig_asplit(const double2* __restrict__ E, const double* __restrict__ v, int ng, int mpad_a, size_t stride,
              __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+  E += (size_t)blockIdx.z * ng * ng;   // frequency of the pass
+  hi += blockIdx.z * stride;
+  lo += blockIdx.z * stride;
   const int r0 = blockIdx.x * 64;
   const int kb = blockIdx.y;
   for (int e = threadIdx.x; e < 64 * 32; e += 256) {
@@ -1267,7 +1271,7 @@ k_sig_asplit(const double2* __restrict__ E, const double* __restrict__ v, int ng
 
 }  // namespace
 
-chi0_status sig_tc_plan(chi0_ctx* c, int64_t T, int ng) {
+chi0_status sig_tc_plan(chi0_ctx* c, int64_t T, int ng, int nw) {
   if (!c->sig_tc) c->sig_tc = new SigTc();
   SigTc& t = *static_cast<SigTc*>(c->sig_tc);
   t.T = T;
@@ -1282,12 +1286,20 @@ chi0_status sig_tc_plan(chi0_ctx* c, int64_t T, int ng) {
     return ctx_fail(c, CHI0_EUNSUPPORTED, "too many transitions in the quasiparticle window for one contraction");
   chi0_status s;
   const size_t opa = (size_t)t.mpad_a * t.kpad * 2, opb = (size_t)t.mpad_b * t.kpad * 2;
-  if ((s = ctx_ensure(c, t.ah, opa, "W^delta hi")) != CHI0_OK) return s;
-  if ((s = ctx_ensure(c, t.al, opa, "W^delta lo")) != CHI0_OK) return s;
+  // W^d of eight frequencies per split (50 blocks at N_G = 300 for one), and as
+  // many frequencies per contraction launch as leave the two Y's that it writes
+  // and the dot products read within L2
+  t.nsplit = std::max(1, std::min(kPrepGroup, nw));
+  t.per = (double)t.nI * t.nJ * 4096 * 8 <= 48e6 ? std::min(2, t.nsplit) : 1;
+  if ((s = ctx_ensure(c, t.ah, opa * t.nsplit, "W^delta hi")) != CHI0_OK) return s;
+  if ((s = ctx_ensure(c, t.al, opa * t.nsplit, "W^delta lo")) != CHI0_OK) return s;
   if ((s = ctx_ensure(c, t.bh, opb, "rho hi")) != CHI0_OK) return s;
   if ((s = ctx_ensure(c, t.bl, opb, "rho lo")) != CHI0_OK) return s;
-  if (!make_map(&t.maps.ah[0], t.ah.p, t.kpad, t.mpad_a) || !make_map(&t.maps.al[0], t.al.p, t.kpad, t.mpad_a) ||
-      !make_map(&t.maps.bh, t.bh.p, t.kpad, (int)t.mpad_b) || !make_map(&t.maps.bl, t.bl.p, t.kpad, (int)t.mpad_b))
+  for (int g = 0; g < t.nsplit; ++g)
+    if (!make_map(&t.maps.ah[g], (char*)t.ah.p + g * opa, t.kpad, t.mpad_a) ||
+        !make_map(&t.maps.al[g], (char*)t.al.p + g * opa, t.kpad, t.mpad_a))
+      return ctx_fail(c, CHI0_ECUDA, "cuTensorMapEncodeTiled failed");
+  if (!make_map(&t.maps.bh, t.bh.p, t.kpad, (int)t.mpad_b) || !make_map(&t.maps.bl, t.bl.p, t.kpad, (int)t.mpad_b))
     return ctx_fail(c, CHI0_ECUDA, "cuTensorMapEncodeTiled failed");
   int dev = 0, nsm = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1307,10 +1319,13 @@ cudaError_t sig_tc_split_b(chi0_ctx* c, const float2* R, int nqp, int nb) {
   return cudaGetLastError();
 }
 
-cudaError_t sig_tc_split_a(chi0_ctx* c, const double2* E, const double* vsqrt) {
+int sig_tc_split_freqs(const chi0_ctx* c) { return static_cast<const SigTc*>(c->sig_tc)->nsplit; }
+int sig_tc_freqs(const chi0_ctx* c) { return static_cast<const SigTc*>(c->sig_tc)->per; }
+
+cudaError_t sig_tc_split_a(chi0_ctx* c, const double2* E, const double* vsqrt, int nf) {
   SigTc& t = *static_cast<SigTc*>(c->sig_tc);
-  k_sig_asplit<<<dim3((unsigned)(t.mpad_a / 64), (unsigned)(t.kpad / 64)), 256, 0, c->st>>>(
-      E, vsqrt, t.ng, t.mpad_a, (__nv_bfloat16*)t.ah.p, (__nv_bfloat16*)t.al.p);
+  k_sig_asplit<<<dim3((unsigned)(t.mpad_a / 64), (unsigned)(t.kpad / 64), (unsigned)nf), 256, 0, c->st>>>(
+      E, vsqrt, t.ng, t.mpad_a, (size_t)t.mpad_a * t.kpad, (__nv_bfloat16*)t.ah.p, (__nv_bfloat16*)t.al.p);
   return cudaGetLastError();
 }
 
@@ -1318,14 +1333,22 @@ cudaError_t sig_tc_split_a(chi0_ctx* c, const double2* E, const double* vsqrt) {
 // column tiles, rounded up), one k range per tile, written as Y's 64 x 64
 // complex FP32 tiles; the half of a last wide tile beyond the B rows is not
 // written.
-cudaError_t sig_tc_contract(chi0_ctx* c, float2* Y) {
+cudaError_t sig_tc_contract(chi0_ctx* c, float2* Y, int a0, int nf) {
   SigTc& t = *static_cast<SigTc*>(c->sig_tc);
+  HerkMaps m;
+  for (int g = 0; g < nf; ++g) {
+    m.ah[g] = t.maps.ah[a0 + g];
+    m.al[g] = t.maps.al[a0 + g];
+  }
+  m.bh = t.maps.bh;
+  m.bl = t.maps.bl;
+  m.own = 0;
   const int ntiles = t.nI * ((t.nJ + 1) / 2);
   const int total_kb = (int)(t.kpad / kBK);
-  const unsigned grid = (unsigned)std::min(ntiles, t.nsm);
-  k_herk_wide<<<grid, kWThreads, kWSmemBytes, c->st>>>(t.maps, total_kb, total_kb, t.mpad_a,
-                                                        reinterpret_cast<double2*>(Y), ntiles, ntiles, ntiles,
-                                                        (int*)c->d_err.p, t.nI, nullptr, 1, (int)t.mpad_b, 1, 0);
+  const unsigned grid = (unsigned)std::min(ntiles * nf, t.nsm);
+  k_herk_wide<<<grid, kWThreads, kWSmemBytes, c->st>>>(m, total_kb, total_kb, t.mpad_a, reinterpret_cast<double2*>(Y),
+                                                        ntiles, ntiles, ntiles * nf, (int*)c->d_err.p, t.nI, nullptr, 1,
+                                                        (int)t.mpad_b, 1, (size_t)t.nI * t.nJ * 4096);
   return cudaGetLastError();
 }
 
