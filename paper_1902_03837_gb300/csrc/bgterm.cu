@@ -17,26 +17,58 @@ namespace chi0 {
 
 namespace {
 
+// P[iw][d] for 32 vectors d per block and up to eight frequencies: eight warps
+// take every eighth state and add up (one thread per (d, frequency) walked over
+// all states, one load after the other).  Bound by the FP64 units, to which the
+// conversions of an FP32 density belong: each is converted once for the eight
+// frequencies (768 states, 1760 vectors, 16 frequencies 217 -> 159 us).
+constexpr int kBgW = 8, kBgF = 8;
 template <typename TOUT>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * kBgW)
 k_bg_sum(const TOUT* __restrict__ rd, const BgChunks ch, const double* __restrict__ wbar, int64_t ntd,
-         int nd, double2* __restrict__ P) {
-  const int d = blockIdx.x * blockDim.x + threadIdx.x;
-  const int iw = blockIdx.y;
-  if (d >= nd) return;
-  int c = 0;
-  while (c + 1 < ch.n && d >= ch.start[c + 1]) ++c;
-  const int64_t stride = ch.start[c + 1] - ch.start[c];
-  const TOUT* p = rd + ch.off[c] + (d - ch.start[c]);
-  const double* w = wbar + (size_t)iw * ntd;
-  double sx = 0.0, sy = 0.0;
-  for (int64_t t = 0; t < ntd; ++t) {
-    const double wt = w[t];
-    const TOUT v = p[t * stride];
-    sx = fma(wt, (double)v.x, sx);
-    sy = fma(wt, (double)v.y, sy);
+         int nd, int nw, double2* __restrict__ P) {
+  __shared__ double2 sums[kBgW][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int d = blockIdx.x * 32 + lane;
+  const int iw0 = blockIdx.y * kBgF, nf = min(kBgF, nw - iw0);
+  const double* w = wbar + (size_t)iw0 * ntd;
+  double2 s[kBgF];
+#pragma unroll
+  for (int f = 0; f < kBgF; ++f) s[f] = make_double2(0.0, 0.0);
+  if (d < nd) {
+    int c = 0;
+    while (c + 1 < ch.n && d >= ch.start[c + 1]) ++c;
+    const int64_t stride = ch.start[c + 1] - ch.start[c];
+    const TOUT* p = rd + ch.off[c] + (d - ch.start[c]);
+#pragma unroll 2
+    for (int64_t t = warp; t < ntd; t += kBgW) {
+      const TOUT v = p[t * stride];
+      const double vx = (double)v.x, vy = (double)v.y;
+#pragma unroll
+      for (int f = 0; f < kBgF; ++f) {
+        if (f < nf) {
+          const double wt = w[(size_t)f * ntd + t];
+          s[f].x = fma(wt, vx, s[f].x);
+          s[f].y = fma(wt, vy, s[f].y);
+        }
+      }
+    }
   }
-  P[(size_t)iw * nd + d] = make_double2(sx, sy);
+#pragma unroll
+  for (int f = 0; f < kBgF; ++f) {
+    if (f >= nf) break;
+    sums[warp][lane] = s[f];
+    __syncthreads();
+    if (warp == 0 && d < nd) {
+      double2 a = s[f];
+      for (int q = 1; q < kBgW; ++q) {
+        a.x += sums[q][lane].x;
+        a.y += sums[q][lane].y;
+      }
+      P[(size_t)(iw0 + f) * nd + d] = a;
+    }
+    __syncthreads();
+  }
 }
 
 // chi[iw][i][j] += v, chi[iw][j][i] += conj(v) for i >= j, with
@@ -72,7 +104,8 @@ template <typename TOUT>
 cudaError_t launch_bg_sum(const TOUT* rd, const BgChunks& ch, const double* wbar, int64_t ntd, int nd,
                           int nw, double2* P, cudaStream_t s) {
   if (nd <= 0 || nw <= 0) return cudaSuccess;
-  k_bg_sum<TOUT><<<dim3((unsigned)((nd + 127) / 128), (unsigned)nw), 128, 0, s>>>(rd, ch, wbar, ntd, nd, P);
+  k_bg_sum<TOUT><<<dim3((unsigned)((nd + 31) / 32), (unsigned)((nw + kBgF - 1) / kBgF)), 32 * kBgW, 0, s>>>(
+      rd, ch, wbar, ntd, nd, nw, P);
   return cudaGetLastError();
 }
 
