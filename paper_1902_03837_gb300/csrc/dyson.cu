@@ -97,7 +97,8 @@ struct PivotSmem {
   double2 row[2][kNB], col[2][kNB], dinv[2];
   int bad[2];
 };
-__device__ __forceinline__ bool pivot_inverse(double2 (&x)[2], int nb, bool general, PivotSmem& sm) {
+template <bool general>
+__device__ __forceinline__ bool pivot_inverse(double2 (&x)[2], int nb, PivotSmem& sm) {
   const int r = threadIdx.x >> 3, c0 = (threadIdx.x & 7) * 2;
   if (threadIdx.x < 2) sm.bad[threadIdx.x] = 0;
   __syncthreads();
@@ -151,8 +152,9 @@ __device__ __forceinline__ void put_pivot(const double2 (&x)[2], double2* __rest
 }
 
 // P of the first block; a matrix of at most 16 rows is done with it.
+template <bool full>
 __global__ void __launch_bounds__(kThreads)
-k_gj_first(Mats m, int nb, double2* __restrict__ pinv, int* __restrict__ err, int general) {
+k_gj_first(Mats m, int nb, double2* __restrict__ pinv, int* __restrict__ err) {
   __shared__ PivotSmem sm;
   const int iw = blockIdx.x;
   const int r = threadIdx.x >> 3, c0 = (threadIdx.x & 7) * 2;
@@ -160,7 +162,7 @@ k_gj_first(Mats m, int nb, double2* __restrict__ pinv, int* __restrict__ err, in
 #pragma unroll
   for (int u = 0; u < 2; ++u)
     x[u] = r < nb && c0 + u < nb ? m.get(iw, r, c0 + u, true) : make_double2(0.0, 0.0);
-  if (!pivot_inverse(x, nb, general, sm)) {
+  if (!pivot_inverse<full>(x, nb, sm)) {
     if (threadIdx.x == 0) atomicExch(err, 1);
     return;
   }
@@ -180,9 +182,10 @@ k_gj_first(Mats m, int nb, double2* __restrict__ pinv, int* __restrict__ err, in
 // One thread per (column e, k), eight columns per block: the panels of one
 // matrix spread over ng / 8 blocks (the FP64 rate of a single SM is low, and
 // this step sits on the critical path of every pivot block).
+template <bool full>
 __global__ void __launch_bounds__(kThreads)
 k_gj_panels(Mats m, int b0, int nb, const double2* __restrict__ pinv, double2* __restrict__ colp,
-            double2* __restrict__ rowp, int full) {
+            double2* __restrict__ rowp) {
   __shared__ double2 base[kPE][kNB];  // A_b0+l,e of the block's columns
   const int iw = blockIdx.y, ng = m.ng;
   const bool first = b0 == 0;
@@ -221,9 +224,10 @@ k_gj_panels(Mats m, int b0, int nb, const double2* __restrict__ pinv, double2* _
 // blocks (one waits for its loads while the other computes) then fit beside a
 // tensor-core contraction block, and the Dyson step of one frequency uses the
 // FP64 units while the contraction of the next occupies the tensor cores.
+template <bool full>
 __global__ void __launch_bounds__(kThreads, 12)
 k_gj_update(Mats m, int nw, int b0, int nb, double2* __restrict__ pinv, const double2* __restrict__ colp,
-            const double2* __restrict__ rowp, int* __restrict__ err, int full) {
+            const double2* __restrict__ rowp, int* __restrict__ err) {
   __shared__ PivotSmem sm;
   const int ng = m.ng;
   const int nt = (ng + kNB - 1) / kNB, pt = b0 / kNB;
@@ -247,7 +251,7 @@ k_gj_update(Mats m, int nw, int b0, int nb, double2* __restrict__ pinv, const do
           for (int u = 0; u < 2; ++u)
             if (c0 + u < nbn) cmsub(x[u], a, rb[(size_t)k * ng + u]);
         }
-      if (!pivot_inverse(x, nbn, full, sm)) {
+      if (!pivot_inverse<full>(x, nbn, sm)) {
         if (threadIdx.x == 0) atomicExch(err, 1);
         return;
       }
@@ -311,19 +315,19 @@ k_gj_update(Mats m, int nw, int b0, int nb, double2* __restrict__ pinv, const do
 // Blocks of the update: two per SM, fewer when there are fewer tiles.
 constexpr int kUpdateBlocks = 2 * 152;
 
-cudaError_t launch_gj(const Mats& m, int nw, double2* colp, double2* rowp, double2* pinv, int* err, int full,
-                      cudaStream_t s) {
+template <bool full>
+cudaError_t launch_gj(const Mats& m, int nw, double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s) {
   const int ng = m.ng, nt = (ng + kNB - 1) / kNB;
-  k_gj_first<<<nw, kThreads, 0, s>>>(m, ng < kNB ? ng : kNB, pinv, err, full);
+  k_gj_first<full><<<nw, kThreads, 0, s>>>(m, ng < kNB ? ng : kNB, pinv, err);
   if (nt > 1)
     for (int b0 = 0; b0 < ng; b0 += kNB) {
       const int nb = ng - b0 < kNB ? ng - b0 : kNB;
       const bool last = b0 + kNB >= ng;
-      k_gj_panels<<<dim3((ng + kPE - 1) / kPE, nw), kThreads, 0, s>>>(m, b0, nb, pinv, colp, rowp, full);
+      k_gj_panels<full><<<dim3((ng + kPE - 1) / kPE, nw), kThreads, 0, s>>>(m, b0, nb, pinv, colp, rowp);
       const int64_t tiles = (int64_t)(full ? nt * nt : nt * (nt + 1) / 2) * nw;
       const int spare = last ? kUpdateBlocks : nw < kUpdateBlocks / 2 ? kUpdateBlocks - nw : kUpdateBlocks / 2;
       const int workers = (int)(tiles < spare ? tiles : spare);
-      k_gj_update<<<workers + (last ? 0 : nw), kThreads, 0, s>>>(m, nw, b0, nb, pinv, colp, rowp, err, full);
+      k_gj_update<full><<<workers + (last ? 0 : nw), kThreads, 0, s>>>(m, nw, b0, nb, pinv, colp, rowp, err);
     }
   return cudaGetLastError();
 }
@@ -336,7 +340,9 @@ int dyson_launches(int ng) {
 }
 
 cudaError_t dyson_prepare() {
-  const void* fns[] = {(const void*)k_gj_first, (const void*)k_gj_panels, (const void*)k_gj_update};
+  const void* fns[] = {(const void*)k_gj_first<false>,  (const void*)k_gj_first<true>,
+                       (const void*)k_gj_panels<false>, (const void*)k_gj_panels<true>,
+                       (const void*)k_gj_update<false>, (const void*)k_gj_update<true>};
   for (const void* f : fns) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                cudaSharedmemCarveoutMaxShared);
@@ -347,7 +353,7 @@ cudaError_t dyson_prepare() {
 
 cudaError_t launch_dyson(const double2* chi, const double* vsqrt, int ng, int nw, double2* A,
                          double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s) {
-  return launch_gj(Mats{chi, vsqrt, A, ng}, nw, colp, rowp, pinv, err, 0, s);
+  return launch_gj<false>(Mats{chi, vsqrt, A, ng}, nw, colp, rowp, pinv, err, s);
 }
 
 // General (non-Hermitian) eps~ of real-axis frequencies: the same blocked
@@ -358,7 +364,7 @@ cudaError_t launch_dyson(const double2* chi, const double* vsqrt, int ng, int nw
 // vanishes all the same is reported through the error flag.
 cudaError_t launch_dyson_general(const double2* chi, const double* vsqrt, int ng, int nw, double2* A,
                                  double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s) {
-  return launch_gj(Mats{chi, vsqrt, A, ng}, nw, colp, rowp, pinv, err, 1, s);
+  return launch_gj<true>(Mats{chi, vsqrt, A, ng}, nw, colp, rowp, pinv, err, s);
 }
 
 }  // namespace chi0
