@@ -157,6 +157,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// One 32-byte store (a whole L2 sector: a lane's neighbours write other rows, so
+// smaller pieces would each reach L2 as a partial sector).
+__device__ __forceinline__ void store32(void* p, const float (&v)[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ void store32(void* p, const double (&v)[4]) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+               : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major tile of 128-byte rows written by
 // TMA with 128-byte swizzle; 8-row atoms 1024 bytes apart.
 __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
@@ -450,22 +462,28 @@ k_herk_wide(const __grid_constant__ HerkMaps maps, int total_kb, int kb_per_spli
           float2* out = reinterpret_cast<float2*>(part) + (u / upf) * f32stride + ((size_t)Jn * nI + I) * (size_t)(kBM / 2) * (kBN / 2) +
                         (size_t)il * (kBN / 2) + (odd ? 4 : 0);
 #pragma unroll
-          for (int cb = 0; cb < kBN / 16; ++cb)
+          for (int cb = 0; cb < kBN / 16; ++cb) {
+            float v[8];
 #pragma unroll
             for (int jj = 0; jj < 4; ++jj) {
               const int e = cb * 4 + jj;
-              out[cb * 8 + jj] = make_float2(accs[e][0] + accc[e][0], accs[e][1] + accc[e][1]);
+              v[2 * jj] = accs[e][0] + accc[e][0];
+              v[2 * jj + 1] = accs[e][1] + accc[e][1];
             }
+            store32(out + cb * 8, v);
+          }
         }
       } else {
         double2* out = part + (size_t)u * kWPart + (size_t)il * (kWN / 2) + hcol * (kBN / 2) + (odd ? 4 : 0);
 #pragma unroll
         for (int cb = 0; cb < kBN / 16; ++cb)
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
+          for (int jj = 0; jj < 4; jj += 2) {
             const int e = cb * 4 + jj;
-            out[cb * 8 + jj] = make_double2((double)accs[e][0] + (double)accc[e][0],
-                                            (double)accs[e][1] + (double)accc[e][1]);
+            const double v[4] = {(double)accs[e][0] + (double)accc[e][0], (double)accs[e][1] + (double)accc[e][1],
+                                 (double)accs[e + 1][0] + (double)accc[e + 1][0],
+                                 (double)accs[e + 1][1] + (double)accc[e + 1][1]};
+            store32(out + cb * 8 + jj, v);
           }
       }
     }
