@@ -65,32 +65,57 @@ chi0_status ensure(chi0_ctx* c, DevBuf& b, size_t bytes, const char* what) {
 }  // namespace
 
 namespace chi0 {
+constexpr int64_t kTimedAll = 512, kTimedStep = 16;
+constexpr size_t kFoldAt = 1024;   // events
+
+// the recorded pairs' times into acc (the pairs must have finished)
+static void stage_fold(chi0_ctx::Stage& st) {
+  for (size_t p = 0; p + 1 < st.used; p += 2) {
+    float t = 0.f;
+    if (cudaEventElapsedTime(&t, st.ev[p], st.ev[p + 1]) == cudaSuccess) st.acc += (double)t * st.weight[p / 2];
+    cudaGetLastError();
+  }
+  st.used = 0;
+}
+
 void stage_begin(chi0_ctx* c, int stage) {
   if (c->capturing) return;
   auto& st = c->stage[stage];
+  const int64_t i = st.count++;
+  st.timed = i < kTimedAll || i % kTimedStep == 0;
+  if (!st.timed) return;
+  if (st.used >= kFoldAt) {
+    // the last pairs of every stream in use must have finished (and nothing is
+    // asked of events while the caller captures the stream)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    bool done = cudaStreamIsCapturing(c->st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    for (size_t p = 1; done && p <= 8; ++p) done = cudaEventQuery(st.ev[st.used + 1 - 2 * p]) == cudaSuccess;
+    cudaGetLastError();
+    if (done) stage_fold(st);
+  }
   if (st.used + 2 > st.ev.size()) {
     cudaEvent_t a = nullptr, b = nullptr;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) {
       cudaGetLastError();
+      if (a) cudaEventDestroy(a);
+      st.timed = false;
       return;
     }
     st.ev.push_back(a);
     st.ev.push_back(b);
+    st.weight.push_back(1);
   }
+  st.weight[st.used / 2] = i < kTimedAll ? 1 : (int)kTimedStep;
   cudaEventRecord(st.ev[st.used], c->st);
 }
 void stage_end(chi0_ctx* c, int stage, int kernels) {
   auto& st = c->stage[stage];
-  if (c->capturing) {
-    st.launches += kernels;
-    c->launches += kernels;
-    return;
-  }
-  if (st.used + 2 > st.ev.size()) return;  // begin failed to get events
-  cudaEventRecord(st.ev[st.used + 1], c->st);
-  st.used += 2;
   st.launches += kernels;
   c->launches += kernels;
+  if (c->capturing || !st.timed) return;
+  cudaEventRecord(st.ev[st.used + 1], c->st);
+  st.used += 2;
+  st.timed = false;
 }
 chi0_status ctx_fail(chi0_ctx* c, chi0_status s, const char* msg) { c->err = msg; return s; }
 chi0_status ctx_ensure(chi0_ctx* c, DevBuf& b, size_t bytes, const char* what) { return ensure(c, b, bytes, what); }
@@ -1942,18 +1967,10 @@ chi0_status chi0_get_stats(chi0_ctx* c, double* ms, double* bytes, double* flops
   CK(cudaStreamSynchronize(c->st), "synchronize");
   for (int k = 0; k < CHI0_NSTAGES; ++k) {
     auto& st = c->stage[k];
-    if (st.used) {
-      double tot = 0.0;
-      for (size_t p = 0; p + 1 < st.used; p += 2) {
-        float t = 0.f;
-        if (cudaEventElapsedTime(&t, st.ev[p], st.ev[p + 1]) == cudaSuccess) tot += t;
-        cudaGetLastError();
-      }
-      st.ms = tot;
-      st.used = 0;
-    } else {
-      st.ms = 0.0;
-    }
+    chi0::stage_fold(st);
+    st.ms = st.acc;
+    st.acc = 0.0;
+    st.count = 0;
     if (ms) ms[k] = st.ms;
     if (bytes) bytes[k] = st.bytes;
     if (flops) flops[k] = st.flops;

@@ -137,11 +137,18 @@ struct chi0_ctx {
   DevBuf d_sigR, d_sigRT, d_sigWd, d_sigY, d_sigI;
   void* sig_tc = nullptr;
 
-  // per-stage device time: CUDA event pairs on the context's stream, summed
-  // over every launch of the stage since the last chi0_get_stats
+  // per-stage device time: CUDA event pairs on the context's stream.  A pair
+  // costs the stream about 4 us, half of a small problem's pass, and pairs
+  // kept until the next readout pile up in a program that never reads them, so
+  // after kTimedAll instances every kTimedStep-th stands for its neighbours,
+  // and finished pairs are folded into ms and used again.
   struct Stage {
     std::vector<cudaEvent_t> ev;  // start, stop, start, stop, ...
-    size_t used = 0;              // events recorded since the last readout
+    std::vector<int> weight;      // instances that each pair stands for
+    size_t used = 0;              // events recorded since the last fold
+    int64_t count = 0;            // instances since the last readout
+    bool timed = false;           // the open instance has a pair
+    double acc = 0;               // folded time since the last readout (ms)
     double ms = 0, bytes = 0, flops = 0;
     int64_t launches = 0;
   };
