@@ -10,10 +10,14 @@
 //   1. every problem's host set-up runs once (chi0_batch_create).  The
 //      problems of one system (one context at several q indices) share its
 //      coefficients and its mixed grids, computed once per system;
-//   2. the oscillator strengths of all problems run in one persistent launch
-//      per grid size (the column transforms are compiled per size) over a
-//      device task table: blocks take the next (problem, k-pair, n, m-chunk)
-//      work item from a counter, so uneven problems balance;
+//   2. the oscillator strengths run in one persistent launch per grid size (the
+//      column transforms are compiled per size) over a device task table:
+//      blocks take the next (problem, k-pair, n, m-chunk) work item from a
+//      counter, so uneven problems balance.  In the mixed form the first problem
+//      of every stream comes first; the others' follow once those problems'
+//      contractions are done, with one block per SM, so that the Dyson steps of
+//      the first problems have the FP64 units meanwhile (nine metals on four
+//      streams: 15.8 -> 15.0 ms);
 //   3. the remaining kernels of every problem (weights, operand split,
 //      contraction, reduction, Dyson) go on a few helper streams.  Problems
 //      are assigned to the streams longest first, each to the stream with the
@@ -48,6 +52,7 @@ struct chi0_batch {
   std::vector<void*> chi_outs;   // chi0 per problem (NULL: not copied out)
   std::vector<int> stream_of;    // helper stream of each problem
   std::vector<int> order;        // problems in launch order (per stream: longest first)
+  std::vector<char> late;        // its rho comes after the first problems' contractions
   std::vector<double> cost;      // estimated device time of each problem (model units)
   std::vector<std::vector<DevBuf>> arena;  // [helper stream][scratch slot] shared buffers
   float tuned_split_ms = 0.f;    // summed best contraction time of the split tuning
@@ -57,9 +62,11 @@ struct chi0_batch {
   cudaGraphExec_t exec = nullptr;
   cudaStream_t capture_stream = nullptr;
   bool fp64 = false;
-  // the rho tasks in groups of one grid size (RhoGeom::nfft), each group one
-  // persistent launch with its own block counter
+  // the rho tasks in groups of one grid size (RhoGeom::nfft), first those of the
+  // streams' first problems, each group one persistent launch with its own
+  // block counter
   struct RhoGroup {
+    bool late;
     int nfft, first, count;
     int64_t total;
     size_t smem;
@@ -83,12 +90,16 @@ chi0_status build_tasks(chi0_batch* b, int jm_max, std::vector<chi0::RhoTask<T, 
                         std::vector<chi0_batch::RhoGroup>& groups) {
   tasks.clear();
   groups.clear();
-  std::vector<chi0_ctx*> items;
-  for (chi0_ctx* c : b->items)
-    if (c->nt > 0) items.push_back(c);
-  std::stable_sort(items.begin(), items.end(),
-                   [](const chi0_ctx* x, const chi0_ctx* y) { return x->geom.nfft < y->geom.nfft; });
-  for (chi0_ctx* c : items) {
+  std::vector<int> items;
+  for (size_t i = 0; i < b->items.size(); ++i)
+    if (b->items[i]->nt > 0) items.push_back((int)i);
+  std::stable_sort(items.begin(), items.end(), [&](int x, int y) {
+    if (b->late[x] != b->late[y]) return b->late[x] < b->late[y];
+    return b->items[x]->geom.nfft < b->items[y]->geom.nfft;
+  });
+  for (int i : items) {
+    chi0_ctx* c = b->items[i];
+    const bool late = b->late[i] != 0;
     chi0::RhoTask<T, TOUT> tk;
     size_t sm = 0;
     int64_t nb = 0;
@@ -98,8 +109,8 @@ chi0_status build_tasks(chi0_batch* b, int jm_max, std::vector<chi0::RhoTask<T, 
         (const typename chi0::C2<T>::t*)c->d_tw1.p, (const typename chi0::C2<T>::t*)c->d_tw2.p,
         (TOUT*)c->d_R.p, jm_max, &tk, &sm, &nb);
     if (e != cudaSuccess) return CHI0_EUNSUPPORTED;
-    if (groups.empty() || groups.back().nfft != c->geom.nfft)
-      groups.push_back({c->geom.nfft, (int)tasks.size(), 0, 0, 0});
+    if (groups.empty() || groups.back().late != late || groups.back().nfft != c->geom.nfft)
+      groups.push_back({late, c->geom.nfft, (int)tasks.size(), 0, 0, 0});
     chi0_batch::RhoGroup& g = groups.back();
     tk.block0 = g.total;
     g.total += nb;
@@ -130,20 +141,28 @@ chi0_status upload_tasks(chi0_batch* b, int jm) {
   return CHI0_OK;
 }
 
+// the groups of one kind on per_sm blocks per SM; counters zeroed with the first
 template <typename T, typename TOUT>
-cudaError_t launch_tasks(chi0_batch* b, cudaStream_t st) {
+cudaError_t launch_tasks(chi0_batch* b, bool late, int per_sm, cudaStream_t st) {
   if (b->groups.empty()) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(b->counter.p, 0, b->groups.size() * 8, st);
+  cudaError_t e = late ? cudaSuccess : cudaMemsetAsync(b->counter.p, 0, b->groups.size() * 8, st);
   for (size_t i = 0; i < b->groups.size() && e == cudaSuccess; ++i) {
     const chi0_batch::RhoGroup& g = b->groups[i];
+    if (g.late != late) continue;
     e = chi0::launch_rho_batch<T, TOUT>((const chi0::RhoTask<T, TOUT>*)b->tasks.p + g.first, g.count, g.total, g.nfft,
-                                        b->jm, g.smem, (unsigned long long*)b->counter.p + i, b->nsm, st);
+                                        b->jm, g.smem, (unsigned long long*)b->counter.p + i, per_sm * b->nsm, st);
   }
   return e;
 }
 
-cudaError_t launch_batched_rho(chi0_batch* b, cudaStream_t st) {
-  return b->fp64 ? launch_tasks<double, double2>(b, st) : launch_tasks<float, float2>(b, st);
+cudaError_t launch_batched_rho(chi0_batch* b, bool late, int per_sm, cudaStream_t st) {
+  return b->fp64 ? launch_tasks<double, double2>(b, late, per_sm, st) : launch_tasks<float, float2>(b, late, per_sm, st);
+}
+
+// every group (the tuning)
+cudaError_t launch_all_rho(chi0_batch* b, cudaStream_t st) {
+  const cudaError_t e = launch_batched_rho(b, false, 2, st);
+  return e == cudaSuccess ? launch_batched_rho(b, true, 2, st) : e;
 }
 
 chi0_status set_tasks(chi0_batch* b, int jm) {
@@ -179,12 +198,12 @@ chi0_status autotune(chi0_batch* b, cudaStream_t st) {
   float best_ms = 1e30f;
   for (int jm : {4, 2, 1}) {
     if (set_tasks(b, jm) != CHI0_OK) continue;
-    if (launch_batched_rho(b, st) != cudaSuccess) {  // warm-up
+    if (launch_all_rho(b, st) != cudaSuccess) {  // warm-up
       cudaGetLastError();
       continue;
     }
     cudaEventRecord(e0, st);
-    cudaError_t le = launch_batched_rho(b, st);
+    cudaError_t le = launch_all_rho(b, st);
     cudaEventRecord(e1, st);
     float ms = 0.f;
     if (le != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
@@ -340,9 +359,13 @@ chi0_status chi0_batch_create(chi0_ctx* const* ctxs, const int* iqs, void* const
     std::stable_sort(b->order.begin(), b->order.end(), [&](int x, int y) { return b->cost[x] > b->cost[y]; });
     std::vector<double> load(ns, 0.0);
     b->stream_of.assign(n, 0);
+    b->late.assign(n, 0);
     for (int i : b->order) {
       const int h = (int)(std::min_element(load.begin(), load.end()) - load.begin());
       b->stream_of[i] = h;
+      // in the mixed form every problem but its stream's first waits with rho
+      // (in the FP64 form rho needs the units of the Dyson step itself)
+      b->late[i] = !b->fp64 && load[h] > 0.0;
       load[h] += b->cost[i];
     }
     // shared scratch of each stream: every slot as large as its largest user
@@ -394,7 +417,7 @@ chi0_status chi0_batch_create(chi0_ctx* const* ctxs, const int* iqs, void* const
     if (cudaStreamCreateWithFlags(&hs, cudaStreamNonBlocking) != cudaSuccess) s = CHI0_ECUDA;
     else b->helpers.push_back(hs);
   }
-  for (int k = 0; k < 2 * ns + 2 && s == CHI0_OK; ++k) {
+  for (int k = 0; k < 2 * ns + 3 && s == CHI0_OK; ++k) {
     cudaEvent_t e = nullptr;
     if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) s = CHI0_ECUDA;
     else b->evs.push_back(e);
@@ -464,13 +487,29 @@ chi0_status chi0_batch_run(chi0_batch* b, void* stream) {
       s = chi0::launch_rho(c, false);
     }
     join(0);
-    if (s == CHI0_OK && launch_batched_rho(b, st) != cudaSuccess) s = CHI0_ECUDA;
+    if (s == CHI0_OK && launch_batched_rho(b, false, 2, st) != cudaSuccess) s = CHI0_ECUDA;
     if (!b->items.empty()) b->items[0]->launches += (int64_t)b->groups.size();
     // the rest of every problem on its stream, in the planned order
     fork(b->evs[2 * ns + 1]);
-    for (int i : b->order) {
-      if (s != CHI0_OK) break;
+    // (the first problem of a stream comes before its others)
+    std::vector<int> seq;
+    for (int i : b->order)
+      if (!b->late[i]) seq.push_back(i);
+    const size_t nearly = seq.size();
+    for (int i : b->order)
+      if (b->late[i]) seq.push_back(i);
+    for (size_t pos = 0; pos < seq.size() && s == CHI0_OK; ++pos) {
+      const int i = seq[pos];
       chi0_ctx* c = b->items[i];
+      if (pos == nearly) {   // the late problems' rho, behind the contractions queued so far
+        for (size_t q = 0; q < nearly; ++q)
+          if (chi0::overlaps_dyson(b->items[seq[q]]) && b->outs[seq[q]])
+            cudaStreamWaitEvent(st, b->items[seq[q]]->ev_join_ct, 0);
+        if (launch_batched_rho(b, true, 1, st) != cudaSuccess) s = CHI0_ECUDA;
+        cudaEventRecord(b->evs[2 * ns + 2], st);
+        for (cudaStream_t h : b->helpers) cudaStreamWaitEvent(h, b->evs[2 * ns + 2], 0);
+        if (s != CHI0_OK) break;
+      }
       c->st = b->helpers[b->stream_of[i]];
       c->rho_iq = c->plan_rho_iq;
       s = b->outs[i] ? chi0::launch_chi0_eps(c) : chi0::launch_chi0(c);

@@ -1252,13 +1252,17 @@ chi0_status launch_eps(chi0_ctx* c) {
   return CHI0_OK;
 }
 
+bool overlaps_dyson(const chi0_ctx* c) {
+  return !(c->fp64 || c->term_params || c->nt == 0 || c->cfg.nw < 2 || c->stream_nb > 0);
+}
+
 chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
   const int iq = c->plan_chi_iq;
   if (copied) *copied = false;
   if (iq < 0 || c->plan_eps_iq != iq) return fail(c, CHI0_ESTATE, "build and Dyson step not planned");
   const int nw = c->cfg.nw, ng = c->cfg.ng;
   chi0_status s;
-  if (c->fp64 || c->term_params || c->nt == 0 || nw < 2 || c->stream_nb > 0) {
+  if (!overlaps_dyson(c)) {
     // FP64 contraction and Dyson share the FP64 pipe; the learned terminator
     // needs every frequency of chi0 first: no overlap to gain
     if ((s = launch_chi0(c)) != CHI0_OK) return s;

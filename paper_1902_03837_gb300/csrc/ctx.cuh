@@ -270,4 +270,6 @@ chi0_status launch_eps(chi0_ctx* c);
 // the Dyson stream; *copied tells whether it was written (only the
 // overlapped pipeline does so)
 chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out = nullptr, bool* copied = nullptr);
+// whether it does so (then ev_join_ct marks the end of the contractions)
+bool overlaps_dyson(const chi0_ctx* c);
 }  // namespace chi0

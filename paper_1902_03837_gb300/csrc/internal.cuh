@@ -120,10 +120,10 @@ cudaError_t rho_task_make(const RhoGeom& g, const typename C2<T>::t* U, const in
 
 // Persistent rho over many tasks of one nfft in one launch (tasks_dev: device
 // array with block0 prefix offsets; total: all blocks; counter: device
-// scratch, zero when the launch starts).
+// scratch, zero when the launch starts; grid: blocks at most).
 template <typename T, typename TOUT>
 cudaError_t launch_rho_batch(const RhoTask<T, TOUT>* tasks_dev, int ntasks, int64_t total, int nfft, int jm,
-                             size_t smem, unsigned long long* counter, int nsm, cudaStream_t s);
+                             size_t smem, unsigned long long* counter, int grid, cudaStream_t s);
 
 // Kernels of rho_fft.cuh by grid size (rho_fft32.cu, rho_fft64.cu).
 namespace rfft {
@@ -135,7 +135,7 @@ cudaError_t rho_dispatch(const RhoTask<T, typename C2<T>::t>& tk, size_t smem, i
                          cudaStream_t s);
 template <typename T>
 cudaError_t batch_dispatch(int nfft, const RhoTask<T, typename C2<T>::t>* tasks, int ntasks, int64_t total,
-                           size_t smem, unsigned long long* counter, int nsm, cudaStream_t s);
+                           size_t smem, unsigned long long* counter, int grid, cudaStream_t s);
 }  // namespace rfft
 
 // a3: real transition weights w[iw][t] (FP64), or w[iw][row] of the nrow

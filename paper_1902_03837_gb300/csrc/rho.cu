@@ -881,11 +881,10 @@ cudaError_t launch_rho_pairs(const RhoGeom& g, const typename C2<T>::t* U, const
 
 template <typename T, typename TOUT>
 cudaError_t launch_rho_batch(const RhoTask<T, TOUT>* tasks_dev, int ntasks, int64_t total, int nfft, int jm,
-                             size_t smem, unsigned long long* counter, int nsm, cudaStream_t s) {
+                             size_t smem, unsigned long long* counter, int grid, cudaStream_t s) {
   if (ntasks == 0 || total == 0) return cudaSuccess;
-  if (nfft) return rfft::batch_dispatch<T>(nfft, tasks_dev, ntasks, total, smem, counter, nsm, s);
+  if (nfft) return rfft::batch_dispatch<T>(nfft, tasks_dev, ntasks, total, smem, counter, grid, s);
   cudaError_t e = cudaSuccess;
-  const int grid = nsm * 2;
   switch (jm) {
     case 4:
       e = cudaFuncSetAttribute(k_rho_batch<T, 4, TOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -320,12 +320,11 @@ cudaError_t rho_launch(const RhoTask<T, typename C2<T>::t>& tk, size_t smem, int
 
 template <typename T, int N>
 cudaError_t batch_launch(const RhoTask<T, typename C2<T>::t>* tasks, int ntasks, int64_t total, size_t smem,
-                         unsigned long long* counter, int nsm, cudaStream_t s) {
+                         unsigned long long* counter, int grid, cudaStream_t s) {
   cudaError_t e =
       cudaFuncSetAttribute(k_rho_fft_batch<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int64_t grid = total < 2 * nsm ? total : 2 * nsm;
-  k_rho_fft_batch<T, N><<<(unsigned)grid, kMaxThreads, smem, s>>>(tasks, ntasks, total, counter);
+  k_rho_fft_batch<T, N><<<(unsigned)(total < grid ? total : grid), kMaxThreads, smem, s>>>(tasks, ntasks, total, counter);
   return cudaGetLastError();
 }
 
@@ -362,8 +361,8 @@ cudaError_t rho_dispatch(const RhoTask<T, typename C2<T>::t>& tk, size_t smem, i
 }
 template <typename T>
 cudaError_t batch_dispatch(int nfft, const RhoTask<T, typename C2<T>::t>* tasks, int ntasks, int64_t total,
-                           size_t smem, unsigned long long* counter, int nsm, cudaStream_t s) {
-#define CHI0_CALL(n) batch_launch<T, n>(tasks, ntasks, total, smem, counter, nsm, s)
+                           size_t smem, unsigned long long* counter, int grid, cudaStream_t s) {
+#define CHI0_CALL(n) batch_launch<T, n>(tasks, ntasks, total, smem, counter, grid, s)
   CHI0_RHO_FFT_SWITCH(nfft, CHI0_CALL)
 #undef CHI0_CALL
 }

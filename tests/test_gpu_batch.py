@@ -136,3 +136,40 @@ def test_batch_validation(lib):
     with pytest.raises(lib.Chi0Error, match="EINVAL"):      # a problem without output
         lib.Batch([c], [0], [None])
     c.close()
+
+
+@pytest.mark.parametrize("nstreams", [1, 3])
+def test_batch_order_of_rho(lib, nstreams):
+    """In the mixed form a stream's first problem runs its rho ahead of the
+    others'.  Problems with and without a Dyson step or a chi0 output, one with
+    a single frequency (no overlap of contraction and Dyson step), in every
+    place of that order, against the one-at-a-time path: the same kernels, the
+    tuned split may group the FP32 sums differently (1e-6)."""
+    import torch
+    stream = torch.cuda.current_stream().cuda_stream
+    systems = [s for s, _ in _systems("c64")]   # system b twice, the same object
+    one = make_system(cfg_tiny(seed=64, kgrid=(2, 2, 2), q_frac=((0.5, 0.0, 0.5),), fft=(22, 22, 22), ng=90,
+                               n_occ=4, n_bands=14, npw_target=60, a=8.0, freqs=(0.3j,), eta=0.0,
+                               coef_dtype="c64"))
+    probs = [(systems[0], 0), (systems[1], 0), (one, 0), (systems[1], 1), (systems[3], 0)]
+    ref = [[t.cpu().numpy() for t in _single(lib, s, iq, 1, stream)] for s, iq in probs]
+    ctx_of = {}
+    for s, _ in probs:
+        if id(s) not in ctx_of:
+            ctx_of[id(s)] = lib.Chi0.for_system(s, precision=1, stream=stream)
+            ctx_of[id(s)].load_system(s)
+    ctxs = [ctx_of[id(s)] for s, _ in probs]
+    for drop in range(len(probs)):   # the problem without a Dyson step; the one after it without a chi0 output
+        buf = [torch.zeros((s.freqs.size, s.ng, s.ng), dtype=torch.complex128, device="cuda") for s, _ in probs]
+        chis = [torch.zeros_like(o) for o in buf]
+        outs = [None if i == drop else o for i, o in enumerate(buf)]
+        chi_out = [None if i == (drop + 1) % len(probs) else c for i, c in enumerate(chis)]
+        batch = lib.Batch(ctxs, [iq for _, iq in probs], outs, nstreams=nstreams, chi_out=chi_out)
+        batch.run(stream)
+        batch.synchronize()
+        batch.close()
+        for (chi_r, inv_r), c, o in zip(ref, chi_out, outs):
+            assert c is None or _rel(c.cpu().numpy(), chi_r) < 1e-6
+            assert o is None or _rel(o.cpu().numpy(), inv_r) < 1e-6
+    for c in ctx_of.values():
+        c.close()
