@@ -105,6 +105,28 @@ __device__ __forceinline__ C cfma_i(const C a, const T s, const C b) {
   return r;
 }
 
+// A constant of the transforms with the part that its rounding to T drops (0 in
+// FP64).  In FP32 the few constants of a column act on every transition alike,
+// so their rounding (up to 3e-8 each) would not average out: nine columns make
+// up a rho, and the gain of a 24-point one is 1e-8 off with rounded constants,
+// 1e-10 with these (extrapolar chi0 of N_G = 220 against 64 bits: 1.3e-7 -> 5e-8
+// for 2% of its time).  sum() is c a + s b with one rounding of the rest.
+template <typename T>
+struct Const {
+  T hi, lo;
+  constexpr Const(double v) : hi((T)v), lo((T)(v - (double)(T)v)) {}
+};
+template <typename T>
+__device__ __forceinline__ T times(const Const<T> c, const T a) {
+  if constexpr (sizeof(T) == 4) return fma(c.hi, a, c.lo * a);
+  else return c.hi * a;
+}
+template <typename T>
+__device__ __forceinline__ T sum(const Const<T> c, const T a, const Const<T> s, const T b) {
+  if constexpr (sizeof(T) == 4) return fma(c.hi, a, fma(s.hi, b, fma(c.lo, a, s.lo * b)));
+  else return fma(c.hi, a, s.hi * b);
+}
+
 // a e^{2 pi i P / Q}
 template <int P, int Q, typename C>
 __device__ __forceinline__ C twiddle(const C a) {
@@ -122,10 +144,15 @@ __device__ __forceinline__ C twiddle(const C a) {
   } else if constexpr (4 * p == 3 * Q) {
     r.x = a.y;
     r.y = -a.x;
+  } else if constexpr (sizeof(T) == 4 && 8 * p % Q == 0) {   // |cos| = |sin|
+    constexpr Const<std::remove_const_t<T>> c(cos_frac(p, Q));
+    constexpr bool same = 8 * p == Q || 8 * p == 5 * Q;
+    r.x = times(c, same ? a.x - a.y : a.x + a.y);
+    r.y = times(c, same ? a.y + a.x : a.y - a.x);
   } else {
-    constexpr double c = cos_frac(p, Q), s = sin_frac(p, Q);
-    r.x = fma((std::remove_const_t<T>)c, a.x, (std::remove_const_t<T>)(-s) * a.y);
-    r.y = fma((std::remove_const_t<T>)c, a.y, (std::remove_const_t<T>)s * a.x);
+    constexpr Const<std::remove_const_t<T>> c(cos_frac(p, Q)), s(sin_frac(p, Q)), ms(-sin_frac(p, Q));
+    r.x = sum(c, a.x, ms, a.y);
+    r.y = sum(c, a.y, s, a.x);
   }
   return r;
 }
@@ -169,12 +196,20 @@ __device__ __forceinline__ void column(C (&a)[N]) {
     a[1] = csub(a[0], b);
     a[0] = cadd(a[0], b);
   } else if constexpr (N == 3) {
-    constexpr T s = (T)sin_frac(1, 3);
+    constexpr Const<T> s(sin_frac(1, 3));
     const C t = cadd(a[1], a[2]), d = csub(a[1], a[2]);
     const C m = cfma(a[0], (T)-0.5, t);
     a[0] = cadd(a[0], t);
-    a[1] = cfma_i(m, s, d);
-    a[2] = cfma_i(m, (T)-s, d);
+    if constexpr (sizeof(T) == 4) {
+      C e;
+      e.x = times(s, d.x);
+      e.y = times(s, d.y);
+      a[1] = cadd_i(m, e);
+      a[2] = csub_i(m, e);
+    } else {
+      a[1] = cfma_i(m, s.hi, d);
+      a[2] = cfma_i(m, -s.hi, d);
+    }
   } else if constexpr (N == 4) {
     const C s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]);
     const C s13 = cadd(a[1], a[3]), d13 = csub(a[1], a[3]);
@@ -183,14 +218,23 @@ __device__ __forceinline__ void column(C (&a)[N]) {
     a[2] = csub(s02, s13);
     a[3] = csub_i(d02, d13);
   } else if constexpr (N == 5) {
-    constexpr T c1 = (T)cos_frac(1, 5), c2 = (T)cos_frac(2, 5), s1 = (T)sin_frac(1, 5), s2 = (T)sin_frac(2, 5);
+    constexpr Const<T> c1(cos_frac(1, 5)), c2(cos_frac(2, 5));
+    constexpr Const<T> s1(sin_frac(1, 5)), s2(sin_frac(2, 5)), ms1(-sin_frac(1, 5));
     const C t1 = cadd(a[1], a[4]), t2 = cadd(a[2], a[3]), d1 = csub(a[1], a[4]), d2 = csub(a[2], a[3]);
-    const C m1 = cfma(cfma(a[0], c1, t1), c2, t2), m2 = cfma(cfma(a[0], c2, t1), c1, t2);
-    C e1, e2;
-    e1.x = fma(s1, d1.x, s2 * d2.x);
-    e1.y = fma(s1, d1.y, s2 * d2.y);
-    e2.x = fma(s2, d1.x, -s1 * d2.x);
-    e2.y = fma(s2, d1.y, -s1 * d2.y);
+    C m1, m2, e1, e2;
+    if constexpr (sizeof(T) == 4) {
+      m1.x = a[0].x + sum(c1, t1.x, c2, t2.x);
+      m1.y = a[0].y + sum(c1, t1.y, c2, t2.y);
+      m2.x = a[0].x + sum(c2, t1.x, c1, t2.x);
+      m2.y = a[0].y + sum(c2, t1.y, c1, t2.y);
+    } else {
+      m1 = cfma(cfma(a[0], c1.hi, t1), c2.hi, t2);
+      m2 = cfma(cfma(a[0], c2.hi, t1), c1.hi, t2);
+    }
+    e1.x = sum(s1, d1.x, s2, d2.x);
+    e1.y = sum(s1, d1.y, s2, d2.y);
+    e2.x = sum(s2, d1.x, ms1, d2.x);
+    e2.y = sum(s2, d1.y, ms1, d2.y);
     a[0] = cadd(a[0], cadd(t1, t2));
     a[1] = cadd_i(m1, e1);
     a[4] = csub_i(m1, e1);

@@ -222,8 +222,19 @@ __device__ __forceinline__ void rho_fft_block(const RhoTask<T, typename C2<T>::t
     }
     __syncthreads();
   }
-  // x columns of the pairs, put in the order of the response set in zs
-  const T scale = (T)(1.0 / ((double)N * N * N));
+  // x columns of the pairs, put in the order of the response set in zs.  1 / N^3
+  // in FP32 carries its rounding error along: rounded alone it would shift every
+  // rho by the same 3e-8 and chi0 by twice that, which no sum averages out.
+  constexpr double inv = 1.0 / ((double)N * N * N);
+  constexpr T scale = (T)inv;
+  auto scaled = [&](T v) {
+    if constexpr (sizeof(T) == 4) {
+      constexpr T rest = (T)(inv - (double)scale);
+      return fma(v, scale, v * rest);
+    } else {
+      return v * scale;
+    }
+  };
   for (int u = tid; u < cm * P; u += nth) {
     const int j = u / P, p = u - j * P;
     T2 a[N];
@@ -237,8 +248,8 @@ __device__ __forceinline__ void rho_fft_block(const RhoTask<T, typename C2<T>::t
       if ((unsigned)(h - hx_base) < (unsigned)HX) {
         const int k = __ldg(lut + h * P);
         if (k >= 0) {
-          a[i].x *= scale;
-          a[i].y *= scale;
+          a[i].x = scaled(a[i].x);
+          a[i].y = scaled(a[i].y);
           o[k] = a[i];
         }
       }
