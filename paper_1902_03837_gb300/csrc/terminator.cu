@@ -165,7 +165,7 @@ struct TrainSmem {
   MlpWeights w;
   alignas(16) float h1[kS * kLd], h2[kS * kLd], d2[kS * kLd], d1[kS * kLd];   // rounded operands
   alignas(16) float r2[kS * kLd], r1[kS * kLd];                               // dz2, dz1 as computed
-  float xs[kS * kI], ys[kS * kO], red[kThreads / 32];
+  float xs[kS * kI], ys[kS * kO], red[32];
 };
 __global__ void __launch_bounds__(kThreads, 1)
 k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const float* __restrict__ t, int64_t batch,
@@ -213,11 +213,14 @@ k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const fl
     lsum = r * r;
     sm.ys[tid] = r / (float)batch;
   }
-#pragma unroll
-  for (int w = 16; w > 0; w >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, w);
-  if (lane == 0) sm.red[warp] = lsum;
+  if (warp == 1) sm.red[lane] = lsum;
   __syncthreads();
-  if (tid == 0) loss_part[blockIdx.x] = 0.5f * (sm.red[0] + sm.red[1]) / (float)batch;   // kS kO = 64 values
+  if (warp == 0) {   // kS kO = 64 values
+    lsum += sm.red[lane];
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, w);
+    if (lane == 0) loss_part[blockIdx.x] = 0.5f * lsum / (float)batch;
+  }
   // dz2 = (dy W3) * (1 - h2^2)
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -338,32 +341,28 @@ k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const fl
 static_assert(sizeof(MlpWeights) % 16 == 0 && kLd % 4 == 0, "16-byte pieces");
 static_assert(kS * kO == 64 && kThreads == 2 * kH && kO * kH == kThreads, "thread maps of k_mlp_train");
 
-// Sum of the block partials in a fixed order: four interleaved sums per
-// parameter (their loads are independent), then the four.
-constexpr int kRedP = 64, kRedW = 4;
-__global__ void __launch_bounds__(kRedP * kRedW)
+// Sum of the block partials, block by block: the order is that of the samples,
+// whatever their number.  32 loads of a thread are in flight; the chain of
+// additions (128 at the minibatch of 4096, 0.3 us) is not what the kernel waits for.
+constexpr int kRedP = 64;
+__global__ void __launch_bounds__(kRedP)
 k_mlp_reduce(const float* __restrict__ part, int nblk, const float* __restrict__ lpart, float* __restrict__ grad,
              float* __restrict__ loss) {
-  __shared__ float sums[kRedW][kRedP];
-  const int p = blockIdx.x * kRedP + threadIdx.x % kRedP, w = threadIdx.x / kRedP;
+  const int p = blockIdx.x * kRedP + threadIdx.x;
+  if (p > kP || (p == kP && !loss)) return;
+  const float* src = p < kP ? part + p : lpart;
+  const size_t stride = p < kP ? kP : 1;
   float g = 0.f;
-  if (p < kP) {
-#pragma unroll 8
-    for (int b = w; b < nblk; b += kRedW) g += part[(size_t)b * kP + p];
-  }
-  sums[w][threadIdx.x % kRedP] = g;
-  __syncthreads();
-  if (w == 0 && p < kP) {
-    for (int q = 1; q < kRedW; ++q) g += sums[q][threadIdx.x];
-    grad[p] = g;
-  }
-  if (blockIdx.x == 0 && loss && threadIdx.x < 32) {
-    float l = 0.f;
-    for (int b = threadIdx.x; b < nblk; b += 32) l += lpart[b];
+  int b = 0;
+  for (; b + 32 <= nblk; b += 32) {
+    float v[32];
 #pragma unroll
-    for (int q = 16; q > 0; q >>= 1) l += __shfl_xor_sync(0xffffffffu, l, q);
-    if (threadIdx.x == 0) *loss = l;
+    for (int i = 0; i < 32; ++i) v[i] = src[(size_t)(b + i) * stride];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) g += v[i];
   }
+  for (; b < nblk; ++b) g += src[(size_t)b * stride];
+  *(p < kP ? grad + p : loss) = g;
 }
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -389,7 +388,7 @@ cudaError_t mlp_loss_grad(const float* prm, const float* x, const float* t, int6
   cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(TrainSmem));
   if (e != cudaSuccess) return e;
   k_mlp_train<<<nblk, kThreads, sizeof(TrainSmem), st>>>(prm, x, t, batch, bf16, part, lpart);
-  k_mlp_reduce<<<(kP + kRedP - 1) / kRedP, kRedP * kRedW, 0, st>>>(part, nblk, lpart, grad, loss);
+  k_mlp_reduce<<<kP / kRedP + 1, kRedP, 0, st>>>(part, nblk, lpart, grad, loss);
   return cudaGetLastError();
 }
 
