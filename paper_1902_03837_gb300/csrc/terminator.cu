@@ -109,28 +109,26 @@ __device__ __forceinline__ float layer3(const MlpWeights& w, const float* __rest
   return z;
 }
 
-// Prediction: two blocks per SM stay for the whole launch and take kSP samples
-// at a time, so that the parameters are staged once per block.  Bound by the
-// FP32 pipe (17.3 k multiply-adds and 256 tanh per sample): 10^6 samples 5180 ->
-// 929 us (0.67 ms of issue slots).
+// Prediction with FP32 operands: two blocks per SM stay for the whole launch and
+// take kSP samples at a time, so that the parameters are staged once per block.
+// Bound by the FP32 pipe (17.3 k multiply-adds and 256 tanh per sample): 10^6
+// samples 5180 -> 929 us (0.67 ms of issue slots).
 struct PredictSmem {
   MlpWeights w;
   alignas(16) float h[kSP * kLd];
   float xs[kSP * kI];
 };
 __global__ void __launch_bounds__(kThreads, 2)
-k_mlp_predict(const float* __restrict__ prm, const float* __restrict__ x, int64_t batch, int bf16,
-              float* __restrict__ y) {
+k_mlp_predict(const float* __restrict__ prm, const float* __restrict__ x, int64_t batch, float* __restrict__ y) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PredictSmem& sm = *reinterpret_cast<PredictSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  load_weights(sm.w, prm, bf16);
+  load_weights(sm.w, prm, 0);
   for (int64_t s0 = (int64_t)blockIdx.x * kSP; s0 < batch; s0 += (int64_t)gridDim.x * kSP) {
     const int ns = (int)min((int64_t)kSP, batch - s0);
-    for (int e = tid; e < kSP * kI; e += kThreads) sm.xs[e] = e < ns * kI ? rb(x[s0 * kI + e], bf16) : 0.f;
+    for (int e = tid; e < kSP * kI; e += kThreads) sm.xs[e] = e < ns * kI ? x[s0 * kI + e] : 0.f;
     __syncthreads();
-    for (int s = tid / kH; s < kSP; s += kThreads / kH)
-      sm.h[s * kLd + tid % kH] = rb(layer1(sm.w, sm.xs, s, tid % kH), bf16);
+    for (int s = tid / kH; s < kSP; s += kThreads / kH) sm.h[s * kLd + tid % kH] = layer1(sm.w, sm.xs, s, tid % kH);
     __syncthreads();
     float acc[kSP / 8][4];
 #pragma unroll
@@ -143,7 +141,7 @@ k_mlp_predict(const float* __restrict__ prm, const float* __restrict__ x, int64_
     for (int i = 0; i < kSP / 8; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        sm.h[(i * 8 + (lane >> 2)) * kLd + j * 32 + warp * 4 + (lane & 3)] = rb(tanhf(acc[i][j]), bf16);
+        sm.h[(i * 8 + (lane >> 2)) * kLd + j * 32 + warp * 4 + (lane & 3)] = tanhf(acc[i][j]);
     __syncthreads();
     if (tid < kSP * kO) {
       const int s = tid % kSP, o = tid / kSP;
@@ -152,6 +150,227 @@ k_mlp_predict(const float* __restrict__ prm, const float* __restrict__ x, int64_
     }
     // the next pass writes xs (read before the last barrier but one) and h
     // (behind its own first barrier)
+  }
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ float low_bf16(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float high_bf16(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+// c += a b^T, 16 x 8 x 16, BF16 operands, FP32 sums.  With g = lane / 4 and t =
+// lane % 4: a = rows g, g + 8 at k = 2t, 2t + 1, then both at k + 8; b = row g at
+// the same k; c = rows g, g + 8 at columns 2t, 2t + 1.
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// four 8 x 8 matrices of BF16 (lane l gives the address of row l % 8 of matrix
+// l / 8): lane l gets row l / 4, columns 2 (l % 4), + 1 of each
+__device__ __forceinline__ void ldsm(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p))
+               : "memory");
+}
+
+// Prediction with BF16 operands: the 128 x 128 layer on the tensor cores.  A warp
+// takes 16 samples from input to output without a barrier: its lanes compute the
+// first layer where the matrix instruction wants the operand and the last one
+// where it leaves the sums.  256 tanh and 900 multiply-adds per sample remain on
+// the FP32 pipe and bound the kernel, not the matrix product (so the register
+// form of the instruction does, and TMEM's extra trips would not be hidden).
+//
+// h2 = bf16(tanh(z)) keeps the value that the chain of FP32 multiply-adds in the
+// order of k gives (as the training kernel computes it): the tensor core's z
+// differs from the chain's by its rounding only, so the two can round apart
+// only next to a rounding boundary.  Where z +- kDoubt sum_k |W2[h][k]| straddles
+// one (some 16 of a warp's 2048 values), the value goes on a list, and the chain
+// is run for up to 32 of the list at a time, one per lane.  kDoubt is three times
+// the largest rounding error of the chain seen over 2.6 million values (3.9e-8 of
+// that sum); a value it misses would be off by one rounding of an operand.
+// 10^6 samples: 929 us on the FP32 pipe -> 348 us (0.26 ms of issue slots).
+constexpr float kDoubt = 1.f / 8388608.f;
+constexpr int kLdb = kH + 8;        // padded row of BF16: eight rows' 16-byte pieces fall into distinct banks
+constexpr int kPredWarps = 8;
+constexpr int kList = 32 + 128;     // below 32 before a step, which adds 128 at most
+struct PredictBf16Smem {
+  alignas(16) __nv_bfloat16 w2[kH * kLdb];
+  alignas(16) __nv_bfloat16 h1[kPredWarps][16 * kLdb];
+  float4 w1[kH];                    // inputs 0..3
+  float4 w3[kH / 2];                // both outputs' weights of two inputs
+  float2 w1b[kH];                   // input 4, bias
+  float2 b2[kH / 2], doubt[kH / 2];
+  uint32_t list[kPredWarps][kList]; // h2 as the tensor core's z gives it | sample | column
+};
+static_assert(kPredWarps * 32 == kThreads, "a warp per tile");
+__global__ void __launch_bounds__(kThreads, 2)
+k_mlp_predict_bf16(const float* __restrict__ prm, const float* __restrict__ x, int64_t batch, float* __restrict__ y) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  PredictBf16Smem& sm = *reinterpret_cast<PredictBf16Smem*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+#pragma unroll 8
+  for (int e = tid; e < kH * kH; e += kThreads) sm.w2[(e / kH) * kLdb + e % kH] = __float2bfloat16_rn(prm[kOffW2 + e]);
+  if (tid < kH) {
+    const float* w = prm + kOffW1 + tid * kI;
+    sm.w1[tid] = make_float4(rb(w[0], 1), rb(w[1], 1), rb(w[2], 1), rb(w[3], 1));
+    sm.w1b[tid] = make_float2(rb(w[4], 1), prm[kOffB1 + tid]);
+  } else if (tid < kH + kH / 2) {
+    const int p = tid - kH;
+    const float* w = prm + kOffW3 + 2 * p;
+    sm.w3[p] = make_float4(rb(w[0], 1), rb(w[1], 1), rb(w[kH], 1), rb(w[kH + 1], 1));
+    sm.b2[p] = make_float2(prm[kOffB2 + 2 * p], prm[kOffB2 + 2 * p + 1]);
+  }
+  const float b3 = prm[kOffB3 + (t & 1)];
+  __syncthreads();
+  if (tid < kH) {
+    float s = 0.f;
+    for (int k = 0; k < kH; ++k) s += fabsf(__bfloat162float(sm.w2[tid * kLdb + k]));
+    reinterpret_cast<float*>(sm.doubt)[tid] = kDoubt * s;
+  }
+  __syncthreads();
+  __nv_bfloat16* h1s = sm.h1[warp];
+  uint32_t* list = sm.list[warp];
+  for (int64_t s0 = ((int64_t)blockIdx.x * kPredWarps + warp) * 16; s0 < batch;
+       s0 += (int64_t)gridDim.x * kPredWarps * 16) {
+    float xr[2][kI];   // rows g, g + 8 of the tile
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int i = 0; i < kI; ++i) xr[r][i] = s0 + g + 8 * r < batch ? rb(x[(s0 + g + 8 * r) * kI + i], 1) : 0.f;
+    uint32_t a[kH / 16][4];
+#pragma unroll
+    for (int ks = 0; ks < kH / 16; ++ks)
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        float h[2][2];
+        const int c0 = ks * 16 + half * 8 + t * 2;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const float4 w = sm.w1[c0 + j];
+          const float2 wb = sm.w1b[c0 + j];
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            float z = fmaf(w.x, xr[r][0], wb.y);
+            z = fmaf(w.y, xr[r][1], z);
+            z = fmaf(w.z, xr[r][2], z);
+            z = fmaf(w.w, xr[r][3], z);
+            h[r][j] = tanhf(fmaf(wb.x, xr[r][4], z));
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          a[ks][2 * half + r] = pack_bf16(h[r][0], h[r][1]);
+          *reinterpret_cast<uint32_t*>(h1s + (g + 8 * r) * kLdb + c0) = a[ks][2 * half + r];
+        }
+      }
+    float out[2][kO] = {};
+    int n = 0;   // entries on the list
+    // the chains of the last cnt entries; their h2 in place of the tensor core's
+    auto settle = [&](int cnt) {
+      __syncwarp();
+      n -= cnt;
+      float d = 0.f;
+      int row = 0, col = 0;
+      if (lane < cnt) {
+        const uint32_t e = list[n + lane];
+        row = (e >> 7) & 15;
+        col = e & (kH - 1);
+        float z = reinterpret_cast<const float*>(sm.b2)[col];
+        const uint4* hp = reinterpret_cast<const uint4*>(h1s + row * kLdb);
+        const uint4* wp = reinterpret_cast<const uint4*>(sm.w2 + col * kLdb);
+#pragma unroll 4
+        for (int k = 0; k < kH / 8; ++k) {
+          const uint4 h = hp[k], w = wp[k];
+          const uint32_t hv[4] = {h.x, h.y, h.z, h.w}, wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            z = fmaf(low_bf16(wv[q]), low_bf16(hv[q]), z);
+            z = fmaf(high_bf16(wv[q]), high_bf16(hv[q]), z);
+          }
+        }
+        d = rb(tanhf(z), 1) - high_bf16(e);
+      }
+      for (uint32_t m = __ballot_sync(0xffffffffu, !(d == 0.f)); m; m &= m - 1) {
+        const int b = __ffs(m) - 1;
+        const int rr = __shfl_sync(0xffffffffu, row, b), cc = __shfl_sync(0xffffffffu, col, b);
+        const float dd = __shfl_sync(0xffffffffu, d, b);
+        const float* w = reinterpret_cast<const float*>(sm.w3 + (cc >> 1)) + (cc & 1);
+        if (lane == (rr & 7) * 4) {
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+            if (rr >> 3 == r) {
+              out[r][0] = fmaf(w[0], dd, out[r][0]);
+              out[r][1] = fmaf(w[2], dd, out[r][1]);
+            }
+        }
+      }
+      __syncwarp();
+    };
+    for (int n0 = 0; n0 < kH; n0 += 16) {
+      float c[2][4];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float2 b2 = sm.b2[n0 / 2 + 4 * j + t];
+        c[j][0] = c[j][2] = b2.x;
+        c[j][1] = c[j][3] = b2.y;
+      }
+#pragma unroll
+      for (int ks = 0; ks < kH / 16; ++ks) {
+        uint32_t b[4];
+        ldsm(b, sm.w2 + (n0 + (lane & 7) + (lane >> 4) * 8) * kLdb + ks * 16 + ((lane >> 3) & 1) * 8);
+        mma_bf16(c[0], a[ks], b[0], b[1]);
+        mma_bf16(c[1], a[ks], b[2], b[3]);
+      }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int p = n0 / 2 + 4 * j + t;
+        const float4 w = sm.w3[p];
+        const float2 dz = sm.doubt[p];
+        uint32_t h[2], open[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const float h0 = tanhf(c[j][2 * r]), h1 = tanhf(c[j][2 * r + 1]);
+          // dz times the slope of tanh, and an ulp for tanhf itself
+          const float e0 = fmaf(dz.x, fmaf(-h0, h0, 1.f), 1.2e-7f), e1 = fmaf(dz.y, fmaf(-h1, h1, 1.f), 1.2e-7f);
+          h[r] = pack_bf16(h0, h1);
+          open[r] = pack_bf16(h0 + e0, h1 + e1) ^ pack_bf16(h0 - e0, h1 - e1);
+          const float r0 = low_bf16(h[r]), r1 = high_bf16(h[r]);
+          out[r][0] = fmaf(w.y, r1, fmaf(w.x, r0, out[r][0]));
+          out[r][1] = fmaf(w.w, r1, fmaf(w.z, r0, out[r][1]));
+        }
+        if (__any_sync(0xffffffffu, (open[0] | open[1]) != 0)) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {   // row g + 8 (v / 2), column 2 p + v % 2
+            const uint32_t o = v & 1 ? open[v >> 1] >> 16 : open[v >> 1] & 0xffffu;
+            const uint32_t m = __ballot_sync(0xffffffffu, o != 0);
+            if (o != 0)
+              list[n + __popc(m & ((1u << lane) - 1))] =
+                  (v & 1 ? h[v >> 1] & 0xffff0000u : h[v >> 1] << 16) | (uint32_t)((g + 8 * (v >> 1)) << 7) |
+                  (uint32_t)(2 * p + (v & 1));
+            n += __popc(m);
+          }
+          while (n >= 32) settle(32);
+        }
+      }
+    }
+    if (n > 0) settle(n);
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int o = 0; o < kO; ++o) {
+        out[r][o] += __shfl_xor_sync(0xffffffffu, out[r][o], 1);
+        out[r][o] += __shfl_xor_sync(0xffffffffu, out[r][o], 2);
+      }
+    // lane t writes output t % 2 of row g + 8 (t / 2)
+    const float lo = t & 1 ? out[0][1] : out[0][0], hi = t & 1 ? out[1][1] : out[1][0];
+    const int64_t row = s0 + g + 8 * (t >> 1);
+    if (row < batch) y[row * kO + (t & 1)] = (t & 2 ? hi : lo) + b3;
+    __syncwarp();   // h1 of the next tile
   }
 }
 
@@ -394,12 +613,12 @@ cudaError_t mlp_loss_grad(const float* prm, const float* x, const float* t, int6
 
 cudaError_t mlp_predict(const float* prm, const float* x, int64_t batch, int bf16, float* y,
                         cudaStream_t st) {
-  const int64_t passes = (batch + kSP - 1) / kSP;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_mlp_predict, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(PredictSmem));
+  const int64_t rows = bf16 ? 16 * kPredWarps : kSP, passes = (batch + rows - 1) / rows;
+  const size_t smem = bf16 ? sizeof(PredictBf16Smem) : sizeof(PredictSmem);
+  auto kernel = bf16 ? k_mlp_predict_bf16 : k_mlp_predict;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_mlp_predict<<<(unsigned)(passes < 2 * 152 ? passes : 2 * 152), kThreads, sizeof(PredictSmem), st>>>(prm, x, batch,
-                                                                                                       bf16, y);
+  kernel<<<(unsigned)(passes < 2 * 152 ? passes : 2 * 152), kThreads, smem, st>>>(prm, x, batch, y);
   return cudaGetLastError();
 }
 
