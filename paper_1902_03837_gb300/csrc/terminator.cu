@@ -30,6 +30,7 @@ constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kH * kI, kOffW2 = kOffB1 + kH, kOffB
 constexpr int kS = 32;         // samples per block of the training kernel
 constexpr int kSP = 64;        // samples per pass of the prediction kernel
 constexpr int kThreads = 256;
+constexpr int kTrainThreads = 512;
 constexpr int kLd = kH + 4;    // padded row: eight rows' 16-byte pieces fall into distinct banks
 
 __device__ __forceinline__ float rb(float v, int bf16) {
@@ -37,7 +38,7 @@ __device__ __forceinline__ float rb(float v, int bf16) {
 }
 
 // acc[i][j] += sum_k A[s_i][k] B[h_j][k], k ascending (rows of kLd floats in
-// shared memory; s_i = 8 i + lane / 4, h_j = 32 j + 4 warp + lane % 4).  Both
+// shared memory; s_i = 8 i + lane / 4, h_j = 32 j + 4 (warp % 8) + lane % 4).  Both
 // layers of the network are bound by the FP32 pipe once the operands come as
 // 16-byte pieces for NS x 4 outputs per thread (one load per 2 NS x 8 / (NS + 4)
 // multiply-adds; a scalar pair of loads per multiply-add was bound by shared
@@ -45,7 +46,7 @@ __device__ __forceinline__ float rb(float v, int bf16) {
 // order of k, so the results do not depend on the tiling.
 template <int NS>
 __device__ __forceinline__ void rows_dot(const float* __restrict__ A, const float* __restrict__ B, float (&acc)[NS][4]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) & 7;
   const float* a = A + (lane >> 2) * kLd;
   const float* b = B + (warp * 4 + (lane & 3)) * kLd;
 #pragma unroll 2
@@ -73,13 +74,14 @@ struct alignas(16) MlpWeights {
   alignas(16) float w3[kO * kH];
   float w1[kH * kI], b1[kH], b2[kH], b3[kO];
 };
+template <int NT>   // threads of the block
 __device__ __forceinline__ void load_weights(MlpWeights& w, const float* __restrict__ prm, int bf16) {
   const int tid = threadIdx.x;
-#pragma unroll 8
-  for (int e = tid; e < kH * kH; e += kThreads)   // (the caller's vector is only 4-byte aligned)
+#pragma unroll 16
+  for (int e = tid; e < kH * kH; e += NT)   // (the caller's vector is only 4-byte aligned)
     w.W2[(e / kH) * kLd + e % kH] = rb(prm[kOffW2 + e], bf16);
-  for (int e = tid; e < kH * kI; e += kThreads) w.w1[e] = rb(prm[kOffW1 + e], bf16);
-  for (int e = tid; e < kO * kH; e += kThreads) w.w3[e] = rb(prm[kOffW3 + e], bf16);
+  for (int e = tid; e < kH * kI; e += NT) w.w1[e] = rb(prm[kOffW1 + e], bf16);
+  for (int e = tid; e < kO * kH; e += NT) w.w3[e] = rb(prm[kOffW3 + e], bf16);
   if (tid < kH) {
     w.b1[tid] = prm[kOffB1 + tid];
     w.b2[tid] = prm[kOffB2 + tid];
@@ -123,7 +125,7 @@ k_mlp_predict(const float* __restrict__ prm, const float* __restrict__ x, int64_
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PredictSmem& sm = *reinterpret_cast<PredictSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  load_weights(sm.w, prm, 0);
+  load_weights<kThreads>(sm.w, prm, 0);
   for (int64_t s0 = (int64_t)blockIdx.x * kSP; s0 < batch; s0 += (int64_t)gridDim.x * kSP) {
     const int ns = (int)min((int64_t)kSP, batch - s0);
     for (int e = tid; e < kSP * kI; e += kThreads) sm.xs[e] = e < ns * kI ? x[s0 * kI + e] : 0.f;
@@ -377,16 +379,17 @@ k_mlp_predict_bf16(const float* __restrict__ prm, const float* __restrict__ x, i
 // Forward and backward for kS samples per block.  Gradients of the block go to
 // part[block][kP] (summed later in a fixed order).  Per-sample values are the
 // same chains as in the prediction; the three products of 32 x 128 x 128 (h2,
-// dz1, dW2) take 4 x 4, 4 x 4 and 8 x 8 outputs per thread.  A block holds an SM
-// (one per SM at the minibatch of 4096): a training step there, with the
-// reduction and Adam, 91.7 -> 36.3 us.
+// dz1, dW2) take 2 x 4, 2 x 4 and 8 x 4 outputs per thread.  A block holds an SM
+// (one per SM at the minibatch of 4096), so its own 16 warps have to cover the
+// latencies: a training step there, with the reduction and Adam, 91.7 us -> 36.8
+// with 8 warps and twice the outputs per thread -> 34.8 us.
 struct TrainSmem {
   MlpWeights w;
   alignas(16) float h1[kS * kLd], h2[kS * kLd], d2[kS * kLd], d1[kS * kLd];   // rounded operands
   alignas(16) float r2[kS * kLd], r1[kS * kLd];                               // dz2, dz1 as computed
   float xs[kS * kI], ys[kS * kO], red[32];
 };
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kTrainThreads, 1)
 k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const float* __restrict__ t, int64_t batch,
             int bf16, float* __restrict__ part, float* __restrict__ loss_part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -394,15 +397,15 @@ k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const fl
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t s0 = (int64_t)blockIdx.x * kS;
   const int ns = (int)min((int64_t)kS, batch - s0);
-  load_weights(sm.w, prm, bf16);
-  for (int e = tid; e < kS * kI; e += kThreads) sm.xs[e] = e < ns * kI ? rb(x[s0 * kI + e], bf16) : 0.f;
+  load_weights<kTrainThreads>(sm.w, prm, bf16);
+  for (int e = tid; e < kS * kI; e += kTrainThreads) sm.xs[e] = e < ns * kI ? rb(x[s0 * kI + e], bf16) : 0.f;
   __syncthreads();
-  const int sr = lane >> 2;                        // rows sr + 8 i
-  const int hc = warp * 4 + (lane & 3);            // layer 2: columns hc + 32 j
-  const int kc = hc * 4;                           // layer 1: columns kc + j
-  float h1v[4][4], h2v[4][4];
+  const int r0 = (warp >> 3) * 16, sr = r0 + (lane >> 2);   // rows sr + 8 i of the warp's half
+  const int hc = (warp & 7) * 4 + (lane & 3);               // layer 2: columns hc + 32 j
+  const int kc = hc * 4;                                    // layer 1: columns kc + j
+  float h1v[2][4], h2v[2][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < 2; ++i) {
     float4 r;
 #pragma unroll
     for (int j = 0; j < 4; ++j) h1v[i][j] = layer1(sm.w, sm.xs, sr + 8 * i, kc + j);
@@ -411,12 +414,12 @@ k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const fl
   }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) h2v[i][j] = sm.w.b2[hc + 32 * j];
-  rows_dot(sm.h1, sm.w.W2, h2v);
+  rows_dot(sm.h1 + r0 * kLd, sm.w.W2, h2v);
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       h2v[i][j] = tanhf(h2v[i][j]);
@@ -442,7 +445,7 @@ k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const fl
   }
   // dz2 = (dy W3) * (1 - h2^2)
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int s = sr + 8 * i, h = hc + 32 * j;
@@ -457,20 +460,20 @@ k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const fl
   __syncthreads();
   // dz1 = (dz2 W2) * (1 - h1^2), h ascending
   {
-    float g[4][4];
+    float g[2][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) g[i][j] = 0.f;
 #pragma unroll 2
     for (int h = 0; h < kH; h += 4) {
-      float4 dv[4], wv[4];
+      float4 dv[2], wv[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) dv[i] = *reinterpret_cast<const float4*>(sm.d2 + (sr + 8 * i) * kLd + h);
+      for (int i = 0; i < 2; ++i) dv[i] = *reinterpret_cast<const float4*>(sm.d2 + (sr + 8 * i) * kLd + h);
 #pragma unroll
       for (int q = 0; q < 4; ++q) wv[q] = *reinterpret_cast<const float4*>(sm.w.W2 + (h + q) * kLd + kc);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < 2; ++i) {
         const float dq[4] = {dv[i].x, dv[i].y, dv[i].z, dv[i].w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -482,7 +485,7 @@ k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const fl
       }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 2; ++i) {
       const int s = sr + 8 * i;
       float d[4];
 #pragma unroll
@@ -499,66 +502,68 @@ k_mlp_train(const float* __restrict__ prm, const float* __restrict__ x, const fl
   float* gp = part + (size_t)blockIdx.x * kP;
   // dW2[h][k] = sum_s dz2[s][h] h1[s][k]
   {
-    const int h0 = (tid >> 4) * 8, k0 = (tid & 15) * 8;
-    float g[8][8];
+    const int h0 = (tid >> 5) * 8, k0 = lane * 4;
+    float g[8][4];
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
-      for (int b = 0; b < 8; ++b) g[a][b] = 0.f;
+      for (int b = 0; b < 4; ++b) g[a][b] = 0.f;
+#pragma unroll 4
     for (int s = 0; s < kS; ++s) {
       const float4 d0 = *reinterpret_cast<const float4*>(sm.d2 + s * kLd + h0);
       const float4 d1 = *reinterpret_cast<const float4*>(sm.d2 + s * kLd + h0 + 4);
       const float4 a0 = *reinterpret_cast<const float4*>(sm.h1 + s * kLd + k0);
-      const float4 a1 = *reinterpret_cast<const float4*>(sm.h1 + s * kLd + k0 + 4);
       const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
-      const float h[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float h[4] = {a0.x, a0.y, a0.z, a0.w};
 #pragma unroll
       for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b) g[a][b] = fmaf(d[a], h[b], g[a][b]);
+        for (int b = 0; b < 4; ++b) g[a][b] = fmaf(d[a], h[b], g[a][b]);
     }
     if (((uintptr_t)gp & 7) == 0) {   // kP and kOffW2 are even: 8-byte pieces where the caller's buffer allows
 #pragma unroll
       for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; b += 2)
+        for (int b = 0; b < 4; b += 2)
           *reinterpret_cast<float2*>(gp + kOffW2 + (h0 + a) * kH + k0 + b) = make_float2(g[a][b], g[a][b + 1]);
     } else {
 #pragma unroll
       for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b) gp[kOffW2 + (h0 + a) * kH + k0 + b] = g[a][b];
+        for (int b = 0; b < 4; ++b) gp[kOffW2 + (h0 + a) * kH + k0 + b] = g[a][b];
     }
   }
-  // dW3[o][h] = sum_s dy[s][o] h2[s][h];  db3
-  {
+  if (tid < 2 * kH) {
+    // dW3[o][h] = sum_s dy[s][o] h2[s][h]
     const int o = tid / kH, h = tid % kH;
     float g = 0.f;
+#pragma unroll 8
     for (int s = 0; s < kS; ++s) g = fmaf(rb(sm.ys[s * kO + o], bf16), sm.h2[s * kLd + h], g);
     gp[kOffW3 + tid] = g;
-  }
-  if (tid < kO) {
-    float g = 0.f;
-    for (int s = 0; s < kS; ++s) g += sm.ys[s * kO + tid];
-    gp[kOffB3 + tid] = g;
-  }
-  {  // db2, db1
-    const int h = tid % kH;
+    // db2, db1
     const float* r = tid < kH ? sm.r2 : sm.r1;
-    float g = 0.f;
+    g = 0.f;
+#pragma unroll 8
     for (int s = 0; s < kS; ++s) g += r[s * kLd + h];
     gp[(tid < kH ? kOffB2 : kOffB1) + h] = g;
-  }
-  // dW1[h][i] = sum_s dz1[s][h] x[s][i]
-  for (int e = tid; e < kH * kI; e += kThreads) {
-    const int h = e / kI, i = e % kI;
-    float g = 0.f;
-    for (int s = 0; s < kS; ++s) g = fmaf(sm.d1[s * kLd + h], sm.xs[s * kI + i], g);
-    gp[kOffW1 + e] = g;
+  } else {
+    // dW1[h][i] = sum_s dz1[s][h] x[s][i];  db3
+    for (int e = tid - 2 * kH; e < kH * kI; e += kTrainThreads - 2 * kH) {
+      const int h = e / kI, i = e % kI;
+      float g = 0.f;
+#pragma unroll 8
+      for (int s = 0; s < kS; ++s) g = fmaf(sm.d1[s * kLd + h], sm.xs[s * kI + i], g);
+      gp[kOffW1 + e] = g;
+    }
+    if (tid - 2 * kH < kO) {
+      float g = 0.f;
+      for (int s = 0; s < kS; ++s) g += sm.ys[s * kO + tid - 2 * kH];
+      gp[kOffB3 + tid - 2 * kH] = g;
+    }
   }
 }
 static_assert(sizeof(MlpWeights) % 16 == 0 && kLd % 4 == 0, "16-byte pieces");
-static_assert(kS * kO == 64 && kThreads == 2 * kH && kO * kH == kThreads, "thread maps of k_mlp_train");
+static_assert(kS == 32 && kTrainThreads == 4 * kH && kO == 2, "thread maps of k_mlp_train");
 
 // Sum of the block partials, block by block: the order is that of the samples,
 // whatever their number.  32 loads of a thread are in flight; the chain of
@@ -606,7 +611,7 @@ cudaError_t mlp_loss_grad(const float* prm, const float* x, const float* t, int6
   const int nblk = (int)((batch + kS - 1) / kS);
   cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(TrainSmem));
   if (e != cudaSuccess) return e;
-  k_mlp_train<<<nblk, kThreads, sizeof(TrainSmem), st>>>(prm, x, t, batch, bf16, part, lpart);
+  k_mlp_train<<<nblk, kTrainThreads, sizeof(TrainSmem), st>>>(prm, x, t, batch, bf16, part, lpart);
   k_mlp_reduce<<<kP / kRedP + 1, kRedP, 0, st>>>(part, nblk, lpart, grad, loss);
   return cudaGetLastError();
 }
