@@ -73,7 +73,7 @@ k_sig_gemm64(const double2* __restrict__ Wd, const double2* __restrict__ R, int 
     Y[((size_t)(t / 64) * nI + i / 64) * 4096 + (size_t)(i % 64) * 64 + t % 64] = make_double2(sx, sy);
 }
 
-constexpr int kDotUnroll = 8;   // values of i per thread between FP64 sums
+constexpr int kDotUnroll = 4;   // values of i per thread between compensated sums
 
 __device__ __forceinline__ size_t tile_off(int64_t t, int i, int nI) {
   return ((size_t)(t >> 6) * nI + (i >> 6)) * 4096 + (size_t)(i & 63) * 64 + (t & 63);
@@ -131,8 +131,13 @@ struct DotSum {
 // Each thread reads its column of Y and the columns (g, a) of RT (tile
 // layout, both coalesced across the warp), A partners per pass.  Products in
 // the element type of rho, summed kDotUnroll at a time into a DotSum.
+// Bound by the latency of its loads (the data comes mostly from L2): all of a
+// step's loads are issued together, the last ragged step's as well (its rows
+// repeat the last one, with Y as 0), and with kQuad (FP32, a multiple of A
+// partners, so that a group's columns start on 16 bytes) two partners come per
+// load: N_G = 300, 16384 columns, two frequencies 55 -> 46 us.
 constexpr int kDotP = 8;
-template <typename TR, typename TY, int A>
+template <typename TR, typename TY, int A, bool kQuad>
 __global__ void __launch_bounds__(32 * kDotP, (sizeof(TR) == 8 && A == 4) ? 3 : 1)
 k_sig_dot(const TR* __restrict__ RT, const TY* __restrict__ Y, int ng, int64_t T, int nqp, int nI, double pref,
           double2* __restrict__ out, size_t ystride, size_t ostride) {
@@ -153,45 +158,40 @@ k_sig_dot(const TR* __restrict__ RT, const TY* __restrict__ Y, int ng, int64_t T
     DotSum<F> sx[A], sy[A];
     if (live) {
       for (int i0 = ph; i0 < ng; i0 += kDotP * kDotUnroll) {
+        TY yv[kDotUnroll];
+        TR rv[kDotUnroll][A];
+#pragma unroll
+        for (int r = 0; r < kDotUnroll; ++r) {
+          const int i = i0 + kDotP * r, ic = i < ng ? i : ng - 1;
+          const size_t ro = (size_t)(ic >> 6) * 4096 + (size_t)(ic & 63) * 64;
+          yv[r] = Ycol[ro];
+          if (i >= ng) yv[r].x = yv[r].y = 0;
+          if constexpr (kQuad) {
+#pragma unroll
+            for (int q = 0; q < A; q += 2) {
+              const float4 v = *reinterpret_cast<const float4*>(col[q] + ro);
+              rv[r][q].x = v.x;
+              rv[r][q].y = v.y;
+              rv[r][q + 1].x = v.z;
+              rv[r][q + 1].y = v.w;
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < A; ++q) rv[r][q] = col[q][ro];
+          }
+        }
         F cx[A], cy[A];
 #pragma unroll
         for (int q = 0; q < A; ++q) cx[q] = cy[q] = 0;
-        if (i0 + kDotP * (kDotUnroll - 1) < ng) {
-          // a full block of kDotUnroll values of i: no guards, so that every
-          // load of the block can be in flight at once
-          TY yv[kDotUnroll];
 #pragma unroll
-          for (int r = 0; r < kDotUnroll; ++r) {
-            const int i = i0 + kDotP * r;
-            yv[r] = Ycol[(size_t)(i >> 6) * 4096 + (size_t)(i & 63) * 64];
-          }
+        for (int r = 0; r < kDotUnroll; ++r) {
+          const F yx = (F)yv[r].x, yy = (F)yv[r].y;
 #pragma unroll
-          for (int r = 0; r < kDotUnroll; ++r) {
-            const int i = i0 + kDotP * r;
-            const size_t ro = (size_t)(i >> 6) * 4096 + (size_t)(i & 63) * 64;
-            const F yx = (F)yv[r].x, yy = (F)yv[r].y;
-#pragma unroll
-            for (int q = 0; q < A; ++q)
-              if (a0 + q < nqp) {
-                const TR v = col[q][ro];
-                cx[q] += v.x * yx - v.y * yy;
-                cy[q] += v.x * yy + v.y * yx;
-              }
-          }
-        } else {
-          for (int r = 0; r < kDotUnroll; ++r) {
-            const int i = i0 + kDotP * r;
-            if (i >= ng) break;
-            const size_t ro = (size_t)(i >> 6) * 4096 + (size_t)(i & 63) * 64;
-            const TY yd = Ycol[ro];
-            const F yx = (F)yd.x, yy = (F)yd.y;
-#pragma unroll
-            for (int q = 0; q < A; ++q)
-              if (a0 + q < nqp) {
-                const TR v = col[q][ro];
-                cx[q] += v.x * yx - v.y * yy;
-                cy[q] += v.x * yy + v.y * yx;
-              }
+          for (int q = 0; q < A; ++q) {   // (partners past nqp repeat one that is not written)
+            cx[q] = fma(rv[r][q].x, yx, cx[q]);
+            cx[q] = fma(-rv[r][q].y, yy, cx[q]);
+            cy[q] = fma(rv[r][q].x, yy, cy[q]);
+            cy[q] = fma(rv[r][q].y, yx, cy[q]);
           }
         }
 #pragma unroll
@@ -248,10 +248,11 @@ cudaError_t launch_sig_dot(const TR* RT, const TY* Y, int ng, int64_t T, int nqp
                            cudaStream_t s, int nf, size_t ystride, size_t ostride) {
   const int nI = (ng + 63) / 64;
   const dim3 grid((unsigned)((T + 31) / 32), (unsigned)nf);
-  if (nqp <= 4)   // fewer partners per pass: fewer registers, more resident blocks
-    k_sig_dot<TR, TY, 4><<<grid, 32 * kDotP, 0, s>>>(RT, Y, ng, T, nqp, nI, pref, out, ystride, ostride);
-  else
-    k_sig_dot<TR, TY, 8><<<grid, 32 * kDotP, 0, s>>>(RT, Y, ng, T, nqp, nI, pref, out, ystride, ostride);
+  constexpr bool f32 = sizeof(TR) == 8;
+  // up to 4 partners per pass: fewer registers, more resident blocks
+  auto kernel = nqp <= 4 ? (f32 && nqp == 4 ? k_sig_dot<TR, TY, 4, f32> : k_sig_dot<TR, TY, 4, false>)
+                         : (f32 && nqp % 8 == 0 ? k_sig_dot<TR, TY, 8, f32> : k_sig_dot<TR, TY, 8, false>);
+  kernel<<<grid, 32 * kDotP, 0, s>>>(RT, Y, ng, T, nqp, nI, pref, out, ystride, ostride);
   return cudaGetLastError();
 }
 

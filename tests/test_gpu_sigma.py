@@ -176,3 +176,24 @@ def test_sigma_i_argument_checks(lib):
     with pytest.raises(lib.Chi0Error, match="ESTATE"):
         fresh.build_sigma_i(0, 4, 6, inv, out)         # chi0_compute_rho first
     fresh.close()
+
+
+@pytest.mark.parametrize("ng,fft", [(31, 20), (33, 20), (65, 20)])
+def test_sigma_i_windows(lib, ng, fft):
+    """Every way the dot products group the partners of a window (up to 4 or 8
+    at a time, two per load or one), at N_G around the 32 values of i of a step:
+    a window of one size is a block of any wider one, whose entries are the same
+    dot products of the same columns in FP32 (1e-5, the oracle's bound)."""
+    import torch
+    s = _sys("c64", ng=ng, fft=fft)
+    ctx, inv = _eps_inv_gpu(lib, s, 1)
+    ref = _oracle_i(s, inv.cpu().numpy(), list(range(0, 16)))
+    for n in (1, 2, 3, 4, 5, 7, 8, 12, 16):
+        out = torch.zeros((s.freqs.size, s.nk, s.nb, n, n), dtype=torch.complex128, device="cuda")
+        ctx.build_sigma_i(0, 16 - n, 16, inv, out)
+        ctx.synchronize()
+        for iw, w in enumerate(s.freqs):
+            if w.real != 0.0:
+                e = _rel(out[iw].cpu().numpy(), ref[iw][:, :, 16 - n:, 16 - n:])
+                assert e < 1e-5, (n, iw, e)
+    ctx.close()
