@@ -336,6 +336,34 @@ chi0_status plan_geometry(chi0_ctx* c, int iq) {
   return CHI0_OK;
 }
 
+// The column transforms' grid is rounded up to their next size, so its states
+// can take more than those of a caller's grid that is just alias free (30^3
+// against 25 x 25 x 17: 2.5 times).  Where they have to grow and memory would then
+// not hold them, rho and the smallest set of contraction operands (at most two
+// pairs, each of rho's size), the caller's grid is kept.
+static bool column_grid_fits(const chi0_ctx* c) {
+  const RhoGeom& g = c->geom;
+  RhoGeom own = g;
+  own.nfft = 0;
+  own.N1 = c->cfg.fft[0];
+  own.N2 = c->cfg.fft[1];
+  own.N3 = c->cfg.fft[2];
+  if (!g.nfft || c->nt == 0 || chi0::rho_volume(g) <= chi0::rho_volume(own)) return true;
+  const double cb = cplx_bytes(c), vol = (double)chi0::rho_volume(g) * cb;
+  const int bnb = std::max(1, std::min(c->stream_nb, c->Nn));
+  const int bnk = std::max(1, std::min(c->stream_nk > 0 ? c->stream_nk : c->nk, c->nk));
+  const bool streamed = c->stream_nb > 0;
+  const double u = (double)c->nk * (streamed ? c->Nm : c->nb) * vol, ublk = streamed ? (double)bnk * bnb * vol : 0.0;
+  if (u <= (double)c->d_U.bytes) return true;
+  const double r = (double)(streamed ? (int64_t)bnk * bnb * c->Nm : c->nt) * g.ng * cb;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return u + ublk + (c->fp64 ? 1.0 : 3.0) * r <= (double)free_b + c->d_U.bytes + c->d_Ublk.bytes + c->d_R.bytes;
+}
+
 chi0_status plan_rho(chi0_ctx* c, int iq) {
   if (!c) return CHI0_EINVAL;
   if (iq < 0 || iq >= c->cfg.nq) return fail(c, CHI0_EINVAL, "iq %d out of range", iq);
@@ -348,6 +376,12 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
   }
   chi0_status s;
   if ((s = plan_geometry(c, iq)) != CHI0_OK) return s;
+  if (!c->rho_generic && c->rho_need_floor == 0 && !column_grid_fits(c)) {
+    c->rho_generic = true;
+    s = plan_geometry(c, iq);
+    c->rho_generic = false;
+    if (s != CHI0_OK) return s;
+  }
   RhoGeom& g = c->geom;
   const std::vector<int32_t>& rows = c->h_rows;
   const std::vector<int16_t>& lut = c->h_lut;
@@ -372,9 +406,9 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
   const size_t plane_bytes = chi0::rho_volume(g) * cb;
   // streamed: the m-band grids of every k (resident) and one block's n grids
   const size_t ubytes = streamed ? (size_t)c->nk * c->Nm * plane_bytes : (size_t)c->nk * c->nb * plane_bytes;
-  if ((s = ensure(c, c->d_U, ubytes, "mixed-grid wavefunctions")) != CHI0_OK) return s;
+  if ((s = ensure(c, c->d_U, ubytes, "states on the grid")) != CHI0_OK) return s;
   if (streamed &&
-      (s = ensure(c, c->d_Ublk, (size_t)c->blk_nk * c->blk_nb * plane_bytes, "mixed grids of a band block")) != CHI0_OK)
+      (s = ensure(c, c->d_Ublk, (size_t)c->blk_nk * c->blk_nb * plane_bytes, "states of a band block")) != CHI0_OK)
     return s;
   if ((s = ensure(c, c->d_R, (size_t)(streamed ? c->nt_blk : c->nt) * g.ng * cb, "rho")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_gresp, (size_t)g.ng * 12, "G set")) != CHI0_OK) return s;
