@@ -1,7 +1,7 @@
 """Benchmark of the chi0 / eps^-1 path on GB300.
 
 One step = the whole path over one synthetic system resident in HBM:
-wavefunctions -> mixed grid, oscillator strengths rho for every transition,
+wavefunctions -> real space, oscillator strengths rho for every transition,
 transition weights, the chi0 contraction for every frequency, and the FP64
 Dyson inversion eps~^-1 for every frequency (chi0_compute_rho +
 chi0_build_invert, which runs chi0_build_chi0 and chi0_invert_eps as one
@@ -61,8 +61,8 @@ def whole_job_tflops(world, flops_per_step, ms_per_step):
 
 
 # stage -> (binding roof, unit, kernel)
-STAGE_ROOF = {"contract": ("tensor", "TFLOP/s", "k_herk_wide"), "rho": ("alu", "TFLOP/s", "k_rho_pairs"),
-              "wf_grid": ("alu", "TFLOP/s", "k_wf_to_mixed"), "dyson": ("fp64", "TFLOP/s", "k_gj_update"),
+STAGE_ROOF = {"contract": ("tensor", "TFLOP/s", "k_herk_wide"), "rho": ("alu", "TFLOP/s", "k_rho_fft"),
+              "wf_grid": ("alu", "TFLOP/s", "k_wf_fft"), "dyson": ("fp64", "TFLOP/s", "k_gj_update"),
               "weights": ("hbm", "GB/s", "k_prep"), "reduce": ("hbm", "GB/s", "k_tc_reduce")}
 # FP32 FMA: 152 SMs x 128 lanes x 2 flop x 1.93 GHz (the clock seen under this load)
 FP32_PEAK, FP32_SRC = 75.0, "FP32 FMA: 152 SMs x 128 lanes x 2 flop x 1.93 GHz"
@@ -74,8 +74,8 @@ FP64_PEAK, FP64_SRC = 1.25, "FP64 nominal (GB300)"
 #   traffic: <kernel> | <workload> | <bytes per launch> | <source file> <sha256 prefix> | <how>
 # A figure is used only while the kernel's source file still has the hash it
 # had when the counters were taken; after any change it reads as null.
-KERNEL_SOURCE = {"k_herk_bf16x3": "tc.cu", "k_herk_wide": "tc.cu", "k_prep": "tc.cu", "k_rho_pairs": "rho.cu",
-                 "k_wf_to_mixed": "rho.cu", "k_gj_update": "dyson.cu", "k_chi0_fp64": "chi0_fp64.cu"}
+KERNEL_SOURCE = {"k_herk_wide": "tc.cu", "k_prep": "tc.cu", "k_rho_fft": "rho_fft.cuh",
+                 "k_wf_fft": "rho_fft.cuh", "k_gj_update": "dyson.cu", "k_chi0_fp64": "chi0_fp64.cu"}
 
 
 def source_sha(fname):
@@ -635,8 +635,8 @@ def run_ours(args, rank, world, dist):
     per_step_ms = {k: v / args.steps for k, v in st_ms.items()}
     roofs = dict(STAGE_ROOF)
     if args.precision == "fp64":  # every stage on the FP64 units
-        roofs.update({"contract": ("fp64", "TFLOP/s", "k_chi0_fp64"), "rho": ("fp64", "TFLOP/s", "k_rho_pairs"),
-                      "wf_grid": ("fp64", "TFLOP/s", "k_wf_to_mixed")})
+        roofs.update({"contract": ("fp64", "TFLOP/s", "k_chi0_fp64"), "rho": ("fp64", "TFLOP/s", "k_rho_fft"),
+                      "wf_grid": ("fp64", "TFLOP/s", "k_wf_fft")})
     bound, unit, kname = roofs[dom]
     # (complex weights of real frequencies: the same kernel over every tile)
     extra = {}
@@ -692,7 +692,7 @@ def run_ours(args, rank, world, dist):
         "metric": METRIC, "value": value, "unit": "TFLOP/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": ("bf16x3/fp32 (chi0), fp32 (rho), f64 (eps^-1)" if args.precision == "mixed" else "f64"), "data": "synthetic",
-        "config": {"workload": workload_name(args), "n_transitions": nt, "l2": "inputs larger than L2 (mixed grids 32 GB, rho 12 GB)",
+        "config": {"workload": workload_name(args), "n_transitions": nt, "l2": "inputs larger than L2 (states on the grid 11 GB, rho 12 GB)",
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "stage_ms_per_step": per_step_ms,
         "roofline": roof,
@@ -1111,8 +1111,8 @@ def run_terminator(args, rank, world, dist):
 def run_batching(args, rank, world, dist):
     """The batching workload: 16 seeded metallic systems of different sizes,
     every q point of each (4-20 per system, 200 problems), all in one batch
-    (one persistent rho launch, every other kernel in one CUDA graph; the q
-    points of a system share its mixed grids), against the same problems one
+    (persistent rho launches, every other kernel in one CUDA graph; the q
+    points of a system share its states on the grid), against the same problems one
     at a time, and the first problem in the plain FP64 form."""
     import torch
     import __graft_entry__ as g

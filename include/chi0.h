@@ -82,7 +82,8 @@ typedef struct {
   int kgrid[3];           /* Gamma-centred grid, k = (i/N1, j/N2, l/N3), k index = (i*N2+j)*N3+l */
   int nbands;             /* bands per k */
   int npw_max;            /* largest plane-wave sphere over all k */
-  int fft[3];             /* real-space grid (N1, N2, N3) used for rho; must be alias free */
+  int fft[3];             /* real-space grid (N1, N2, N3) of rho; must be alias free.  rho is the same sum on
+                             every alias-free grid: a smaller one is taken where a fast transform has it */
   int ng;                 /* number of response G vectors */
   int nq;                 /* number of q points */
   const double* q_frac;   /* [nq][3] reduced coordinates; each q must be a vector of the k grid;
@@ -198,7 +199,7 @@ chi0_status chi0_get_rho_rows(chi0_ctx* ctx, const int64_t* rows, int64_t nrows,
 /* Band-block streaming for problems whose oscillator strengths do not fit in
  * device memory (the paper distributes the response function's memory over
  * the band indices: Parallelism section, linear response).  With
- * bands_per_block > 0, chi0_compute_rho keeps only the mixed grids of the
+ * bands_per_block > 0, chi0_compute_rho keeps only the grids of the
  * occupied-side bands m (at every k) and chi0_build_chi0 / chi0_build_invert
  * take the transitions in blocks of k_per_block k points (0: all) times
  * bands_per_block bands n: for each block the n grids, rho, the weights and
@@ -258,7 +259,8 @@ chi0_status chi0_get_stats(chi0_ctx* ctx, double* ms, double* bytes, double* flo
  *   out:    device pointer, [nw][ng][ng] complex128, receives eps~^-1;
  *   cuda_stream: cudaStream_t (NULL = default stream).
  * It calls no allocating routine: its scratch (about 2.1 MB: panels for
- * ng <= 2048, the pivot-block inverse, V and an error flag) is one static
+ * ng <= 2048 or several smaller matrices at a time, their pivot blocks, V and
+ * an error flag) is one static
  * device array that every GPU loading this library holds until the process
  * exits.  The first call on a device looks up that array's device address
  * (once per device, with the device current); make that first call before
@@ -279,16 +281,18 @@ chi0_status chi0_invert_eps_noalloc(const void* chi0, const double* v_sqrt, int 
  * because the number of transitions varies.  A batch runs many independent
  * problems -- problem i is context ctxs[i] at q index iqs[i] -- as one unit.
  * A context may appear several times with different q indices (every q point
- * of one system): its problems share its coefficients and its mixed grids,
+ * of one system): its problems share its coefficients and its states on the grid,
  * which are computed once per replay.  At creation: all host set-up; the
  * problems' remaining work is assigned to `nstreams` helper streams, longest
  * first, each to the stream with the least estimated work, and the problems
  * of one stream share one set of scratch buffers (operands, partials, chi0,
  * Dyson panels) sized for the largest of them; the rho tile width and every
  * contraction's transition split are timed on the batch's own data and the
- * fastest kept.  Every replay runs the oscillator strengths of all problems
- * in ONE persistent launch over a device task table, the rest on the helper
- * streams, all captured once into a CUDA graph.
+ * fastest kept.  Every replay runs the oscillator strengths of the problems
+ * in one persistent launch per grid size over a device task table (in the mixed
+ * form those of every stream's first problem ahead, the others' beside the first
+ * problems' Dyson steps), the rest on the helper streams, all captured once
+ * into a CUDA graph.
  *   chi_out: NULL, or n device pointers to [nw_i][ng_i][ng_i] complex128
  *            receiving chi0 of each problem (NULL entries: not returned);
  *   eps_out: NULL, or n device pointers to [nw_i][ng_i][ng_i] complex128
@@ -322,7 +326,7 @@ chi0_status chi0_batch_synchronize(chi0_batch* b);
  * summed time of the fastest split of each contraction during the tuning. */
 chi0_status chi0_batch_info(const chi0_batch* b, int* stream_of, double* tuned_split_ms);
 
-/* m bands per block chosen for the persistent rho launch (1, 2 or 4). */
+/* m bands per block chosen for the persistent rho launches (1, 2 or 4). */
 int chi0_batch_rho_width(const chi0_batch* b);
 
 void chi0_batch_destroy(chi0_batch* b);
@@ -455,7 +459,7 @@ chi0_status chi0_set_double_grid(chi0_ctx* ctx, int nd, const double* eps_dense)
  * The contraction sum_j W^d_ij conj(rho(j)) runs on the tensor cores in the
  * mixed form (BF16x3 products, FP32 accumulation in 128-term pieces, FP64
  * sums), in plain FP64 in the FP64 form.  Requires chi0_compute_rho(iq)
- * (mixed-grid wavefunctions and the response set).  Device memory: rho of
+ * (the states on the grid and the response set).  Device memory: rho of
  * the window (nk nbands nqp ng complex) and an N_G x nk nbands nqp FP64
  * complex work array.
  * Errors: CHI0_EINVAL (window empty or outside [0, nbands), NULL pointer,
