@@ -1268,31 +1268,40 @@ k_sig_bsplit(const float2* __restrict__ R, int64_t T, int nqp, int nb, int ng, i
 
 // A: row 2 i + c, column j holds W^d_ij.c, Eq. (W_delta) with W = V E V:
 // W^d_ij = V_i V_j [ (Im E_ij + Im E_ji) / 2 - i (Re E_ij - Re E_ji) / 2 ].
+// A block takes 32 rows i by 64 columns j; the transposed entries E_ji come
+// through shared memory, so that both reads run along rows of E, and an
+// (i, j) gives both rows c: eight frequencies of N_G = 300 27 -> 20 us.
 __global__ void __launch_bounds__(256)
 k_sig_asplit(const double2* __restrict__ E, const double* __restrict__ v, int ng, int mpad_a, size_t stride,
              __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+  __shared__ double2 et[64][33];
   E += (size_t)blockIdx.z * ng * ng;   // frequency of the pass
   hi += blockIdx.z * stride;
   lo += blockIdx.z * stride;
-  const int r0 = blockIdx.x * 64;
-  const int kb = blockIdx.y;
+  const int i0 = blockIdx.x * 32, kb = blockIdx.y;
   for (int e = threadIdx.x; e < 64 * 32; e += 256) {
-    const int ml = e >> 5, jp = e & 31;
-    const int m = r0 + ml, i = m >> 1;
-    const int j = kb * 64 + 2 * jp;
-    float x[2] = {0.f, 0.f};
+    const int jl = e >> 5, il = e & 31, j = kb * 64 + jl, i = i0 + il;
+    if (j < ng && i < ng) et[jl][il] = E[(size_t)j * ng + i];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 32 * 32; e += 256) {
+    const int il = e >> 5, jp = e & 31, i = i0 + il;
+    float x[2] = {0.f, 0.f}, y[2] = {0.f, 0.f};
     if (i < ng) {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        const int jj = j + q;
-        if (jj < ng) {
-          const double2 a = E[(size_t)i * ng + jj], b = E[(size_t)jj * ng + i];
-          const double f = 0.5 * v[i] * v[jj];
-          x[q] = (float)((m & 1) ? -f * (a.x - b.x) : f * (a.y + b.y));
+        const int j = kb * 64 + 2 * jp + q;
+        if (j < ng) {
+          const double2 a = E[(size_t)i * ng + j], b = et[2 * jp + q][il];
+          const double f = 0.5 * v[i] * v[j];
+          x[q] = (float)(f * (a.y + b.y));
+          y[q] = (float)(-f * (a.x - b.x));
         }
       }
     }
-    split_store(x[0], x[1], hi, lo, ((size_t)kb * mpad_a + m) * 64 + 2 * jp);
+    const size_t off = ((size_t)kb * mpad_a + 2 * i) * 64 + 2 * jp;
+    split_store(x[0], x[1], hi, lo, off);
+    split_store(y[0], y[1], hi, lo, off + 64);
   }
 }
 
