@@ -375,6 +375,13 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
     return CHI0_OK;
   }
   chi0_status s;
+  // From here on the geometry, the k-pairs, the tables and, where a buffer
+  // grows, the states and rho themselves are those of this q point, which may
+  // need another grid than the last one.  A call that fails on the way leaves no
+  // plan and no results: the next one plans from the start.
+  c->rho_planned_epoch = 0;
+  c->plan_rho_iq = -1;
+  c->rho_iq = c->chi_iq = c->eps_iq = -1;
   if ((s = plan_geometry(c, iq)) != CHI0_OK) return s;
   if (!c->rho_generic && c->rho_need_floor == 0 && !column_grid_fits(c)) {
     c->rho_generic = true;
@@ -394,9 +401,8 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
     c->blk_nk = std::max(1, std::min(c->stream_nk > 0 ? c->stream_nk : c->nk, c->nk));
     c->nt_blk = (int64_t)c->blk_nk * c->blk_nb * c->Nm;
   }
-  c->rho_iq = c->chi_iq = c->eps_iq = -1;
-  c->plan_rho_iq = iq;
   if (c->nt == 0) {
+    c->plan_rho_iq = iq;
     c->rho_planned_epoch = c->plan_epoch;
     ++c->rho_plan_serial;
     return CHI0_OK;
@@ -471,6 +477,7 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
       a2.flops = (double)c->nt * (6.0 * n * n * n + col * (n * n + n * g.HZ + g.npair));
     }
   }
+  c->plan_rho_iq = iq;
   c->rho_planned_epoch = c->plan_epoch;
   ++c->rho_plan_serial;
   return CHI0_OK;
