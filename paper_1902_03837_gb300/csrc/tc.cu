@@ -755,8 +755,14 @@ bool make_map(CUtensorMap* m, void* ptr, int64_t kpad, int mpad) {
 chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   if (!c->tc) c->tc = new TcState();
   TcState& t = *static_cast<TcState*>(c->tc);
-  t.mpad = (2 * ng + kBM - 1) / kBM * kBM;
-  t.kpad = (nt + kBK - 1) / kBK * kBK;
+  const int mpad = (2 * ng + kBM - 1) / kBM * kBM;
+  const int64_t kpad = (nt + kBK - 1) / kBK * kBK;
+  // A batch plans every problem twice, the second time on scratch shared by the
+  // problems of a stream, which was sized from the first plan and cannot grow:
+  // the choices made from the free memory then stand, whatever is free now.
+  const bool settled = t.part.borrowed && t.mpad == mpad && t.kpad == kpad;
+  t.mpad = mpad;
+  t.kpad = kpad;
   const int nT = t.mpad / kBM;
   herm_tiles(t);
   t.total_kb = (int)(t.kpad / kBK);
@@ -772,7 +778,7 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   const size_t opb = (size_t)t.mpad * t.kpad * 2;
   // A buffers for up to kPrepGroup frequencies, as far as half of the free
   // device memory allows (one pair is always needed)
-  {
+  if (!settled) {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
       cudaGetLastError();
@@ -807,10 +813,10 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
       }
     nchunks = (t.total_kb + kbpc - 1) / kbpc;
   };
-  choose_split(t.ntiles, t.kbpc, t.nchunks, t.per);
+  if (!settled) choose_split(t.ntiles, t.kbpc, t.nchunks, t.per);
   // the full tile grid of the complex contraction of a real-axis frequency
   t.ntiles_f = nT * t.nJ;
-  choose_split(t.ntiles_f, t.kbpc_f, t.nchunks_f, t.per_f);
+  if (!settled) choose_split(t.ntiles_f, t.kbpc_f, t.nchunks_f, t.per_f);
   if (t.kpad / kPT > 0x7fffffff / t.mpad)
     return ctx_fail(c, CHI0_EUNSUPPORTED, "too many transitions for one contraction");
   chi0_status s;

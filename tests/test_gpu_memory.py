@@ -1,0 +1,85 @@
+"""Calls that have to work with little device memory: a block of the test's own
+leaves the free memory that each one names.  Sizes are some hundred MB, so that
+the 2 MB pieces of the device's allocator do not matter.
+"""
+import contextlib
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module")
+def lib():
+    import torch
+    assert torch.cuda.is_available()
+    import __graft_entry__ as g
+    g.build()
+    from paper_1902_03837_gb300 import chi0
+    return chi0
+
+
+@contextlib.contextmanager
+def _leave(nbytes):
+    """nbytes of device memory left free."""
+    import torch
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    fill = torch.empty(int(torch.cuda.mem_get_info()[0] - nbytes), dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        torch.cuda.synchronize()
+        del fill
+        torch.cuda.empty_cache()
+
+
+def _context(lib, kgrid, L, ng, nocc, nb, nw, qs, fft, seed=1):
+    """A mixed-form context on twelve plane waves per state that reach the
+    corners of the cube |G_a| <= L."""
+    import torch
+    rng = np.random.default_rng(seed)
+    nk = int(np.prod(kgrid))
+    corners = np.array([(L, -L, L), (-L, L, -L), (L, 0, 0), (0, -L, 0), (0, 0, L), (0, 0, 0)])
+    box = np.stack(np.meshgrid(*[np.arange(1, L)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    ctx = lib.Chi0(a=9.0, kgrid=kgrid, nbands=nb, npw_max=12, fft=fft, ng=ng, q_frac=qs,
+                   omega=1j * np.linspace(0.1, 2.0, nw), eta=0.0, precision=lib.CHI0_MIXED_BF16X3,
+                   stream=torch.cuda.current_stream().cuda_stream)
+    for ik in range(nk):
+        g = np.concatenate([corners, box[rng.choice(len(box), 6, replace=False)]]).astype(np.int32)
+        c = rng.standard_normal((nb, 12)) + 1j * rng.standard_normal((nb, 12))
+        ctx.set_wavefunctions(ik, g, (c / np.linalg.norm(c, axis=1, keepdims=True)).astype(np.complex64))
+    e = np.concatenate([rng.uniform(-0.4, 0.0, (nk, nocc)), rng.uniform(0.1, 1.0, (nk, nb - nocc))], 1)
+    ctx.set_energies(e, np.broadcast_to((np.arange(nb) < nocc).astype(float), (nk, nb)).copy())
+    ctx.synchronize()
+    return ctx
+
+
+def test_batch_keeps_its_first_plan(lib):
+    """204,800 transitions of N_G = 250 (390 MB per operand pair): with seven
+    pairs of memory left beside states and rho, a batch plans operands of three
+    of its four frequencies.  On the scratch sized for that it must not find room
+    for the fourth, whose partials would be three times as large."""
+    import torch
+    nocc, nb, ng, nw = 8, 408, 250, 4
+    ctx = _context(lib, (4, 4, 4), 3, ng, nocc, nb, nw, [(0.25, 0.0, 0.0)], (16, 16, 16))
+    out = [torch.zeros((nw, ng, ng), dtype=torch.complex128, device="cuda") for _ in range(2)]
+
+    def run():
+        batch = lib.Batch([ctx], [0], [out[0]], nstreams=1, chi_out=[out[1]])
+        batch.run(torch.cuda.current_stream().cuda_stream)
+        batch.synchronize()
+        batch.close()
+        return [o.cpu().numpy() for o in out]
+
+    ref = run()
+    nt = 64 * nocc * (nb - nocc)
+    pair = 512 * nt * 4
+    with _leave(64 * nb * 12 ** 3 * 8 + nt * ng * 8 + 7 * pair):
+        got = run()
+    ctx.close()
+    for a, b in zip(got, ref):            # the same products, summed in other pieces
+        assert np.linalg.norm(a - b) < 1e-6 * np.linalg.norm(b)
