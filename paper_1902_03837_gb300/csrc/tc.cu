@@ -776,21 +776,16 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
   }
   t.nsm = nsm;
   const size_t opb = (size_t)t.mpad * t.kpad * 2;
-  // A buffers for up to kPrepGroup frequencies, as far as half of the free
-  // device memory allows (one pair is always needed)
-  if (!settled) {
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
-      cudaGetLastError();
-      free_b = 0;
-    }
-    int have = 0;
-    while (have < kPrepGroup && t.ah[have].bytes >= opb && t.al[have].bytes >= opb) ++have;
-    int g = std::min(kPrepGroup, std::max(1, nw));
-    if (c->group_cap > 0) g = std::min(g, c->group_cap);
-    while (g > std::max(1, have) && (double)(g - have) * 2.0 * (double)opb > 0.5 * (double)free_b) --g;
-    t.group = g;
-  }
+  // the unit-weight operand B is read only by the two-operand form (weights
+  // of mixed signs) and by the complex contractions of real frequencies
+  const bool need_b = c->herk_sign == 0 || c->has_real;
+  // a batch problem (group_cap > 0) keeps room for twice the planned
+  // partials, for the split candidates of tc_tune_split
+  const size_t room = c->group_cap > 0 ? 2 : 1;
+  auto part_bytes = [&]() {
+    return 16 * std::max((size_t)t.per * t.nchunks * t.ntiles * room * kWPart,
+                         c->has_real ? (size_t)t.per_f * t.nchunks_f * t.ntiles_f * kWPart : (size_t)0);
+  };
   // Splits of the transitions and frequencies per launch, in units of one
   // k-block's products (0.8 us): whole waves of one CTA per SM, each unit 3
   // for its ramp and the write of its partial, each launch 8, and each split of
@@ -813,27 +808,48 @@ chi0_status tc_plan(chi0_ctx* c, int64_t nt, int ng, int nw) {
       }
     nchunks = (t.total_kb + kbpc - 1) / kbpc;
   };
-  if (!settled) choose_split(t.ntiles, t.kbpc, t.nchunks, t.per);
-  // the full tile grid of the complex contraction of a real-axis frequency
-  t.ntiles_f = nT * t.nJ;
-  if (!settled) choose_split(t.ntiles_f, t.kbpc_f, t.nchunks_f, t.per_f);
+  t.ntiles_f = nT * t.nJ;   // the full tile grid of the complex contraction of a real-axis frequency
+  // A buffers for up to kPrepGroup frequencies, as far as they leave half of the
+  // device memory free that B and the partials do not take (one pair is always
+  // needed).  The transitions with weight differ from q point to q point, so an
+  // earlier pair may be too small: its memory counts as free, and it is given
+  // back, whether a larger one takes its place or not.
+  if (!settled) {
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+      cudaGetLastError();
+      free_b = 0;
+    }
+    int have = 0;
+    while (have < kPrepGroup && t.ah[have].bytes >= opb && t.al[have].bytes >= opb) ++have;
+    double avail = (double)free_b;
+    for (int g = have; g < kPrepGroup; ++g)
+      for (DevBuf* b : {&t.ah[g], &t.al[g]})
+        if (b->p && !b->borrowed && b->bytes < opb) {
+          avail += (double)b->bytes;
+          cudaFree(b->p);
+          *b = DevBuf{};
+        }
+    auto growth = [](const DevBuf& b, size_t bytes) { return b.bytes < bytes ? (double)(bytes - b.bytes) : 0.0; };
+    if (need_b) avail -= growth(t.bh, opb) + growth(t.bl, opb);
+    t.group = std::min(kPrepGroup, std::max(1, nw));
+    if (c->group_cap > 0) t.group = std::min(t.group, c->group_cap);
+    for (;; --t.group) {
+      choose_split(t.ntiles, t.kbpc, t.nchunks, t.per);
+      choose_split(t.ntiles_f, t.kbpc_f, t.nchunks_f, t.per_f);
+      if (t.group <= std::max(1, have) ||
+          (double)(t.group - have) * 2.0 * (double)opb <= 0.5 * (avail - growth(t.part, part_bytes())))
+        break;
+    }
+  }
   if (t.kpad / kPT > 0x7fffffff / t.mpad)
     return ctx_fail(c, CHI0_EUNSUPPORTED, "too many transitions for one contraction");
   chi0_status s;
-  // the unit-weight operand B is read only by the two-operand form (weights
-  // of mixed signs) and by the complex contractions of real frequencies
-  const bool need_b = c->herk_sign == 0 || c->has_real;
   if (need_b) {
     if ((s = ctx_ensure(c, t.bh, opb, "B hi")) != CHI0_OK) return s;
     if ((s = ctx_ensure(c, t.bl, opb, "B lo")) != CHI0_OK) return s;
   }
-  // a batch problem (group_cap > 0) keeps room for twice the planned
-  // partials, for the split candidates of tc_tune_split
-  const size_t room = c->group_cap > 0 ? 2 : 1;
-  const size_t nbytes = std::max((size_t)t.per * t.nchunks * t.ntiles * room * kWPart,
-                                  c->has_real ? (size_t)t.per_f * t.nchunks_f * t.ntiles_f * kWPart : (size_t)0);
-  if ((s = ctx_ensure(c, t.part, nbytes * 16, "chunk partials")) != CHI0_OK)
-    return s;
+  if ((s = ctx_ensure(c, t.part, part_bytes(), "chunk partials")) != CHI0_OK) return s;
   for (int g = 0; g < t.group; ++g) {
     if ((s = ctx_ensure(c, t.ah[g], opb, "A hi")) != CHI0_OK) return s;
     if ((s = ctx_ensure(c, t.al[g], opb, "A lo")) != CHI0_OK) return s;

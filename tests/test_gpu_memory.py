@@ -83,3 +83,38 @@ def test_batch_keeps_its_first_plan(lib):
     ctx.close()
     for a, b in zip(got, ref):            # the same products, summed in other pieces
         assert np.linalg.norm(a - b) < 1e-6 * np.linalg.norm(b)
+
+
+def test_operands_of_the_last_q_point_count_as_memory(lib):
+    """A metal's transitions with weight differ from q point to q point (here a
+    band count per k that differs, 0/1 occupations).  The second q point has more
+    of them, so none of the first one's operand pairs is large enough; they hold
+    half of the memory, and what they hold has to count, or the eight frequencies
+    go in two passes instead of one (seen in the number of kernels launched)."""
+    import torch
+    rng = np.random.default_rng(5)
+    nb, ng, nw = 300, 250, 8
+    qs = [(q / 4, 0.0, 0.0) for q in (1, 2)]
+    nocc = np.repeat(rng.integers(4, 13, 4), 16)          # by k_x
+    ctx = _context(lib, (4, 4, 4), 3, ng, 4, nb, nw, qs, (16, 16, 16))
+    e = rng.uniform(0.1, 1.0, (64, nb))
+    occ = (np.arange(nb)[None] < nocc[:, None]).astype(float)
+    ctx.set_energies(np.where(occ > 0, -e, e), occ)
+    rows = [sum(int(nocc[(16 * (kx - iq - 1)) % 64]) * (nb - int(nocc[16 * kx])) * 16 for kx in range(4)) for iq in range(2)]
+    order = np.argsort(rows)
+    assert rows[order[1]] >= rows[order[0]] + 64
+    out = torch.zeros((nw, ng, ng), dtype=torch.complex128, device="cuda")
+
+    def launches(iq):
+        ctx.compute_rho(iq)
+        before = ctx.get_stats()[3]
+        ctx.build_chi0(iq, out)
+        ctx.synchronize()
+        return ctx.get_stats()[3] - before
+
+    ctx.compute_rho(int(order[0]))                        # states and rho in place
+    pair = 512 * rows[order[0]] * 4
+    with _leave(17 * pair):
+        got = [launches(int(iq)) for iq in order]
+    ctx.close()
+    assert got[0] == got[1]
