@@ -83,7 +83,10 @@ typedef struct {
   int nbands;             /* bands per k */
   int npw_max;            /* largest plane-wave sphere over all k */
   int fft[3];             /* real-space grid (N1, N2, N3) of rho; must be alias free.  rho is the same sum on
-                             every alias-free grid: a smaller one is taken where a fast transform has it */
+                             every alias-free grid: one that a fast transform has is taken where there is
+                             one.  Where its states would take more than those of this grid and the free
+                             device memory does not hold them, this grid is kept: the last bits of rho can
+                             then depend on the free memory at the first call for a q point */
   int ng;                 /* number of response G vectors */
   int nq;                 /* number of q points */
   const double* q_frac;   /* [nq][3] reduced coordinates; each q must be a vector of the k grid;

@@ -10,8 +10,10 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <string>
 #include <tuple>
+#include <utility>
 #include <vector>
 
 #include "../../include/chi0.h"
@@ -161,13 +163,20 @@ void response_set(const chi0_ctx* c, int iq, std::vector<int32_t>& out) {
   const int ng = c->cfg.ng;
   const int m = (int)std::ceil(std::cbrt(3.0 * ng / (4.0 * M_PI))) + 3;
   std::vector<std::tuple<int64_t, int, int, int>> cand;
-  cand.reserve((size_t)(2 * m + 1) * (2 * m + 1) * (2 * m + 1));
-  for (int x = -m; x <= m; ++x)
-    for (int y = -m; y <= m; ++y)
-      for (int z = -m; z <= m; ++z) {
-        const int64_t a = lq[0] + L * x, b = lq[1] + L * y, d = lq[2] + L * z;
-        cand.emplace_back(a * a + b * b + d * d, x, y, z);
-      }
+  // only the vectors of a ball that holds ng lattice points wherever it lies
+  // (4 pi / 3 (r - sqrt(3) / 2)^3 >= ng); every one where the box cuts the ball
+  const double r = (std::cbrt(3.0 * ng / (4.0 * M_PI)) + 0.8661) * (double)L;
+  for (double most : {r * r, 1e300}) {
+    cand.clear();
+    for (int x = -m; x <= m; ++x)
+      for (int y = -m; y <= m; ++y)
+        for (int z = -m; z <= m; ++z) {
+          const int64_t a = lq[0] + L * x, b = lq[1] + L * y, d = lq[2] + L * z;
+          const int64_t n2 = a * a + b * b + d * d;
+          if ((double)n2 <= most) cand.emplace_back(n2, x, y, z);
+        }
+    if ((int64_t)cand.size() >= ng) break;
+  }
   std::sort(cand.begin(), cand.end());
   out.resize((size_t)ng * 3);
   for (int i = 0; i < ng; ++i) {
@@ -226,8 +235,73 @@ namespace chi0 {
 
 constexpr int kBgChunk = 4096;   // difference vectors per launch of the extrapolar densities
 
+// Extents of the response set gresp and of the umklapps g0 in g, which has those
+// of the spheres, and the grid of the states: points per axis (*need) and g.nfft,
+// the smallest cubic grid of the column transforms (rho_fft.cuh) that has them,
+// 0 where they do not reach.
+static chi0_status choose_grid(chi0_ctx* c, const std::vector<int32_t>& gresp, const std::vector<int32_t>& g0,
+                               RhoGeom& g, std::vector<int32_t>& rows, std::vector<int16_t>& lut, int* need_out) {
+  int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-(1 << 30), -(1 << 30), -(1 << 30)};
+  for (int i = 0; i < g.ng; ++i)
+    for (int d = 0; d < 3; ++d) {
+      lo[d] = std::min(lo[d], gresp[3 * i + d]);
+      hi[d] = std::max(hi[d], gresp[3 * i + d]);
+    }
+  g.Mx_lo = lo[0];
+  g.My_lo = lo[1];
+  g.Mz_lo = lo[2];
+  g.HX = hi[0] - lo[0] + 1;
+  g.HY = hi[1] - lo[1] + 1;
+  g.HZ = hi[2] - lo[2] + 1;
+  int g0max = 0;
+  for (int v : g0) g0max = std::max(g0max, std::abs(v));
+  g.g0max = g0max;
+  g.g0z_min = 1 << 30;
+  g.g0z_max = -(1 << 30);
+  for (int ik = 0; ik < c->nk; ++ik) {
+    g.g0z_min = std::min(g.g0z_min, g0[3 * ik + 2]);
+    g.g0z_max = std::max(g.g0z_max, g0[3 * ik + 2]);
+  }
+  // the real-space product must not alias onto the response set,
+  // and a column transform holds frequencies of [-n/2, n/2) only; the
+  // extrapolar correction's densities reach the differences of the set
+  const int L[3] = {g.Lx, g.Ly, g.Lz};
+  int need = 0;
+  for (int d = 0; d < 3; ++d) {
+    const int n = c->cfg.fft[d];
+    const int hmax = std::max(std::abs(lo[d]), std::abs(hi[d])) + g0max;
+    if (n <= 2 * L[d] + hmax)
+      return fail(c, CHI0_EINVAL,
+                  "fft[%d] = %d aliases: need > 2*%d + %d for these spheres and response set", d,
+                  n, L[d], hmax);
+    const int reach = c->bg_on ? std::max(hmax, hi[d] - lo[d]) : hmax;
+    need = std::max({need, 2 * L[d] + reach + 1, 2 * reach + 1});
+  }
+  need = std::max(need, c->rho_need_floor);
+  *need_out = need;
+  // rho does not depend on the grid as long as it is alias free: take the
+  // smallest cubic one the column transforms know (rho_fft.cuh), and the
+  // caller's grid where that does not reach
+  chi0::rho_fft_tables(gresp.data(), g, rows, lut);
+  auto size = [&](const RhoGeom& x) {
+    return c->fp64 ? chi0::rho_fft_size<double>(x, need) : chi0::rho_fft_size<float>(x, need);
+  };
+  g.nfft = c->rho_generic ? 0 : size(g);
+  if (g.nfft && c->bg_on) {   // the difference set's chunks go through the same kernel
+    RhoGeom gd = g;
+    gd.HX = 2 * (hi[0] - lo[0]) + 1;
+    gd.HY = 2 * (hi[1] - lo[1]) + 1;
+    gd.HZ = 2 * (hi[2] - lo[2]) + 1;
+    gd.npair = gd.HY * gd.HZ;
+    gd.ng = kBgChunk;
+    if (size(gd) == 0) g.nfft = 0;
+  }
+  if (g.nfft) g.N1 = g.N2 = g.N3 = g.nfft;
+  return CHI0_OK;
+}
+
 // Host set-up of a q point: response set, k-pairs, transition block, extents
-// and the smallest alias-free grid (rho_need), which is what batch.cu needs of
+// and the grid of the states (rho_need), which is what batch.cu needs of
 // every q point before it shares one system's grids between them.
 chi0_status plan_geometry(chi0_ctx* c, int iq) {
   // ---- q-point setup on the host
@@ -267,30 +341,9 @@ chi0_status plan_geometry(chi0_ctx* c, int iq) {
   g.nb = c->nb;
   g.npw_max = c->npw_max;
   g.ng = c->cfg.ng;
-  int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-(1 << 30), -(1 << 30), -(1 << 30)};
-  for (int i = 0; i < g.ng; ++i)
-    for (int d = 0; d < 3; ++d) {
-      lo[d] = std::min(lo[d], c->h_gresp[3 * i + d]);
-      hi[d] = std::max(hi[d], c->h_gresp[3 * i + d]);
-    }
-  g.Mx_lo = lo[0];
-  g.My_lo = lo[1];
-  g.Mz_lo = lo[2];
-  g.HX = hi[0] - lo[0] + 1;
-  g.HY = hi[1] - lo[1] + 1;
-  g.HZ = hi[2] - lo[2] + 1;
   g.n_lo = c->n_lo;
   g.Nn = c->Nn;
   g.Nm = c->Nm;
-  int g0max = 0;
-  for (int v : c->h_g0) g0max = std::max(g0max, std::abs(v));
-  g.g0max = g0max;
-  g.g0z_min = 1 << 30;
-  g.g0z_max = -(1 << 30);
-  for (int ik = 0; ik < c->nk; ++ik) {
-    g.g0z_min = std::min(g.g0z_min, c->h_g0[3 * ik + 2]);
-    g.g0z_max = std::max(g.g0z_max, c->h_g0[3 * ik + 2]);
-  }
   // response indices in (Gy, Gz, Gx) order
   c->h_gperm.resize(g.ng);
   for (int i = 0; i < g.ng; ++i) c->h_gperm[i] = i;
@@ -301,67 +354,89 @@ chi0_status plan_geometry(chi0_ctx* c, int iq) {
     if (A[2] != B[2]) return A[2] < B[2];
     return A[0] < B[0];
   });
-  // the real-space product must not alias onto the response set,
-  // and a column transform holds frequencies of [-n/2, n/2) only; the
-  // extrapolar correction's densities reach the differences of the set
-  int need = 0;
-  for (int d = 0; d < 3; ++d) {
-    const int n = c->cfg.fft[d];
-    const int hmax = std::max(std::abs(lo[d]), std::abs(hi[d])) + g0max;
-    if (n <= 2 * L[d] + hmax)
-      return fail(c, CHI0_EINVAL,
-                  "fft[%d] = %d aliases: need > 2*%d + %d for these spheres and response set", d,
-                  n, L[d], hmax);
-    const int reach = c->bg_on ? std::max(hmax, hi[d] - lo[d]) : hmax;
-    need = std::max({need, 2 * L[d] + reach + 1, 2 * reach + 1});
+  return choose_grid(c, c->h_gresp, c->h_g0, g, c->h_rows, c->h_lut, &c->rho_need);
+}
+
+// Entries of a state on the caller's grid.
+static size_t own_volume(const chi0_ctx* c) {
+  RhoGeom own = c->geom;
+  own.nfft = 0;
+  own.N1 = c->cfg.fft[0];
+  own.N2 = c->cfg.fft[1];
+  own.N3 = c->cfg.fft[2];
+  return chi0::rho_volume(own);
+}
+
+// Entries of a state that d_U is sized for: the most that any q point of the
+// context needs, so that a loop over them does not find the states to have
+// grown after the contraction has taken its operands from the free memory.
+// Not beyond the caller's grid, which always serves: more only for a q point that
+// is planned (column_grid_fits).
+static size_t states_volume(chi0_ctx* c) {
+  const size_t v = chi0::rho_volume(c->geom), own = own_volume(c);
+  if (c->cfg.nq == 1 || c->rho_need_floor > 0 || v >= own) return v;
+  if (c->states_epoch != c->sphere_epoch) {
+    c->states_most = 0;
+    const std::string err = c->err;
+    std::vector<int32_t> gresp, kq, g0, rows;
+    std::vector<int16_t> lut;
+    const bool generic = c->rho_generic;
+    c->rho_generic = false;
+    for (int q = 0; q < c->cfg.nq && c->states_most < own; ++q) {
+      response_set(c, q, gresp);
+      kpairs(c, q, kq, g0);
+      RhoGeom g = c->geom;
+      g.N1 = c->cfg.fft[0];
+      g.N2 = c->cfg.fft[1];
+      g.N3 = c->cfg.fft[2];
+      int need = 0;
+      if (choose_grid(c, gresp, g0, g, rows, lut, &need) == CHI0_OK)   // (a q point that is refused needs nothing)
+        c->states_most = std::max(c->states_most, chi0::rho_volume(g));
+    }
+    c->rho_generic = generic;
+    c->err = err;
+    c->states_epoch = c->sphere_epoch;
   }
-  c->rho_need = std::max(need, c->rho_need_floor);
-  // rho does not depend on the grid as long as it is alias free: take the
-  // smallest cubic one the column transforms know (rho_fft.cuh), and the
-  // caller's grid where that does not reach
-  chi0::rho_fft_tables(c->h_gresp.data(), g, c->h_rows, c->h_lut);
-  if (!c->rho_generic)
-    g.nfft = c->fp64 ? chi0::rho_fft_size<double>(g, c->rho_need) : chi0::rho_fft_size<float>(g, c->rho_need);
-  if (g.nfft && c->bg_on) {   // the difference set's chunks go through the same kernel
-    RhoGeom gd = g;
-    gd.HX = 2 * (hi[0] - lo[0]) + 1;
-    gd.HY = 2 * (hi[1] - lo[1]) + 1;
-    gd.HZ = 2 * (hi[2] - lo[2]) + 1;
-    gd.npair = gd.HY * gd.HZ;
-    gd.ng = kBgChunk;
-    const int n = c->fp64 ? chi0::rho_fft_size<double>(gd, c->rho_need) : chi0::rho_fft_size<float>(gd, c->rho_need);
-    if (n == 0) g.nfft = 0;
-  }
-  if (g.nfft) g.N1 = g.N2 = g.N3 = g.nfft;
-  return CHI0_OK;
+  return std::max(v, std::min(c->states_most, own));
 }
 
 // The column transforms' grid is rounded up to their next size, so its states
 // can take more than those of a caller's grid that is just alias free (30^3
 // against 25 x 25 x 17: 2.5 times).  Where they have to grow and memory would then
 // not hold them, rho and the smallest set of contraction operands (at most two
-// pairs, each of rho's size), the caller's grid is kept.
+// pairs, each of rho's size), the caller's grid is kept.  What an earlier q point
+// left in these buffers and in the operands counts as memory.
 static bool column_grid_fits(const chi0_ctx* c) {
   const RhoGeom& g = c->geom;
-  RhoGeom own = g;
-  own.nfft = 0;
-  own.N1 = c->cfg.fft[0];
-  own.N2 = c->cfg.fft[1];
-  own.N3 = c->cfg.fft[2];
-  if (!g.nfft || c->nt == 0 || chi0::rho_volume(g) <= chi0::rho_volume(own)) return true;
+  if (!g.nfft || c->nt == 0 || chi0::rho_volume(g) <= own_volume(c)) return true;
   const double cb = cplx_bytes(c), vol = (double)chi0::rho_volume(g) * cb;
   const int bnb = std::max(1, std::min(c->stream_nb, c->Nn));
   const int bnk = std::max(1, std::min(c->stream_nk > 0 ? c->stream_nk : c->nk, c->nk));
   const bool streamed = c->stream_nb > 0;
   const double u = (double)c->nk * (streamed ? c->Nm : c->nb) * vol, ublk = streamed ? (double)bnk * bnb * vol : 0.0;
-  if (u <= (double)c->d_U.bytes) return true;
+  if (u <= (double)c->d_U.bytes && ublk <= (double)c->d_Ublk.bytes) return true;
   const double r = (double)(streamed ? (int64_t)bnk * bnb * c->Nm : c->nt) * g.ng * cb;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
     cudaGetLastError();
     return true;
   }
-  return u + ublk + (c->fp64 ? 1.0 : 3.0) * r <= (double)free_b + c->d_U.bytes + c->d_Ublk.bytes + c->d_R.bytes;
+  return u + ublk + (c->fp64 ? 1.0 : 3.0) * r <=
+         (double)free_b + c->d_U.bytes + c->d_Ublk.bytes + c->d_R.bytes + chi0::tc_operand_bytes(c);
+}
+
+// Where these buffers have to grow by more than the free memory, the
+// contraction's operands, which are planned anew after a new rho, give theirs back.
+static void make_room(chi0_ctx* c, std::initializer_list<std::pair<const DevBuf*, size_t>> bufs) {
+  size_t grow = 0, free_b = 0, total_b = 0;
+  for (const auto& b : bufs)
+    if (!b.first->borrowed && b.first->bytes < b.second) grow += b.second - b.first->bytes;
+  if (grow == 0) return;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (grow > free_b) chi0::tc_drop_operands(c);
 }
 
 chi0_status plan_rho(chi0_ctx* c, int iq) {
@@ -411,12 +486,13 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
   const size_t cb = cplx_bytes(c);
   const size_t plane_bytes = chi0::rho_volume(g) * cb;
   // streamed: the m-band grids of every k (resident) and one block's n grids
-  const size_t ubytes = streamed ? (size_t)c->nk * c->Nm * plane_bytes : (size_t)c->nk * c->nb * plane_bytes;
-  if ((s = ensure(c, c->d_U, ubytes, "states on the grid")) != CHI0_OK) return s;
-  if (streamed &&
-      (s = ensure(c, c->d_Ublk, (size_t)c->blk_nk * c->blk_nb * plane_bytes, "states of a band block")) != CHI0_OK)
-    return s;
-  if ((s = ensure(c, c->d_R, (size_t)(streamed ? c->nt_blk : c->nt) * g.ng * cb, "rho")) != CHI0_OK) return s;
+  const size_t nstates = (size_t)c->nk * (streamed ? c->Nm : c->nb), ubytes = nstates * plane_bytes;
+  const size_t vol_bytes = states_volume(c) * cb, nblk = streamed ? (size_t)c->blk_nk * c->blk_nb : 0;
+  const size_t rbytes = (size_t)(streamed ? c->nt_blk : c->nt) * g.ng * cb;
+  make_room(c, {{&c->d_U, nstates * vol_bytes}, {&c->d_Ublk, nblk * vol_bytes}, {&c->d_R, rbytes}});
+  if ((s = ensure(c, c->d_U, nstates * vol_bytes, "states on the grid")) != CHI0_OK) return s;
+  if (streamed && (s = ensure(c, c->d_Ublk, nblk * vol_bytes, "states of a band block")) != CHI0_OK) return s;
+  if ((s = ensure(c, c->d_R, rbytes, "rho")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_gresp, (size_t)g.ng * 12, "G set")) != CHI0_OK) return s;
   if ((s = ensure(c, c->d_gperm, (size_t)g.ng * 4, "G order")) != CHI0_OK) return s;
   const size_t rows_bytes = (rows.size() * 4 + 15) / 16 * 16;
@@ -1542,6 +1618,7 @@ chi0_status chi0_set_wavefunctions(chi0_ctx* c, int ik, int npw, const int32_t* 
     CK(cudaStreamWaitEvent(c->st, c->ev_up[ik], 0), "upload wait");
   if (new_sphere) {
     ++c->plan_epoch;
+    ++c->sphere_epoch;
     std::memcpy(hg, incoming.data(), (size_t)npw * 12);
     std::memset(hg + (size_t)npw * 3, 0, (size_t)(c->npw_max - npw) * 12);
     c->h_npw[ik] = npw;
@@ -1720,6 +1797,7 @@ chi0_status chi0_set_bg_terminator(chi0_ctx* c, int on, double eps_bar) {
   c->bg_on = on ? 1 : 0;
   c->bg_eps = eps_bar;
   ++c->plan_epoch;
+  ++c->sphere_epoch;
   // the transition block changes (every band n): compute_rho must run again
   c->rho_iq = c->chi_iq = c->eps_iq = -1;
   c->plan_rho_iq = c->plan_chi_iq = c->plan_eps_iq = -1;

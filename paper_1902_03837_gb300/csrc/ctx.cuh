@@ -75,6 +75,10 @@ struct chi0_ctx {
   // that they share one grid, and rho_generic where one of them has none
   int rho_need = 0, rho_need_floor = 0;
   bool rho_generic = false;
+  // most entries of a state on the grid over the q points, for the spheres (and
+  // the extrapolar setting) of states_epoch
+  size_t states_most = 0;
+  uint64_t sphere_epoch = 1, states_epoch = 0;
   std::vector<int32_t> h_rows;
   std::vector<int16_t> h_lut;
   DevBuf d_gresp, d_gperm, d_rtab, d_kq, d_g0, d_tw1, d_tw2, d_U, d_R, d_w, d_part, d_chi, d_A, d_colp, d_rowp,
@@ -212,6 +216,10 @@ chi0_status tc_launch(chi0_ctx* c, const void* R, const double* w, int64_t nt, i
                       const cudaEvent_t* ev_prep = nullptr, const chi0::BgApply* bg = nullptr,
                       const int* vkind = nullptr, int accumulate = 0, const int64_t* perm = nullptr);
 void tc_release(chi0_ctx* c);
+// device memory that the operands and the partials hold, and giving it back (the
+// next plan allocates them again)
+size_t tc_operand_bytes(const chi0_ctx* c);
+void tc_drop_operands(chi0_ctx* c);
 // one bounded mbarrier wait that can never be satisfied (failure detection)
 cudaError_t launch_wait_probe(int* err, cudaStream_t s);
 // self-energy kernel I (Eq. I_c) on the tensor cores: Y(i, t) = sum_j

@@ -1150,6 +1150,23 @@ std::vector<DevBuf*> tc_scratch_slots(chi0_ctx* c) {
   return v;
 }
 
+size_t tc_operand_bytes(const chi0_ctx* c) {
+  size_t n = 0;
+  if (c->tc)
+    for (const DevBuf* b : tc_scratch_slots(const_cast<chi0_ctx*>(c)))
+      if (!b->borrowed) n += b->bytes;
+  return n;
+}
+
+void tc_drop_operands(chi0_ctx* c) {
+  if (!c->tc) return;
+  for (DevBuf* b : tc_scratch_slots(c))
+    if (b->p && !b->borrowed) {
+      cudaFree(b->p);
+      *b = DevBuf{};
+    }
+}
+
 // The contraction of the first entries of the frequency list (those of one
 // launch, their operands split as tc_launch does) timed for the planned transition split and for
 // half and twice as many splits; the fastest is kept for the later launches.

@@ -118,3 +118,67 @@ def test_operands_of_the_last_q_point_count_as_memory(lib):
         got = [launches(int(iq)) for iq in order]
     ctx.close()
     assert got[0] == got[1]
+
+
+# 96,000 states on 12^3 points (1.3 GB) at the first q point and on 15^3 (2.6 GB)
+# at the second, whose response set reaches further along x; rho 47 MB and as
+# much for a pair of the contraction's operands
+NB, NGQ, NWQ = 1500, 61, 8
+QQ = [(0.25, 0.0, 0.0), (0.5, 0.0, 0.0)]
+STATES, RHO = 64 * NB * 8, 64 * (NB - 1) * NGQ * 8
+
+
+def _two_q(lib, fft):
+    return _context(lib, (4, 4, 4), 4, NGQ, 1, NB, NWQ, QQ, fft, seed=2)
+
+
+def _rho_and_chi(ctx, iq):
+    import torch
+    chi = torch.zeros((NWQ, NGQ, NGQ), dtype=torch.complex128, device="cuda")
+    ctx.compute_rho(iq)
+    rho = ctx.get_rho_rows(np.arange(0, 64 * (NB - 1), 997))
+    ctx.build_chi0(iq, chi)
+    ctx.synchronize()
+    return rho, chi.cpu().numpy()
+
+
+@pytest.fixture(scope="module")
+def ample(lib):
+    """The results with all of the memory."""
+    ref = []
+    for iq in range(2):
+        ctx = _two_q(lib, (20, 20, 20))
+        ref.append(_rho_and_chi(ctx, iq))
+        ctx.close()
+    return ref
+
+
+@pytest.mark.parametrize("fft,room", [
+    # what the states of the caller's 20 x 20 grid, 9 planes deep, would take (2.8 GB),
+    # and some: those of both q points fit
+    ((20, 20, 20), STATES * 20 * 20 * 9 + 3 * RHO),
+    # a grid that is just alias free (1404 points): both q points need more than it.
+    # The second one's states fit where the first one's operands are given back
+    ((13, 12, 12), STATES * 15 ** 3 + 5 * RHO)])
+def test_second_q_point_with_larger_states(lib, ample, fft, room):
+    ctx = _two_q(lib, fft)
+    with _leave(room):
+        got = [_rho_and_chi(ctx, iq) for iq in (0, 1, 0)]
+    ctx.close()
+    for (rho, chi), iq in zip(got, (0, 1, 0)):
+        assert np.array_equal(rho, ample[iq][0]), iq     # the same kernels on the same grid
+        assert np.linalg.norm(chi - ample[iq][1]) < 1e-6 * np.linalg.norm(chi)
+
+
+def test_callers_grid_where_the_larger_one_does_not_fit(lib, ample):
+    """1.1 GB for the states on the caller's grid, where 15^3 points would take
+    2.6: the kernels of the caller's grid, the same sums otherwise rounded (FP32:
+    some 15 levels of additions of 6e-8)."""
+    ctx = _two_q(lib, (13, 12, 12))
+    with _leave(STATES * 1404 + 6 * RHO):
+        rho, chi = _rho_and_chi(ctx, 1)
+    again = _rho_and_chi(ctx, 1)          # (the plan holds)
+    ctx.close()
+    assert 0 < np.linalg.norm(rho - ample[1][0]) < 2e-6 * np.linalg.norm(rho)
+    assert np.array_equal(rho, again[0])
+    assert np.linalg.norm(chi - ample[1][1]) < 5e-6 * np.linalg.norm(chi)
