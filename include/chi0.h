@@ -86,7 +86,8 @@ typedef struct {
                              every alias-free grid: one that a fast transform has is taken where there is
                              one.  Where its states would take more than those of this grid and the free
                              device memory does not hold them, this grid is kept: the last bits of rho can
-                             then depend on the free memory at the first call for a q point */
+                             then depend on the free memory at the first call for a q point
+                             (or when a batch is created) */
   int ng;                 /* number of response G vectors */
   int nq;                 /* number of q points */
   const double* q_frac;   /* [nq][3] reduced coordinates; each q must be a vector of the k grid;

@@ -248,6 +248,45 @@ void destroy_batch(chi0_batch* b) {
   delete b;
 }
 
+// The column transforms' grid is rounded up, so its states can take more than
+// those of a caller's grid that is just alias free.  Where the states of all
+// systems, every problem's rho and each stream's smallest set of operands (at most
+// two pairs, each of rho's size) would then not fit the free memory, the
+// caller's grid is kept for as many systems as it takes, those that gain most first.
+void keep_callers_grids(chi0_batch* b, chi0_ctx* const* ctxs, int ns) {
+  struct System {
+    chi0_ctx* base;
+    double more;   // bytes that the column transforms' states take beyond the caller's grid
+  };
+  std::vector<System> sys;
+  const double cb = b->fp64 ? 16.0 : 8.0;
+  double need = 0.0, largest = 0.0;
+  for (size_t i = 0; i < b->items.size(); ++i) {
+    const chi0_ctx* c = b->items[i];
+    if (c->nt == 0) continue;
+    const double r = (double)c->nt * c->cfg.ng * cb;
+    need += r;
+    largest = std::max(largest, r);
+    if (std::find_if(sys.begin(), sys.end(), [&](const System& x) { return x.base == ctxs[i]; }) != sys.end()) continue;
+    const double states = (double)c->nk * c->nb * cb, vol = (double)(c->rho_generic ? chi0::own_volume(c) : chi0::rho_volume(c->geom));
+    need += states * vol;
+    sys.push_back({ctxs[i], c->rho_generic ? 0.0 : states * (vol - (double)chi0::own_volume(c))});
+  }
+  if (!b->fp64) need += 2.0 * largest * ns;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  std::stable_sort(sys.begin(), sys.end(), [](const System& x, const System& y) { return x.more > y.more; });
+  for (const System& x : sys) {
+    if (need <= (double)free_b || x.more <= 0.0) return;
+    for (size_t i = 0; i < b->items.size(); ++i)
+      if (ctxs[i] == x.base) b->items[i]->rho_generic = true;
+    need -= x.more;
+  }
+}
+
 // Estimated device time of a problem (seconds): the tensor-core contraction
 // (3 BF16 products over the lower-triangle tiles, at about 1.1 PFLOP/s
 // issued) or the FP64 one, plus the FP64 Dyson step (about 4 N_G^3 complex
@@ -320,6 +359,7 @@ chi0_status chi0_batch_create(chi0_ctx* const* ctxs, const int* iqs, void* const
         }
       if (pass == 0) s = chi0::plan_geometry(c, b->iqs[i]);
     }
+  if (s == CHI0_OK) keep_callers_grids(b, ctxs, std::min(nstreams, n));
   // plan rho; the first problem of a system with transitions owns the mixed
   // grids, the system's other problems borrow them
   std::vector<chi0_ctx*> owner(n, nullptr);

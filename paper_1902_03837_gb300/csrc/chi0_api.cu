@@ -358,7 +358,7 @@ chi0_status plan_geometry(chi0_ctx* c, int iq) {
 }
 
 // Entries of a state on the caller's grid.
-static size_t own_volume(const chi0_ctx* c) {
+size_t own_volume(const chi0_ctx* c) {
   RhoGeom own = c->geom;
   own.nfft = 0;
   own.N1 = c->cfg.fft[0];

@@ -259,6 +259,7 @@ chi0_status tc_tune_split(chi0_ctx* c, float* best_ms);
 // plan (host set-up, allocation, uploads; may synchronise) and launch
 // (kernels only, capturable) halves of compute_rho / build_chi0 / invert_eps
 chi0_status plan_geometry(chi0_ctx* c, int iq);
+size_t own_volume(const chi0_ctx* c);
 chi0_status plan_rho(chi0_ctx* c, int iq);
 chi0_status launch_rho(chi0_ctx* c, bool with_pairs);
 chi0_status plan_chi0(chi0_ctx* c, int iq);

@@ -182,3 +182,22 @@ def test_callers_grid_where_the_larger_one_does_not_fit(lib, ample):
     assert 0 < np.linalg.norm(rho - ample[1][0]) < 2e-6 * np.linalg.norm(rho)
     assert np.array_equal(rho, again[0])
     assert np.linalg.norm(chi - ample[1][1]) < 5e-6 * np.linalg.norm(chi)
+
+
+@pytest.mark.parametrize("iqs,states", [((1,), 1404), ((1, 0), 1404 + 12 ** 3), ((0, 1), 12 ** 3 + 1404)])
+def test_batch_on_the_callers_grid(lib, ample, iqs, states):
+    """The same in a batch, of one system or of two: 2.6 GB for the states of the
+    second q point do not fit, its 1.1 GB on the caller's grid do, beside the
+    1.3 GB of a first q point of another system."""
+    import torch
+    ctxs = [_two_q(lib, (13, 12, 12)) for _ in iqs]
+    out = [torch.zeros((NWQ, NGQ, NGQ), dtype=torch.complex128, device="cuda") for _ in iqs]
+    with _leave(STATES * states + 16 * RHO):
+        batch = lib.Batch(ctxs, iqs, [None] * len(iqs), nstreams=1, chi_out=out)
+        batch.run(torch.cuda.current_stream().cuda_stream)
+        batch.synchronize()
+        batch.close()
+    for c in ctxs:
+        c.close()
+    for iq, chi in zip(iqs, out):
+        assert np.linalg.norm(chi.cpu().numpy() - ample[iq][1]) < 5e-6 * np.linalg.norm(ample[iq][1])
