@@ -67,7 +67,25 @@ chi0_status ensure(chi0_ctx* c, DevBuf& b, size_t bytes, const char* what) {
 }  // namespace
 
 namespace chi0 {
+// The calls whose stages are timed: those before kTimedAll instances, then one in
+// every kTimedStep, which stands for its neighbours.  Whole calls, because the
+// instances of a stage within one do not take the same time (the transitions' rho
+// and the densities of the extrapolar term, the groups of the Dyson step): every
+// 16th instance would be the same one of them in each call.  At a place of its
+// window that a hash gives (the finaliser of Murmur 3), because a loop over q
+// points would make every 16th call one of the same q point.
 constexpr int64_t kTimedAll = 512, kTimedStep = 16;
+static int call_weight(int64_t instances, int64_t call) {
+  if (instances < kTimedAll) return 1;
+  uint32_t h = (uint32_t)(call / kTimedStep);
+  h = (h ^ h >> 16) * 0x85ebca6bu;
+  h = (h ^ h >> 13) * 0xc2b2ae35u;
+  return call % kTimedStep == (h ^ h >> 16) % kTimedStep ? (int)kTimedStep : 0;
+}
+void begin_call(chi0_ctx* c, int entry) {
+  auto& e = c->calls[c->entry = entry];
+  c->timed_weight = call_weight(e.instances, e.calls++);
+}
 constexpr size_t kFoldAt = 1024;   // events
 
 // the recorded pairs' times into acc (the pairs must have finished)
@@ -83,8 +101,8 @@ static void stage_fold(chi0_ctx::Stage& st) {
 void stage_begin(chi0_ctx* c, int stage) {
   if (c->capturing) return;
   auto& st = c->stage[stage];
-  const int64_t i = st.count++;
-  st.timed = i < kTimedAll || i % kTimedStep == 0;
+  ++c->calls[c->entry].instances;
+  st.timed = c->timed_weight > 0;
   if (!st.timed) return;
   if (st.used >= kFoldAt) {
     // the last pairs of every stream in use must have finished (and nothing is
@@ -107,7 +125,7 @@ void stage_begin(chi0_ctx* c, int stage) {
     st.ev.push_back(b);
     st.weight.push_back(1);
   }
-  st.weight[st.used / 2] = i < kTimedAll ? 1 : (int)kTimedStep;
+  st.weight[st.used / 2] = c->timed_weight;
   cudaEventRecord(st.ev[st.used], c->st);
 }
 void stage_end(chi0_ctx* c, int stage, int kernels) {
@@ -1715,6 +1733,7 @@ chi0_status chi0_set_energies(chi0_ctx* c, const double* eps, const double* occ)
 
 chi0_status chi0_compute_rho(chi0_ctx* c, int iq) {
   if (!c) return CHI0_EINVAL;
+  chi0::begin_call(c, chi0_ctx::kRhoCall);
   chi0_status s;
   if ((s = chi0::plan_rho(c, iq)) != CHI0_OK) return s;
   return chi0::launch_rho(c, true);
@@ -1723,6 +1742,7 @@ chi0_status chi0_compute_rho(chi0_ctx* c, int iq) {
 chi0_status chi0_build_chi0(chi0_ctx* c, int iq, void* out, int out_on_device) {
   if (!c) return CHI0_EINVAL;
   if (iq != c->rho_iq || iq < 0) return fail(c, CHI0_ESTATE, "chi0_compute_rho(%d) must come first", iq);
+  chi0::begin_call(c, chi0_ctx::kChiCall);
   chi0_status s;
   if ((s = chi0::plan_chi0(c, iq)) != CHI0_OK) return s;
   if ((s = chi0::launch_chi0(c)) != CHI0_OK) return s;
@@ -1744,6 +1764,7 @@ chi0_status chi0_invert_eps(chi0_ctx* c, int iq, void* out, int out_on_device) {
   if (iq != c->chi_iq || iq < 0) return fail(c, CHI0_ESTATE, "chi0_build_chi0(%d) must come first", iq);
   if (!out) return fail(c, CHI0_EINVAL, "NULL output");
   const size_t bytes = (size_t)c->cfg.ng * c->cfg.ng * c->cfg.nw * 16;
+  chi0::begin_call(c, chi0_ctx::kEpsCall);
   chi0_status s;
   double2* A;
   if (out_on_device) {
@@ -1767,6 +1788,7 @@ chi0_status chi0_build_invert(chi0_ctx* c, int iq, void* chi_out, void* eps_out,
   if (iq != c->rho_iq || iq < 0) return fail(c, CHI0_ESTATE, "chi0_compute_rho(%d) must come first", iq);
   if (!eps_out) return fail(c, CHI0_EINVAL, "NULL output");
   const size_t bytes = (size_t)c->cfg.ng * c->cfg.ng * c->cfg.nw * 16;
+  chi0::begin_call(c, chi0_ctx::kChiEpsCall);
   chi0_status s;
   double2* A;
   if (out_on_device) {
@@ -1821,6 +1843,7 @@ chi0_status chi0_build_sigma_i(chi0_ctx* c, int iq, int qp_lo, int qp_hi, const 
   const int ng = c->cfg.ng, nb = c->nb;
   const int64_t T = (int64_t)c->nk * nb * nqp;
   const size_t cb = cplx_bytes(c);
+  chi0::begin_call(c, chi0_ctx::kSigmaCall);
   chi0_status s;
   // rho geometry of the window: n in [qp_lo, qp_hi) at k, every band m at k - q
   RhoGeom& g = c->sig_geom;
@@ -2093,11 +2116,12 @@ chi0_status chi0_get_stats(chi0_ctx* c, double* ms, double* bytes, double* flops
     chi0::stage_fold(st);
     st.ms = st.acc;
     st.acc = 0.0;
-    st.count = 0;
     if (ms) ms[k] = st.ms;
     if (bytes) bytes[k] = st.bytes;
     if (flops) flops[k] = st.flops;
   }
+  for (auto& e : c->calls) e = {};
+  c->timed_weight = 1;
   if (launches) *launches = c->launches;
   return CHI0_OK;
 }

@@ -144,19 +144,25 @@ struct chi0_ctx {
   // per-stage device time: CUDA event pairs on the context's stream.  A pair
   // costs the stream about 4 us, half of a small problem's pass, and pairs
   // kept until the next readout pile up in a program that never reads them, so
-  // after kTimedAll instances every kTimedStep-th stands for its neighbours,
-  // and finished pairs are folded into ms and used again.
+  // after kTimedAll instances one call in every kTimedStep stands for its
+  // neighbours, and finished pairs are folded into ms and used again.
   struct Stage {
     std::vector<cudaEvent_t> ev;  // start, stop, start, stop, ...
-    std::vector<int> weight;      // instances that each pair stands for
+    std::vector<int> weight;      // calls that each pair stands for
     size_t used = 0;              // events recorded since the last fold
-    int64_t count = 0;            // instances since the last readout
     bool timed = false;           // the open instance has a pair
     double acc = 0;               // folded time since the last readout (ms)
     double ms = 0, bytes = 0, flops = 0;
     int64_t launches = 0;
   };
   Stage stage[CHI0_NSTAGES];
+  // calls of each entry point, and stages run by them, since the last readout
+  enum { kRhoCall, kChiCall, kEpsCall, kChiEpsCall, kSigmaCall, kEntries };
+  struct {
+    int64_t calls = 0, instances = 0;
+  } calls[kEntries];
+  int entry = kRhoCall;           // of the call that is running
+  int timed_weight = 1;           // calls that it stands for; 0: not timed
   int64_t launches = 0;           // kernels launched since chi0_create
   double tc_issued_flops = 0;     // tensor-core flops issued by the last mixed contraction
 
