@@ -106,12 +106,17 @@ void stage_begin(chi0_ctx* c, int stage) {
   if (!st.timed) return;
   if (st.used >= kFoldAt) {
     // the last pairs of every stream in use must have finished (and nothing is
-    // asked of events while the caller captures the stream)
+    // asked of events while the caller captures the stream).  An event query
+    // would end a capture that another thread has begun in the global mode, so
+    // this thread leaves that mode meanwhile.
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    const bool relaxed = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-    bool done = cudaStreamIsCapturing(c->st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    bool done = relaxed && cudaStreamIsCapturing(c->st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
     for (size_t p = 1; done && p <= 8; ++p) done = cudaEventQuery(st.ev[st.used + 1 - 2 * p]) == cudaSuccess;
     cudaGetLastError();
     if (done) stage_fold(st);
+    if (relaxed) cudaThreadExchangeStreamCaptureMode(&mode);
   }
   if (st.used + 2 > st.ev.size()) {
     cudaEvent_t a = nullptr, b = nullptr;
