@@ -115,7 +115,9 @@ __device__ __forceinline__ bool pivot_inverse(double2 (&x)[2], int nb, PivotSmem
           sm.dinv[b] = make_double2(d.x * inv, -d.y * inv);
         } else {   // Hermitian positive definite: real positive pivots
           if (!(d.x > 1e-150)) sm.bad[b] = 1;
-          sm.dinv[b] = make_double2(recip(d.x), 0.0);
+          // an infinite pivot is no number to go on with: 1 / d = 0 would leave
+          // finite entries everywhere and hide it
+          sm.dinv[b] = make_double2(isinf(d.x) ? d.x - d.x : recip(d.x), 0.0);
         }
       }
       if (r == p) sm.row[b][c] = x[u];
