@@ -190,13 +190,23 @@ __device__ __forceinline__ void ldsm(uint32_t (&r)[4], const __nv_bfloat16* p) {
 // h2 = bf16(tanh(z)) keeps the value that the chain of FP32 multiply-adds in the
 // order of k gives (as the training kernel computes it): the tensor core's z
 // differs from the chain's by its rounding only, so the two can round apart
-// only next to a rounding boundary.  Where z +- kDoubt sum_k |W2[h][k]| straddles
-// one (some 16 of a warp's 2048 values), the value goes on a list, and the chain
-// is run for up to 32 of the list at a time, one per lane.  kDoubt is three times
-// the largest rounding error of the chain seen over 2.6 million values (3.9e-8 of
-// that sum); a value it misses would be off by one rounding of an operand.
-// 10^6 samples: 929 us on the FP32 pipe -> 348 us (0.26 ms of issue slots).
-constexpr float kDoubt = 1.f / 8388608.f;
+// only next to a rounding boundary.  Where z +- kDoubt P straddles one, the value
+// goes on a list, and the chain is run for up to 32 of the list at a time, one per
+// lane.  Both roundings go with the size of the partial sums, the bias among them,
+// and P bounds those: the largest |z| after any of the four steps of 32 terms, and
+// half the largest sum of 32 |W2|, by which a sum can exceed both ends of its
+// step.  128 roundings of half an ulp add up to 3.3 ulp in the mean where all
+// partial sums are equally large (a bias of 0.6 and small weights), and the tensor
+// core drops up to one per 16 terms.  Over 8.4 million values each of eleven
+// networks (initial, trained-like, biases far above the weights, sums that rise
+// and fall) the two differ by 15 2^-23 of the largest partial sum at most, by
+// 0.2-3 in the root mean square, so kDoubt is 16 2^-23: none of their values went
+// unnoticed.  (With 2^-23 sum |W2| for kDoubt P up to 133 did, where a bias was
+// above the weights.)  Some 25 of a warp's 2048 values are listed.
+// 10^6 samples: 929 us on the FP32 pipe -> 424 us (0.26 ms of issue slots; 352 with
+// the narrower doubt, which lists 14).
+constexpr float kDoubt = 1.f / 524288.f;
+constexpr int kTrack = 2;           // products of 16 terms between looks at the sums
 constexpr int kLdb = kH + 8;        // padded row of BF16: eight rows' 16-byte pieces fall into distinct banks
 constexpr int kPredWarps = 8;
 constexpr int kList = 32 + 128;     // below 32 before a step, which adds 128 at most
@@ -206,7 +216,7 @@ struct PredictBf16Smem {
   float4 w1[kH];                    // inputs 0..3
   float4 w3[kH / 2];                // both outputs' weights of two inputs
   float2 w1b[kH];                   // input 4, bias
-  float2 b2[kH / 2], doubt[kH / 2];
+  float2 b2[kH / 2], doubt[kH / 2];   // doubt: kDoubt / 2 of the largest sum of 32 |W2|
   uint32_t list[kPredWarps][kList]; // h2 as the tensor core's z gives it | sample | column
 };
 static_assert(kPredWarps * 32 == kThreads, "a warp per tile");
@@ -230,9 +240,13 @@ k_mlp_predict_bf16(const float* __restrict__ prm, const float* __restrict__ x, i
   const float b3 = prm[kOffB3 + (t & 1)];
   __syncthreads();
   if (tid < kH) {
-    float s = 0.f;
-    for (int k = 0; k < kH; ++k) s += fabsf(__bfloat162float(sm.w2[tid * kLdb + k]));
-    reinterpret_cast<float*>(sm.doubt)[tid] = kDoubt * s;
+    float most = 0.f;
+    for (int k = 0; k < kH; k += 16 * kTrack) {
+      float s = 0.f;
+      for (int q = 0; q < 16 * kTrack; ++q) s += fabsf(__bfloat162float(sm.w2[tid * kLdb + k + q]));
+      most = fmaxf(most, s);
+    }
+    reinterpret_cast<float*>(sm.doubt)[tid] = 0.5f * kDoubt * most;
   }
   __syncthreads();
   __nv_bfloat16* h1s = sm.h1[warp];
@@ -314,12 +328,14 @@ k_mlp_predict_bf16(const float* __restrict__ prm, const float* __restrict__ x, i
       __syncwarp();
     };
     for (int n0 = 0; n0 < kH; n0 += 16) {
-      float c[2][4];
+      float c[2][4], most[2][4];   // sums, and the largest of them so far
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const float2 b2 = sm.b2[n0 / 2 + 4 * j + t];
         c[j][0] = c[j][2] = b2.x;
         c[j][1] = c[j][3] = b2.y;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) most[j][q] = fabsf(c[j][q]);
       }
 #pragma unroll
       for (int ks = 0; ks < kH / 16; ++ks) {
@@ -327,6 +343,12 @@ k_mlp_predict_bf16(const float* __restrict__ prm, const float* __restrict__ x, i
         ldsm(b, sm.w2 + (n0 + (lane & 7) + (lane >> 4) * 8) * kLdb + ks * 16 + ((lane >> 3) & 1) * 8);
         mma_bf16(c[0], a[ks], b[0], b[1]);
         mma_bf16(c[1], a[ks], b[2], b[3]);
+        if (ks % kTrack == kTrack - 1) {
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) most[j][q] = fmaxf(most[j][q], fabsf(c[j][q]));
+        }
       }
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
@@ -337,8 +359,9 @@ k_mlp_predict_bf16(const float* __restrict__ prm, const float* __restrict__ x, i
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           const float h0 = tanhf(c[j][2 * r]), h1 = tanhf(c[j][2 * r + 1]);
-          // dz times the slope of tanh, and an ulp for tanhf itself
-          const float e0 = fmaf(dz.x, fmaf(-h0, h0, 1.f), 1.2e-7f), e1 = fmaf(dz.y, fmaf(-h1, h1, 1.f), 1.2e-7f);
+          // the doubt times the slope of tanh, and an ulp for tanhf itself
+          const float d0 = fmaf(kDoubt, most[j][2 * r], dz.x), d1 = fmaf(kDoubt, most[j][2 * r + 1], dz.y);
+          const float e0 = fmaf(d0, fmaf(-h0, h0, 1.f), 1.2e-7f), e1 = fmaf(d1, fmaf(-h1, h1, 1.f), 1.2e-7f);
           h[r] = pack_bf16(h0, h1);
           open[r] = pack_bf16(h0 + e0, h1 + e1) ^ pack_bf16(h0 - e0, h1 - e1);
           const float r0 = low_bf16(h[r]), r1 = high_bf16(h[r]);
