@@ -1361,15 +1361,26 @@ chi0_status sig_tc_plan(chi0_ctx* c, int64_t T, int ng, int nw) {
     return ctx_fail(c, CHI0_EUNSUPPORTED, "too many transitions in the quasiparticle window for one contraction");
   chi0_status s;
   const size_t opa = (size_t)t.mpad_a * t.kpad * 2, opb = (size_t)t.mpad_b * t.kpad * 2;
-  // W^d of eight frequencies per split (50 blocks at N_G = 300 for one), and as
-  // many frequencies per contraction launch as leave the two Y's that it writes
-  // and the dot products read within L2
-  t.nsplit = std::max(1, std::min(kPrepGroup, nw));
-  t.per = (double)t.nI * t.nJ * 4096 * 8 <= 48e6 ? std::min(2, t.nsplit) : 1;
-  if ((s = ctx_ensure(c, t.ah, opa * t.nsplit, "W^delta hi")) != CHI0_OK) return s;
-  if ((s = ctx_ensure(c, t.al, opa * t.nsplit, "W^delta lo")) != CHI0_OK) return s;
   if ((s = ctx_ensure(c, t.bh, opb, "rho hi")) != CHI0_OK) return s;
   if ((s = ctx_ensure(c, t.bl, opb, "rho lo")) != CHI0_OK) return s;
+  // W^d of eight frequencies per split (50 blocks at N_G = 300 for one), fewer
+  // where they would take more than half of the memory that is left beside Y, and
+  // as many frequencies per contraction launch as leave the two Y's that it writes
+  // and the dot products read within L2
+  const double ybytes = (double)t.nI * t.nJ * 4096 * 8;
+  t.nsplit = std::max(1, std::min(kPrepGroup, nw));
+  if (t.ah.bytes < opa * t.nsplit) {
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+      cudaGetLastError();
+      free_b = 0;
+    }
+    const double room = 0.5 * ((double)free_b - std::max(0.0, ybytes - (double)c->d_sigY.bytes));
+    while (t.nsplit > 1 && t.ah.bytes < opa * t.nsplit && 2.0 * (double)(opa * t.nsplit - t.ah.bytes) > room) t.nsplit /= 2;
+  }
+  t.per = ybytes <= 48e6 ? std::min(2, t.nsplit) : 1;
+  if ((s = ctx_ensure(c, t.ah, opa * t.nsplit, "W^delta hi")) != CHI0_OK) return s;
+  if ((s = ctx_ensure(c, t.al, opa * t.nsplit, "W^delta lo")) != CHI0_OK) return s;
   for (int g = 0; g < t.nsplit; ++g)
     if (!make_map(&t.maps.ah[g], (char*)t.ah.p + g * opa, t.kpad, t.mpad_a) ||
         !make_map(&t.maps.al[g], (char*)t.al.p + g * opa, t.kpad, t.mpad_a))

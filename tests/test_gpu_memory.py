@@ -201,3 +201,25 @@ def test_batch_on_the_callers_grid(lib, ample, iqs, states):
         c.close()
     for iq, chi in zip(iqs, out):
         assert np.linalg.norm(chi.cpu().numpy() - ample[iq][1]) < 5e-6 * np.linalg.norm(ample[iq][1])
+
+
+def test_self_energy_operands_of_fewer_frequencies(lib):
+    """N_G = 3000: the operands of W^delta take 72 MB per frequency, 580 MB for the
+    eight that go through the split at a time.  With 300 MB left fewer do, and the
+    results have the same bits."""
+    import torch
+    ng, nw, nb = 3000, 8, 6
+    ctx = _context(lib, (2, 1, 1), 3, ng, 2, nb, 1, [(0.5, 0.0, 0.0)], (24, 24, 24))
+    ctx.compute_rho(0)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    eps = torch.randn(nw, ng, ng, dtype=torch.complex128, device="cuda", generator=gen)
+    out = torch.zeros((nw, 2, nb, 2, 2), dtype=torch.complex128, device="cuda")
+    ctx.synchronize()
+    with _leave(300 * MB):
+        ctx.build_sigma_i(0, 1, 3, eps, out)
+        ctx.synchronize()
+    got = out.clone()
+    ctx.build_sigma_i(0, 1, 3, eps, out)
+    ctx.synchronize()
+    ctx.close()
+    assert bool((got != 0).any()) and torch.equal(got, out)
