@@ -78,11 +78,13 @@ struct Mats {
 
 // 1 / d in FP64: the FP32 reciprocal (24 bits) and two Newton steps
 // r <- r (2 - d r), each of which doubles the correct bits; the division
-// where d leaves FP32's range.  The reciprocal heads every sweep's chain of
-// dependent FP64 operations.
+// outside 2^-99 <= |d| < 2^100, which FP32 holds with room.  The reciprocal heads
+// every sweep's chain of dependent FP64 operations, of which a comparison is one
+// too, so the range is told from the exponent.  An infinite pivot is no number to
+// go on with: 1 / d = 0 would leave finite entries everywhere and hide it.
 __device__ __forceinline__ double recip(double d) {
-  const double ad = fabs(d);
-  if (!(ad > 1e-30 && ad < 1e30)) return 1.0 / d;
+  const unsigned e = (unsigned)__double2hiint(d) >> 20 & 0x7ffu;
+  if (e - 924u >= 199u) return e == 0x7ffu ? d - d : 1.0 / d;
   double r = (double)(1.0f / (float)d);
   r = fma(r, fma(-d, r, 1.0), r);
   return fma(r, fma(-d, r, 1.0), r);
@@ -115,9 +117,7 @@ __device__ __forceinline__ bool pivot_inverse(double2 (&x)[2], int nb, PivotSmem
           sm.dinv[b] = make_double2(d.x * inv, -d.y * inv);
         } else {   // Hermitian positive definite: real positive pivots
           if (!(d.x > 1e-150)) sm.bad[b] = 1;
-          // an infinite pivot is no number to go on with: 1 / d = 0 would leave
-          // finite entries everywhere and hide it
-          sm.dinv[b] = make_double2(isinf(d.x) ? d.x - d.x : recip(d.x), 0.0);
+          sm.dinv[b] = make_double2(recip(d.x), 0.0);
         }
       }
       if (r == p) sm.row[b][c] = x[u];
