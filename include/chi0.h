@@ -461,11 +461,15 @@ chi0_status chi0_set_double_grid(chi0_ctx* ctx, int nd, const double* eps_dense)
  *            entry [w][k][m][a - qp_lo][b - qp_lo]; device (out_on_device = 1,
  *            asynchronous on the context's stream) or host (synchronises).
  * The contraction sum_j W^d_ij conj(rho(j)) runs on the tensor cores in the
- * mixed form (BF16x3 products, FP32 accumulation in 128-term pieces, FP64
- * sums), in plain FP64 in the FP64 form.  Requires chi0_compute_rho(iq)
- * (the states on the grid and the response set).  Device memory: rho of
- * the window (nk nbands nqp ng complex) and an N_G x nk nbands nqp FP64
- * complex work array.
+ * mixed form (BF16x3 products, FP32 accumulation in 128-term pieces, added in
+ * compensated FP32; the sums over i likewise, in eight parts added in FP64), in
+ * plain FP64 in the FP64 form.  Requires chi0_compute_rho(iq) (the states on
+ * the grid and the response set).  Device memory, kept for the next call: rho of the
+ * window twice (nk nbands nqp ng complex, complex64 in the mixed form, once in
+ * tiles of 64 x 64) and an N_G x nk nbands nqp work array: complex128 in the FP64
+ * form, beside W^d of one frequency; complex64 in the mixed form, of one or two
+ * frequencies, beside BF16 pairs of rho (as large as rho) and of W^d of up to eight
+ * frequencies (as far as half of the free memory holds them).
  * Errors: CHI0_EINVAL (window empty or outside [0, nbands), NULL pointer,
  * nw < 1, |q+G| = 0), CHI0_EUNSUPPORTED (more than 64 bands in the window,
  * or too many transitions for one contraction), CHI0_ESTATE, CHI0_ENOMEM,

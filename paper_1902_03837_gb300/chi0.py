@@ -185,7 +185,7 @@ def ppa_eval(omega_t, R, freqs, eta, out, stream=None):
 
 class Batch:
     """chi0_batch: many (context, q index) problems run as one captured graph.
-    A context may appear with several q indices (they share its mixed grids).
+    A context may appear with several q indices (they share its states on the grid).
     eps_out / chi_out: per problem a complex128 CUDA tensor [nw][ng][ng] or
     None; each problem needs at least one of them."""
 

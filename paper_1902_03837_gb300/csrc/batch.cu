@@ -9,7 +9,7 @@
 //
 //   1. every problem's host set-up runs once (chi0_batch_create).  The
 //      problems of one system (one context at several q indices) share its
-//      coefficients and its mixed grids, computed once per system;
+//      coefficients and its states on the grid, computed once per system;
 //   2. the oscillator strengths run in one persistent launch per grid size (the
 //      column transforms are compiled per size) over a device task table:
 //      blocks take the next (problem, k-pair, n, m-chunk) work item from a
@@ -360,8 +360,8 @@ chi0_status chi0_batch_create(chi0_ctx* const* ctxs, const int* iqs, void* const
       if (pass == 0) s = chi0::plan_geometry(c, b->iqs[i]);
     }
   if (s == CHI0_OK) keep_callers_grids(b, ctxs, std::min(nstreams, n));
-  // plan rho; the first problem of a system with transitions owns the mixed
-  // grids, the system's other problems borrow them
+  // plan rho; the first problem of a system with transitions owns the states,
+  // the system's other problems borrow them
   std::vector<chi0_ctx*> owner(n, nullptr);
   for (int i = 0; i < n && s == CHI0_OK; ++i) {
     chi0_ctx* c = b->items[i];
@@ -374,7 +374,7 @@ chi0_status chi0_batch_create(chi0_ctx* const* ctxs, const int* iqs, void* const
     }
     if ((s = chi0::plan_rho(c, b->iqs[i])) != CHI0_OK) break;
     owner[i] = own ? own : (c->nt > 0 ? c : nullptr);
-    if (!own) s = chi0::launch_rho(c, false);   // the mixed grids (used by the tuning below)
+    if (!own) s = chi0::launch_rho(c, false);   // the states (used by the tuning below)
   }
   // sizing pass: plan the rest of each problem with its own scratch, note the
   // sizes and free them again (one problem's scratch at a time)
@@ -516,7 +516,7 @@ chi0_status chi0_batch_run(chi0_batch* b, void* stream) {
         cudaStreamWaitEvent(st, b->evs[first_event + k], 0);
       }
     };
-    // the mixed grids of every system (its grid owner), spread over the streams
+    // the states of every system (by the problem that owns them), spread over the streams
     fork(b->evs[2 * ns]);
     int nown = 0;
     for (size_t i = 0; i < b->items.size() && s == CHI0_OK; ++i) {

@@ -303,8 +303,8 @@ static chi0_status choose_grid(chi0_ctx* c, const std::vector<int32_t>& gresp, c
   need = std::max(need, c->rho_need_floor);
   *need_out = need;
   // rho does not depend on the grid as long as it is alias free: take the
-  // smallest cubic one the column transforms know (rho_fft.cuh), and the
-  // caller's grid where that does not reach
+  // smallest cubic one with these points that the column transforms know
+  // (rho_fft.cuh), and the caller's grid where that does not reach
   chi0::rho_fft_tables(gresp.data(), g, rows, lut);
   auto size = [&](const RhoGeom& x) {
     return c->fp64 ? chi0::rho_fft_size<double>(x, need) : chi0::rho_fft_size<float>(x, need);
@@ -550,8 +550,8 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
     CK(cudaMemcpyAsync(c->d_tw2.p, t2.data(), t2.size() * 8, cudaMemcpyHostToDevice, c->st), "tw H2D");
     CK(cudaStreamSynchronize(c->st), "synchronize");
   }
-  // mixed grid: coefficients in, U out; transforms along y (NX N2 NY per gz
-  // plane) and x (N1 N2 NX per gz plane)
+  // states: coefficients in, U out; on the mixed grid, transforms along y (NX N2
+  // NY per gz plane) and x (N1 N2 NX per gz plane)
   {
     auto& a1 = c->stage[CHI0_STAGE_WF_GRID];
     a1.bytes = (double)c->nk * c->nb * ((double)c->npw_max * (cb + 12) + ubytes / ((double)c->nk * c->nb));
@@ -582,7 +582,7 @@ chi0_status plan_rho(chi0_ctx* c, int iq) {
   return CHI0_OK;
 }
 
-// wavefunctions to the mixed grid: every k and band (nkr = 0), or the k
+// wavefunctions to the grid: every k and band (nkr = 0), or the k
 // points k0 .. k0 + nkr - 1 and bands b0 .. b0 + nbo - 1 into U[k - k0][b - b0]
 cudaError_t launch_wf_range(chi0_ctx* c, void* U, int k0, int nkr, int b0, int nbo) {
   const RhoGeom& g = c->geom;
@@ -603,7 +603,7 @@ cudaError_t launch_wf_range(chi0_ctx* c, void* U, int k0, int nkr, int b0, int n
   return e;
 }
 
-// kernels of compute_rho (wavefunctions to the mixed grid; rho unless the
+// kernels of compute_rho (wavefunctions to the grid; rho unless the
 // caller runs rho for many problems in one batched launch, or the
 // transitions are streamed in band blocks by build_chi0)
 // rho of the whole problem, pipelined with the coefficient upload: the k
@@ -1422,14 +1422,20 @@ chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
   // least the q matrices whose updates fit into the chain.  Where the
   // contraction takes longer than the Dyson steps, the last groups halve down to
   // q, so that little is left after the last contraction (N_G = 1000: 2, 1, 1);
-  // where the Dyson steps take longer, small last groups would only add
-  // chains.  A group holds frequencies of one kind (imaginary
-  // axis: Hermitian eps~; real axis: general eps~, whose chi0 is first
-  // combined from its two contractions H_r + i H_i).
-  // Consecutive groups alternate between two Dyson streams, each with its
-  // own panel scratch (the group's slice of the per-frequency buffers), so
-  // that the pivot-block inverses of one group (one SM per matrix) overlap
-  // the rank-32 updates of the other.
+  // where the Dyson steps take longer, small last groups would only add chains.
+  // Which of the two is longer is told from the updates at 0.85 of the FP64 rate
+  // (64 of 74 us of a step of twelve matrices of N_G = 300 are multiply-adds) and
+  // from the issued products at 1.2e15 per second (N_G = 400; 1.46e15 at 1000).  Few
+  // large groups against halved last ones, with the Dyson steps taking 3.3 times
+  // as long as the contraction 49.1 / 50.5 ms (N_G = 1000, ten frequencies), 1.8 times
+  // 16.2 / 16.5 and 37.0 / 37.3 ms (600, 800), 0.6 to 0.75 times 12.45 / 12.46, 23.8 /
+  // 24.1 and 49.9 / 49.9 ms (431, 600, 800): near the line it matters little.
+  // A group holds frequencies of one kind (imaginary axis: Hermitian eps~; real
+  // axis: general eps~, whose chi0 is first combined from its two contractions
+  // H_r + i H_i).  Consecutive groups alternate between two Dyson streams, each
+  // with its own panel scratch (the group's slice of the per-frequency buffers),
+  // so that the chain of one group (panels, and the next pivot inverted by one
+  // block per matrix within each update) overlaps the updates of the other.
   int grp = 0;
   const double nt16 = (ng + 15) / 16;
   const double step_s = 54.0 * (c->has_real ? nt16 * nt16 : 0.5 * nt16 * (nt16 + 1.0)) / 1.93e9;   // of one matrix
@@ -1842,9 +1848,9 @@ chi0_status chi0_build_sigma_i(chi0_ctx* c, int iq, int qp_lo, int qp_hi, const 
   if (nqp > 64) return fail(c, CHI0_EUNSUPPORTED, "at most 64 bands in the quasiparticle window");
   if (iq != c->rho_iq) return fail(c, CHI0_ESTATE, "chi0_compute_rho(%d) must come first", iq);
   if (c->stream_nb > 0)
-    return fail(c, CHI0_EUNSUPPORTED, "the self-energy kernel needs every band's mixed grids (no band-block streaming)");
+    return fail(c, CHI0_EUNSUPPORTED, "the self-energy kernel needs every band's states on the grid (no band-block streaming)");
   if (c->nt == 0)
-    return fail(c, CHI0_ESTATE, "no transitions at this q: the mixed-grid wavefunctions were not built");
+    return fail(c, CHI0_ESTATE, "no transitions at this q: the states on the grid were not built");
   const int ng = c->cfg.ng, nb = c->nb;
   const int64_t T = (int64_t)c->nk * nb * nqp;
   const size_t cb = cplx_bytes(c);

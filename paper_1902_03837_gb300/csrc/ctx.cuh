@@ -39,7 +39,7 @@ struct chi0_ctx {
   int rho_iq = -1, chi_iq = -1, eps_iq = -1;      // completed (launched) steps
   int plan_rho_iq = -1, plan_chi_iq = -1, plan_eps_iq = -1;  // planned steps
   double2* plan_eps_out = nullptr;
-  // batch problems: grid_shared = the mixed grids d_U belong to another
+  // batch problems: grid_shared = the states d_U belong to another
   // problem of the same system (launch_rho then skips the wavefunction
   // transforms); group_cap > 0 limits the frequencies per operand-split pass
   bool grid_shared = false;

@@ -91,7 +91,8 @@ int rho_fft_size(const RhoGeom& g, int need);
 // lut[hx][pair] = response index or -1.
 void rho_fft_tables(const int32_t* gset, RhoGeom& g, std::vector<int32_t>& rows, std::vector<int16_t>& lut);
 
-// a1: sphere -> mixed grid U[k][band][x][gz][y] for every k and band, or
+// a1: sphere -> states on the grid (g.nfft: U[k][band][x][z][y], else mixed grids
+// U[k][band][x][gz][y]) for every k and band, or
 // (nkr > 0) for the k points k0 .. k0 + nkr - 1 and bands b0 .. b0 + nbo - 1
 // only, written as U[k - k0][band - b0] (coefficients indexed globally).
 template <typename T>

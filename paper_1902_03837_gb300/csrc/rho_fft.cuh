@@ -1,11 +1,13 @@
-// Oscillator strengths through in-register transforms on the smallest
-// alias-free grid (kernels; instantiated per type in rho_fft32.cu / rho_fft64.cu).
+// Oscillator strengths through in-register transforms on a small alias-free
+// grid (kernels; instantiated per type in rho_fft32.cu / rho_fft64.cu).
 //
 //   rho(G) = 1/N^3 sum_r conj(u_n(r)) u_m(r) e^{i h.r},   h = G - G0,
 //
 // is exact on every grid with N > 2 L + max|h| per axis (L: largest Miller
-// index of the spheres), so the states are put on the smallest such N^3 grid
-// that the column transform (fft.cuh) knows, whatever grid the caller set.
+// index of the spheres, over both signs and every k), so the states are put on
+// the smallest such N^3 grid that the column transform (fft.cuh) knows, whatever
+// grid the caller set.  The bound is sufficient, not necessary: spheres and response
+// sets that lie off-centre can be alias free with a few points less.
 // For the 48^3 grid of the precision workload that is 24^3: an eighth of the
 // points.  The result is the same sum; only its rounding differs.
 //

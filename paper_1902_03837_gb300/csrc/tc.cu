@@ -213,9 +213,9 @@ __device__ __forceinline__ void nsum(float& s, float& c, float x) {
 // epilogue warps drain them, two per TMEM lane quadrant, each holding the
 // compensated sums of 128 of the 256 columns.  Warps 0..3 (producer, MMA issuer, two idle) give registers to the
 // epilogue warpgroups: 384 threads launched at 144 registers (55,296), then
-// 4 x 32 x 40 + 8 x 32 x 192 = 54,272 after the hand-over, which leaves a
-// 128-thread, 64-register Dyson block room beside it (10,240 registers,
-// 2,816 per sub-partition).
+// 4 x 32 x 40 + 8 x 32 x 192 = 54,272 after the hand-over, which leaves 10,240
+// beside it (2,816 per sub-partition): two blocks of the Dyson update, 128 threads
+// of 40 registers each.
 // Tiles: (I, J) with I in [2J, nI), nI = mpad / 128 row tiles of A and nJ =
 // ceil(mpad / 256) column tiles of B: every real entry (r, c) with r >= c lies
 // in one of them.  Where mpad is an odd multiple of 128, the second box of the
