@@ -79,6 +79,12 @@ struct RhoTask {
   int64_t block0;  // first global block of this task in a batched launch
 };
 
+// Limit of the dynamic shared memory of a kernel that has `own` bytes of static
+// shared memory: all that a block can have, whatever a launch needs, because
+// the limit belongs to the kernel and threads that launch it with different
+// sizes would lower it for each other between setting it and launching.
+constexpr int smem_limit(size_t own = 0) { return (int)((227 << 10) - (own + 15) / 16 * 16); }
+
 // ---- launchers (stream-ordered; return cudaGetLastError()) ----
 
 // Smallest grid the column transforms take that has at least `need` points

@@ -702,7 +702,7 @@ cudaError_t launch_wf_to_mixed(const RhoGeom& g, const int32_t* gvec, const int3
   const size_t smem = ((size_t)g.NZ * g.NX * g.NY + (size_t)g.NX * g.N2) * sizeof(T2);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(k_wf_to_mixed<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+                                       smem_limit());
   if (e != cudaSuccess) return e;
   k_wf_to_mixed<T><<<nkr * nbo, 256, smem, s>>>(g, gvec, npw, coef, tw1, tw2, U, k0, b0, nbo);
   return cudaGetLastError();
@@ -711,7 +711,7 @@ cudaError_t launch_wf_to_mixed(const RhoGeom& g, const int32_t* gvec, const int3
 template <typename T, int JM, typename TOUT>
 static cudaError_t launch_rho_jm(const RhoTask<T, TOUT>& tk, size_t smem, int64_t nblocks, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(k_rho_pairs<T, JM, TOUT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit());
   if (e != cudaSuccess) return e;
   if (nblocks > 0x7fffffff) return cudaErrorInvalidValue;
   k_rho_pairs<T, JM, TOUT><<<(unsigned)nblocks, kRhoThreads, smem, s>>>(tk);
@@ -887,17 +887,20 @@ cudaError_t launch_rho_batch(const RhoTask<T, TOUT>* tasks_dev, int ntasks, int6
   cudaError_t e = cudaSuccess;
   switch (jm) {
     case 4:
-      e = cudaFuncSetAttribute(k_rho_batch<T, 4, TOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = cudaFuncSetAttribute(k_rho_batch<T, 4, TOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               smem_limit(sizeof(RhoTask<T, TOUT>) + 8));
       if (e != cudaSuccess) return e;
       k_rho_batch<T, 4, TOUT><<<grid, kRhoThreads, smem, s>>>(tasks_dev, ntasks, total, counter);
       break;
     case 2:
-      e = cudaFuncSetAttribute(k_rho_batch<T, 2, TOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = cudaFuncSetAttribute(k_rho_batch<T, 2, TOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               smem_limit(sizeof(RhoTask<T, TOUT>) + 8));
       if (e != cudaSuccess) return e;
       k_rho_batch<T, 2, TOUT><<<grid, kRhoThreads, smem, s>>>(tasks_dev, ntasks, total, counter);
       break;
     default:
-      e = cudaFuncSetAttribute(k_rho_batch<T, 1, TOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = cudaFuncSetAttribute(k_rho_batch<T, 1, TOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               smem_limit(sizeof(RhoTask<T, TOUT>) + 8));
       if (e != cudaSuccess) return e;
       k_rho_batch<T, 1, TOUT><<<grid, kRhoThreads, smem, s>>>(tasks_dev, ntasks, total, counter);
   }

@@ -315,7 +315,7 @@ cudaError_t wf_launch(const RhoGeom& g, const int32_t* gvec, const int32_t* npw,
   const size_t smem = box + xc * per;
   if (smem > (227 << 10)) return cudaErrorInvalidValue;
   cudaError_t e =
-      cudaFuncSetAttribute(k_wf_fft<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_wf_fft<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit());
   if (e != cudaSuccess) return e;
   k_wf_fft<T, N><<<nkr * nbo, kMaxThreads, smem, s>>>(g, gvec, npw, coef, U, k0, b0, nbo, xc);
   return cudaGetLastError();
@@ -325,7 +325,7 @@ template <typename T, int N>
 cudaError_t rho_launch(const RhoTask<T, typename C2<T>::t>& tk, size_t smem, int threads, int64_t nblocks,
                        cudaStream_t s) {
   cudaError_t e =
-      cudaFuncSetAttribute(k_rho_fft<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_rho_fft<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit());
   if (e != cudaSuccess) return e;
   k_rho_fft<T, N><<<(unsigned)nblocks, threads, smem, s>>>(tk);
   return cudaGetLastError();
@@ -334,8 +334,8 @@ cudaError_t rho_launch(const RhoTask<T, typename C2<T>::t>& tk, size_t smem, int
 template <typename T, int N>
 cudaError_t batch_launch(const RhoTask<T, typename C2<T>::t>* tasks, int ntasks, int64_t total, size_t smem,
                          unsigned long long* counter, int grid, cudaStream_t s) {
-  cudaError_t e =
-      cudaFuncSetAttribute(k_rho_fft_batch<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_rho_fft_batch<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem_limit(sizeof(RhoTask<T, typename C2<T>::t>) + 8));
   if (e != cudaSuccess) return e;
   k_rho_fft_batch<T, N><<<(unsigned)(total < grid ? total : grid), kMaxThreads, smem, s>>>(tasks, ntasks, total, counter);
   return cudaGetLastError();
