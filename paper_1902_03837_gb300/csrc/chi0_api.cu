@@ -1376,9 +1376,9 @@ chi0_status launch_eps(chi0_ctx* c) {
     double2* out = c->plan_eps_out + (size_t)i0 * n2;
     cudaError_t e = general
         ? chi0::launch_dyson_general(chi, (const double*)c->d_vsqrt.p, ng, i1 - i0, out, (double2*)c->d_colp.p,
-                                     (double2*)c->d_rowp.p, (double2*)c->d_pinv.p, (int*)c->d_err.p, c->st)
+                                     (double2*)c->d_rowp.p, (double2*)c->d_pinv.p, (int*)c->d_err.p, c->st, c->capturing)
         : chi0::launch_dyson(chi, (const double*)c->d_vsqrt.p, ng, i1 - i0, out, (double2*)c->d_colp.p,
-                             (double2*)c->d_rowp.p, (double2*)c->d_pinv.p, (int*)c->d_err.p, c->st);
+                             (double2*)c->d_rowp.p, (double2*)c->d_pinv.p, (int*)c->d_err.p, c->st, c->capturing);
     if (e != cudaSuccess) return cuda_fail(c, e, "dyson launch");
     nlaunch += chi0::dyson_launches(ng);
     i0 = i1;
@@ -1430,6 +1430,9 @@ chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
   // as long as the contraction 49.1 / 50.5 ms (N_G = 1000, ten frequencies), 1.8 times
   // 16.2 / 16.5 and 37.0 / 37.3 ms (600, 800), 0.6 to 0.75 times 12.45 / 12.46, 23.8 /
   // 24.1 and 49.9 / 49.9 ms (431, 600, 800): near the line it matters little.
+  // Matrices whose update alone exceeds the chain make up two groups at least, so
+  // that one group's panels and last blocks lie beside the other's updates (six of
+  // N_G = 3000 578 -> 563 ms, four real frequencies of N_G = 2000 229 -> 221).
   // A group holds frequencies of one kind (imaginary axis: Hermitian eps~; real
   // axis: general eps~, whose chi0 is first combined from its two contractions
   // H_r + i H_i).  Consecutive groups alternate between two Dyson streams, each
@@ -1437,17 +1440,17 @@ chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
   // so that the chain of one group (panels, and the next pivot inverted by one
   // block per matrix within each update) overlaps the updates of the other.
   int grp = 0;
-  const double nt16 = (ng + 15) / 16;
-  const double step_s = 54.0 * (c->has_real ? nt16 * nt16 : 0.5 * nt16 * (nt16 + 1.0)) / 1.93e9;   // of one matrix
-  const int q = std::max(1, (int)std::min(30e-6 / step_s, 1e6)), size = std::max(4, q);
-  const bool dyson_bound = nt16 * step_s / 0.85 > c->tc_issued_flops / nw / 1.2e15;
+  const double step_s = chi0::dyson_update_seconds(ng, c->has_real);
+  const int q = std::max(1, (int)std::min(chi0::kDysonChain / step_s, 1e6)), size = std::max(4, q);
+  const bool dyson_bound = (ng + 15) / 16 * step_s / 0.85 > c->tc_issued_flops / nw / 1.2e15;
   auto general = [&](int iw) { return c->has_real && c->h_vi[iw] >= 0; };
   auto first_v = [&](int iw) { return c->has_real ? c->h_vr[iw] : iw; };   // list entries of frequency iw
   auto last_v = [&](int iw) { return general(iw) ? c->h_vi[iw] : first_v(iw); };
   for (int w0 = 0; w0 < nw && s == CHI0_OK;) {
     const int r = nw - w0;
     int gw;
-    if (dyson_bound) gw = r <= size + size / 2 ? r : size;
+    if (dyson_bound && w0 == 0 && step_s >= chi0::kDysonChain && r > 1 && r <= size + size / 2) gw = (r + 1) / 2;
+    else if (dyson_bound) gw = r <= size + size / 2 ? r : size;
     else if (r > size) gw = std::min(size, r - size);
     else gw = r <= q ? r : std::max(q, r / 2);
     for (int g = 1; g < gw; ++g)
@@ -1477,9 +1480,9 @@ chi0_status launch_chi0_eps(chi0_ctx* c, void* host_out, bool* copied) {
     double2* rowp = (double2*)c->d_rowp.p + (size_t)w0 * ng * 16;
     double2* pinv = (double2*)c->d_pinv.p + (size_t)w0 * 512;
     e = general(w0) ? chi0::launch_dyson_general(chi, (const double*)c->d_vsqrt.p, ng, gw, out, colp, rowp, pinv,
-                                                 (int*)c->d_err.p, c->st)
+                                                 (int*)c->d_err.p, c->st, true)
                     : chi0::launch_dyson(chi, (const double*)c->d_vsqrt.p, ng, gw, out, colp, rowp, pinv,
-                                         (int*)c->d_err.p, c->st);
+                                         (int*)c->d_err.p, c->st, true);
     if (e != cudaSuccess) s = cuda_fail(c, e, "dyson launch");
     chi0::stage_end(c, CHI0_STAGE_DYSON, chi0::dyson_launches(ng));
     // a host output receives each group as soon as it is inverted, so that

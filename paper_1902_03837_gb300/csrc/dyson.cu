@@ -222,10 +222,11 @@ k_gj_panels(Mats m, int b0, int nb, const double2* __restrict__ pinv, double2* _
 // (two entries of a row per lane), so that an SM's four FP64 units share every
 // tile and the last one costs a quarter of what a tile per warp does.  The
 // panels come straight from L1/L2: three loads of 16 bytes for eight
-// multiply-adds, which take a warp's unit 512 clocks.  At most 40 registers: two
-// blocks (one waits for its loads while the other computes) then fit beside a
-// tensor-core contraction block, and the Dyson step of one frequency uses the
-// FP64 units while the contraction of the next occupies the tensor cores.
+// multiply-adds, which take a warp's unit 512 clocks.  At most 40 registers:
+// twelve blocks per SM hide the loads of a large matrix (96% of the FP64 rate at
+// N_G = 3000, 88% with two), and two fit beside a tensor-core contraction block,
+// so that the Dyson step of one frequency uses the FP64 units while the
+// contraction of the next occupies the tensor cores.
 template <bool full>
 __global__ void __launch_bounds__(kThreads, 12)
 k_gj_update(Mats m, int nw, int b0, int nb, double2* __restrict__ pinv, const double2* __restrict__ colp,
@@ -314,12 +315,33 @@ k_gj_update(Mats m, int nw, int b0, int nb, double2* __restrict__ pinv, const do
   }
 }
 
-// Blocks of the update: two per SM, fewer when there are fewer tiles.
-constexpr int kUpdateBlocks = 2 * 152;
+}  // namespace
+
+// 54 clocks of an SM's FP64 units per 16 x 16 tile
+double dyson_update_seconds(int ng, bool general) {
+  const double nt = (ng + kNB - 1) / kNB;
+  return 54.0 * (general ? nt * nt : 0.5 * nt * (nt + 1.0)) / 1.93e9;
+}
+
+namespace {
 
 template <bool full>
-cudaError_t launch_gj(const Mats& m, int nw, double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s) {
+cudaError_t launch_gj(const Mats& m, int nw, double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s,
+                      bool beside) {
   const int ng = m.ng, nt = (ng + kNB - 1) / kNB;
+  // Blocks of the update, fewer when there are fewer tiles.  As many per SM as its
+  // registers allow hide the loads best, but the next pivot shares its SM's FP64
+  // units with them and has to end before they do.  Alone that is so from five times
+  // the chain on (four matrices of N_G = 3000 420 -> 382 ms against two per SM, three
+  // of 1000 12.2 -> 11.7; two of 900 6.32 ms with two, 6.57 with twelve, three of 431
+  // 1.40 and 1.54).  Beside a contraction, where two groups share the SMs, from one
+  // matrix as long as the chain on (two of N_G = 750 4.15 -> 3.80 ms, the precision
+  // workload on 6x6x6 k 291 -> 282, six of N_G = 3000 664 -> 583); below, a contraction
+  // cannot start while blocks of the higher-priority Dyson step wait (nine metals of
+  // N_G = 178 to 330 in a batch 15.4 ms with two, 16.6 with twelve).
+  const double work = dyson_update_seconds(ng, full);
+  const bool longer = beside ? work >= kDysonChain : work * nw >= 5.0 * kDysonChain;
+  const int most = (longer ? 12 : 2) * 152;
   k_gj_first<full><<<nw, kThreads, 0, s>>>(m, ng < kNB ? ng : kNB, pinv, err);
   if (nt > 1)
     for (int b0 = 0; b0 < ng; b0 += kNB) {
@@ -327,7 +349,7 @@ cudaError_t launch_gj(const Mats& m, int nw, double2* colp, double2* rowp, doubl
       const bool last = b0 + kNB >= ng;
       k_gj_panels<full><<<dim3((ng + kPE - 1) / kPE, nw), kThreads, 0, s>>>(m, b0, nb, pinv, colp, rowp);
       const int64_t tiles = (int64_t)(full ? nt * nt : nt * (nt + 1) / 2) * nw;
-      const int spare = last ? kUpdateBlocks : nw < kUpdateBlocks / 2 ? kUpdateBlocks - nw : kUpdateBlocks / 2;
+      const int spare = last ? most : nw < most / 2 ? most - nw : most / 2;
       const int workers = (int)(tiles < spare ? tiles : spare);
       k_gj_update<full><<<workers + (last ? 0 : nw), kThreads, 0, s>>>(m, nw, b0, nb, pinv, colp, rowp, err);
     }
@@ -354,8 +376,8 @@ cudaError_t dyson_prepare() {
 }
 
 cudaError_t launch_dyson(const double2* chi, const double* vsqrt, int ng, int nw, double2* A,
-                         double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s) {
-  return launch_gj<false>(Mats{chi, vsqrt, A, ng}, nw, colp, rowp, pinv, err, s);
+                         double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s, bool beside) {
+  return launch_gj<false>(Mats{chi, vsqrt, A, ng}, nw, colp, rowp, pinv, err, s, beside);
 }
 
 // General (non-Hermitian) eps~ of real-axis frequencies: the same blocked
@@ -365,8 +387,8 @@ cudaError_t launch_dyson(const double2* chi, const double* vsqrt, int ng, int nw
 // (anti-Hermitian) part, which every Schur complement inherits; a pivot that
 // vanishes all the same is reported through the error flag.
 cudaError_t launch_dyson_general(const double2* chi, const double* vsqrt, int ng, int nw, double2* A,
-                                 double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s) {
-  return launch_gj<true>(Mats{chi, vsqrt, A, ng}, nw, colp, rowp, pinv, err, s);
+                                 double2* colp, double2* rowp, double2* pinv, int* err, cudaStream_t s, bool beside) {
+  return launch_gj<true>(Mats{chi, vsqrt, A, ng}, nw, colp, rowp, pinv, err, s, beside);
 }
 
 }  // namespace chi0

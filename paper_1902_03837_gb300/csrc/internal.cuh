@@ -209,13 +209,18 @@ cudaError_t launch_chi0_reduce(const double2* part, int nchunks, int ng, int nw,
 
 // a5: eps~ = 1 - V chi V, then blocked Gauss-Jordan inverse in A (which may be
 // chi).  Scratch per matrix: ng * 16 entries in each panel, 512 in pinv.
+// beside: while a contraction, or other problems of a batch, run as well.
 cudaError_t launch_dyson(const double2* chi, const double* vsqrt, int ng, int nw, double2* A,
                          double2* colpanel, double2* rowpanel, double2* pinv, int* err_flag,
-                         cudaStream_t s);
+                         cudaStream_t s, bool beside = false);
 // The same for general eps~ (real-axis frequencies): every tile, no symmetry.
 cudaError_t launch_dyson_general(const double2* chi, const double* vsqrt, int ng, int nw, double2* A,
                                  double2* colpanel, double2* rowpanel, double2* pinv, int* err_flag,
-                                 cudaStream_t s);
+                                 cudaStream_t s, bool beside = false);
+// Time of one matrix's update with a pivot block on the whole GPU (s), and that of
+// the step of a chain of pivot blocks, whatever the size.
+double dyson_update_seconds(int ng, bool general);
+constexpr double kDysonChain = 30e-6;
 // Kernel launches of either.
 int dyson_launches(int ng);
 // The Dyson kernels prefer the whole shared-memory carveout, the setting of
