@@ -245,7 +245,7 @@ enum {
 
 /* Device time of every stage summed over the launches since the previous
  * chi0_get_stats (ms, CUDA events on the context's stream; beyond 512
- * stages one call in every 16 is timed and stands for 16), the algorithmic
+ * stages one call in every 16 is timed, and the others count as their mean), the algorithmic
  * bytes and flops of the most recent instance of each stage, and the number
  * of kernels this context has launched since chi0_create.  Any pointer may
  * be NULL; arrays have CHI0_NSTAGES entries.  Synchronises. */

@@ -68,23 +68,24 @@ chi0_status ensure(chi0_ctx* c, DevBuf& b, size_t bytes, const char* what) {
 
 namespace chi0 {
 // The calls whose stages are timed: those before kTimedAll instances, then one in
-// every kTimedStep, which stands for its neighbours.  Whole calls, because the
-// instances of a stage within one do not take the same time (the transitions' rho
-// and the densities of the extrapolar term, the groups of the Dyson step): every
-// 16th instance would be the same one of them in each call.  At a place of its
-// window that a hash gives (the finaliser of Murmur 3), because a loop over q
-// points would make every 16th call one of the same q point.
+// every kTimedStep; the readout takes the mean of the latter for those in between.
+// Whole calls, because the instances of a stage within one do not take the same
+// time (the transitions' rho and the densities of the extrapolar term, the groups
+// of the Dyson step): every 16th instance would be the same one of them in each
+// call.  At a place of its window that a hash gives (the finaliser of Murmur 3),
+// because a loop over q points would make every 16th call one of the same q point.
 constexpr int64_t kTimedAll = 512, kTimedStep = 16;
-static int call_weight(int64_t instances, int64_t call) {
-  if (instances < kTimedAll) return 1;
+static bool sampled_call(int64_t call) {
   uint32_t h = (uint32_t)(call / kTimedStep);
   h = (h ^ h >> 16) * 0x85ebca6bu;
   h = (h ^ h >> 13) * 0xc2b2ae35u;
-  return call % kTimedStep == (h ^ h >> 16) % kTimedStep ? (int)kTimedStep : 0;
+  return call % kTimedStep == (h ^ h >> 16) % kTimedStep;
 }
 void begin_call(chi0_ctx* c, int entry) {
   auto& e = c->calls[c->entry = entry];
-  c->timed_weight = call_weight(e.instances, e.calls++);
+  const int64_t call = e.calls++;
+  c->phase = e.instances < kTimedAll ? chi0_ctx::kFull : sampled_call(call) ? chi0_ctx::kSampled : chi0_ctx::kUntimed;
+  if (c->phase != chi0_ctx::kUntimed) ++e.timed[c->phase];
 }
 constexpr size_t kFoldAt = 1024;   // events
 
@@ -92,17 +93,28 @@ constexpr size_t kFoldAt = 1024;   // events
 static void stage_fold(chi0_ctx::Stage& st) {
   for (size_t p = 0; p + 1 < st.used; p += 2) {
     float t = 0.f;
-    if (cudaEventElapsedTime(&t, st.ev[p], st.ev[p + 1]) == cudaSuccess) st.acc += (double)t * st.weight[p / 2];
+    const auto& tag = st.tag[p / 2];
+    if (cudaEventElapsedTime(&t, st.ev[p], st.ev[p + 1]) == cudaSuccess) st.acc[tag.first][tag.second] += (double)t;
     cudaGetLastError();
   }
   st.used = 0;
+}
+
+// time of a stage over all calls of an entry point
+static double stage_ms(const chi0_ctx* c, const chi0_ctx::Stage& st, int entry) {
+  const auto& e = c->calls[entry];
+  const double* a = st.acc[entry];
+  const double rest = (double)(e.calls - e.timed[chi0_ctx::kFull]);
+  if (rest <= 0.0) return a[chi0_ctx::kFull];
+  const int from = e.timed[chi0_ctx::kSampled] > 0 ? chi0_ctx::kSampled : chi0_ctx::kFull;
+  return a[chi0_ctx::kFull] + (e.timed[from] > 0 ? a[from] / (double)e.timed[from] * rest : 0.0);
 }
 
 void stage_begin(chi0_ctx* c, int stage) {
   if (c->capturing) return;
   auto& st = c->stage[stage];
   ++c->calls[c->entry].instances;
-  st.timed = c->timed_weight > 0;
+  st.timed = c->phase != chi0_ctx::kUntimed;
   if (!st.timed) return;
   if (st.used >= kFoldAt) {
     // the last pairs of every stream in use must have finished (and nothing is
@@ -128,9 +140,9 @@ void stage_begin(chi0_ctx* c, int stage) {
     }
     st.ev.push_back(a);
     st.ev.push_back(b);
-    st.weight.push_back(1);
+    st.tag.emplace_back();
   }
-  st.weight[st.used / 2] = c->timed_weight;
+  st.tag[st.used / 2] = {c->entry, c->phase};
   cudaEventRecord(st.ev[st.used], c->st);
 }
 void stage_end(chi0_ctx* c, int stage, int kernels) {
@@ -2128,14 +2140,17 @@ chi0_status chi0_get_stats(chi0_ctx* c, double* ms, double* bytes, double* flops
   for (int k = 0; k < CHI0_NSTAGES; ++k) {
     auto& st = c->stage[k];
     chi0::stage_fold(st);
-    st.ms = st.acc;
-    st.acc = 0.0;
+    st.ms = 0.0;
+    for (int e = 0; e < chi0_ctx::kEntries; ++e) {
+      st.ms += chi0::stage_ms(c, st, e);
+      st.acc[e][0] = st.acc[e][1] = 0.0;
+    }
     if (ms) ms[k] = st.ms;
     if (bytes) bytes[k] = st.bytes;
     if (flops) flops[k] = st.flops;
   }
   for (auto& e : c->calls) e = {};
-  c->timed_weight = 1;
+  c->phase = chi0_ctx::kFull;
   if (launches) *launches = c->launches;
   return CHI0_OK;
 }

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/chi0.h"
@@ -146,23 +147,23 @@ struct chi0_ctx {
   // kept until the next readout pile up in a program that never reads them, so
   // after kTimedAll instances one call in every kTimedStep stands for its
   // neighbours, and finished pairs are folded into ms and used again.
+  enum { kRhoCall, kChiCall, kEpsCall, kChiEpsCall, kSigmaCall, kEntries };
+  enum { kFull, kSampled, kUntimed };   // calls that are all timed, then one of many, and the others
   struct Stage {
     std::vector<cudaEvent_t> ev;  // start, stop, start, stop, ...
-    std::vector<int> weight;      // calls that each pair stands for
+    std::vector<std::pair<int, int>> tag;   // entry point and phase of each pair
     size_t used = 0;              // events recorded since the last fold
     bool timed = false;           // the open instance has a pair
-    double acc = 0;               // folded time since the last readout (ms)
+    double acc[kEntries][2] = {};   // folded time since the last readout (ms)
     double ms = 0, bytes = 0, flops = 0;
     int64_t launches = 0;
   };
   Stage stage[CHI0_NSTAGES];
   // calls of each entry point, and stages run by them, since the last readout
-  enum { kRhoCall, kChiCall, kEpsCall, kChiEpsCall, kSigmaCall, kEntries };
   struct {
-    int64_t calls = 0, instances = 0;
+    int64_t calls = 0, timed[2] = {}, instances = 0;
   } calls[kEntries];
-  int entry = kRhoCall;           // of the call that is running
-  int timed_weight = 1;           // calls that it stands for; 0: not timed
+  int entry = kRhoCall, phase = kFull;   // of the call that is running
   int64_t launches = 0;           // kernels launched since chi0_create
   double tc_issued_flops = 0;     // tensor-core flops issued by the last mixed contraction
 
